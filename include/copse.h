@@ -456,6 +456,14 @@ copse_status copse_tune_fused(copse_ctx *ctx, copse_model *model, const uint32_t
                               size_t n_queries, int reps, float *ms, uint32_t *best);
 /* Set the fused crossover copse_tune_fused would choose (default: always fused). */
 copse_status copse_ctx_set_ntt_fused_max(copse_ctx *ctx, uint32_t max_fused);
+/* Which kernel multiplies an encrypted model's diagonals with the rotations (the products of
+ * Section 4.3 with the diagonals encrypted, Section 8.3): COPSE_ENC_MAC_AUTO (the default)
+ * takes the one expected to be faster for each matrix size and number of query ciphertexts,
+ * the others fix one.  Results are the same residues.  EINVAL for another value. */
+#define COPSE_ENC_MAC_AUTO 0
+#define COPSE_ENC_MAC_TENSOR 1
+#define COPSE_ENC_MAC_INTEGER 2
+copse_status copse_ctx_set_enc_mac(copse_ctx *ctx, int kernel);
 
 /* Baby-step sizes (copse_model_set_bsgs): the reshuffle candidates g_r[] are
  * timed by the reshuffle stage with the level plan held, then the level

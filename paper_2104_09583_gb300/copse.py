@@ -66,6 +66,7 @@ _SIG = {
     "copse_model_set_bsgs": (C.c_int, [vp, C.c_uint32, C.c_uint32]),
     "copse_ctx_set_ntt_cluster_max": (C.c_int, [vp, C.c_uint32]),
     "copse_ctx_set_ntt_fused_max": (C.c_int, [vp, C.c_uint32]),
+    "copse_ctx_set_enc_mac": (C.c_int, [vp, C.c_int]),
     "copse_tune_fused": (C.c_int, [vp, vp, u32p, C.c_size_t, C.c_size_t, C.c_int, C.POINTER(C.c_float),
                                    C.POINTER(C.c_uint32)]),
     "copse_model_set_encrypted": (C.c_int, [vp, C.c_int]),
@@ -279,6 +280,14 @@ def copse_ctx_set_ntt_cluster_max(ctx, max_cluster):
 
 def copse_ctx_set_ntt_fused_max(ctx, max_fused):
     _check(_lib.copse_ctx_set_ntt_fused_max(ctx, max_fused))
+
+
+ENC_MAC = {"auto": 0, "tensor": 1, "integer": 2}
+
+
+def copse_ctx_set_enc_mac(ctx, kernel):
+    """kernel: "auto", "tensor" or "integer" (see include/copse.h)."""
+    _check(_lib.copse_ctx_set_enc_mac(ctx, ENC_MAC[kernel]))
 
 
 def copse_tune_fused(ctx, model, cands=(64, 128, 256, 512, 1 << 30), n_queries=1, reps=3):

@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_enc_mac_tc(const TcArgs P) {
         const int nj16 = R.nk * TC_KS, r = (int)(I.e >> P.logN);
         const uint32_t a_mn = (uint32_t)nj16 * 16, pos = (uint32_t)(I.e & nmask);
         const PrimeDev pd = P.pr[r];
+        const u64 mst = mask_state(P.seed, r, pos, P.logN);
         uint8_t *A1 = A0 + TC_MX * a_mn;
         ulonglong2 cw[AB_PAIRS];
 #pragma unroll
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_enc_mac_tc(const TcArgs P) {
                 u64 d0 = 0, d1 = 0;
                 if (id != ~0u) {
                     d0 = h ? cw[k].y : cw[k].x;
-                    d1 = seeded_mask(P.seed, MODEL_STREAM + 2ull * id, r, pos, P.logN, pd);
+                    d1 = mask_at(mst, id, pd);
                 }
                 const uint32_t off = (uint32_t)x * a_mn + (uint32_t)((j + h) >> 3) * 128 + (uint32_t)((j + h) & 7) * 16;
                 *(uint4 *)(A0 + off) = digits8(d0, pd.q);
@@ -621,8 +622,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_enc_mac_tc(const TcArgs P) {
 }
 
 // rot [nb][2][n_el] of query ciphertext b -> R [n_el][nc][nq][64][2] (baby step j in chunk
-// j / 64 at j % 64), each residue v stored centred and biased, v' + 0x0080808080808080: 32 elements x 32 rows (j, c) per block through shared memory, reads
-// coalesced along the elements, writes along the rows
+// j / 64 at j % 64): 32 elements x 32 rows (j, c) per block through shared memory, reads
+// coalesced along the elements, writes along the rows.  Each residue v is stored centred and
+// biased, v' + 0x0080808080808080, for the tensor cores' digits, or (SPLIT) as its low 28 bits
+// and the rest in the two halves of the word, for the integer kernel's products.
+template <bool SPLIT>
 __global__ void k_rot_to_elements(const u64 *__restrict__ rot, u64 *__restrict__ R, int nb, int nq, int b,
                                   size_t n_el, int logN, const PrimeDev *__restrict__ pr) {
     __shared__ u64 t[32][33];
@@ -641,7 +645,7 @@ __global__ void k_rot_to_elements(const u64 *__restrict__ rot, u64 *__restrict__
             const int j = row >> 1;
             const u64 q = pr[e >> logN].q, v = t[threadIdx.x][i];
             R[((e * nc + j / TC_CJ) * nq + b) * (TC_CJ * 2) + (j % TC_CJ) * 2 + (row & 1)] =
-                (v > (q >> 1) ? v - q : v) + DIGIT_BIAS;
+                SPLIT ? ((v >> 28) << 32) | (v & 0x0FFFFFFFu) : (v > (q >> 1) ? v - q : v) + DIGIT_BIAS;
         }
     }
 }
@@ -728,11 +732,13 @@ double enc_mac_tc_flops(const EncModel::MacMat &M, int nq, int logN) {
     return n_el * n_mt * nqp * (double)nb16 * 2.0 /* d0, d1 */ * 2.0 * 128 * (TC_QP * 2 * 8);
 }
 
-copse_status rot_to_elements(copse_ctx *c, const u64 *rot, int nb, int nq, int b, int ell, u64 *R, cudaStream_t s) {
+copse_status rot_to_elements(copse_ctx *c, const u64 *rot, int nb, int nq, int b, int ell, u64 *R, bool split,
+                             cudaStream_t s) {
     const size_t n_el = (size_t)ell << c->logN;
     const dim3 grid((unsigned)((n_el + 31) / 32), (unsigned)((2 * nb + 31) / 32));
     TIMED("rot_layout", 16.0 * (double)n_el * 2.0 * nb, s,
-          k_rot_to_elements<<<grid, dim3(32, 8), 0, s>>>(rot, R, nb, nq, b, n_el, c->logN, c->d_prime));
+          (split ? k_rot_to_elements<true> : k_rot_to_elements<false>)<<<grid, dim3(32, 8), 0, s>>>(
+              rot, R, nb, nq, b, n_el, c->logN, c->d_prime));
     LAUNCH_CHECK();
     return COPSE_OK;
 }

@@ -307,6 +307,8 @@ copse_status enc_matmul(copse_ctx *c, const copse_evk *evk, const EncModel &E, c
         Scratch sc(s);
         // baby steps: rotations of every query ciphertext of the group (one ModUp each), moved
         // into the element-major layout [ell N][nb / 64][ng][64][2] of the multiply-accumulate
+        const bool on_int = c->enc_mac == COPSE_ENC_MAC_INTEGER ||
+                            (c->enc_mac == COPSE_ENC_MAC_AUTO && enc_mac_use_int(E.mac[kind], ng));
         u64 *Rb = nullptr, *rot = nullptr;
         if ((st = sc.get(c, &Rb, (size_t)ng * nb64 * per))) break;
         {
@@ -314,7 +316,7 @@ copse_status enc_matmul(copse_ctx *c, const copse_evk *evk, const EncModel &E, c
             if ((st = sr.get(c, &rot, (size_t)nb * per))) break;
             for (int q = 0; q < ng && st == COPSE_OK; q++) {
                 st = op_rotations(c, evk, v[g0 + q], G.baby, rot, s);
-                if (st == COPSE_OK) st = rot_to_elements(c, rot, nb, ng, q, ell, Rb, s);
+                if (st == COPSE_OK) st = rot_to_elements(c, rot, nb, ng, q, ell, Rb, on_int, s);
             }
         }
         // matrix by matrix: products, relinearisation, giant steps (+ mask)
@@ -340,8 +342,12 @@ copse_status enc_matmul(copse_ctx *c, const copse_evk *evk, const EncModel &E, c
                 for (int y = 0; y < nm; y++)
                     for (int j = 0; j < nb; j++) present += G.acc[x0 + y].diag[j] >= 0;
                 const double bytes = 8.0 * (double)n_el * ((double)present + 2.0 * nb * ng + 3.0 * nm * ng);
-                TIMED_OPS("enc_mac", bytes, enc_mac_tc_flops(M, ng, c->logN), s,
-                          st = enc_mac_tc(c, M, Rb, ng, acc3, (size_t)nm * per3, E.seed, s));
+                if (on_int)
+                    TIMED_OPS("enc_mac_int", bytes, 4.0 * (double)n_el * (double)present * ng, s,
+                              st = enc_mac_int(c, M, Rb, ng, acc3, (size_t)nm * per3, E.seed, s));
+                else
+                    TIMED_OPS("enc_mac", bytes, enc_mac_tc_flops(M, ng, c->logN), s,
+                              st = enc_mac_tc(c, M, Rb, ng, acc3, (size_t)nm * per3, E.seed, s));
                 if (st) break;
             }
             // one relinearisation per (query ciphertext, accumulator), then the giant steps

@@ -126,9 +126,24 @@ __device__ __forceinline__ void mac128(Acc128 &a, u64 x, u64 y) {
     a.lo += plo;
     a.hi += phi + (a.lo < plo);
 }
-__device__ __forceinline__ u64 reduce128(const Acc128 &a, const PrimeDev &P) {
-    return add_mod(mul_shoup(barrett_wide(0, a.hi, P), P.r64, P.r64_sh, P.q), barrett_wide(0, a.lo, P), P.q);
+// x mod q up to one q: x - floor(x floor(2^64 / q) / 2^64) q in [0, 2q) for any 64-bit x.  For a
+// prime above 2^32 floor(2^64 / q) fits 32 bits: three 32-bit products for the quotient and its
+// multiple where a full 64-bit quotient takes seven (smaller primes, which short prime sizes at
+// large rings reach, take that).
+__device__ __forceinline__ u64 reduce64_lazy(u64 x, const PrimeDev &P) {
+    if (P.one_sh >> 32) return mul_shoup_lazy(x, 1, P.one_sh, P.q);
+    const uint32_t c = (uint32_t)P.one_sh;
+    const uint32_t h = (uint32_t)(((x >> 32) * c + __umulhi((uint32_t)x, c)) >> 32);
+    return x - (u64)h * P.q;
 }
+// (hi 2^64 + lo) mod q in [0, q) for any two words: hi (2^64 mod q) by its Shoup quotient and lo
+// each below 2q, one correction of their sum
+__device__ __forceinline__ u64 reduce_words(u64 hi, u64 lo, const PrimeDev &P) {
+    u64 s = mul_shoup_lazy(hi, P.r64, P.r64_sh, P.q) + reduce64_lazy(lo, P);
+    if (s >= 2 * P.q) s -= 2 * P.q;
+    return s >= P.q ? s - P.q : s;
+}
+__device__ __forceinline__ u64 reduce128(const Acc128 &a, const PrimeDev &P) { return reduce_words(a.hi, a.lo, P); }
 // Exact sums of products of operands below 2^56 (residues of primes below 2^55 and
 // sums of two of them) from 32 x 32 -> 64-bit multiply-adds: x = x1 2^28 + x0 with
 // x0, x1 < 2^28, so x y = x1 y1 2^56 + (x1 y0 + x0 y1) 2^28 + x0 y0 and every partial
@@ -181,11 +196,14 @@ __device__ __forceinline__ uint32_t galois_src(uint32_t n, u64 g, int logN) {
 
 // SplitMix64 (Steele, Lea, Flood, OOPSLA 2014) in counter form: output number
 // (stream * 2^40 + idx + 1) of the sequence whose state starts at `seed`.
-__device__ __forceinline__ u64 rng_word(u64 seed, u64 stream, u64 idx) {
-    u64 z = seed + 0x9E3779B97F4A7C15ULL * ((stream << 40) + idx + 1ULL);
+constexpr u64 RNG_STEP = 0x9E3779B97F4A7C15ULL;
+__device__ __forceinline__ u64 rng_mix(u64 z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
+}
+__device__ __forceinline__ u64 rng_word(u64 seed, u64 stream, u64 idx) {
+    return rng_mix(seed + RNG_STEP * ((stream << 40) + idx + 1ULL));
 }
 
 // Encrypted-model ciphertexts are secret-key encryptions whose mask a is drawn from the
@@ -194,11 +212,21 @@ __device__ __forceinline__ u64 rng_word(u64 seed, u64 stream, u64 idx) {
 // (evaluation point psi_r^(2 brev(pos) + 1)) a is the uniform residue number r N + brev(pos)
 // of the stream: two 64-bit words hi, lo give (hi 2^64 + lo) mod q.
 constexpr u64 MODEL_STREAM = 0x800000ull;
+// The generator's state before model ciphertext 0's mask at one element, and the mask of model
+// ciphertext id there (id's stream lies 2 id 2^40 outputs further: RNG_STEP (id << 41) mod 2^64
+// takes one 32-bit product).  Loops over many ciphertexts at one element use the pair.
+__device__ __forceinline__ u64 mask_state(u64 seed, int r, uint32_t pos, int logN) {
+    const u64 j = bit_reverse(pos, logN);
+    return seed + RNG_STEP * ((MODEL_STREAM << 40) + 2 * (((u64)r << logN) + j) + 1ULL);
+}
+__device__ __forceinline__ u64 mask_at(u64 state, uint32_t id, const PrimeDev &P) {
+    const u64 z = state + ((u64)((uint32_t)RNG_STEP * id) << 41);
+    return reduce_words(rng_mix(z), rng_mix(z + RNG_STEP), P);
+}
 __device__ __forceinline__ u64 seeded_mask(u64 seed, u64 stream, int r, uint32_t pos, int logN, const PrimeDev &P) {
     const u64 j = bit_reverse(pos, logN);
     const u64 idx = 2 * (((u64)r << logN) + j);
-    const u64 hi = rng_word(seed, stream, idx), lo = rng_word(seed, stream, idx + 1);
-    return add_mod(mul_shoup(barrett_wide(0, hi, P), P.r64, P.r64_sh, P.q), barrett_wide(0, lo, P), P.q);
+    return reduce_words(rng_word(seed, stream, idx), rng_word(seed, stream, idx + 1), P);
 }
 
 // 16-byte asynchronous copies global -> shared (cp.async, grouped per thread)
@@ -292,6 +320,7 @@ struct copse_ctx {
     long ntt_cluster_max = 1L << 30;
     long ntt_fused_max = 1L << 30;    // the same crossover for the transforms fused with base conversions
     bool ntt_cluster16 = false;       // N = 2^15: the device places 16-CTA clusters (non-portable size)
+    int enc_mac = 0;                  // COPSE_ENC_MAC_*: the encrypted products' kernel
     // device status word: kernels whose bounded waits ran out set bits here (COPSE_DEV_*);
     // read and cleared by copse_ctx_device_status
     int *d_status = nullptr;
@@ -581,11 +610,18 @@ copse_status enc_matmul(copse_ctx *c, const copse_evk *evk, const EncModel &E, c
 // written (not added to).
 copse_status enc_mac_tc(copse_ctx *c, const EncModel::MacMat &M, const u64 *R, int nq, u64 *acc, size_t a_ct,
                         u64 seed, cudaStream_t s);
-// rotations [nb][2][ell N] of query ciphertext b into the element-major layout of enc_mac_tc
+// the same sums on the integer pipe (encmac_int.cu)
+copse_status enc_mac_int(copse_ctx *c, const EncModel::MacMat &M, const u64 *R, int nq, u64 *acc, size_t a_ct,
+                         u64 seed, cudaStream_t s);
+// whether the integer kernel is the faster one for nq query ciphertexts of these matrices
+bool enc_mac_use_int(const std::vector<EncModel::MacMat> &mats, int nq);
+// rotations [nb][2][ell N] of query ciphertext b into the element-major layout of enc_mac_tc, or
+// (split) of enc_mac_int: the same places, each word the residue's low 28 bits and the rest in its halves
 // f16 multiply-add operations (2 per digit product) the tensor cores issue for one enc_mac_tc
 // launch of nq query ciphertexts (padding rows, columns and baby steps included)
 double enc_mac_tc_flops(const EncModel::MacMat &M, int nq, int logN);
-copse_status rot_to_elements(copse_ctx *c, const u64 *rot, int nb, int nq, int b, int ell, u64 *R, cudaStream_t s);
+copse_status rot_to_elements(copse_ctx *c, const u64 *rot, int nb, int nq, int b, int ell, u64 *R, bool split,
+                             cudaStream_t s);
 // c0 of nc model ciphertexts [nc][ell N] into matrix M at positions pos[i] (device array)
 copse_status mac_scatter(copse_ctx *c, const u64 *c0, const uint32_t *pos, int nc, const EncModel::MacMat &M,
                          cudaStream_t s);

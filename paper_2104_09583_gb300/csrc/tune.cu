@@ -230,6 +230,13 @@ extern "C" copse_status copse_ctx_set_ntt_fused_max(copse_ctx *c, uint32_t max_f
     return COPSE_OK;
 }
 
+extern "C" copse_status copse_ctx_set_enc_mac(copse_ctx *c, int kernel) {
+    if (!c) { set_error("null context"); return COPSE_EINVAL; }
+    if (kernel < COPSE_ENC_MAC_AUTO || kernel > COPSE_ENC_MAC_INTEGER) { set_error("unknown multiply-accumulate kernel"); return COPSE_EINVAL; }
+    c->enc_mac = kernel;
+    return COPSE_OK;
+}
+
 extern "C" copse_status copse_tune_fused(copse_ctx *c, copse_model *m, const uint32_t *cands, size_t n,
                                          size_t n_queries, int reps, float *ms, uint32_t *best) {
     if (!c || !m || !cands || !ms || !best || n < 1 || reps < 1) {
