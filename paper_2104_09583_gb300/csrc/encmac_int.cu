@@ -43,18 +43,9 @@ struct IntMacArgs {
     const PrimeDev *pr;
 };
 
-// partial sums of split products: x0 y0, x1 y1, (x0 + x1)(y0 + y1)
-struct AccK {
-    u64 lo, hi, s;
-};
-__device__ __forceinline__ void mac_k(AccK &a, uint2 x, uint32_t xs, uint2 y, uint32_t ys) {
-    a.lo += (u64)x.x * y.x;
-    a.hi += (u64)x.y * y.y;
-    a.s += (u64)xs * ys;
-}
 using u128 = unsigned __int128;
 __device__ __forceinline__ void fold(u128 &t, AccK &a) {
-    t += (u128)a.lo + ((u128)(a.s - a.lo - a.hi) << 28) + ((u128)a.hi << 56);
+    t += acc_value(a);
     a = AccK{0, 0, 0};
 }
 __device__ __forceinline__ u128 shfl_down_u128(u128 v, int d) {

@@ -173,6 +173,25 @@ __device__ __forceinline__ Acc128 acc3w_value(const Acc3w &a) {
     v.hi += (a.hi >> 8) + (v.lo < h);
     return v;
 }
+// The same sums with three multiply-adds a product (Karatsuba): x0 y0, x1 y1 and
+// (x0 + x1)(y0 + y1), the middle term by subtraction when the sums are taken as a 128-bit value.
+// Operands below 2^55 (x0 + x1 < 1.5 2^28): 64 products at most; sums of two such operands: 16.
+struct AccK {
+    u64 lo, hi, s;
+};
+__device__ __forceinline__ void mac_k(AccK &a, uint2 x, uint32_t xs, uint2 y, uint32_t ys) {
+    a.lo += (u64)x.x * y.x;
+    a.hi += (u64)x.y * y.y;
+    a.s += (u64)xs * ys;
+}
+__device__ __forceinline__ unsigned __int128 acc_value(const AccK &a) {
+    return (unsigned __int128)a.lo + ((unsigned __int128)(a.s - a.lo - a.hi) << 28) + ((unsigned __int128)a.hi << 56);
+}
+__device__ __forceinline__ uint2 split_k(u64 x) { return make_uint2((uint32_t)x & 0x0FFFFFFFu, (uint32_t)(x >> 28)); }
+__device__ __forceinline__ u64 acc_reduce(const AccK &a, const PrimeDev &P) {
+    const unsigned __int128 v = acc_value(a);
+    return reduce_words((u64)(v >> 64), (u64)v, P);
+}
 // Montgomery reduction (P. Montgomery, Math. Comp. 1985) of a 128-bit value x < q 2^64:
 // x 2^-64 mod q in [0, q).  Key-switching keys are stored in Montgomery form k 2^64 mod q,
 // so a dot product of residues with key words summed exactly in 128 bits (mac128; nd

@@ -23,10 +23,12 @@ namespace {
 
 constexpr int TPB = 256;
 constexpr int MAX_ALPHA = 40;
-constexpr int MAX_ACC = 8;
+constexpr int MM_ACC = 32;            // accumulators per launch (their diagonals' addresses are kernel parameters)
+constexpr int MM_DEEP = 2;            // rotations a thread loads at a time
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
-constexpr int MM_PARTS = 8;  // rotation ranges with their own partial sums in k_mm_fused
+constexpr int MM_PARTS = 8;           // rotation ranges with their own partial sums at most
+constexpr int MM_BLOCKS = 1400;       // blocks that a launch is split up to (about three waves)
 constexpr int RS_CHUNK = 32; // giant-step terms per k_rotsum launch
 
 inline unsigned nblk(size_t n) { return (unsigned)((n + TPB - 1) / TPB); }
@@ -43,13 +45,6 @@ __global__ void k_add(const u64 *a, const u64 *b, u64 *out, int ncomp, int level
     int r = (int)((e >> logN) % level);
     u64 q = pr[r].q;
     out[e] = neg ? sub_mod(a[e], b[e], q) : add_mod(a[e], b[e], q);
-}
-
-// c0 += p (p: [level][N]) on component 0 only
-__global__ void k_add_plain(u64 *ct, const u64 *p, int level, int logN, const PrimeDev *pr) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ((size_t)level << logN)) return;
-    ct[e] = add_mod(ct[e], p[e], pr[e >> logN].q);
 }
 
 __global__ void k_affine(const u64 *x, const u64 *m, const u64 *addp, u64 *out, int level, int logN,
@@ -242,13 +237,13 @@ __global__ void k_moddown_conv(const u64 *u, size_t ustride, u64 *W, size_t wstr
     }
 }
 
-// Diagonal products over shared rotations with one ModDown per sum (double
-// hoisting).  For every element (r, n) of the extended basis and each rotation k
-// of the chunk:
+// Diagonal products over shared rotations with one ModDown per sum (double hoisting).  For
+// every element (r, n) of the extended basis and each rotation k of the chunk:
 //   R_k = sum_j tau_k(yhat_j) * ksk_k[j]  (+ P * tau_k(c0) on component 0 at q-primes)
-//   acc_a += pt[a][k] * R_k
-// The key-switched ciphertexts are never written: each key, each diagonal and
-// each accumulator is read once per chunk.
+//   acc_a = sum_k pt[a][k] * R_k   (added to the earlier chunks' sum unless this is the first)
+// The diagonal products are summed exactly from split 28-bit products (at most CHUNK_ROT terms)
+// and reduced once.  grid.y / the block's part splits the chunk's rotations into contiguous
+// ranges with their own partial sums at acc + part * part_stride (summed later).
 struct MmJob {
     const u64 *ksk;  // [ndig][2][L+alpha][N] NTT domain
     u64 g;           // Galois element
@@ -256,16 +251,19 @@ struct MmJob {
 };
 struct MmTable {
     MmJob job[CHUNK_ROT];
-    const u64 *pt[MAX_ACC * CHUNK_ROT];  // [acc][rotation], [ell+alpha][N], null = zero diagonal
-    u64 *acc[MAX_ACC];                   // [2][ell+alpha][N]
+    const u64 *pt[MM_ACC * CHUNK_ROT];  // [acc][rotation], [ell+alpha][N], null = zero diagonal
+    u64 *acc;                           // [acc][2][ell+alpha][N]
 };
 
-// grid.y splits the chunk's rotations into gridDim.y contiguous ranges; range y
-// accumulates into its own partial sums at acc + y * part_stride (summed later).
-template <int NA>
-__global__ void __launch_bounds__(256) k_mm_fused(const u64 *yhat, const u64 *c0, int nrot, const MmTable tab,
-                                                  size_t part_stride, int ell, int alpha, int L, int logN,
-                                                  const PrimeDev *pr, KsTables T) {
+// one accumulator: the key switch of each rotation inline, so that no R_k is written
+struct MmFusedTable {
+    MmJob job[CHUNK_ROT];
+    const u64 *pt[CHUNK_ROT];
+    u64 *acc;
+};
+__global__ void __launch_bounds__(256) k_mm_fused(const u64 *yhat, const u64 *c0, int nrot, int first,
+                                                  const __grid_constant__ MmFusedTable tab, size_t part_stride, int ell,
+                                                  int alpha, int L, int logN, const PrimeDev *pr, KsTables T) {
     const int N = 1 << logN;
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t n_el = (size_t)nx << logN;
@@ -274,102 +272,91 @@ __global__ void __launch_bounds__(256) k_mm_fused(const u64 *yhat, const u64 *c0
     const int per = (nrot + (int)gridDim.y - 1) / (int)gridDim.y;
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
-    const size_t poff = (size_t)blockIdx.y * part_stride;
+    u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride;
     const int r = (int)(e >> logN);
     const uint32_t n = (uint32_t)(e & (N - 1));
     const int g = r < ell ? r : L + (r - ell);
     const PrimeDev P = pr[g];
     const u64 Pm = r < ell ? T.md_P[r] : 0;
-    // the accumulators' diagonal products summed lazily (at most CHUNK_ROT terms per
-    // launch on a residue < q), reduced once at the end
-    u64 a0[NA], a1[NA];
-#pragma unroll
-    for (int x = 0; x < NA; x++) {
-        a0[x] = tab.acc[x][poff + e];
-        a1[x] = tab.acc[x][poff + n_el + e];
-    }
+    AccK a0{0, 0, 0}, a1{0, 0, 0};
     for (int k = k0; k < k1; k++) {
         const MmJob J = tab.job[k];
         u64 u0 = 0, u1 = 0;
-        if (J.R) {
-            u0 = J.R[e];
-            u1 = J.R[n_el + e];
-        } else {
-            const uint32_t src = galois_src(n, J.g, logN);
-            ks_dot(yhat + ((size_t)r << logN) + src, (size_t)nx << logN, J.ksk + ((size_t)g << logN) + n,
-                   (size_t)NB << logN, nd, P, u0, u1);
-            if (r < ell) u0 = add_mod(u0, mul_mod(Pm, c0[((size_t)r << logN) + src], P), P.q);
-        }
-#pragma unroll
-        for (int x = 0; x < NA; x++) {
-            const u64 *p = tab.pt[x * nrot + k];
-            if (!p) continue;
-            const u64 pv = p[e];
-            a0[x] = add_mod(a0[x], mul_mod(pv, u0, P), P.q);
-            a1[x] = add_mod(a1[x], mul_mod(pv, u1, P), P.q);
-        }
+        const uint32_t src = galois_src(n, J.g, logN);
+        const uint2 p = split_k(tab.pt[k][e]);
+        ks_dot(yhat + ((size_t)r << logN) + src, (size_t)nx << logN, J.ksk + ((size_t)g << logN) + n,
+               (size_t)NB << logN, nd, P, u0, u1);
+        if (r < ell) u0 = add_mod(u0, mul_mod(Pm, c0[((size_t)r << logN) + src], P), P.q);
+        const uint2 v0 = split_k(u0), v1 = split_k(u1);
+        mac_k(a0, p, p.x + p.y, v0, v0.x + v0.y);
+        mac_k(a1, p, p.x + p.y, v1, v1.x + v1.y);
     }
-#pragma unroll
-    for (int x = 0; x < NA; x++) {
-        tab.acc[x][poff + e] = a0[x];
-        tab.acc[x][poff + n_el + e] = a1[x];
-    }
+    const u64 s0 = acc_reduce(a0, P), s1 = acc_reduce(a1, P);
+    acc[e] = first ? s0 : add_mod(acc[e], s0, P.q);
+    acc[n_el + e] = first ? s1 : add_mod(acc[n_el + e], s1, P.q);
 }
 
-// The same accumulation with every R_k precomputed: a streaming multiply-accumulate
-// whose loads for rotation k + 1 are issued before the products of rotation k.
+// The same sums for a tile of NA accumulators per thread over precomputed R_k: two residue
+// products per diagonal word.  Reduced products made this the integer pipe's at 2.0 TB/s; exact
+// sums (six multiply-adds and no reduction per word) reach 4.0 TB/s (69 + 378 accumulators of 64
+// rotations at N = 2^15: 8.5 -> 4.2 ms), the multiplier's pipe 65-70% busy.  Blocks run over the
+// launch's accumulator tiles fastest, so that the tiles of one element range find its R_k in L2;
+// each thread has the loads of MM_DEEP rotations in flight (four at two blocks per SM: 1% slower).
 template <int NA>
-__global__ void __launch_bounds__(256) k_mm_mac(int nrot, const MmTable tab, size_t part_stride, int ell, int alpha,
-                                                int L, int logN, const PrimeDev *pr) {
-    const int nx = ell + alpha;
+__global__ void __launch_bounds__(256, 3) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
+                                                   size_t part_stride, int ell, int alpha, int L, int logN,
+                                                   const PrimeDev *pr) {
+    const int nx = ell + alpha, tiles = (nacc + NA - 1) / NA;
     const size_t n_el = (size_t)nx << logN;
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int x0 = (int)(blockIdx.x % tiles) * NA, na = min(NA, nacc - x0);
+    const size_t e = (size_t)(blockIdx.x / tiles) * blockDim.x + threadIdx.x;
     if (e >= n_el) return;
     const int per = (nrot + (int)gridDim.y - 1) / (int)gridDim.y;
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
-    const size_t poff = (size_t)blockIdx.y * part_stride;
     const int r = (int)(e >> logN);
     const PrimeDev P = pr[r < ell ? r : L + (r - ell)];
-    u64 a0[NA], a1[NA];
+    AccK a[NA][2];
 #pragma unroll
-    for (int x = 0; x < NA; x++) {
-        a0[x] = tab.acc[x][poff + e];
-        a1[x] = tab.acc[x][poff + n_el + e];
-    }
-    u64 r0, r1, pv[NA];
-    auto load = [&](int k, u64 &x0, u64 &x1, u64 *v) {
-        const u64 *R = tab.job[k].R;
-        x0 = R[e];
-        x1 = R[n_el + e];
+    for (int x = 0; x < NA; x++) a[x][0] = a[x][1] = AccK{0, 0, 0};
+    for (int kb = k0; kb < k1; kb += MM_DEEP) {
+        u64 R[MM_DEEP][2], pv[MM_DEEP][NA];
 #pragma unroll
-        for (int x = 0; x < NA; x++) {
-            const u64 *p = tab.pt[x * nrot + k];
-            v[x] = p ? p[e] : 0;
+        for (int i = 0; i < MM_DEEP; i++) {
+            const int k = kb + i;
+            R[i][0] = R[i][1] = 0;
+            if (k < k1) {
+                R[i][0] = tab.job[k].R[e];
+                R[i][1] = tab.job[k].R[n_el + e];
+            }
+#pragma unroll
+            for (int x = 0; x < NA; x++) {
+                const u64 *p = k < k1 && x < na ? tab.pt[(x0 + x) * nrot + k] : nullptr;
+                pv[i][x] = p ? __ldcs(p + e) : 0;
+            }
         }
-    };
-    load(k0, r0, r1, pv);
-    for (int k = k0; k < k1; k++) {
-        u64 n0 = 0, n1 = 0, nv[NA];
 #pragma unroll
-        for (int x = 0; x < NA; x++) nv[x] = 0;
-        if (k + 1 < k1) load(k + 1, n0, n1, nv);
+        for (int i = 0; i < MM_DEEP; i++) {
+            const uint2 r0 = split_k(R[i][0]), r1 = split_k(R[i][1]);
 #pragma unroll
-        for (int x = 0; x < NA; x++) {
-            if (!tab.pt[x * nrot + k]) continue;
-            a0[x] = add_mod(a0[x], mul_mod(pv[x], r0, P), P.q);
-            a1[x] = add_mod(a1[x], mul_mod(pv[x], r1, P), P.q);
+            for (int x = 0; x < NA; x++) {
+                const uint2 p = split_k(pv[i][x]);
+                mac_k(a[x][0], p, p.x + p.y, r0, r0.x + r0.y);
+                mac_k(a[x][1], p, p.x + p.y, r1, r1.x + r1.y);
+            }
         }
-        r0 = n0;
-        r1 = n1;
-#pragma unroll
-        for (int x = 0; x < NA; x++) pv[x] = nv[x];
     }
+    u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride + (size_t)x0 * 2 * n_el + e;
 #pragma unroll
-    for (int x = 0; x < NA; x++) {
-        tab.acc[x][poff + e] = a0[x];
-        tab.acc[x][poff + n_el + e] = a1[x];
-    }
+    for (int x = 0; x < NA; x++)
+        if (x < na) {
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                u64 *o = acc + (size_t)(2 * x + c) * n_el;
+                const u64 s = acc_reduce(a[x][c], P);
+                *o = first ? s : add_mod(*o, s, P.q);
+            }
+        }
 }
 
 // Giant steps of a baby-step / giant-step product: for every element (r, n) of
@@ -1158,17 +1145,22 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
     // extended-basis accumulators [nacc][2][ell+alpha][N] and the Q-basis results [nacc][2][ell][N]
     u64 *acc = nullptr, *res = raw_out;
     if (!res) STATUS_TRY(sc.get(c, &res, (size_t)nacc * per));
-    CUDA_TRY(cudaMemsetAsync(res, 0, (size_t)nacc * per * sizeof(u64), s));
-    if (!ks_idx.empty()) {
-        // rotations of a chunk are split into `parts` ranges with their own partial sums
-        // (more independent threads to hide the gathers' latency), summed before ModDown
-        // (with many accumulators the launches over accumulator chunks already fill the GPU)
-        const int parts = nacc > MAX_ACC ? 1 : (int)std::min<size_t>(MM_PARTS, (ks_idx.size() + 7) / 8);
+    if (ks_idx.empty()) {
+        CUDA_TRY(cudaMemsetAsync(res, 0, (size_t)nacc * per * sizeof(u64), s));
+    } else {
+        // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
+        // partial sums where the elements and accumulators alone make too few blocks
+        const int tiles = nacc < MM_PRECOMPUTE_ACC ? 1 : (std::min(nacc, MM_ACC) + 3) / 4;
+        const size_t blocks = (size_t)nblk((size_t)nx * N) * tiles;
+        const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
+                                                 (MM_BLOCKS + blocks - 1) / blocks});
         const size_t part_stride = (size_t)nacc * ext;
         u64 *part = nullptr;
         STATUS_TRY(sc.get(c, &acc, (size_t)nacc * ext));
-        STATUS_TRY(sc.get(c, &part, (size_t)parts * part_stride));
-        CUDA_TRY(cudaMemsetAsync(part, 0, (size_t)parts * part_stride * sizeof(u64), s));
+        if (parts > 1)
+            STATUS_TRY(sc.get(c, &part, (size_t)parts * part_stride));
+        else
+            part = acc;
         u64 *yhat = nullptr;
         STATUS_TRY(ks_modup(c, v.data + (size_t)ell * N, ell, sc, &yhat, s));
         const int nd = (ell + A - 1) / A;
@@ -1193,48 +1185,53 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         }
         for (size_t k0 = 0; k0 < ks_idx.size(); k0 += CHUNK_ROT) {
             const int nr = (int)std::min<size_t>(CHUNK_ROT, ks_idx.size() - k0);
-            for (int a0 = 0; a0 < nacc; a0 += MAX_ACC) {
-                const int na = std::min(MAX_ACC, nacc - a0);
-                MmTable tab;
-                memset(&tab, 0, sizeof(tab));
+            const int first = k0 == 0 ? 1 : 0;
+            for (int a0 = 0; a0 < nacc; a0 += MM_ACC) {
+                const int na = std::min(MM_ACC, nacc - a0);
                 int nz_pt = 0;
+                auto point = [&](int a, int x) {
+                    const u64 *p = pt[a0 + a][ks_idx[k0 + x]];
+                    nz_pt += p != nullptr;
+                    return p;
+                };
+                MmTable tab;
+                MmFusedTable ftab;
+                tab.acc = ftab.acc = part + (size_t)a0 * ext;
                 for (int x = 0; x < nr; x++) {
                     const int r = ks_idx[k0 + x];
-                    tab.job[x] = MmJob{evk->find(gal[r]), gal[r], Rall ? Rall + (k0 + x) * ext : nullptr};
-                    for (int a = 0; a < na; a++) {
-                        tab.pt[a * nr + x] = pt[a0 + a][r];
-                        nz_pt += pt[a0 + a][r] != nullptr;
-                    }
+                    tab.job[x] = ftab.job[x] = MmJob{evk->find(gal[r]), gal[r], Rall ? Rall + (k0 + x) * ext : nullptr};
+                    for (int a = 0; a < na; a++) tab.pt[a * nr + x] = point(a, x);
+                    ftab.pt[x] = tab.pt[x];
                 }
-                for (int a = 0; a < na; a++) tab.acc[a] = part + (size_t)(a0 + a) * ext;
                 // algorithmic bytes: keys, diagonals, accumulators in and out, the rotated
                 // digits and c0 once (with R_k precomputed: R_k in place of the keys, digits and c0)
                 const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * na * nx * parts +
                                                 (Rall ? (double)nr * 2 * nx
                                                       : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
-                const dim3 grid(nblk((size_t)nx * N), parts);
-#define MM_CASE(K)                                                                                        \
-    case K:                                                                                               \
-        if (Rall)                                                                                         \
-            TIMED("mm_fused", bytes, s,                                                                   \
-                  k_mm_mac<K><<<grid, TPB, 0, s>>>(nr, tab, part_stride, ell, A, c->L, c->logN, c->d_prime)); \
-        else                                                                                              \
-            TIMED("mm_fused", bytes, s,                                                                   \
-                  k_mm_fused<K><<<grid, TPB, 0, s>>>(yhat, v.data, nr, tab, part_stride, ell, A, c->L,      \
-                                                      c->logN, c->d_prime, c->ks));          \
-        break;
-                switch (na) {
-                    MM_CASE(1) MM_CASE(2) MM_CASE(3) MM_CASE(4) MM_CASE(5) MM_CASE(6) MM_CASE(7) MM_CASE(8)
-                    default: set_error("internal: accumulator count"); return COPSE_EINVAL;
-                }
-#undef MM_CASE
+                const unsigned eb = nblk((size_t)nx * N);
+#define MM_MAC(K)                                                                                              \
+    k_mm_mac<K><<<dim3(eb * (unsigned)((na + K - 1) / K), parts), TPB, 0, s>>>(nr, na, first, tab, part_stride, \
+                                                                               ell, A, c->L, c->logN, c->d_prime)
+                if (!Rall)
+                    TIMED("mm_fused", bytes, s,
+                          k_mm_fused<<<dim3(eb, parts), TPB, 0, s>>>(yhat, v.data, nr, first, ftab, part_stride, ell, A,
+                                                                     c->L, c->logN, c->d_prime, c->ks));
+                else if (na <= 2)
+                    TIMED("mm_fused", bytes, s, MM_MAC(2));
+                else if (na == 3)
+                    TIMED("mm_fused", bytes, s, MM_MAC(3));
+                else
+                    TIMED("mm_fused", bytes, s, MM_MAC(4));
+#undef MM_MAC
                 LAUNCH_CHECK();
             }
         }
-        TIMED("sum_parts", 8.0 * (double)(parts + 1) * part_stride, s,
-              k_sum_parts<<<nblk(part_stride), TPB, 0, s>>>(part, part_stride, parts, acc, part_stride, ell, A,
-                                                            c->L, c->logN, c->d_prime));
-        LAUNCH_CHECK();
+        if (parts > 1) {
+            TIMED("sum_parts", 8.0 * (double)(parts + 1) * part_stride, s,
+                  k_sum_parts<<<nblk(part_stride), TPB, 0, s>>>(part, part_stride, parts, acc, part_stride, ell, A,
+                                                                c->L, c->logN, c->d_prime));
+            LAUNCH_CHECK();
+        }
         // one ModDown per accumulator (both components)
         STATUS_TRY(moddown_batch(c, acc, nacc, ell, res, s));
     }
