@@ -320,8 +320,10 @@ struct copse_ctx {
     u64 *d_psi_sh = nullptr;
     u64 *d_ipsi = nullptr;            // [NP][N] psi^-brev(k)
     u64 *d_ipsi_sh = nullptr;
-    u64 *d_stw_f = nullptr;           // N >= 2^12: each cluster CTA's / row tile's row-stage twiddles,
-    u64 *d_stw_i = nullptr;           //   (w, w') pairs in staging order, [NP][N / 2048][2048][2]
+    u64 *d_tw_f = nullptr;            // N >= 2^12: (w, w') pairs of psi^brev(k), [NP][N][2],
+    u64 *d_tw_i = nullptr;            //   and of psi^-brev(k)
+    u64 *d_low_f = nullptr;           // the low row stages' pairs in the order of the threads that use
+    u64 *d_low_i = nullptr;           //   them, [NP][N / 2048][pairs][128][2] (ntt_core.cuh)
     uint32_t *d_slot_index = nullptr; // [N] NTT(mod t) position of slot s
     KsTables ks{};
     std::vector<void *> owned;        // device allocations freed with the context
@@ -410,7 +412,7 @@ struct NttBatch {
     // N^-1 (the first step of the base conversion that reads it folded in: N^-1 * c mod q)
     const Shoup *scale = nullptr;
 };
-// the staged row twiddles of the cluster transforms (context creation)
+// the transforms' twiddle tables (context creation)
 copse_status ntt_stage_tables(copse_ctx *ctx);
 copse_status ntt_forward(copse_ctx *ctx, const NttBatch &b, cudaStream_t s);
 copse_status ntt_inverse(copse_ctx *ctx, const NttBatch &b, cudaStream_t s);

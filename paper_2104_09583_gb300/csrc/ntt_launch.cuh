@@ -1,0 +1,124 @@
+// Launching the transforms: which form a batch takes, and the timing families.
+#pragma once
+
+#include <atomic>
+
+#include "ntt_core.cuh"
+
+// one block per residue polynomial, in place (N <= 2^11; ntt.cu)
+copse_status ntt_small(copse_ctx *ctx, const NttBatch &b, cudaStream_t s, bool inverse);
+
+namespace {
+
+// kernel-timer family of each transform variant
+template <class IO> constexpr const char *io_family(bool inv) { return inv ? "ntt_inv" : "ntt_fwd"; }
+template <> constexpr const char *io_family<CopyIO>(bool) { return "ntt_inv_copy"; }
+template <> constexpr const char *io_family<GatherIO>(bool) { return "ntt_inv_copy"; }
+template <> constexpr const char *io_family<MsIO>(bool) { return "ntt_fwd_ms"; }
+template <> constexpr const char *io_family<MdIO>(bool) { return "ntt_fwd_md"; }
+template <> constexpr const char *io_family<MuIO>(bool) { return "ntt_fwd_mu"; }
+template <> constexpr const char *io_family<MddIO>(bool) { return "ntt_fwd_mdd"; }
+
+// butterflies of a batch (N/2 log2 N per transformed residue polynomial): the integer
+// roof's unit for the transforms
+inline double butterflies(const copse_ctx *ctx, const NttBatch &b) {
+    return (double)b.npoly * b.nr * (ctx->N / 2) * ctx->logN;
+}
+
+template <bool INV>
+NttTables tables(const copse_ctx *c) {
+    return NttTables{c->d_prime, (const ulonglong2 *)(INV ? c->d_tw_i : c->d_tw_f),
+                     (const ulonglong2 *)(INV ? c->d_low_i : c->d_low_f), c->L};
+}
+
+// the 16-block clusters of N = 2^15 are above the portable size: opted in once per device
+template <class K>
+copse_status cluster_attr(K kernel, int device, std::atomic<uint64_t> &done) {
+    if (device >= 0 && device < 64 && (done.load(std::memory_order_acquire) & (1ull << device))) return COPSE_OK;
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (device >= 0 && device < 64) done.fetch_or(1ull << device, std::memory_order_release);
+    return COPSE_OK;
+}
+
+template <int LOGN, bool INV, class IO>
+copse_status launch_cluster(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s) {
+    const unsigned grid = (unsigned)b.npoly * (unsigned)b.nr * Shape<LOGN>::TILES;
+    const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;  // one read and one write of each residue polynomial
+    if constexpr (LOGN == 15) {
+        static std::atomic<uint64_t> done{0};
+        if constexpr (INV)
+            STATUS_TRY(cluster_attr(k_ntt_inv_cluster<LOGN, IO>, ctx->device, done));
+        else
+            STATUS_TRY(cluster_attr(k_ntt_fwd_cluster<LOGN, IO>, ctx->device, done));
+    }
+    TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
+        if constexpr (INV)
+            k_ntt_inv_cluster<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io);
+        else
+            k_ntt_fwd_cluster<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io);
+    });
+    LAUNCH_CHECK();
+    return COPSE_OK;
+}
+
+// two launches; the partial transform in `mid`
+template <int LOGN, bool INV, class IO>
+copse_status launch_tiled(copse_ctx *ctx, const NttBatch &b, const IO &io, const Mid &mid, cudaStream_t s) {
+    const unsigned grid = (unsigned)b.npoly * (unsigned)b.nr * Shape<LOGN>::TILES;
+    const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;
+    TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
+        if constexpr (INV) {
+            k_ntt_inv_rows<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io, mid);
+            k_ntt_inv_cols<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io, mid);
+        } else {
+            k_ntt_fwd_cols<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io, mid);
+            k_ntt_fwd_rows<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io, mid);
+        }
+    });
+    LAUNCH_CHECK();
+    return COPSE_OK;
+}
+
+// A batch of b with this IO: clusters up to max_cluster residue polynomials (N = 2^15 only where
+// 16-block clusters are opted in), else two launches through `data` (in place) or, when it is
+// null, through scratch.
+template <int LOGN, bool INV, class IO>
+copse_status launch_ring(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *data, long max_cluster, cudaStream_t s) {
+    if (ctx->ntt_clusters && (long)b.npoly * b.nr <= max_cluster && (LOGN < 15 || ctx->ntt_cluster16))
+        return launch_cluster<LOGN, INV, IO>(ctx, b, io, s);
+    if (data) return launch_tiled<LOGN, INV, IO>(ctx, b, io, Mid{data, b.stride, 0}, s);
+    u64 *scratch = nullptr;
+    STATUS_TRY(dev_alloc(ctx, (void **)&scratch, ((size_t)b.npoly * b.nr << LOGN) * sizeof(u64), s));
+    const copse_status st = launch_tiled<LOGN, INV, IO>(ctx, b, io, Mid{scratch, (size_t)b.nr << LOGN, b.r0}, s);
+    dev_free(scratch, s);
+    return st;
+}
+template <bool INV, class IO>
+copse_status launch_io(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *data, long max_cluster, cudaStream_t s) {
+    switch (ctx->logN) {
+        case 12: return launch_ring<12, INV, IO>(ctx, b, io, data, max_cluster, s);
+        case 13: return launch_ring<13, INV, IO>(ctx, b, io, data, max_cluster, s);
+        case 14: return launch_ring<14, INV, IO>(ctx, b, io, data, max_cluster, s);
+        default: return launch_ring<15, INV, IO>(ctx, b, io, data, max_cluster, s);
+    }
+}
+
+// in place
+template <bool INV>
+copse_status launch_plain(copse_ctx *ctx, const NttBatch &b, cudaStream_t s) {
+    if (b.npoly <= 0 || b.nr <= 0) return COPSE_OK;
+    if (ctx->logN < 12) return ntt_small(ctx, b, s, INV);
+    return launch_io<INV>(ctx, b, PlainIO{b.data, b.stride, ctx->logN}, b.data, ctx->ntt_cluster_max, s);
+}
+
+// fused with the IO (*done = false, nothing launched, below 2^12 and with the fused forms off)
+template <bool INV = false, class IO>
+copse_status launch_fused(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s, bool *done) {
+    *done = b.npoly <= 0 || b.nr <= 0;
+    if (*done || !ctx->ntt_clusters || ctx->logN < 12) return COPSE_OK;
+    STATUS_TRY((launch_io<INV>(ctx, b, io, (u64 *)nullptr, ctx->ntt_fused_max, s)));
+    *done = true;
+    return COPSE_OK;
+}
+
+}  // namespace
