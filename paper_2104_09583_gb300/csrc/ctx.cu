@@ -270,30 +270,59 @@ static copse_status build_tables(copse_ctx *c) {
             mdd_Binv[(size_t)ell * L + i] = mk_shoup(h_inv(B, qi), qi);
         }
     }
-    // Montgomery forms of the conversion factors and of the negated corrections
+    // the fused conversions' factors (Montgomery form, split at 28 bits) and centring constants
     auto mont = [&](u64 x, int g) { return h_mul(x % c->primes[g], c->hprime[g].r64, c->primes[g]); };
-    auto neg = [&](u64 x, int g) { const u64 q = c->primes[g], r = x % q; return r ? q - r : 0; };
-    std::vector<u64> modup_hat_m(modup_hat.size()), modup_negq_m(modup_qhat.size());
+    auto split = [](u64 x) { return ((x >> 28) << 32) | (x & 0x0FFFFFFFull); };
+    // c -= ((b - 1) / 2) f mod prime g
+    auto centre = [&](u64 &sum, u64 b, u64 f, int g) {
+        const u64 q = c->primes[g];
+        sum = (sum + q - h_mul(((b - 1) / 2) % q, f, q)) % q;
+    };
+    std::vector<u64> modup_f(modup_hat.size()), modup_c(modup_hat.size(), 0);
     for (int ell = 1; ell <= L; ell++)
         for (int i = 0; i < ell; i++)
             for (int g = 0; g < NP; g++) {
                 const size_t ti = ((size_t)ell * L + i) * NP + g;
-                modup_hat_m[ti] = mont(modup_hat[ti].w, g);
-                modup_negq_m[ti] = mont(neg(modup_qhat[ti], g), g);
+                const u64 f = mont(modup_hat[ti].w, g);
+                modup_f[ti] = split(f);
+                centre(modup_c[((size_t)ell * L + i / A * A) * NP + g], c->primes[i], f, g);
             }
-    std::vector<u64> md_hat_m(md_hat.size()), md_negP_m(L);
+    std::vector<u64> md_f(md_hat.size()), md_c(L, 0), mdd_f(mdd_hat.size(), 0), mdd_c(mdd_B.size(), 0);
     for (int k = 0; k < A; k++)
-        for (int i = 0; i < L; i++) md_hat_m[(size_t)k * L + i] = mont(md_hat[(size_t)k * L + i].w, i);
-    for (int i = 0; i < L; i++) md_negP_m[i] = mont(neg(md_P[i], i), i);
-    std::vector<u64> mdd_hat_m(mdd_hat.size()), mdd_negB_m(mdd_B.size());
-    for (size_t x = 0; x < mdd_hat.size(); x++) mdd_hat_m[x] = mont(mdd_hat[x].w, (int)(x % L));
-    for (size_t x = 0; x < mdd_B.size(); x++) mdd_negB_m[x] = mont(neg(mdd_B[x], (int)(x % L)), (int)(x % L));
-    STATUS_TRY(upload(c, &c->ks.modup_hat_m, modup_hat_m));
-    STATUS_TRY(upload(c, &c->ks.modup_negq_m, modup_negq_m));
-    STATUS_TRY(upload(c, &c->ks.md_hat_m, md_hat_m));
-    STATUS_TRY(upload(c, &c->ks.md_negP_m, md_negP_m));
-    STATUS_TRY(upload(c, &c->ks.mdd_hat_m, mdd_hat_m));
-    STATUS_TRY(upload(c, &c->ks.mdd_negB_m, mdd_negB_m));
+        for (int i = 0; i < L; i++) {
+            const u64 f = mont(md_hat[(size_t)k * L + i].w, i);
+            md_f[(size_t)k * L + i] = split(f);
+            centre(md_c[i], c->primes[L + k], f, i);
+        }
+    for (int ell = 2; ell <= L; ell++)
+        for (int k = 0; k < nb; k++)
+            for (int i = 0; i < ell - 1; i++) {
+                const size_t x = ((size_t)ell * nb + k) * L + i;
+                const u64 f = mont(mdd_hat[x].w, i);
+                mdd_f[x] = split(f);
+                centre(mdd_c[(size_t)ell * L + i], c->primes[k == 0 ? ell - 1 : L + k - 1], f, i);
+            }
+    // -t times the finishes' inverses
+    auto neg_t = [&](const Shoup &inv, int i) {
+        const u64 q = c->primes[i], x = h_mul(c->t % q, inv.w, q);
+        return mk_shoup(x ? q - x : 0, q);
+    };
+    std::vector<Shoup> ms_ntq(ms_qinv.size()), md_ntP(L), mdd_ntB(mdd_Binv.size());
+    for (int i = 0; i < L; i++) md_ntP[i] = neg_t(md_Pinv[i], i);
+    for (int ell = 2; ell <= L; ell++)
+        for (int i = 0; i < ell - 1; i++) {
+            ms_ntq[(size_t)ell * L + i] = neg_t(ms_qinv[(size_t)ell * L + i], i);
+            mdd_ntB[(size_t)ell * L + i] = neg_t(mdd_Binv[(size_t)ell * L + i], i);
+        }
+    STATUS_TRY(upload(c, &c->ks.modup_f, modup_f));
+    STATUS_TRY(upload(c, &c->ks.modup_c, modup_c));
+    STATUS_TRY(upload(c, &c->ks.md_f, md_f));
+    STATUS_TRY(upload(c, &c->ks.md_c, md_c));
+    STATUS_TRY(upload(c, &c->ks.mdd_f, mdd_f));
+    STATUS_TRY(upload(c, &c->ks.mdd_c, mdd_c));
+    STATUS_TRY(upload(c, &c->ks.ms_ntq, ms_ntq));
+    STATUS_TRY(upload(c, &c->ks.md_ntP, md_ntP));
+    STATUS_TRY(upload(c, &c->ks.mdd_ntB, mdd_ntB));
     // first-step factors times N^-1: the scales of the inverse transforms feeding the conversions
     auto scaled = [&](const Shoup &f, int g) { return mk_shoup(h_mul(f.w, c->hprime[g].ninv, c->primes[g]), c->primes[g]); };
     std::vector<Shoup> mu_scale(modup_inv.size()), md_scale(A), ms_scale(L + 1), mdd_scale(mdd_inv.size());

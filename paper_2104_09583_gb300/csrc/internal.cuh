@@ -298,11 +298,13 @@ struct KsTables {
     Shoup *mdd_hat;     // [(L+1) * (alpha+1) * L]
     u64 *mdd_B;         // [(L+1) * L]
     Shoup *mdd_Binv;    // [(L+1) * L]
-    // The conversion factors in Montgomery form (x 2^64 mod the target prime), indexed like
-    // the factors above, for the fused transforms' loads: a conversion sums its products
-    // exactly in 128 bits, adds the negated correction of every centred negative digit
-    // (modup_negq_m = -modup_qhat, md_negP_m = -P, mdd_negB_m = -B) and reduces once.
-    u64 *modup_hat_m, *modup_negq_m, *md_hat_m, *md_negP_m, *mdd_hat_m, *mdd_negB_m;
+    // The fused transforms' conversions (ntt_io.cuh) take the factors in Montgomery form (x 2^64
+    // mod the target prime) split at 28 bits (low word, high word), indexed like the factors above:
+    // modup_f, md_f, mdd_f; and the centring of all digits together, -sum of (b_k - 1) / 2 times
+    // the factors: modup_c [ell][first prime of the digit][g], md_c [i], mdd_c [ell][i].  Their
+    // finishes take -t times the inverse: ms_ntq, md_ntP, mdd_ntB, indexed like the inverses.
+    u64 *modup_f, *modup_c, *md_f, *md_c, *mdd_f, *mdd_c;
+    Shoup *ms_ntq, *md_ntP, *mdd_ntB;
     // gadget factor of key-switching keys: P mod q_i (i < L)
 };
 
@@ -411,7 +413,13 @@ struct NttBatch {
     // inverse transforms: when set, residue r's result is scaled by scale[r - r0] instead of
     // N^-1 (the first step of the base conversion that reads it folded in: N^-1 * c mod q)
     const Shoup *scale = nullptr;
+    // inverse transforms (2^12 <= N): results x stored as digits of a fused conversion,
+    // x + (q - 1) / 2 mod q split at 28 bits (low word, high word)
+    bool digits = false;
 };
+// whether the conversions around key switches and modulus switches run fused with the transforms
+// (their digits are then stored as above)
+inline bool ntt_fuses(const copse_ctx *c) { return c->ntt_clusters && c->logN >= 12; }
 // the transforms' twiddle tables (context creation)
 copse_status ntt_stage_tables(copse_ctx *ctx);
 copse_status ntt_forward(copse_ctx *ctx, const NttBatch &b, cudaStream_t s);
@@ -465,16 +473,16 @@ struct MddFuse {
 };
 copse_status ntt_forward_moddown_drop(copse_ctx *ctx, const MddFuse &f, int npoly, cudaStream_t s, bool *done);
 copse_status moddown_drop_unfused(copse_ctx *ctx, const MddFuse &f, int npoly, cudaStream_t s);
-// The fused forms run on the cluster transform (2^12 <= N <= 2^15); *done = false
-// (nothing launched) otherwise, and the caller takes the unfused sequence.
+// The fused forms run where ntt_fuses says (2^12 <= N); *done = false (nothing launched)
+// otherwise, and the caller takes the unfused sequence.
 copse_status ntt_forward_modswitch(copse_ctx *ctx, const MsFuse &f, int nc, cudaStream_t s, bool *done);
 copse_status ntt_forward_moddown(copse_ctx *ctx, const MdFuse &f, int njobs, cudaStream_t s, bool *done);
 // out-of-place inverse transform of residues [0, nr) (prime `fixed` when >= 0) of npoly
-// polynomials src + p sstride into dst + p dstride
+// polynomials src + p sstride into dst + p dstride, as digits of a conversion (NttBatch::digits)
 copse_status ntt_inverse_copy(copse_ctx *ctx, const u64 *src, size_t sstride, u64 *dst, size_t dstride, int npoly,
                               int nr, int fixed, cudaStream_t s, bool *done, const Shoup *scale = nullptr);
 // the same for one residue (prime `fixed`) of npoly <= MS_POLYS polynomials held at
-// separate addresses src[p] ([N] each) into dst + p N
+// separate addresses src[p] ([N] each) into dst + p N (as digits where ntt_fuses, else plain)
 struct GatherSrc {
     const u64 *p[MS_POLYS];
 };

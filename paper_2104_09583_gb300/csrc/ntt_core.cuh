@@ -58,8 +58,8 @@ __device__ __forceinline__ bool ntt_skipped(const NttBatch &b, int p, int r) {
 
 // Forward butterfly without a correction step: the Shoup product V is below 2q for any
 // 64-bit input, so x' = U + V and y' = U - V + 2q only grow by 2q per stage.  From inputs
-// below q, values stay below (2 log2 N + 1) q <= 31 q < 2^60 for primes below 2^55 (the
-// context's limit); the final store reduces them once (fwd_reduce).
+// below 2q, values stay below (2 log2 N + 2) q <= 32 q <= 2^60 for primes below 2^55 (the
+// context's limit); the final store reduces them once.
 __device__ __forceinline__ void bf_fwd(u64 &x, u64 &y, ulonglong2 w, u64 q, u64 q2) {
     const u64 U = x;
     const u64 V = mul_shoup_lazy(y, w.x, w.y, q);
@@ -207,7 +207,7 @@ __device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int 
 }
 
 // Forward row half: v holds coefficients i + m SB of the thread's row (i = t mod SB); all LB row
-// stages, the values reduced and stored through io.
+// stages, the values stored through io (reduced unless it takes them raw).
 template <int LOGN, class IO>
 __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T,
                                          const ulonglong2 *low, const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
@@ -230,7 +230,10 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
     for (int h = 0; h < 4; h++) {
         u64 x[4];
 #pragma unroll
-        for (int m = 0; m < 4; m++) x[m] = fwd_reduce(sm[pad(f0 + 32 * (4 * h + m))], P);
+        for (int m = 0; m < 4; m++) {
+            x[m] = sm[pad(f0 + 32 * (4 * h + m))];
+            if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
+        }
         store_n(io, p, r, g, ((size_t)tile << 11) + f0 + 128 * h, 32, x);
     }
 }
@@ -266,7 +269,7 @@ __device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int 
 // column stages, scaled and stored through io.
 template <int LOGN, class IO>
 __device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T, Shoup sc,
-                                         u64 q, u64 *sm, u64 (&v)[16]) {
+                                         bool digits, u64 q, u64 *sm, u64 (&v)[16]) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
     stages_inv<S::A - 4>(v, q, 2 * q, TwInvColLow<S::A>{T, i});
@@ -277,8 +280,14 @@ __device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int 
     for (int m = 0; m < 16; m++) v[m] = sm[((i + m * S::SA) << S::LC) + c];
     stages_inv<4>(v, q, (2 * q) << (S::A - 4), TwInvColTop{T});
 #pragma unroll
-    for (int m = 0; m < 16; m++)
-        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, mul_shoup(v[m], sc, q));
+    for (int m = 0; m < 16; m++) {
+        u64 x = mul_shoup(v[m], sc, q);
+        if (digits) {  // centred, offset by (q - 1) / 2, split at 28 bits
+            x = add_mod(x, (q - 1) / 2, q);
+            x = ((x >> 28) << 32) | (x & 0x0FFFFFFFu);
+        }
+        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, x);
+    }
 }
 
 // ---------------------------------------------------------------- tiled: two launches
@@ -376,7 +385,7 @@ __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_cols(const __grid_
     for (int m = 0; m < 16; m++) v[m] = in[(size_t)(16 * i + m) << S::LB];
     const PrimeDev P = tb.pr[t.g];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), sc, P.q, sm, v);
+    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), sc, b.digits, P.q, sm, v);
 }
 
 // ---------------------------------------------------------------- clusters: one launch
@@ -439,7 +448,7 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = colt[((16 * ic + m) << S::LC) + c];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, T, sc, P.q, colt, v);
+    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, T, sc, b.digits, P.q, colt, v);
 }
 
 }  // namespace

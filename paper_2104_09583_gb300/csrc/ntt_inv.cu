@@ -16,6 +16,7 @@ copse_status ntt_inverse_copy(copse_ctx *ctx, const u64 *src, size_t sstride, u6
                               int nr, int fixed, cudaStream_t s, bool *done, const Shoup *scale) {
     NttBatch b{nullptr, 0, npoly, 0, nr, nr, fixed};
     b.scale = scale;
+    b.digits = true;
     return launch_fused<true>(ctx, b, CopyIO{src, sstride, dst, dstride, ctx->logN}, s, done);
 }
 
@@ -24,6 +25,7 @@ copse_status ntt_inverse_gather(copse_ctx *ctx, const GatherSrc &src, int npoly,
     if (npoly > MS_POLYS) { set_error("internal: too many polynomials in one gathered transform"); return COPSE_EINVAL; }
     NttBatch b{nullptr, 0, npoly, 0, 1, 1, fixed};
     b.scale = scale;
+    b.digits = true;
     STATUS_TRY(launch_fused<true>(ctx, b, GatherIO{src, dst, ctx->logN}, s, done));
     if (*done) return COPSE_OK;
     // a gather, then the in-place transform

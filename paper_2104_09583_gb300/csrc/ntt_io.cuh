@@ -62,9 +62,10 @@ __device__ __forceinline__ void mdd_store(const MddFuse &f, const PrimeDev *pr, 
     f.outp[p >> 1][at] = res;
 }
 
-// Load / store of the forward cluster transform: coefficient n of residue r (global
-// prime g) of batch polynomial p in; NTT-domain value v (in [0, q)) at position k out.
+// Load / store of the transforms: coefficient n of residue r (global prime g) of batch
+// polynomial p in; value v at position k out, in [0, q), or (RAW) unreduced below 2^60.
 struct PlainIO {
+    static constexpr bool RAW = false;
     u64 *data;
     size_t stride;
     int logN;
@@ -79,6 +80,7 @@ struct PlainIO {
 
 // out-of-place transform: residue r of polynomial p from src into dst
 struct CopyIO {
+    static constexpr bool RAW = false;
     const u64 *src;
     size_t sstride;
     u64 *dst;
@@ -95,6 +97,7 @@ struct CopyIO {
 
 // one residue of polynomials at separate addresses in, contiguous residues out
 struct GatherIO {
+    static constexpr bool RAW = false;
     GatherSrc src;
     u64 *dst;
     int logN;
@@ -110,6 +113,7 @@ struct GatherIO {
 // y [item][nd][ell+alpha][N]; a digit's own residues (skipped by the transform) are
 // copied from the input, which already holds them in NTT form
 struct MuIO {
+    static constexpr bool RAW = false;
     const u64 *xc;     // [item][ell][N] coefficient form
     const u64 *x_ntt;  // item i at x_ntt + i * xs, [ell][N] NTT domain
     size_t xs;
@@ -117,22 +121,6 @@ struct MuIO {
     int ell, alpha, nd, L, NP, logN;
     const PrimeDev *pr;
     KsTables T;
-    __device__ __forceinline__ u64 load(int p, int, int g, size_t n) const {
-        const int item = p / nd, j = p - item * nd;
-        const int lo = j * alpha, hi = min(lo + alpha, ell);
-        const u64 qg = pr[g].q;
-        const u64 *x = xc + (size_t)item * ell * ((size_t)1 << logN);
-        u64 acc = 0;
-        for (int i = lo; i < hi; i++) {
-            const u64 qi = pr[i].q;
-            const u64 v = x[((size_t)i << logN) + n];  // already times modup_inv (inverse transform's scale)
-            const size_t ti = ((size_t)ell * L + i) * NP + g;
-            u64 w = mul_shoup(v, T.modup_hat[ti], qg);
-            if (v > (qi - 1) / 2) w = sub_mod(w, T.modup_qhat[ti], qg);
-            acc = add_mod(acc, w, qg);
-        }
-        return acc;
-    }
     __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
         y[(((size_t)p * (ell + alpha) + r) << logN) + k] = v;
     }
@@ -147,59 +135,31 @@ struct MuIO {
 
 // modulus switch: load the centred conversion of the last prime's residue, store the finish
 struct MsIO {
+    static constexpr bool RAW = true;
     MsFuse f;
     const PrimeDev *pr;
     KsTables T;
     int L, logN;
-    __device__ __forceinline__ u64 load(int p, int r, int, size_t n) const {
-        const u64 ql = pr[f.ell - 1].q;
-        const u64 w = f.last[((size_t)p << logN) + n];  // already times t^-1 (inverse transform's scale)
-        // |centred w| < q_{ell-1}/2 < q_r: the chain is in decreasing order
-        return w > (ql - 1) / 2 ? pr[r].q - (ql - w) : w;
-    }
-    __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
-        ms_store(f, pr, T, L, logN, p, r, k, v);
-    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
 // ModDown: load the conversion of the alpha special residues, store the finish
 struct MdIO {
+    static constexpr bool RAW = true;
     MdFuse f;
     const PrimeDev *pr;
     KsTables T;
     int L, alpha, logN;
-    __device__ __forceinline__ u64 load(int p, int r, int, size_t n) const {
-        const u64 *up = f.U + (size_t)p * f.ustride;
-        const u64 qi = pr[r].q;
-        u64 acc = 0;
-        for (int k = 0; k < alpha; k++) {
-            const u64 pk = pr[L + k].q;
-            const u64 y = up[((size_t)(f.ell + k) << logN) + n];  // already times md_inv[k] (inverse transform's scale)
-            u64 v = mul_shoup(y, T.md_hat[(size_t)k * L + r], qi);
-            if (y > (pk - 1) / 2) v = sub_mod(v, T.md_P[r], qi);
-            acc = add_mod(acc, v, qi);
-        }
-        return acc;
-    }
-    __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
-        md_store(f, pr, T, logN, p, r, k, v);
-    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
 // relinearise-and-drop ModDown: load the conversion from the q_{ell-1} P basis, store the finish
 struct MddIO {
+    static constexpr bool RAW = true;
     MddFuse f;
     const PrimeDev *pr;
     KsTables T;
     int L, alpha, logN;
-    __device__ __forceinline__ u64 load(int p, int r, int, size_t n) const {
-        return mdd_load(f, pr, T, L, alpha, logN, p, r, n);
-    }
-    __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
-        mdd_store(f, pr, T, L, logN, p, r, k, v);
-    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
@@ -219,33 +179,50 @@ __device__ __forceinline__ void store_n(const IO &io, int p, int r, int g, size_
     for (int i = 0; i < K; i++) io.store(p, r, g, k0 + (size_t)i * dk, v[i]);
 }
 
-// A base conversion sum_k [y_k]_centred * f_k mod q as one lazy sum: with f_k in Montgomery form
-// F_k = f_k 2^64 mod q and C = (-c) 2^64 mod q for the correction c that every centred negative
-// digit takes (the product of the basis, the same for all of them),
-// S = sum_k y_k F_k + #{k: y_k > (b_k - 1) / 2} C is summed exactly (the products split at 28 bits,
-// three multiply-adds each, at most 64 of them) and reduced once, S 2^-64 mod q (Montgomery).
-// S < m 2^(2 bits) + m q < q 2^64 for m < 2^(63 - bits) terms of residues below 2^bits.
-struct ConvSum {
-    AccK a;
-    uint32_t neg;
-};
-template <int K>
-__device__ __forceinline__ void conv_term(ConvSum (&s)[K], const u64 (&y)[K], u64 F, u64 half) {
-    const uint2 f = split_k(F);
-    const uint32_t fs = f.x + f.y;
+// A base conversion sum_k c_k f_k mod q of centred digits c_k = [y_k] in (-b_k / 2, b_k / 2).
+// The inverse transform that makes the digits stores them as y_k + (b_k - 1) / 2 mod b_k
+// (NttBatch::digits), so that c_k is that value less (b_k - 1) / 2 and the centring of every
+// digit is one constant per target prime: with f_k in Montgomery form F_k = f_k 2^64 mod q and
+// C = -sum_k ((b_k - 1) / 2) F_k mod q,
+//   S = C + sum_k (y_k + (b_k - 1) / 2 mod b_k) F_k
+// is summed exactly (digits and factors are stored split at 28 bits: three multiply-adds a
+// product, at most 64 products) and reduced once, S 2^-64 mod q (Montgomery).
+// S < m 2^(2 bits) + q < q 2^64 for m < 2^(63 - bits) terms of residues below 2^bits; the result
+// stays below 2q, which the transform takes (its values stay below (2 log2 N + 2) q).
+// The digits of the next factor are loaded while this one's are multiplied.
+// Taking the centring out of the sums (a comparison and a count per product before) and the
+// factors and digits apart beforehand, with finishes of one combined reduction: ModDown with six
+// special primes at N = 2^15 83 -> 66 ms over a batch of 16 encrypted query ciphertexts, ModUp
+// 52 -> 44, relinearise-and-drop 17 -> 13; a batch of 16 residue polynomials at N = 2^14 34 -> 28 us.
+template <int K, class FAC>
+__device__ __forceinline__ void conv_sum(const u64 *y, size_t ystep, size_t dn, int m, u64 C, const PrimeDev &P,
+                                         FAC fac, u64 (&v)[K]) {
+    AccK s[K];
+    uint2 d[K];
 #pragma unroll
     for (int i = 0; i < K; i++) {
-        const uint2 v = split_k(y[i]);
-        mac_k(s[i].a, v, v.x + v.y, f, fs);
-        s[i].neg += y[i] > half;
+        s[i] = AccK{C, 0, C};
+        d[i] = *(const uint2 *)(y + (size_t)i * dn);
     }
-}
-template <int K>
-__device__ __forceinline__ void conv_reduce(const ConvSum (&s)[K], u64 C, const PrimeDev &P, u64 (&v)[K]) {
+    for (int k = 0; k < m; k++) {
+        uint2 nx[K];
+        y += k + 1 < m ? ystep : 0;
+#pragma unroll
+        for (int i = 0; i < K; i++) nx[i] = *(const uint2 *)(y + (size_t)i * dn);
+        const u64 F = __ldg(fac(k));
+        const uint2 f = make_uint2((uint32_t)F, (uint32_t)(F >> 32));
+        const uint32_t fs = f.x + f.y;
+#pragma unroll
+        for (int i = 0; i < K; i++) {
+            mac_k(s[i], d[i], d[i].x + d[i].y, f, fs);
+            d[i] = nx[i];
+        }
+    }
 #pragma unroll
     for (int i = 0; i < K; i++) {
-        const unsigned __int128 x = acc_value(s[i].a) + (u64)s[i].neg * C;
-        v[i] = mont_reduce(Acc128{(u64)x, (u64)(x >> 64)}, P);
+        const unsigned __int128 x = acc_value(s[i]);
+        const u64 lo = (u64)x, mm = lo * P.qinv_neg;
+        v[i] = (u64)(x >> 64) + __umul64hi(mm, P.q) + (lo != 0);
     }
 }
 
@@ -253,81 +230,62 @@ template <int K>
 __device__ __forceinline__ void load_n(const MuIO &io, int p, int, int g, size_t n0, size_t dn, u64 (&v)[K]) {
     const int item = p / io.nd, j = p - item * io.nd;
     const int lo = j * io.alpha, hi = min(lo + io.alpha, io.ell);
-    const u64 *x = io.xc + (size_t)item * io.ell * ((size_t)1 << io.logN) + n0;
-    ConvSum s[K];
-#pragma unroll
-    for (int i = 0; i < K; i++) s[i] = ConvSum{AccK{0, 0, 0}, 0};
-    for (int i = lo; i < hi; i++) {
-        const size_t ti = ((size_t)io.ell * io.L + i) * io.NP + g;
-        const u64 *xi = x + ((size_t)i << io.logN);
-        u64 y[K];
-#pragma unroll
-        for (int k = 0; k < K; k++) y[k] = xi[(size_t)k * dn];  // already times modup_inv (the inverse transform's scale)
-        conv_term(s, y, io.T.modup_hat_m[ti], (io.pr[i].q - 1) / 2);
-    }
-    conv_reduce(s, io.T.modup_negq_m[((size_t)io.ell * io.L + lo) * io.NP + g], io.pr[g], v);
+    const size_t N = (size_t)1 << io.logN, t0 = ((size_t)io.ell * io.L + lo) * io.NP + g;
+    conv_sum(io.xc + ((size_t)item * io.ell + lo) * N + n0, N, dn, hi - lo, io.T.modup_c[t0], io.pr[g],
+             [&](int k) { return io.T.modup_f + t0 + (size_t)k * io.NP; }, v);
 }
 
 template <int K>
 __device__ __forceinline__ void load_n(const MdIO &io, int p, int r, int, size_t n0, size_t dn, u64 (&v)[K]) {
-    const u64 *up = io.f.U + (size_t)p * io.f.ustride + ((size_t)io.f.ell << io.logN) + n0;
-    const u64 C = io.T.md_negP_m[r];
-    ConvSum s[K];
-#pragma unroll
-    for (int i = 0; i < K; i++) s[i] = ConvSum{AccK{0, 0, 0}, 0};
-    for (int k = 0; k < io.alpha; k++) {
-        const u64 *yk = up + ((size_t)k << io.logN);
-        u64 y[K];
-#pragma unroll
-        for (int i = 0; i < K; i++) y[i] = yk[(size_t)i * dn];  // already times md_inv[k] (the inverse transform's scale)
-        conv_term(s, y, io.T.md_hat_m[(size_t)k * io.L + r], (io.pr[io.L + k].q - 1) / 2);
-    }
-    conv_reduce(s, C, io.pr[r], v);
+    const size_t N = (size_t)1 << io.logN;
+    conv_sum(io.f.U + (size_t)p * io.f.ustride + (size_t)io.f.ell * N + n0, N, dn, io.alpha, io.T.md_c[r], io.pr[r],
+             [&](int k) { return io.T.md_f + (size_t)k * io.L + r; }, v);
 }
 
 template <int K>
 __device__ __forceinline__ void load_n(const MddIO &io, int p, int r, int, size_t n0, size_t dn, u64 (&v)[K]) {
-    const int ell = io.f.ell, nb = io.alpha + 1;
-    const u64 *up = io.f.U + (size_t)p * io.f.ustride + ((size_t)(ell - 1) << io.logN) + n0;
-    const u64 C = io.T.mdd_negB_m[(size_t)ell * io.L + r];
-    ConvSum s[K];
-#pragma unroll
-    for (int i = 0; i < K; i++) s[i] = ConvSum{AccK{0, 0, 0}, 0};
-    for (int k = 0; k < nb; k++) {
-        const u64 bk = k == 0 ? io.pr[ell - 1].q : io.pr[io.L + k - 1].q;
-        const u64 *yk = up + ((size_t)k << io.logN);
-        u64 y[K];
-#pragma unroll
-        for (int i = 0; i < K; i++) y[i] = yk[(size_t)i * dn];  // scaled by the inverse transform
-        conv_term(s, y, io.T.mdd_hat_m[((size_t)ell * nb + k) * io.L + r], (bk - 1) / 2);
-    }
-    conv_reduce(s, C, io.pr[r], v);
+    const size_t N = (size_t)1 << io.logN, t0 = (size_t)io.f.ell * (io.alpha + 1) * io.L + r;
+    conv_sum(io.f.U + (size_t)p * io.f.ustride + (size_t)(io.f.ell - 1) * N + n0, N, dn, io.alpha + 1,
+             io.T.mdd_c[(size_t)io.f.ell * io.L + r], io.pr[r],
+             [&](int k) { return io.T.mdd_f + t0 + (size_t)k * io.L; }, v);
 }
 
+// the one digit of a modulus switch: c = d - (q_{ell-1} - 1) / 2, |c| < q_r as the chain is in
+// decreasing order
 template <int K>
 __device__ __forceinline__ void load_n(const MsIO &io, int p, int r, int, size_t n0, size_t dn, u64 (&v)[K]) {
-    const u64 ql = io.pr[io.f.ell - 1].q, qr = io.pr[r].q, half = (ql - 1) / 2;
+    const u64 up = io.pr[r].q - (io.pr[io.f.ell - 1].q - 1) / 2;
     const u64 *w = io.f.last + ((size_t)p << io.logN) + n0;  // already times t^-1
 #pragma unroll
     for (int i = 0; i < K; i++) {
-        const u64 x = w[(size_t)i * dn];
-        v[i] = x > half ? qr - (ql - x) : x;  // |centred x| < q_{ell-1} / 2 < q_r
+        const uint2 d = *(const uint2 *)(w + (size_t)i * dn);
+        v[i] = ((u64)d.y << 28) + d.x + up;
     }
 }
 
-// the finishes of ms_store, md_store and mdd_store for K positions of one residue
+// x a + v b mod q for constants a, b (Shoup pairs), x < q and any v < 2^60, in [0, q): the two
+// quotients are subtracted together, so the sum lies below 3q
+__device__ __forceinline__ u64 mul2_shoup(u64 x, Shoup a, u64 v, Shoup b, u64 q) {
+    const u64 h = __umul64hi(x, a.wp) + __umul64hi(v, b.wp);
+    u64 r = x * a.w + v * b.w - h * q;
+    if (r >= 2 * q) r -= 2 * q;
+    return r >= q ? r - q : r;
+}
+
+// the finishes of ms_store, md_store and mdd_store for K positions of one residue, from the
+// transform's unreduced values: (U - t v) B^-1 = U B^-1 + v (-t B^-1)
 template <int K>
 __device__ __forceinline__ void store_n(const MsIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K]) {
     const MsFuse &f = io.f;
     const u64 q = io.pr[r].q;
-    const Shoup tm{io.pr[r].t_mod, io.pr[r].t_mod_sh}, qinv = io.T.ms_qinv[(size_t)f.ell * io.L + r];
+    const Shoup qinv = io.T.ms_qinv[(size_t)f.ell * io.L + r], tq = io.T.ms_ntq[(size_t)f.ell * io.L + r];
     const u64 *x = (f.xp[0] ? f.xp[p] : f.x + (size_t)p * f.ell * ((size_t)1 << io.logN)) + ((size_t)r << io.logN);
     u64 *o = (f.outp[0] ? f.outp[p] : f.out + (size_t)p * (f.ell - 1) * ((size_t)1 << io.logN)) + ((size_t)r << io.logN);
     u64 xv[K];
 #pragma unroll
     for (int i = 0; i < K; i++) xv[i] = x[k0 + (size_t)i * dk];
 #pragma unroll
-    for (int i = 0; i < K; i++) o[k0 + (size_t)i * dk] = mul_shoup(sub_mod(xv[i], mul_shoup(v[i], tm, q), q), qinv, q);
+    for (int i = 0; i < K; i++) o[k0 + (size_t)i * dk] = mul2_shoup(xv[i], qinv, v[i], tq, q);
 }
 
 template <int K>
@@ -335,13 +293,13 @@ __device__ __forceinline__ void store_n(const MdIO &io, int p, int r, int, size_
     const MdFuse &f = io.f;
     const int job = p >> 1, c = p & 1;
     const u64 q = io.pr[r].q;
-    const Shoup tm{io.pr[r].t_mod, io.pr[r].t_mod_sh}, pinv = io.T.md_Pinv[r];
+    const Shoup pinv = io.T.md_Pinv[r], tp = io.T.md_ntP[r];
     const u64 *U = f.U + (size_t)p * f.ustride + ((size_t)r << io.logN);
     u64 res[K];
 #pragma unroll
     for (int i = 0; i < K; i++) res[i] = U[k0 + (size_t)i * dk];
 #pragma unroll
-    for (int i = 0; i < K; i++) res[i] = mul_shoup(sub_mod(res[i], mul_shoup(v[i], tm, q), q), pinv, q);
+    for (int i = 0; i < K; i++) res[i] = mul2_shoup(res[i], pinv, v[i], tp, q);
     if (c < f.add_comps && f.add[job]) {
         const u64 *a = f.add[job] + (size_t)c * f.acomp + ((size_t)r << io.logN);
         const u64 gal = f.gal[job];
@@ -364,13 +322,13 @@ __device__ __forceinline__ void store_n(const MddIO &io, int p, int r, int, size
     const MddFuse &f = io.f;
     const u64 q = io.pr[r].q;
     const size_t n = (size_t)1 << io.logN;
-    const Shoup tm{io.pr[r].t_mod, io.pr[r].t_mod_sh}, binv = io.T.mdd_Binv[(size_t)f.ell * io.L + r];
+    const Shoup binv = io.T.mdd_Binv[(size_t)f.ell * io.L + r], tb = io.T.mdd_ntB[(size_t)f.ell * io.L + r];
     const u64 *U = f.U + (size_t)p * f.ustride + ((size_t)r << io.logN);
     u64 res[K];
 #pragma unroll
     for (int i = 0; i < K; i++) res[i] = U[k0 + (size_t)i * dk];
 #pragma unroll
-    for (int i = 0; i < K; i++) res[i] = mul_shoup(sub_mod(res[i], mul_shoup(v[i], tm, q), q), binv, q);
+    for (int i = 0; i < K; i++) res[i] = mul2_shoup(res[i], binv, v[i], tb, q);
     u64 *out;
     if (!f.outp[0]) {
         out = f.out + ((size_t)p * (f.ell - 1) + r) * n;

@@ -115,7 +115,7 @@ copse_status launch_plain(copse_ctx *ctx, const NttBatch &b, cudaStream_t s) {
 template <bool INV = false, class IO>
 copse_status launch_fused(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s, bool *done) {
     *done = b.npoly <= 0 || b.nr <= 0;
-    if (*done || !ctx->ntt_clusters || ctx->logN < 12) return COPSE_OK;
+    if (*done || !ntt_fuses(ctx)) return COPSE_OK;
     STATUS_TRY((launch_io<INV>(ctx, b, io, (u64 *)nullptr, ctx->ntt_fused_max, s)));
     *done = true;
     return COPSE_OK;

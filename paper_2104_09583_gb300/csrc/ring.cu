@@ -708,6 +708,7 @@ copse_status moddown_apply(copse_ctx *c, u64 *U, int ell, int nj, MdFuse &f, Scr
     f.ell = ell;
     NttBatch ib = batch(U, (size_t)nx * N, 2 * nj, ell, A, ell);
     ib.scale = c->ks.md_scale;  // the conversion's first step (md_inv) folded in
+    ib.digits = ntt_fuses(c);
     STATUS_TRY(ntt_inverse(c, ib, s));
     bool done = false;
     STATUS_TRY(ntt_forward_moddown(c, f, nj, s, &done));
@@ -952,6 +953,7 @@ static copse_status mul_group(copse_ctx *c, const copse_evk *evk, const std::vec
     // conversion + transform + finish (or conversion, transform, finish)
     NttBatch ib = batch(U, (size_t)nx * N, 2 * nj, ell - 1, A + 1, ell);
     ib.scale = c->ks.mdd_scale + (size_t)ell * (A + 1);  // the conversion's first step (mdd_inv) folded in
+    ib.digits = ntt_fuses(c);
     STATUS_TRY(ntt_inverse(c, ib, s));
     if (join_lane >= 0) {
         STATUS_TRY(fork_join(c, s, 1, join_lane));
