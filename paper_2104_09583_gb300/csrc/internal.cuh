@@ -322,9 +322,9 @@ struct copse_ctx {
     u64 *d_psi_sh = nullptr;
     u64 *d_ipsi = nullptr;            // [NP][N] psi^-brev(k)
     u64 *d_ipsi_sh = nullptr;
-    u64 *d_tw_f = nullptr;            // N >= 2^12: (w, w') pairs of psi^brev(k), [NP][N][2],
+    u64 *d_tw_f = nullptr;            // N >= 2^8: (w, w') pairs of psi^brev(k), [NP][N][2],
     u64 *d_tw_i = nullptr;            //   and of psi^-brev(k)
-    u64 *d_low_f = nullptr;           // the low row stages' pairs in the order of the threads that use
+    u64 *d_low_f = nullptr;           // N >= 2^12: the low row stages' pairs in the order of the threads that use
     u64 *d_low_i = nullptr;           //   them, [NP][N / 2048][pairs][128][2] (ntt_core.cuh)
     uint32_t *d_slot_index = nullptr; // [N] NTT(mod t) position of slot s
     KsTables ks{};
@@ -413,13 +413,13 @@ struct NttBatch {
     // inverse transforms: when set, residue r's result is scaled by scale[r - r0] instead of
     // N^-1 (the first step of the base conversion that reads it folded in: N^-1 * c mod q)
     const Shoup *scale = nullptr;
-    // inverse transforms (2^12 <= N): results x stored as digits of a fused conversion,
+    // inverse transforms (N >= 2^8): results x stored as digits of a fused conversion,
     // x + (q - 1) / 2 mod q split at 28 bits (low word, high word)
     bool digits = false;
 };
 // whether the conversions around key switches and modulus switches run fused with the transforms
 // (their digits are then stored as above)
-inline bool ntt_fuses(const copse_ctx *c) { return c->ntt_clusters && c->logN >= 12; }
+inline bool ntt_fuses(const copse_ctx *c) { return c->ntt_clusters && c->logN >= 8; }
 // the transforms' twiddle tables (context creation)
 copse_status ntt_stage_tables(copse_ctx *ctx);
 copse_status ntt_forward(copse_ctx *ctx, const NttBatch &b, cudaStream_t s);
@@ -473,7 +473,7 @@ struct MddFuse {
 };
 copse_status ntt_forward_moddown_drop(copse_ctx *ctx, const MddFuse &f, int npoly, cudaStream_t s, bool *done);
 copse_status moddown_drop_unfused(copse_ctx *ctx, const MddFuse &f, int npoly, cudaStream_t s);
-// The fused forms run where ntt_fuses says (2^12 <= N); *done = false (nothing launched)
+// The fused forms run where ntt_fuses says (N >= 2^8); *done = false (nothing launched)
 // otherwise, and the caller takes the unfused sequence.
 copse_status ntt_forward_modswitch(copse_ctx *ctx, const MsFuse &f, int nc, cudaStream_t s, bool *done);
 copse_status ntt_forward_moddown(copse_ctx *ctx, const MdFuse &f, int njobs, cudaStream_t s, bool *done);

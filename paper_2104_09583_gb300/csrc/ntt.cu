@@ -11,8 +11,8 @@
 //
 // Rings of N >= 2^12 run as N = N1 x N2, N1 rows of N2 contiguous coefficients: the first
 // log2(N1) forward stages pair coefficients of one column, the others of one row
-// (ntt_core.cuh; the launches in ntt_launch.cuh, ntt_fwd.cu and ntt_inv.cu).  Smaller rings
-// use one block per polynomial (here).
+// (ntt_core.cuh; the launches in ntt_launch.cuh, ntt_fwd.cu, ntt_fwd_ks.cu and ntt_inv.cu).
+// Smaller rings use one block per polynomial (below 2^8: here).
 #include <cstdlib>
 
 #include "ntt_launch.cuh"
@@ -167,7 +167,7 @@ copse_status ntt_small(copse_ctx *ctx, const NttBatch &b, cudaStream_t s, bool i
 }
 
 copse_status ntt_stage_tables(copse_ctx *ctx) {
-    if (ctx->logN < 12) return COPSE_OK;   // one block per transform below 2^12
+    if (ctx->logN < 8) return COPSE_OK;
     if (ctx->logN == 15) {
         // 16-block clusters are above the portable size: an option (COPSE_NTT_CLUSTER16=1) where
         // the device can place at least one
@@ -188,20 +188,23 @@ copse_status ntt_stage_tables(copse_ctx *ctx) {
         ctx->ntt_cluster16 = e == cudaSuccess && nclusters > 0 && opt && opt[0] == '1';
         cudaGetLastError();
     }
+    // one block per transform below 2^12: no low row stages
     const int lb = ctx->logN - ctx->logN / 2, pairs = lb == 8 ? 15 : (lb == 7 ? 14 : 12);
-    const size_t n = (size_t)ctx->NP * ctx->N, nl = (size_t)ctx->NP * (ctx->N / TILE) * pairs * NTHR;
+    const size_t n = (size_t)ctx->NP * ctx->N;
+    const size_t nl = ctx->logN < 12 ? 0 : (size_t)ctx->NP * (ctx->N / TILE) * pairs * NTHR;
     for (int inv = 0; inv < 2; inv++) {
         void *p = nullptr, *l = nullptr;
         CUDA_TRY(cudaMalloc(&p, n * sizeof(ulonglong2)));
         ctx->owned.push_back(p);
-        CUDA_TRY(cudaMalloc(&l, nl * sizeof(ulonglong2)));
-        ctx->owned.push_back(l);
         const u64 *W = inv ? ctx->d_ipsi : ctx->d_psi, *Wp = inv ? ctx->d_ipsi_sh : ctx->d_psi_sh;
         k_pairs<<<(unsigned)((n + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)p, n);
         CUDA_TRY(cudaGetLastError());
+        (inv ? ctx->d_tw_i : ctx->d_tw_f) = (u64 *)p;
+        if (!nl) continue;
+        CUDA_TRY(cudaMalloc(&l, nl * sizeof(ulonglong2)));
+        ctx->owned.push_back(l);
         k_low_pairs<<<(unsigned)((nl + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)l, ctx->NP, ctx->logN, pairs, inv);
         CUDA_TRY(cudaGetLastError());
-        (inv ? ctx->d_tw_i : ctx->d_tw_f) = (u64 *)p;
         (inv ? ctx->d_low_i : ctx->d_low_f) = (u64 *)l;
     }
     CUDA_TRY(cudaDeviceSynchronize());

@@ -1,4 +1,4 @@
-// The transform kernels for 2^12 <= N <= 2^15: N = 2^A rows of 2^LB coefficients, the first A
+// The transform kernels.  For 2^12 <= N <= 2^15: N = 2^A rows of 2^LB coefficients, the first A
 // forward stages over columns, the last LB over rows, the inverse the other way round (the
 // stage order, twiddle order and lazy ranges are stated in ntt.cu).
 //
@@ -265,6 +265,17 @@ __device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int 
     for (int m = 0; m < 16; m++) v[m] = reduce64_lazy(v[m], P);
 }
 
+// an inverse transform's result: scaled, and stored as a conversion's digit where asked (centred,
+// offset by (q - 1) / 2, split at 28 bits)
+__device__ __forceinline__ u64 inv_result(u64 v, Shoup sc, bool digits, u64 q) {
+    u64 x = mul_shoup(v, sc, q);
+    if (digits) {
+        x = add_mod(x, (q - 1) / 2, q);
+        x = ((x >> 28) << 32) | (x & 0x0FFFFFFFu);
+    }
+    return x;
+}
+
 // Inverse column half: v holds rows 16 b .. 16 b + 15 of the thread's column (below 2q); all A
 // column stages, scaled and stored through io.
 template <int LOGN, class IO>
@@ -280,14 +291,8 @@ __device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int 
     for (int m = 0; m < 16; m++) v[m] = sm[((i + m * S::SA) << S::LC) + c];
     stages_inv<4>(v, q, (2 * q) << (S::A - 4), TwInvColTop{T});
 #pragma unroll
-    for (int m = 0; m < 16; m++) {
-        u64 x = mul_shoup(v[m], sc, q);
-        if (digits) {  // centred, offset by (q - 1) / 2, split at 28 bits
-            x = add_mod(x, (q - 1) / 2, q);
-            x = ((x >> 28) << 32) | (x & 0x0FFFFFFFu);
-        }
-        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, x);
-    }
+    for (int m = 0; m < 16; m++)
+        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m], sc, digits, q));
 }
 
 // ---------------------------------------------------------------- tiled: two launches
@@ -449,6 +454,101 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     for (int m = 0; m < 16; m++) v[m] = colt[((16 * ic + m) << S::LC) + c];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
     inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, T, sc, b.digits, P.q, colt, v);
+}
+
+// ---------------------------------------------------------------- 2^8 <= N <= 2^11: one block
+// A block of N / 16 threads holds one residue polynomial, 16 coefficients a thread: the first
+// four stages, the next four and the remaining LOGN - 8 in registers, with an exchange through
+// shared memory between them (a stage per exchange before: 5.6 us at N = 2^10 and 9.6 us at
+// N = 2^11 for any batch that fits the GPU).
+template <int LOGN, class IO>
+__global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_constant__ NttBatch b, NttTables tb,
+                                                                 const __grid_constant__ IO io) {
+    constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;  // SP: threads per sixteenth
+    __shared__ u64 sm[(1 << LOGN) + NT];
+    const TileAt t = tile_at(b, tb.L, 1);
+    if (ntt_skipped(b, t.p, t.r)) {
+        io.skip(t.p, t.r, 0, 1);
+        return;
+    }
+    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    const PrimeDev P = tb.pr[t.g];
+    const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
+    u64 v[16];
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+        u64 x[4];
+        load_n(io, t.p, t.r, t.g, (size_t)(th + 4 * h * NT), NT, x);
+#pragma unroll
+        for (int m = 0; m < 4; m++) v[4 * h + m] = x[m];
+    }
+    stages_fwd<4>(v, P.q, 2 * P.q, TwColTop{T});
+#pragma unroll
+    for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
+    stages_fwd<4>(v, P.q, 2 * P.q, TwRowTop<4>{T, blk});
+    if (LS > 0) {
+#pragma unroll
+        for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = v[m];
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
+        stages_fwd<LS>(v, P.q, 2 * P.q, [&](int s, int il) { return ldg2(T + (1 << (8 + s)) + ((16 * th) >> (LS - s)) + il); });
+    }
+#pragma unroll
+    for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+        u64 x[4];
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            x[m] = sm[pad(th + (4 * h + m) * NT)];
+            if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
+        }
+        store_n(io, t.p, t.r, t.g, (size_t)(th + 4 * h * NT), NT, x);
+    }
+}
+
+template <int LOGN, class IO>
+__global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_constant__ NttBatch b, NttTables tb,
+                                                                 const __grid_constant__ IO io) {
+    constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;
+    __shared__ u64 sm[(1 << LOGN) + NT];
+    const TileAt t = tile_at(b, tb.L, 1);
+    if (ntt_skipped(b, t.p, t.r)) return;
+    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    const PrimeDev P = tb.pr[t.g];
+    const u64 q = P.q;
+    const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
+    u64 v[16];
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] = io.load(t.p, t.r, t.g, (size_t)(th + m * NT));
+#pragma unroll
+    for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
+    __syncthreads();
+    if (LS > 0) {
+#pragma unroll
+        for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
+        stages_inv<LS>(v, q, q, [&](int s, int il) { return ldg2(T + (1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il); });
+#pragma unroll
+        for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
+    stages_inv<4>(v, q, q << LS, TwInvRowTop<4>{T, blk});
+#pragma unroll
+    for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = reduce64_lazy(v[m], P);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] = sm[pad(th + m * NT)];
+    stages_inv<4>(v, q, 2 * q, TwInvColTop{T});
+    const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
+#pragma unroll
+    for (int m = 0; m < 16; m++) io.store(t.p, t.r, t.g, (size_t)(th + m * NT), inv_result(v[m], sc, b.digits, q));
 }
 
 }  // namespace

@@ -5,7 +5,7 @@
 
 #include "ntt_core.cuh"
 
-// one block per residue polynomial, in place (N <= 2^11; ntt.cu)
+// one block per residue polynomial, in place, a stage per barrier (N <= 2^7; ntt.cu)
 copse_status ntt_small(copse_ctx *ctx, const NttBatch &b, cudaStream_t s, bool inverse);
 
 namespace {
@@ -79,6 +79,20 @@ copse_status launch_tiled(copse_ctx *ctx, const NttBatch &b, const IO &io, const
     return COPSE_OK;
 }
 
+template <int LOGN, bool INV, class IO>
+copse_status launch_one(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s) {
+    const unsigned grid = (unsigned)b.npoly * (unsigned)b.nr;
+    const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;
+    TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
+        if constexpr (INV)
+            k_ntt_inv_one<LOGN, IO><<<grid, 1 << (LOGN - 4), 0, s>>>(b, tables<true>(ctx), io);
+        else
+            k_ntt_fwd_one<LOGN, IO><<<grid, 1 << (LOGN - 4), 0, s>>>(b, tables<false>(ctx), io);
+    });
+    LAUNCH_CHECK();
+    return COPSE_OK;
+}
+
 // A batch of b with this IO: clusters up to max_cluster residue polynomials (N = 2^15 only where
 // 16-block clusters are opted in), else two launches through `data` (in place) or, when it is
 // null, through scratch.
@@ -96,6 +110,10 @@ copse_status launch_ring(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *d
 template <bool INV, class IO>
 copse_status launch_io(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *data, long max_cluster, cudaStream_t s) {
     switch (ctx->logN) {
+        case 8: return launch_one<8, INV, IO>(ctx, b, io, s);
+        case 9: return launch_one<9, INV, IO>(ctx, b, io, s);
+        case 10: return launch_one<10, INV, IO>(ctx, b, io, s);
+        case 11: return launch_one<11, INV, IO>(ctx, b, io, s);
         case 12: return launch_ring<12, INV, IO>(ctx, b, io, data, max_cluster, s);
         case 13: return launch_ring<13, INV, IO>(ctx, b, io, data, max_cluster, s);
         case 14: return launch_ring<14, INV, IO>(ctx, b, io, data, max_cluster, s);
@@ -107,11 +125,11 @@ copse_status launch_io(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *dat
 template <bool INV>
 copse_status launch_plain(copse_ctx *ctx, const NttBatch &b, cudaStream_t s) {
     if (b.npoly <= 0 || b.nr <= 0) return COPSE_OK;
-    if (ctx->logN < 12) return ntt_small(ctx, b, s, INV);
+    if (ctx->logN < 8) return ntt_small(ctx, b, s, INV);
     return launch_io<INV>(ctx, b, PlainIO{b.data, b.stride, ctx->logN}, b.data, ctx->ntt_cluster_max, s);
 }
 
-// fused with the IO (*done = false, nothing launched, below 2^12 and with the fused forms off)
+// fused with the IO (*done = false, nothing launched, below 2^8 and with the fused forms off)
 template <bool INV = false, class IO>
 copse_status launch_fused(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s, bool *done) {
     *done = b.npoly <= 0 || b.nr <= 0;

@@ -1,5 +1,5 @@
-"""The transforms of every ring of two passes (N = 2^12 .. 2^15: each split into columns and rows
-has its own stage counts and tile shapes), in one launch (clusters) and in two (tiled), plain and
+"""The transforms of every ring from N = 2^8 on (each has its own stage counts and tile shapes: one
+block below 2^12, else columns and rows in one launch, clusters, and in two, tiled), plain and
 fused with the base conversions, against the oracle coefficient for coefficient (tolerance zero):
 import and export (plain both ways), a product (ModUp; relinearise and drop), a rotation (ModUp;
 ModDown with a permuted addend), a modulus switch, at 55-bit primes and digits of one, two and
@@ -22,7 +22,7 @@ from test_gpu_parity import assert_same  # noqa: E402
 ALWAYS = 1 << 30
 
 
-@pytest.mark.parametrize("log_n,dnum", [(12, 5), (12, 2), (13, 3), (14, 2), (15, 3)])
+@pytest.mark.parametrize("log_n,dnum", [(8, 3), (9, 5), (10, 2), (11, 3), (12, 5), (12, 2), (13, 3), (14, 2), (15, 3)])
 def test_ring_operations_match_the_oracle(log_n, dnum):
     L, N = 5, 1 << log_n
     P = B.Params(logN=log_n, L=L, bits=55, dnum=dnum)
@@ -58,7 +58,7 @@ def test_ring_operations_match_the_oracle(log_n, dnum):
         K.copse_ctx_destroy(ctx)
 
 
-@pytest.mark.parametrize("log_n", [12, 13])
+@pytest.mark.parametrize("log_n", [8, 9, 11, 12, 13])
 @pytest.mark.parametrize("most", [ALWAYS, 0])
 def test_negacyclic_product_matches_the_oracle(log_n, most):
     P = B.Params(logN=log_n, L=3, bits=55, dnum=3)
