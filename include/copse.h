@@ -454,7 +454,8 @@ copse_status copse_ctx_set_ntt_cluster_max(copse_ctx *ctx, uint32_t max_cluster)
  * is the current setting. */
 copse_status copse_tune_fused(copse_ctx *ctx, copse_model *model, const uint32_t *cands, size_t n,
                               size_t n_queries, int reps, float *ms, uint32_t *best);
-/* Set the fused crossover copse_tune_fused would choose (default: always clusters). */
+/* Set the fused crossover copse_tune_fused would choose (default: as
+ * many residue polynomials as the GPU holds clusters of at once). */
 copse_status copse_ctx_set_ntt_fused_max(copse_ctx *ctx, uint32_t max_fused);
 /* Which kernel multiplies an encrypted model's diagonals with the rotations (the products of
  * Section 4.3 with the diagonals encrypted, Section 8.3): COPSE_ENC_MAC_AUTO (the default)

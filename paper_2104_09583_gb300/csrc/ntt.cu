@@ -128,6 +128,7 @@ __global__ void k_md_finish_io(const MdFuse f, const u64 *W, int njobs, const Pr
 // forward stage s of thread t takes 16 >> (K - s) pairs of transform stage A + 4 + s from
 // coefficient 16 t of its tile on, inverse stage s takes 8 >> s pairs of distance 2^s
 // (K = LB - 4 low stages).
+constexpr long CLUSTER_BLOCKS = 400;
 __global__ void k_pairs(const u64 *W, const u64 *Wp, ulonglong2 *out, size_t n) {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e < n) out[e] = make_ulonglong2(W[e], Wp[e]);
@@ -171,10 +172,12 @@ copse_status ntt_stage_tables(copse_ctx *ctx) {
     if (ctx->logN == 15) {
         // 16-block clusters are above the portable size: an option (COPSE_NTT_CLUSTER16=1) where
         // the device can place at least one
-        CUDA_TRY(cudaFuncSetAttribute(k_ntt_fwd_cluster<15, PlainIO>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        std::atomic<uint64_t> none{0};
+        STATUS_TRY(cluster_attr<15>(k_ntt_fwd_cluster<15, PlainIO>, -1, none));
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(16);
         cfg.blockDim = dim3(NTHR);
+        cfg.dynamicSmemBytes = sizeof(ClusterSmem<15>);
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = 16;
@@ -188,6 +191,12 @@ copse_status ntt_stage_tables(copse_ctx *ctx) {
         ctx->ntt_cluster16 = e == cudaSuccess && nclusters > 0 && opt && opt[0] == '1';
         cudaGetLastError();
     }
+    // Clusters up to about the blocks that fit the GPU at once (three of a cluster kernel's blocks
+    // per SM), two launches above; the tuner or the caller may set other crossovers.  Measured at
+    // N = 2^14 (us a forward transform in a graph, clusters / tiled): 16 residue polynomials
+    // 9.5 / 8.1, 32: 9.8 / 10.1, 48: 12.5 / 12.9, 64: 22.2 / 15.5, 128: 32.9 / 23.7; whole
+    // inferences are flat between 32 and 64.
+    if (ctx->logN >= 12 && ctx->logN < 15) ctx->ntt_cluster_max = ctx->ntt_fused_max = CLUSTER_BLOCKS >> (ctx->logN - 11);
     // one block per transform below 2^12: no low row stages
     const int lb = ctx->logN - ctx->logN / 2, pairs = lb == 8 ? 15 : (lb == 7 ? 14 : 12);
     const size_t n = (size_t)ctx->NP * ctx->N;

@@ -16,13 +16,14 @@
 // in global memory between them, any batch size.  Cluster: N / 2048 blocks of a thread-block
 // cluster own one residue polynomial and hand the tiles over through distributed shared memory,
 // each thread writing its 16 outputs of the first half into the blocks that take them on: one
-// launch, for batches too small to fill the GPU.
+// launch, for batches too small to fill the GPU (one residue polynomial at N = 2^14: 7.1 us in a
+// graph, 7.9 with 512 threads and four coefficients a thread).
 //
 // Measured (us, forward / inverse; before = a radix-4 / radix-8 pass per two or three stages with
 // 512 / 256 threads and every twiddle staged through shared memory): N = 2^15, 1024 residue
 // polynomials 616 / 644 before, 331 / 359 now (0.76 / 0.70 T butterflies/s of the 0.95 that the
 // multiplier alone reaches), 64: 43 / 47 before, 29 / 31 now; N = 2^14, 1024 in clusters
-// 269 / 313 before, 178 / 185 now.
+// 269 / 313 before, 163 / 178 tiled now.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -116,27 +117,33 @@ __device__ __forceinline__ void stages_inv(u64 (&v)[16], u64 q, u64 c0, TW tw) {
     }
 }
 
-__device__ __forceinline__ ulonglong2 ldg2(const ulonglong2 *p) { return __ldg(p); }
+// a twiddle pair from global memory, or (SH) from the block's copy in shared memory
+template <bool SH>
+__device__ __forceinline__ ulonglong2 pair_at(const ulonglong2 *p) {
+    if constexpr (SH) return *p;
+    else return __ldg(p);
+}
 // Row tiles keep coefficient f of the tile at word f + f / 16 of shared memory: 16 threads that
 // read 16 consecutive coefficients each hit different banks, as do 16 that read a run.
 constexpr int PTILE = TILE + TILE / 16;
 __device__ __forceinline__ int pad(int f) { return f + (f >> 4); }
 
 // twiddles of the passes (T: the prime's pairs in natural order, low: this tile's low row pairs
-// of this thread, [pair][thread])
+// of this thread, [pair][thread]); the column stages use the first 2^A pairs only
 //
 // forward column stages 0..3: the whole transform's first 15 twiddles
+template <bool SH>
 struct TwColTop {
     const ulonglong2 *T;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return ldg2(T + (1 << s) + il); }
+    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return pair_at<SH>(T + (1 << s) + il); }
 };
 // forward column stages 4..A-1 of rows 16 b ..
-template <int A>
+template <int A, bool SH>
 struct TwColLow {
     const ulonglong2 *T;
     int b;
     __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return ldg2(T + (1 << (4 + s)) + ((16 * b) >> (A - 4 - s)) + il);
+        return pair_at<SH>(T + (1 << (4 + s)) + ((16 * b) >> (A - 4 - s)) + il);
     }
 };
 // forward row stages 0..3 of one row
@@ -145,31 +152,43 @@ struct TwRowTop {
     const ulonglong2 *T;
     int row;
     __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return ldg2(T + (1 << (A + s)) + (row << s) + il);
+        return pair_at<false>(T + (1 << (A + s)) + (row << s) + il);
+    }
+};
+// the same, and the last four inverse row stages, from a copy of the 15 pairs of each of a tile's
+// R rows, those of 2^u groups per row at R (2^u - 1) (gr: the row within the tile)
+template <int R, bool INV>
+struct TwRowTopSh {
+    const ulonglong2 *W;
+    int gr;
+    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
+        const int u = INV ? 3 - s : s;
+        return W[R * ((1 << u) - 1) + (gr << u) + il];
     }
 };
 // low row stages in thread order: the pairs of stage s follow those of the stages before
-template <int K, bool INV>
+template <int K, bool INV, bool SH>
 struct TwRowLow {
     const ulonglong2 *low;
     __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
         const int off = INV ? 16 - (16 >> s) : (16 >> (K - s)) - (16 >> K);
-        return ldg2(low + (off + il) * NTHR);
+        return pair_at<SH>(low + (off + il) * NTHR);
     }
 };
 // inverse column stages of distance 2^s rows, rows 16 b ..
-template <int A>
+template <int A, bool SH>
 struct TwInvColLow {
     const ulonglong2 *T;
     int b;
     __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return ldg2(T + (1 << (A - 1 - s)) + ((16 * b) >> (s + 1)) + il);
+        return pair_at<SH>(T + (1 << (A - 1 - s)) + ((16 * b) >> (s + 1)) + il);
     }
 };
 // the last four inverse column stages
+template <bool SH>
 struct TwInvColTop {
     const ulonglong2 *T;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return ldg2(T + (1 << (3 - s)) + il); }
+    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return pair_at<SH>(T + (1 << (3 - s)) + il); }
 };
 // the last four inverse row stages of one row
 template <int A>
@@ -177,72 +196,82 @@ struct TwInvRowTop {
     const ulonglong2 *T;
     int row;
     __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return ldg2(T + (1 << (A + 3 - s)) + (row << (3 - s)) + il);
+        return pair_at<false>(T + (1 << (A + 3 - s)) + (row << (3 - s)) + il);
     }
 };
 
 // ---------------------------------------------------------------- the halves of a transform
-// Forward column half: the tile's coefficients through io.load, all A column stages; the
-// thread ends with rows 16 b .. 16 b + 15 of its column.
-template <int LOGN, class IO>
+// Forward column half: the tile's coefficients through io (KL at a time), all A column stages;
+// the thread ends with rows 16 b .. 16 b + 15 of its column.  SH: the first 2^A pairs at T are
+// the block's copy, complete after `arrived`.
+template <int LOGN, int KL, bool SH, class IO, class ARR>
 __device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T, u64 q,
-                                         u64 *sm, u64 (&v)[16]) {
+                                         u64 *sm, u64 (&v)[16], ARR arrived) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
     const size_t n0 = ((size_t)i << S::LB) + (tile << S::LC) + c, dn = (size_t)S::SA << S::LB;
 #pragma unroll
-    for (int h = 0; h < 4; h++) {
-        u64 x[4];
-        load_n(io, p, r, g, n0 + 4 * h * dn, dn, x);
+    for (int h = 0; h < 16 / KL; h++) {
+        u64 x[KL];
+        load_n(io, p, r, g, n0 + KL * h * dn, dn, x);
 #pragma unroll
-        for (int m = 0; m < 4; m++) v[4 * h + m] = x[m];
+        for (int m = 0; m < KL; m++) v[KL * h + m] = x[m];
     }
-    stages_fwd<4>(v, q, 2 * q, TwColTop{T});
+    arrived();
+    stages_fwd<4>(v, q, 2 * q, TwColTop<SH>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[((i + m * S::SA) << S::LC) + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((16 * i + m) << S::LC) + c];
-    stages_fwd<S::A - 4>(v, q, 2 * q, TwColLow<S::A>{T, i});
+    stages_fwd<S::A - 4>(v, q, 2 * q, TwColLow<S::A, SH>{T, i});
 }
 
 // Forward row half: v holds coefficients i + m SB of the thread's row (i = t mod SB); all LB row
-// stages, the values stored through io (reduced unless it takes them raw).
-template <int LOGN, class IO>
-__device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T,
-                                         const ulonglong2 *low, const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
+// stages, the values stored through io (reduced unless it takes them raw).  u: the finishes'
+// operands where they are loaded ahead (EARLY), in the order of the stores.
+template <int LOGN, bool EARLY, class IO, class TOP, class LOW>
+__device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int tile, TOP top, LOW low,
+                                         const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, i = t & (S::SB - 1), gr = t / S::SB;
     const u64 q = P.q;
-    stages_fwd<4>(v, q, 2 * q, TwRowTop<S::A>{T, (tile << S::LR) + gr});
+    const int f0 = (t & ~31) * 16 + (t & 31);
+    const size_t k0 = ((size_t)tile << 11) + f0;
+    u64 u[4][4];
+    if (EARLY) {
+#pragma unroll
+        for (int h = 0; h < 4; h++) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
+    }
+    stages_fwd<4>(v, q, 2 * q, top);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad((gr << S::LB) + i + m * S::SB)] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * t + m)];
-    stages_fwd<S::LB - 4>(v, q, 2 * q, TwRowLow<S::LB - 4, false>{low});
+    stages_fwd<S::LB - 4>(v, q, 2 * q, low);
     // to runs of 32 coefficients per warp access, within the warp's 512
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(16 * t + m)] = v[m];
     __syncwarp();
-    const int f0 = (t & ~31) * 16 + (t & 31);
 #pragma unroll
     for (int h = 0; h < 4; h++) {
         u64 x[4];
+        if (!EARLY) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
 #pragma unroll
         for (int m = 0; m < 4; m++) {
             x[m] = sm[pad(f0 + 32 * (4 * h + m))];
             if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
         }
-        store_n(io, p, r, g, ((size_t)tile << 11) + f0 + 128 * h, 32, x);
+        store_n(io, p, r, g, k0 + 128 * h, 32, x, u[h]);
     }
 }
 
 // Inverse row half: the tile through io.load, all LB row stages; the thread ends with
-// coefficients i + m SB of its row, reduced below 2q.
-template <int LOGN, class IO>
-__device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T,
-                                         const ulonglong2 *low, const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
+// coefficients i + m SB of its row, reduced below 2q.  `arrived`: the twiddles' copies complete.
+template <int LOGN, class IO, class TOP, class LOW, class ARR>
+__device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int tile, TOP top, LOW low,
+                                         const PrimeDev &P, u64 *sm, u64 (&v)[16], ARR arrived) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, i = t & (S::SB - 1), gr = t / S::SB;
     const u64 q = P.q;
@@ -251,16 +280,17 @@ __device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int 
     for (int m = 0; m < 16; m++) v[m] = io.load(p, r, g, ((size_t)tile << 11) + f0 + 32 * m);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(f0 + 32 * m)] = v[m];
+    arrived();
     __syncwarp();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * t + m)];
-    stages_inv<S::LB - 4>(v, q, q, TwRowLow<S::LB - 4, true>{low});
+    stages_inv<S::LB - 4>(v, q, q, low);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(16 * t + m)] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad((gr << S::LB) + i + m * S::SB)];
-    stages_inv<4>(v, q, q << (S::LB - 4), TwInvRowTop<S::A>{T, (tile << S::LR) + gr});
+    stages_inv<4>(v, q, q << (S::LB - 4), top);
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = reduce64_lazy(v[m], P);
 }
@@ -278,18 +308,18 @@ __device__ __forceinline__ u64 inv_result(u64 v, Shoup sc, bool digits, u64 q) {
 
 // Inverse column half: v holds rows 16 b .. 16 b + 15 of the thread's column (below 2q); all A
 // column stages, scaled and stored through io.
-template <int LOGN, class IO>
+template <int LOGN, bool SH, class IO>
 __device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T, Shoup sc,
                                          bool digits, u64 q, u64 *sm, u64 (&v)[16]) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
-    stages_inv<S::A - 4>(v, q, 2 * q, TwInvColLow<S::A>{T, i});
+    stages_inv<S::A - 4>(v, q, 2 * q, TwInvColLow<S::A, SH>{T, i});
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[((16 * i + m) << S::LC) + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((i + m * S::SA) << S::LC) + c];
-    stages_inv<4>(v, q, (2 * q) << (S::A - 4), TwInvColTop{T});
+    stages_inv<4>(v, q, (2 * q) << (S::A - 4), TwInvColTop<SH>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++)
         io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m], sc, digits, q));
@@ -316,6 +346,11 @@ __device__ __forceinline__ TileAt tile_at(const NttBatch &b, int L, int tiles) {
     t.g = ntt_prime(b, t.r, L);
     return t;
 }
+// the low row pairs of a tile within their table
+template <int LOGN>
+__device__ __forceinline__ size_t low_at(const TileAt &t) {
+    return ((size_t)t.g * Shape<LOGN>::TILES + t.tile) * Shape<LOGN>::PAIRS * NTHR;
+}
 // constant tables of a launch
 struct NttTables {
     const PrimeDev *pr;
@@ -336,7 +371,7 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_cols(const __grid_
         return;
     }
     u64 v[16];
-    fwd_cols<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), tb.pr[t.g].q, sm, v);
+    fwd_cols<LOGN, 4, false>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), tb.pr[t.g].q, sm, v, [] {});
     const int c = threadIdx.x & (S::C - 1), i = threadIdx.x >> S::LC;
     u64 *o = mid.base + t.p * mid.ps + ((size_t)(t.r - mid.r0) << LOGN) + ((size_t)t.tile << S::LC) + c;
 #pragma unroll
@@ -356,8 +391,9 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_rows(const __grid_
     u64 v[16];
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = in[m * S::SB];
-    fwd_rows<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN),
-                   tb.low + ((size_t)t.g * S::TILES + t.tile) * S::PAIRS * NTHR + th, tb.pr[t.g], sm, v);
+    fwd_rows<LOGN, false>(io, t.p, t.r, t.g, t.tile,
+                          TwRowTop<S::A>{tb.tw + ((size_t)t.g << LOGN), (t.tile << S::LR) + gr},
+                          TwRowLow<S::LB - 4, false, false>{tb.low + low_at<LOGN>(t) + th}, tb.pr[t.g], sm, v);
 }
 
 template <int LOGN, class IO>
@@ -369,8 +405,9 @@ __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_rows(const __grid_
     if (ntt_skipped(b, t.p, t.r)) return;
     const int th = threadIdx.x, i = th & (S::SB - 1), gr = th / S::SB;
     u64 v[16];
-    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN),
-                   tb.low + ((size_t)t.g * S::TILES + t.tile) * S::PAIRS * NTHR + th, tb.pr[t.g], sm, v);
+    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile,
+                   TwInvRowTop<S::A>{tb.tw + ((size_t)t.g << LOGN), (t.tile << S::LR) + gr},
+                   TwRowLow<S::LB - 4, true, false>{tb.low + low_at<LOGN>(t) + th}, tb.pr[t.g], sm, v, [] {});
     u64 *o = mid.base + t.p * mid.ps + ((size_t)(t.r - mid.r0) << LOGN) + ((size_t)t.tile << 11) + (gr << S::LB) + i;
 #pragma unroll
     for (int m = 0; m < 16; m++) o[m * S::SB] = v[m];
@@ -390,15 +427,44 @@ __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_cols(const __grid_
     for (int m = 0; m < 16; m++) v[m] = in[(size_t)(16 * i + m) << S::LB];
     const PrimeDev P = tb.pr[t.g];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), sc, b.digits, P.q, sm, v);
+    inv_cols<LOGN, false>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), sc, b.digits, P.q, sm, v);
 }
 
 // ---------------------------------------------------------------- clusters: one launch
+// A batch this small waits for memory more than for the multiplier, so every twiddle of the
+// block is copied to shared memory from the start (asynchronous copies, in flight with the
+// coefficients), the conversions take eight coefficients at a time, and the finishes' operands
+// are loaded before the row stages.
+template <int LOGN>
+struct ClusterSmem {
+    u64 colt[TILE], rowt[PTILE];
+    ulonglong2 low[Shape<LOGN>::PAIRS * NTHR];  // [pair][thread]
+    ulonglong2 top[15 * Shape<LOGN>::R];        // TwRowTopSh
+    ulonglong2 col[1 << Shape<LOGN>::A];        // the prime's first 2^A pairs
+};
+// each thread copies the low pairs that it uses itself
+template <int LOGN>
+__device__ __forceinline__ void copy_twiddles(ClusterSmem<LOGN> &S, const NttTables &tb, const TileAt &t) {
+    using H = Shape<LOGN>;
+    const int th = threadIdx.x;
+    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN), *low = tb.low + low_at<LOGN>(t);
+    for (int e = th; e < (1 << H::A); e += NTHR) cp_async16(&S.col[e], T + e);
+    for (int e = th; e < 15 * H::R; e += NTHR) {
+        // entry R (2^u - 1) + k: pair 2^(A + u) + (row0 << u) + k
+        const int u = 31 - __clz(e / H::R + 1), k = e - H::R * ((1 << u) - 1);
+        cp_async16(&S.top[e], T + (1 << (H::A + u)) + ((t.tile << H::LR) << u) + k);
+    }
+#pragma unroll
+    for (int k = 0; k < H::PAIRS; k++) cp_async16(&S.low[k * NTHR + th], low + k * NTHR + th);
+    cp_async_commit();
+}
+
 template <int LOGN, class IO>
 __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTHR)
     k_ntt_fwd_cluster(const __grid_constant__ NttBatch b, NttTables tb, const __grid_constant__ IO io) {
     using S = Shape<LOGN>;
-    __shared__ u64 colt[TILE], rowt[PTILE];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    ClusterSmem<LOGN> &M = *reinterpret_cast<ClusterSmem<LOGN> *>(dyn_smem);
     cg::cluster_group cl = cg::this_cluster();
     const TileAt t = tile_at(b, tb.L, S::TILES);  // tile = the block's rank
     if (ntt_skipped(b, t.p, t.r)) {  // the same for every block of the cluster
@@ -406,54 +472,59 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
         return;
     }
     cl.barrier_arrive();  // every block runs: its row tile may be written
-    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    copy_twiddles<LOGN>(M, tb, t);
     const PrimeDev P = tb.pr[t.g];
     u64 v[16];
-    fwd_cols<LOGN>(io, t.p, t.r, t.g, t.tile, T, P.q, colt, v);
+    fwd_cols<LOGN, 8, true>(io, t.p, t.r, t.g, t.tile, M.col, P.q, M.colt, v, [] {
+        cp_async_wait<0>();
+        __syncthreads();
+    });
     cl.barrier_wait();
     const int th = threadIdx.x, c = th & (S::C - 1), ic = th >> S::LC, i = th & (S::SB - 1), gr = th / S::SB;
 #pragma unroll
     for (int h = 0; h < 16; h += (S::R < 16 ? S::R : 16)) {
         // rows 16 ic + h .. belong to one block: R rows a block, R a power of two >= 8
-        u64 *dst = cl.map_shared_rank(rowt, (16 * ic + h) >> S::LR);
+        u64 *dst = cl.map_shared_rank(M.rowt, (16 * ic + h) >> S::LR);
 #pragma unroll
         for (int m = h; m < h + (S::R < 16 ? S::R : 16); m++)
             dst[pad((((16 * ic + m) & (S::R - 1)) << S::LB) + (t.tile << S::LC) + c)] = v[m];
     }
     cl.sync();
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = rowt[pad((gr << S::LB) + i + m * S::SB)];
-    fwd_rows<LOGN>(io, t.p, t.r, t.g, t.tile, T, tb.low + ((size_t)t.g * S::TILES + t.tile) * S::PAIRS * NTHR + th, P,
-                   rowt, v);
+    for (int m = 0; m < 16; m++) v[m] = M.rowt[pad((gr << S::LB) + i + m * S::SB)];
+    fwd_rows<LOGN, true>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, false>{M.top, gr},
+                         TwRowLow<S::LB - 4, false, true>{M.low + th}, P, M.rowt, v);
 }
 
 template <int LOGN, class IO>
 __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTHR)
     k_ntt_inv_cluster(const __grid_constant__ NttBatch b, NttTables tb, const __grid_constant__ IO io) {
     using S = Shape<LOGN>;
-    __shared__ u64 colt[TILE], rowt[PTILE];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    ClusterSmem<LOGN> &M = *reinterpret_cast<ClusterSmem<LOGN> *>(dyn_smem);
     cg::cluster_group cl = cg::this_cluster();
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) return;
     cl.barrier_arrive();
-    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    copy_twiddles<LOGN>(M, tb, t);
     const PrimeDev P = tb.pr[t.g];
     const int th = threadIdx.x, i = th & (S::SB - 1), gr = th / S::SB, c = th & (S::C - 1), ic = th >> S::LC;
     u64 v[16];
-    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile, T, tb.low + ((size_t)t.g * S::TILES + t.tile) * S::PAIRS * NTHR + th, P,
-                   rowt, v);
+    // the low pairs are the thread's own copies; the others' are complete after the exchange's barrier
+    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, true>{M.top, gr},
+                   TwRowLow<S::LB - 4, true, true>{M.low + th}, P, M.rowt, v, [] { cp_async_wait<0>(); });
     cl.barrier_wait();
     const int row = (t.tile << S::LR) + gr;
 #pragma unroll
     for (int m = 0; m < 16; m++) {
         const int col = i + m * S::SB;
-        cl.map_shared_rank(colt, col >> S::LC)[(row << S::LC) + (col & (S::C - 1))] = v[m];
+        cl.map_shared_rank(M.colt, col >> S::LC)[(row << S::LC) + (col & (S::C - 1))] = v[m];
     }
     cl.sync();
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = colt[((16 * ic + m) << S::LC) + c];
+    for (int m = 0; m < 16; m++) v[m] = M.colt[((16 * ic + m) << S::LC) + c];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN>(io, t.p, t.r, t.g, t.tile, T, sc, b.digits, P.q, colt, v);
+    inv_cols<LOGN, true>(io, t.p, t.r, t.g, t.tile, M.col, sc, b.digits, P.q, M.colt, v);
 }
 
 // ---------------------------------------------------------------- 2^8 <= N <= 2^11: one block
@@ -461,41 +532,52 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
 // four stages, the next four and the remaining LOGN - 8 in registers, with an exchange through
 // shared memory between them (a stage per exchange before: 5.6 us at N = 2^10 and 9.6 us at
 // N = 2^11 for any batch that fits the GPU).
+template <int LOGN>
+__device__ __forceinline__ void copy_pairs(ulonglong2 *dst, const ulonglong2 *src) {
+#pragma unroll
+    for (int k = 0; k < 16; k++) cp_async16(dst + threadIdx.x + (k << (LOGN - 4)), src + threadIdx.x + (k << (LOGN - 4)));
+    cp_async_commit();
+}
 template <int LOGN, class IO>
 __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_constant__ NttBatch b, NttTables tb,
                                                                  const __grid_constant__ IO io) {
     constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;  // SP: threads per sixteenth
     __shared__ u64 sm[(1 << LOGN) + NT];
+    __shared__ ulonglong2 T[1 << LOGN];
     const TileAt t = tile_at(b, tb.L, 1);
     if (ntt_skipped(b, t.p, t.r)) {
         io.skip(t.p, t.r, 0, 1);
         return;
     }
-    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    copy_pairs<LOGN>(T, tb.tw + ((size_t)t.g << LOGN));
     const PrimeDev P = tb.pr[t.g];
     const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
-    u64 v[16];
+    u64 v[16], u[4][4];
 #pragma unroll
-    for (int h = 0; h < 4; h++) {
-        u64 x[4];
-        load_n(io, t.p, t.r, t.g, (size_t)(th + 4 * h * NT), NT, x);
+    for (int h = 0; h < 2; h++) {
+        u64 x[8];
+        load_n(io, t.p, t.r, t.g, (size_t)(th + 8 * h * NT), NT, x);
 #pragma unroll
-        for (int m = 0; m < 4; m++) v[4 * h + m] = x[m];
+        for (int m = 0; m < 8; m++) v[8 * h + m] = x[m];
     }
-    stages_fwd<4>(v, P.q, 2 * P.q, TwColTop{T});
+    cp_async_wait<0>();
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 4; h++) operand_n(io, t.p, t.r, (size_t)(th + 4 * h * NT), NT, u[h]);
+    stages_fwd<4>(v, P.q, 2 * P.q, TwColTop<true>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
-    stages_fwd<4>(v, P.q, 2 * P.q, TwRowTop<4>{T, blk});
+    stages_fwd<4>(v, P.q, 2 * P.q, [&](int s, int il) { return T[(1 << (4 + s)) + (blk << s) + il]; });
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = v[m];
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
-        stages_fwd<LS>(v, P.q, 2 * P.q, [&](int s, int il) { return ldg2(T + (1 << (8 + s)) + ((16 * th) >> (LS - s)) + il); });
+        stages_fwd<LS>(v, P.q, 2 * P.q, [&](int s, int il) { return T[(1 << (8 + s)) + ((16 * th) >> (LS - s)) + il]; });
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
@@ -508,7 +590,7 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_co
             x[m] = sm[pad(th + (4 * h + m) * NT)];
             if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
         }
-        store_n(io, t.p, t.r, t.g, (size_t)(th + 4 * h * NT), NT, x);
+        store_n(io, t.p, t.r, t.g, (size_t)(th + 4 * h * NT), NT, x, u[h]);
     }
 }
 
@@ -517,9 +599,10 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
                                                                  const __grid_constant__ IO io) {
     constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;
     __shared__ u64 sm[(1 << LOGN) + NT];
+    __shared__ ulonglong2 T[1 << LOGN];
     const TileAt t = tile_at(b, tb.L, 1);
     if (ntt_skipped(b, t.p, t.r)) return;
-    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN);
+    copy_pairs<LOGN>(T, tb.tw + ((size_t)t.g << LOGN));
     const PrimeDev P = tb.pr[t.g];
     const u64 q = P.q;
     const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
@@ -528,24 +611,25 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
     for (int m = 0; m < 16; m++) v[m] = io.load(t.p, t.r, t.g, (size_t)(th + m * NT));
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
+    cp_async_wait<0>();
     __syncthreads();
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
-        stages_inv<LS>(v, q, q, [&](int s, int il) { return ldg2(T + (1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il); });
+        stages_inv<LS>(v, q, q, [&](int s, int il) { return T[(1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il]; });
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
         __syncthreads();
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
-    stages_inv<4>(v, q, q << LS, TwInvRowTop<4>{T, blk});
+    stages_inv<4>(v, q, q << LS, [&](int s, int il) { return T[(1 << (7 - s)) + (blk << (3 - s)) + il]; });
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = reduce64_lazy(v[m], P);
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(th + m * NT)];
-    stages_inv<4>(v, q, 2 * q, TwInvColTop{T});
+    stages_inv<4>(v, q, 2 * q, TwInvColTop<true>{T});
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
 #pragma unroll
     for (int m = 0; m < 16; m++) io.store(t.p, t.r, t.g, (size_t)(th + m * NT), inv_result(v[m], sc, b.digits, q));

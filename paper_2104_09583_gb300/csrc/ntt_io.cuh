@@ -140,6 +140,9 @@ struct MsIO {
     const PrimeDev *pr;
     KsTables T;
     int L, logN;
+    __device__ __forceinline__ const u64 *operand(int p, int r) const {
+        return (f.xp[0] ? f.xp[p] : f.x + (size_t)p * f.ell * ((size_t)1 << logN)) + ((size_t)r << logN);
+    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
@@ -150,6 +153,9 @@ struct MdIO {
     const PrimeDev *pr;
     KsTables T;
     int L, alpha, logN;
+    __device__ __forceinline__ const u64 *operand(int p, int r) const {
+        return f.U + (size_t)p * f.ustride + ((size_t)r << logN);
+    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
@@ -160,6 +166,9 @@ struct MddIO {
     const PrimeDev *pr;
     KsTables T;
     int L, alpha, logN;
+    __device__ __forceinline__ const u64 *operand(int p, int r) const {
+        return f.U + (size_t)p * f.ustride + ((size_t)r << logN);
+    }
     __device__ __forceinline__ void skip(int, int, int, int) const {}
 };
 
@@ -174,9 +183,23 @@ __device__ __forceinline__ void load_n(const IO &io, int p, int r, int g, size_t
     for (int i = 0; i < K; i++) v[i] = io.load(p, r, g, n0 + (size_t)i * dn);
 }
 template <int K, class IO>
-__device__ __forceinline__ void store_n(const IO &io, int p, int r, int g, size_t k0, size_t dk, const u64 (&v)[K]) {
+__device__ __forceinline__ void store_n(const IO &io, int p, int r, int g, size_t k0, size_t dk, const u64 (&v)[K],
+                                        const u64 (&)[K]) {
 #pragma unroll
     for (int i = 0; i < K; i++) io.store(p, r, g, k0 + (size_t)i * dk, v[i]);
+}
+// The operand of a finish (the value whose switched-down remainder the transform makes), loaded
+// ahead of its store: u[i] for position k0 + i dk.
+template <int K, class IO>
+__device__ __forceinline__ void operand_n(const IO &io, int p, int r, size_t k0, size_t dk, u64 (&u)[K]) {
+    if constexpr (IO::RAW) {
+        const u64 *x = io.operand(p, r);
+#pragma unroll
+        for (int i = 0; i < K; i++) u[i] = x[k0 + (size_t)i * dk];
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; i++) u[i] = 0;
+    }
 }
 
 // A base conversion sum_k c_k f_k mod q of centred digits c_k = [y_k] in (-b_k / 2, b_k / 2).
@@ -275,31 +298,26 @@ __device__ __forceinline__ u64 mul2_shoup(u64 x, Shoup a, u64 v, Shoup b, u64 q)
 // the finishes of ms_store, md_store and mdd_store for K positions of one residue, from the
 // transform's unreduced values: (U - t v) B^-1 = U B^-1 + v (-t B^-1)
 template <int K>
-__device__ __forceinline__ void store_n(const MsIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K]) {
+__device__ __forceinline__ void store_n(const MsIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K],
+                                        const u64 (&u)[K]) {
     const MsFuse &f = io.f;
     const u64 q = io.pr[r].q;
     const Shoup qinv = io.T.ms_qinv[(size_t)f.ell * io.L + r], tq = io.T.ms_ntq[(size_t)f.ell * io.L + r];
-    const u64 *x = (f.xp[0] ? f.xp[p] : f.x + (size_t)p * f.ell * ((size_t)1 << io.logN)) + ((size_t)r << io.logN);
     u64 *o = (f.outp[0] ? f.outp[p] : f.out + (size_t)p * (f.ell - 1) * ((size_t)1 << io.logN)) + ((size_t)r << io.logN);
-    u64 xv[K];
 #pragma unroll
-    for (int i = 0; i < K; i++) xv[i] = x[k0 + (size_t)i * dk];
-#pragma unroll
-    for (int i = 0; i < K; i++) o[k0 + (size_t)i * dk] = mul2_shoup(xv[i], qinv, v[i], tq, q);
+    for (int i = 0; i < K; i++) o[k0 + (size_t)i * dk] = mul2_shoup(u[i], qinv, v[i], tq, q);
 }
 
 template <int K>
-__device__ __forceinline__ void store_n(const MdIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K]) {
+__device__ __forceinline__ void store_n(const MdIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K],
+                                        const u64 (&u)[K]) {
     const MdFuse &f = io.f;
     const int job = p >> 1, c = p & 1;
     const u64 q = io.pr[r].q;
     const Shoup pinv = io.T.md_Pinv[r], tp = io.T.md_ntP[r];
-    const u64 *U = f.U + (size_t)p * f.ustride + ((size_t)r << io.logN);
     u64 res[K];
 #pragma unroll
-    for (int i = 0; i < K; i++) res[i] = U[k0 + (size_t)i * dk];
-#pragma unroll
-    for (int i = 0; i < K; i++) res[i] = mul2_shoup(res[i], pinv, v[i], tp, q);
+    for (int i = 0; i < K; i++) res[i] = mul2_shoup(u[i], pinv, v[i], tp, q);
     if (c < f.add_comps && f.add[job]) {
         const u64 *a = f.add[job] + (size_t)c * f.acomp + ((size_t)r << io.logN);
         const u64 gal = f.gal[job];
@@ -318,17 +336,15 @@ __device__ __forceinline__ void store_n(const MdIO &io, int p, int r, int, size_
 }
 
 template <int K>
-__device__ __forceinline__ void store_n(const MddIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K]) {
+__device__ __forceinline__ void store_n(const MddIO &io, int p, int r, int, size_t k0, size_t dk, const u64 (&v)[K],
+                                        const u64 (&u)[K]) {
     const MddFuse &f = io.f;
     const u64 q = io.pr[r].q;
     const size_t n = (size_t)1 << io.logN;
     const Shoup binv = io.T.mdd_Binv[(size_t)f.ell * io.L + r], tb = io.T.mdd_ntB[(size_t)f.ell * io.L + r];
-    const u64 *U = f.U + (size_t)p * f.ustride + ((size_t)r << io.logN);
     u64 res[K];
 #pragma unroll
-    for (int i = 0; i < K; i++) res[i] = U[k0 + (size_t)i * dk];
-#pragma unroll
-    for (int i = 0; i < K; i++) res[i] = mul2_shoup(res[i], binv, v[i], tb, q);
+    for (int i = 0; i < K; i++) res[i] = mul2_shoup(u[i], binv, v[i], tb, q);
     u64 *out;
     if (!f.outp[0]) {
         out = f.out + ((size_t)p * (f.ell - 1) + r) * n;

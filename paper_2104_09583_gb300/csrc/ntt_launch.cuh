@@ -31,11 +31,14 @@ NttTables tables(const copse_ctx *c) {
                      (const ulonglong2 *)(INV ? c->d_low_i : c->d_low_f), c->L};
 }
 
-// the 16-block clusters of N = 2^15 are above the portable size: opted in once per device
-template <class K>
+// A cluster kernel's shared memory, and the opt-in to 16-block clusters (N = 2^15, above the
+// portable size): function attributes, raised once per kernel and device.  Threads that race
+// here raise them twice, which is harmless.
+template <int LOGN, class K>
 copse_status cluster_attr(K kernel, int device, std::atomic<uint64_t> &done) {
     if (device >= 0 && device < 64 && (done.load(std::memory_order_acquire) & (1ull << device))) return COPSE_OK;
-    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterSmem<LOGN>)));
+    if (LOGN == 15) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     if (device >= 0 && device < 64) done.fetch_or(1ull << device, std::memory_order_release);
     return COPSE_OK;
 }
@@ -44,18 +47,17 @@ template <int LOGN, bool INV, class IO>
 copse_status launch_cluster(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s) {
     const unsigned grid = (unsigned)b.npoly * (unsigned)b.nr * Shape<LOGN>::TILES;
     const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;  // one read and one write of each residue polynomial
-    if constexpr (LOGN == 15) {
-        static std::atomic<uint64_t> done{0};
-        if constexpr (INV)
-            STATUS_TRY(cluster_attr(k_ntt_inv_cluster<LOGN, IO>, ctx->device, done));
-        else
-            STATUS_TRY(cluster_attr(k_ntt_fwd_cluster<LOGN, IO>, ctx->device, done));
-    }
+    const size_t smem = sizeof(ClusterSmem<LOGN>);
+    static std::atomic<uint64_t> done{0};
+    if constexpr (INV)
+        STATUS_TRY(cluster_attr<LOGN>(k_ntt_inv_cluster<LOGN, IO>, ctx->device, done));
+    else
+        STATUS_TRY(cluster_attr<LOGN>(k_ntt_fwd_cluster<LOGN, IO>, ctx->device, done));
     TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
         if constexpr (INV)
-            k_ntt_inv_cluster<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io);
+            k_ntt_inv_cluster<LOGN, IO><<<grid, NTHR, smem, s>>>(b, tables<true>(ctx), io);
         else
-            k_ntt_fwd_cluster<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io);
+            k_ntt_fwd_cluster<LOGN, IO><<<grid, NTHR, smem, s>>>(b, tables<false>(ctx), io);
     });
     LAUNCH_CHECK();
     return COPSE_OK;
