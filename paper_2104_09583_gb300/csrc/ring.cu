@@ -22,6 +22,7 @@
 namespace {
 
 constexpr int TPB = 256;
+constexpr int KS_TPB = 128;           // threads of the key-switch kernels (two elements each)
 constexpr int MAX_ALPHA = 40;
 constexpr int MM_ACC = 32;            // accumulators per launch (their diagonals' addresses are kernel parameters)
 constexpr int MM_DEEP = 2;            // rotations a thread loads at a time
@@ -150,20 +151,89 @@ __global__ void k_modup(const u64 *x, const u64 *x_ntt, size_t xs, u64 *y, int e
     }
 }
 
-// sum_j y_j * k_j over the nd key-switching digits of one element and both key
-// components: the key words are in Montgomery form (k 2^64 mod q), the products are summed
-// exactly in 128 bits and reduced once (mont_reduce).  yh: digit j's value at
-// yh[j * ystride]; key component c of digit j at key[(2 j + c) * kstride].
-__device__ __forceinline__ void ks_dot(const u64 *yh, size_t ystride, const u64 *key, size_t kstride, int nd,
-                                       const PrimeDev &P, u64 &o0, u64 &o1) {
-    Acc128 a0{0, 0}, a1{0, 0};
-    for (int j = 0; j < nd; j++) {
-        const u64 y = yh[(size_t)j * ystride];
-        mac128(a0, y, key[(size_t)(2 * j) * kstride]);
-        mac128(a1, y, key[(size_t)(2 * j + 1) * kstride]);
+// sum_j y_j * k_j over the nd key-switching digits of two adjacent elements n, n + 1 (n even) and
+// both key components: the key words are in Montgomery form (k 2^64 mod q), the products are
+// summed exactly (split at 28 bits, at most 64 of them) and reduced once (mont_reduce).  yh:
+// digit j's residue at yh + j * ystride, read at the pair that holds the two sources, in order or
+// (flip) exchanged: an automorphism takes an aligned pair of positions of the bit-reversed
+// transform to an aligned pair (their exponents differ by N, and so do the images').  Key
+// component c of digit j at key + (2 j + c) * kstride.  Every access is 16 bytes.
+struct Pair2 {
+    u64 x0, x1;
+};
+__device__ __forceinline__ Pair2 ld_pair(const u64 *p, bool flip = false) {
+    const ulonglong2 v = *(const ulonglong2 *)p;
+    return flip ? Pair2{v.y, v.x} : Pair2{v.x, v.y};
+}
+__device__ __forceinline__ void st_pair(u64 *p, Pair2 v) { *(ulonglong2 *)p = make_ulonglong2(v.x0, v.x1); }
+__device__ __forceinline__ Pair2 add_pair(Pair2 a, Pair2 b, u64 q) {
+    return Pair2{add_mod(a.x0, b.x0, q), add_mod(a.x1, b.x1, q)};
+}
+__device__ __forceinline__ Pair2 mul_pair(u64 c, Pair2 a, const PrimeDev &P) {
+    return Pair2{mul_mod(c, a.x0, P), mul_mod(c, a.x1, P)};
+}
+__device__ __forceinline__ u64 mont_acc(const AccK &a, const PrimeDev &P) {
+    const unsigned __int128 v = acc_value(a);
+    return mont_reduce(Acc128{(u64)v, (u64)(v >> 64)}, P);
+}
+struct DotAcc {
+    AccK a[2][2];  // [component][element]
+};
+__device__ __forceinline__ void dot_term(DotAcc &d, Pair2 y, Pair2 k0, Pair2 k1) {
+    const u64 yv[2] = {y.x0, y.x1}, kv[2][2] = {{k0.x0, k0.x1}, {k1.x0, k1.x1}};
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+        const uint2 ys = split_k(yv[e]);
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const uint2 ks = split_k(kv[c][e]);
+            mac_k(d.a[c][e], ys, ys.x + ys.y, ks, ks.x + ks.y);
+        }
     }
-    o0 = mont_reduce(a0, P);
-    o1 = mont_reduce(a1, P);
+}
+// ND > 0: nd at compile time, every word loaded before the first product; ND = 0: the next
+// digit's words loaded before this digit's products
+template <int ND>
+__device__ __forceinline__ void ks_dot(const u64 *yh, size_t ystride, bool flip, const u64 *key, size_t kstride, int nd,
+                                       const PrimeDev &P, Pair2 &o0, Pair2 &o1) {
+    DotAcc d;
+#pragma unroll
+    for (int c = 0; c < 2; c++) d.a[c][0] = d.a[c][1] = AccK{0, 0, 0};
+    if constexpr (ND > 0) {
+        Pair2 y[ND], k0[ND], k1[ND];
+#pragma unroll
+        for (int j = 0; j < ND; j++) {
+            k0[j] = ld_pair(key + (size_t)(2 * j) * kstride);
+            k1[j] = ld_pair(key + (size_t)(2 * j + 1) * kstride);
+            y[j] = ld_pair(yh + (size_t)j * ystride, flip);
+        }
+#pragma unroll
+        for (int j = 0; j < ND; j++) dot_term(d, y[j], k0[j], k1[j]);
+    } else {
+        Pair2 y = ld_pair(yh, flip), k0 = ld_pair(key), k1 = ld_pair(key + kstride);
+        for (int j = 1; j < nd; j++) {
+            yh += ystride;
+            key += 2 * kstride;
+            const Pair2 ny = ld_pair(yh, flip), n0 = ld_pair(key), n1 = ld_pair(key + kstride);
+            dot_term(d, y, k0, k1);
+            y = ny;
+            k0 = n0;
+            k1 = n1;
+        }
+        dot_term(d, y, k0, k1);
+    }
+    o0 = Pair2{mont_acc(d.a[0][0], P), mont_acc(d.a[0][1], P)};
+    o1 = Pair2{mont_acc(d.a[1][0], P), mont_acc(d.a[1][1], P)};
+}
+// the pair of positions that tau_g takes to n, n + 1 (n even), and whether exchanged
+__device__ __forceinline__ uint32_t galois_pair(uint32_t n, u64 g, int logN, bool &flip) {
+    if (g == 1) {
+        flip = false;
+        return n;
+    }
+    const uint32_t src = galois_src(n, g, logN);
+    flip = src & 1;
+    return src & ~1u;
 }
 
 struct InnerJob {
@@ -179,32 +249,35 @@ struct InnerJobs {
     InnerJob j[CHUNK_ROT];
 };
 
-// (u0, u1)[r][n] = sum_j yhat[j][r][tau_g n] * ksk[j][c][ext_prime(r)][n]
-__global__ void k_ks_inner(const u64 *yhat, const InnerJobs jobs, int ell, int alpha, int L, int logN,
-                           const PrimeDev *pr, const u64 *mdP) {
-    const int N = 1 << logN;
-    const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha;
-    const int NB = L + alpha;
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ((size_t)nx << logN)) return;
-    const InnerJob J = jobs.j[blockIdx.y];
+// (u0, u1)[r][n] = sum_j yhat[j][r][tau_g n] * ksk[j][c][ext_prime(r)][n]; two elements a thread.
+// Bound by HBM, each key read once: 6.3 TB/s of algorithmic bytes on the rotations of 16 encrypted
+// query ciphertexts (N = 2^15; 40.9 -> 28.8 ms).  Words one by one and products reduced from 128
+// bits: 4.4 TB/s; 16-byte words a digit ahead: 4.7; all digits' words first: 6.3 (256 threads: 5.9).
+template <int ND>
+__global__ void __launch_bounds__(KS_TPB) k_ks_inner(const u64 *yhat, const __grid_constant__ InnerJobs jobs, int ell,
+                                                  int alpha, int L, int logN, const PrimeDev *pr, const u64 *mdP) {
+    const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
+    const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x), n_el = (size_t)nx << logN;
+    if (e >= n_el) return;
+    const InnerJob &J = jobs.j[blockIdx.y];
     const int r = (int)(e >> logN);
-    const uint32_t n = (uint32_t)(e & (N - 1));
+    const uint32_t n = (uint32_t)(e & ((1u << logN) - 1));
     const int g = r < ell ? r : L + (r - ell);
     const PrimeDev P = pr[g];
-    const uint32_t src = J.g == 1 ? n : galois_src(n, J.g, logN);
+    bool flip;
+    const uint32_t src = galois_pair(n, J.g, logN, flip);
     const u64 *yh = J.y ? J.y : yhat;
-    u64 acc0, acc1;
-    ks_dot(yh + ((size_t)r << logN) + src, (size_t)nx << logN, J.ksk + ((size_t)g << logN) + n, (size_t)NB << logN,
-           nd, P, acc0, acc1);
+    Pair2 a0, a1;
+    ks_dot<ND>(yh + ((size_t)r << logN) + src, n_el, flip, J.ksk + ((size_t)g << logN) + n, (size_t)NB << logN, nd, P, a0, a1);
     if (J.pd && r < ell) {
         const u64 Pm = mdP[r];
-        acc0 = add_mod(acc0, mul_mod(Pm, J.pd[((size_t)r << logN) + n], P), P.q);
-        acc1 = add_mod(acc1, mul_mod(Pm, J.pd[((size_t)(ell + r) << logN) + n], P), P.q);
+        a0 = add_pair(a0, mul_pair(Pm, ld_pair(J.pd + ((size_t)r << logN) + n), P), P.q);
+        a1 = add_pair(a1, mul_pair(Pm, ld_pair(J.pd + ((size_t)(ell + r) << logN) + n), P), P.q);
     }
-    if (J.pc0 && r < ell) acc0 = add_mod(acc0, mul_mod(mdP[r], J.pc0[((size_t)r << logN) + src], P), P.q);
-    J.out[e] = acc0;
-    J.out[((size_t)nx << logN) + e] = acc1;
+    if (J.pc0 && r < ell)
+        a0 = add_pair(a0, mul_pair(mdP[r], ld_pair(J.pc0 + ((size_t)r << logN) + src, flip), P), P.q);
+    st_pair(J.out + e, a0);
+    st_pair(J.out + n_el + e, a1);
 }
 
 // ModDown conversion: u polys (stride ustride) whose residues ell..ell+alpha-1 are in
@@ -261,39 +334,43 @@ struct MmFusedTable {
     const u64 *pt[CHUNK_ROT];
     u64 *acc;
 };
-__global__ void __launch_bounds__(256) k_mm_fused(const u64 *yhat, const u64 *c0, int nrot, int first,
+template <int ND>
+__global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 *c0, int nrot, int first,
                                                   const __grid_constant__ MmFusedTable tab, size_t part_stride, int ell,
                                                   int alpha, int L, int logN, const PrimeDev *pr, KsTables T) {
-    const int N = 1 << logN;
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t n_el = (size_t)nx << logN;
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= n_el) return;
     const int per = (nrot + (int)gridDim.y - 1) / (int)gridDim.y;
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
     u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride;
     const int r = (int)(e >> logN);
-    const uint32_t n = (uint32_t)(e & (N - 1));
+    const uint32_t n = (uint32_t)(e & ((1u << logN) - 1));
     const int g = r < ell ? r : L + (r - ell);
     const PrimeDev P = pr[g];
     const u64 Pm = r < ell ? T.md_P[r] : 0;
-    AccK a0{0, 0, 0}, a1{0, 0, 0};
+    DotAcc a;
+#pragma unroll
+    for (int c = 0; c < 2; c++) a.a[c][0] = a.a[c][1] = AccK{0, 0, 0};
     for (int k = k0; k < k1; k++) {
         const MmJob J = tab.job[k];
-        u64 u0 = 0, u1 = 0;
-        const uint32_t src = galois_src(n, J.g, logN);
-        const uint2 p = split_k(tab.pt[k][e]);
-        ks_dot(yhat + ((size_t)r << logN) + src, (size_t)nx << logN, J.ksk + ((size_t)g << logN) + n,
-               (size_t)NB << logN, nd, P, u0, u1);
-        if (r < ell) u0 = add_mod(u0, mul_mod(Pm, c0[((size_t)r << logN) + src], P), P.q);
-        const uint2 v0 = split_k(u0), v1 = split_k(u1);
-        mac_k(a0, p, p.x + p.y, v0, v0.x + v0.y);
-        mac_k(a1, p, p.x + p.y, v1, v1.x + v1.y);
+        bool flip;
+        const uint32_t src = galois_pair(n, J.g, logN, flip);
+        const Pair2 p = ld_pair(tab.pt[k] + e);
+        Pair2 u0, u1;
+        ks_dot<ND>(yhat + ((size_t)r << logN) + src, n_el, flip, J.ksk + ((size_t)g << logN) + n, (size_t)NB << logN, nd, P,
+               u0, u1);
+        if (r < ell) u0 = add_pair(u0, mul_pair(Pm, ld_pair(c0 + ((size_t)r << logN) + src, flip), P), P.q);
+        dot_term(a, p, u0, u1);
     }
-    const u64 s0 = acc_reduce(a0, P), s1 = acc_reduce(a1, P);
-    acc[e] = first ? s0 : add_mod(acc[e], s0, P.q);
-    acc[n_el + e] = first ? s1 : add_mod(acc[n_el + e], s1, P.q);
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        Pair2 s{acc_reduce(a.a[c][0], P), acc_reduce(a.a[c][1], P)};
+        if (!first) s = add_pair(s, ld_pair(acc + c * n_el + e), P.q);
+        st_pair(acc + c * n_el + e, s);
+    }
 }
 
 // The same sums for a tile of NA accumulators per thread over precomputed R_k: two residue
@@ -373,31 +450,36 @@ struct RsTable {
     RsTerm t[RS_CHUNK];
 };
 
-__global__ void __launch_bounds__(256) k_rotsum(const RsTable tab, int nterm, u64 *acc, int ell, int alpha, int L,
-                                                int logN, const PrimeDev *pr, KsTables T) {
-    const int N = 1 << logN;
+template <int ND>
+__global__ void __launch_bounds__(KS_TPB) k_rotsum(const __grid_constant__ RsTable tab, int nterm, int first, u64 *acc,
+                                                int ell, int alpha, int L, int logN, const PrimeDev *pr, KsTables T) {
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t n_el = (size_t)nx << logN;
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= n_el) return;
     const int r = (int)(e >> logN);
-    const uint32_t n = (uint32_t)(e & (N - 1));
+    const uint32_t n = (uint32_t)(e & ((1u << logN) - 1));
     const int g = r < ell ? r : L + (r - ell);
     const PrimeDev P = pr[g];
     const u64 Pm = r < ell ? T.md_P[r] : 0;
-    u64 a0 = acc[e], a1 = acc[n_el + e];
-    for (int k = 0; k < nterm; k++) {
-        const RsTerm J = tab.t[k];
-        const uint32_t src = galois_src(n, J.g, logN);
-        u64 t0, t1;
-        ks_dot(J.yhat + ((size_t)r << logN) + src, (size_t)nx << logN, J.ksk + ((size_t)g << logN) + n,
-               (size_t)NB << logN, nd, P, t0, t1);
-        a0 = add_mod(a0, t0, P.q);
-        a1 = add_mod(a1, t1, P.q);
-        if (r < ell) a0 = add_mod(a0, mul_mod(Pm, J.c0[((size_t)r << logN) + src], P), P.q);
+    Pair2 a0{0, 0}, a1{0, 0};
+    if (!first) {
+        a0 = ld_pair(acc + e);
+        a1 = ld_pair(acc + n_el + e);
     }
-    acc[e] = a0;
-    acc[n_el + e] = a1;
+    for (int k = 0; k < nterm; k++) {
+        const RsTerm &J = tab.t[k];
+        bool flip;
+        const uint32_t src = galois_pair(n, J.g, logN, flip);
+        Pair2 t0, t1;
+        ks_dot<ND>(J.yhat + ((size_t)r << logN) + src, n_el, flip, J.ksk + ((size_t)g << logN) + n, (size_t)NB << logN, nd, P,
+               t0, t1);
+        a0 = add_pair(a0, t0, P.q);
+        a1 = add_pair(a1, t1, P.q);
+        if (r < ell) a0 = add_pair(a0, mul_pair(Pm, ld_pair(J.c0 + ((size_t)r << logN) + src, flip), P), P.q);
+    }
+    st_pair(acc + e, a0);
+    st_pair(acc + n_el + e, a1);
 }
 
 // out[i] = sum_y part[y * stride + i] over nparts partial sums of extended-basis
@@ -647,6 +729,22 @@ __global__ void k_add_one(u64 *c0, int ell, int logN, const PrimeDev *pr) {
 }
 
 // ---------------------------------------------------------------- helpers
+inline unsigned ks_blocks(size_t n_el) { return (unsigned)((n_el / 2 + KS_TPB - 1) / KS_TPB); }
+// a key-switch kernel by its number of digits
+#define KS_DISPATCH(nd, kernel, grid, args)                          \
+    switch (nd) {                                                    \
+        case 1: kernel<1><<<grid, KS_TPB, 0, s>>> args; break;       \
+        case 2: kernel<2><<<grid, KS_TPB, 0, s>>> args; break;       \
+        case 3: kernel<3><<<grid, KS_TPB, 0, s>>> args; break;       \
+        case 4: kernel<4><<<grid, KS_TPB, 0, s>>> args; break;       \
+        default: kernel<0><<<grid, KS_TPB, 0, s>>> args; break;      \
+    }
+void ks_inner_launch(copse_ctx *c, const u64 *yhat, const InnerJobs &jobs, int nj, int ell, cudaStream_t s) {
+    const int A = c->alpha, nd = (ell + A - 1) / A;
+    KS_DISPATCH(nd, k_ks_inner, dim3(ks_blocks((size_t)(ell + A) * c->N), nj),
+                (yhat, jobs, ell, A, c->L, c->logN, c->d_prime, c->ks.md_P));
+}
+
 NttBatch batch(u64 *data, size_t stride, int npoly, int r0, int nr, int ell, int fixed = -1) {
     return NttBatch{data, stride, npoly, r0, nr, ell, fixed};
 }
@@ -730,13 +828,12 @@ copse_status ks_apply(copse_ctx *c, const u64 *yhat, int ell, const std::vector<
     if (nj > CHUNK_ROT || nj > MD_JOBS) { set_error("internal: too many key-switch jobs in one launch"); return COPSE_EINVAL; }
     InnerJobs jobs;
     for (int i = 0; i < nj; i++) jobs.j[i] = jobs_h[i];
-    dim3 grid(nblk((size_t)nx * N), nj);
     const int ndg = (ell + A - 1) / A;
     // algorithmic bytes: the digits once, per job the two key components of every digit and
     // the output; products: two per digit and element
     TIMED_OPS("ks_inner", 8.0 * N * ((double)ndg * nx + (double)nj * (2.0 * ndg * nx + 2.0 * nx)),
               2.0 * N * (double)nj * ndg * nx, s,
-              k_ks_inner<<<grid, TPB, 0, s>>>(yhat, jobs, ell, A, c->L, c->logN, c->d_prime, c->ks.md_P));
+              ks_inner_launch(c, yhat, jobs, nj, ell, s));
     LAUNCH_CHECK();
     return moddown_apply(c, U, ell, nj, f, sc, s);
 }
@@ -946,8 +1043,7 @@ static copse_status mul_group(copse_ctx *c, const copse_evk *evk, const std::vec
     for (int k = 0; k < nj; k++)
         ij.j[k] = InnerJob{evk->rlk, U + (size_t)k * 2 * nx * N, 1, yhat + (size_t)k * nd * nx * N, d + (size_t)k * per3};
     TIMED_OPS("ks_inner", 8.0 * N * nj * (3.0 * nd * nx + 2.0 * nx + 2.0 * ell), 2.0 * N * (double)nj * nd * nx, s,
-              k_ks_inner<<<dim3(nblk((size_t)nx * N), nj), TPB, 0, s>>>(yhat, ij, ell, A, c->L, c->logN, c->d_prime,
-                                                                         c->ks.md_P));
+              ks_inner_launch(c, yhat, ij, nj, ell, s));
     LAUNCH_CHECK();
     // the dropped prime's and the special residues to coefficients, then the fused
     // conversion + transform + finish (or conversion, transform, finish)
@@ -1152,8 +1248,8 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
     } else {
         // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
         // partial sums where the elements and accumulators alone make too few blocks
-        const int tiles = nacc < MM_PRECOMPUTE_ACC ? 1 : (std::min(nacc, MM_ACC) + 3) / 4;
-        const size_t blocks = (size_t)nblk((size_t)nx * N) * tiles;
+        const size_t blocks = nacc < MM_PRECOMPUTE_ACC ? ks_blocks((size_t)nx * N)
+                                                       : (size_t)nblk((size_t)nx * N) * ((std::min(nacc, MM_ACC) + 3) / 4);
         const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
                                                  (MM_BLOCKS + blocks - 1) / blocks});
         const size_t part_stride = (size_t)nacc * ext;
@@ -1180,8 +1276,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                     jobs.j[i] = InnerJob{evk->find(gal[r]), Rall + (k0 + i) * ext, gal[r], nullptr, nullptr, v.data};
                 }
                 TIMED_OPS("ks_inner", 8.0 * N * nj * (2.0 * nd * nx + 2.0 * nx + ell), 2.0 * N * (double)nj * nd * nx, s,
-                          k_ks_inner<<<dim3(nblk((size_t)nx * N), nj), TPB, 0, s>>>(yhat, jobs, ell, A, c->L, c->logN,
-                                                                                     c->d_prime, c->ks.md_P));
+                          ks_inner_launch(c, yhat, jobs, nj, ell, s));
                 LAUNCH_CHECK();
             }
         }
@@ -1216,8 +1311,9 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                                                                                ell, A, c->L, c->logN, c->d_prime)
                 if (!Rall)
                     TIMED("mm_fused", bytes, s,
-                          k_mm_fused<<<dim3(eb, parts), TPB, 0, s>>>(yhat, v.data, nr, first, ftab, part_stride, ell, A,
-                                                                     c->L, c->logN, c->d_prime, c->ks));
+                          KS_DISPATCH(nd, k_mm_fused, dim3(ks_blocks((size_t)nx * N), parts),
+                                      (yhat, v.data, nr, first, ftab, part_stride, ell, A, c->L, c->logN, c->d_prime,
+                                       c->ks)));
                 else if (na <= 2)
                     TIMED("mm_fused", bytes, s, MM_MAC(2));
                 else if (na == 3)
@@ -1290,13 +1386,15 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
         // per matrix, the rotated accumulators key-switched into one extended-basis sum
         // (the ModUps of a matrix's terms batched), one ModDown for all matrices
         STATUS_TRY(sc.get(c, &acc, (size_t)n_mat * ext));
-        CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)n_mat * ext * sizeof(u64), s));
         for (int a = 0; a < n_mat; a++) {
             int x0 = 0;
             while (x0 < nacc && (acc_mat[x0] != a || gal[x0] == 1)) x0++;
             int x1 = x0;
             while (x1 < nacc && acc_mat[x1] == a && gal[x1] != 1) x1++;
-            if (x0 == x1) continue;
+            if (x0 == x1) {  // no rotated term
+                CUDA_TRY(cudaMemsetAsync(acc + (size_t)a * ext, 0, ext * sizeof(u64), s));
+                continue;
+            }
             for (int x = x1; x < nacc; x++)
                 if (acc_mat[x] == a && gal[x] != 1) {
                     set_error("internal: giant steps of a matrix not contiguous");
@@ -1316,8 +1414,8 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
                 }
                 const double bytes = 8.0 * N * ((double)nt * (2.0 * nd * nx + (double)nd * nx + ell) + 4.0 * nx);
                 TIMED("rotsum", bytes, s,
-                      k_rotsum<<<nblk((size_t)nx * N), TPB, 0, s>>>(tab, nt, acc + (size_t)a * ext, ell, A, c->L,
-                                                                    c->logN, c->d_prime, c->ks));
+                      KS_DISPATCH(nd, k_rotsum, ks_blocks((size_t)nx * N),
+                                  (tab, nt, k0 == x0, acc + (size_t)a * ext, ell, A, c->L, c->logN, c->d_prime, c->ks)));
                 LAUNCH_CHECK();
             }
         }
