@@ -539,15 +539,9 @@ extern "C" copse_status copse_encrypt_features(copse_ctx *c, const copse_keys *k
     auto buf = std::make_unique<copse_ctbuf>();
     buf->ctx = c;
     buf->stream = s;
-    // query ciphertext q holds queries [q per_ct, (q + 1) per_ct); its plane i is encryption q p + i
-    copse_status st = COPSE_OK;
-    for (size_t j0 = 0, q = 0; st == COPSE_OK && (j0 < nq || (nq == 0 && q == 0)); j0 += per_ct, q++) {
-        const size_t n = std::min(per_ct, nq - j0);
-        st = encrypt_planes(c, k, d_feats + j0 * f.n_features, (int)n, (int)f.n_features, (int)f.K, (int)f.q,
-                            (int)f.pd(), (int)f.block, (int)f.n_seg, (int)f.precision, seed, buf->cts, s, nullptr,
-                            (int)(q * f.precision));
-        if (nq == 0) break;
-    }
+    const int nct = (int)std::max<size_t>(1, (nq + per_ct - 1) / per_ct);
+    const copse_status st = encrypt_planes(c, k, d_feats, (int)nq, nct, (int)f.n_features, (int)f.K, (int)f.q, (int)f.pd(),
+                                           (int)f.block, (int)f.n_seg, (int)f.precision, seed, buf->cts, s);
     if (tmp) dev_free(tmp, s);
     if (st) return st;
     *out = buf.release();
@@ -870,23 +864,27 @@ extern "C" copse_status copse_decrypt_labels(copse_ctx *c, const copse_keys *k, 
     const size_t per_ct = (size_t)(c->N / f.span());
     if (nq > per_ct * res->cts.size()) { set_error("more queries than slot blocks"); return COPSE_EINVAL; }
     cudaStream_t s = as_stream(stream);
-    u64 *slots = nullptr;
     uint8_t *bits = on_device ? out_bits : nullptr;
-    STATUS_TRY(dev_alloc(c, (void **)&slots, (size_t)c->N * 8, s));
     const size_t n_out = f.n_out();
     if (!on_device) STATUS_TRY(dev_alloc(c, (void **)&bits, std::max<size_t>(nq * n_out, 1), s));
-    // query j is block j mod per_ct of result ciphertext j / per_ct
-    for (size_t j0 = 0, q = 0; j0 < nq || (nq == 0 && q == 0); j0 += per_ct, q++) {
-        const size_t n = std::min(per_ct, nq - j0);
-        STATUS_TRY(decrypt_slots_dev(c, k, res->cts[q], slots, s));
-        STATUS_TRY(extract_bits(c, slots, (int)n, seg_layout(f), bits + j0 * n_out, s));
-        if (nq == 0) break;
+    // query j is block j mod per_ct of result ciphertext j / per_ct; runs of ciphertexts at one level
+    // (an inference's results share theirs) go together
+    const size_t used = std::max<size_t>(1, (nq + per_ct - 1) / per_ct);
+    copse_status st = COPSE_OK;
+    for (size_t i = 0, n; i < used && st == COPSE_OK; i += n) {
+        n = 1;
+        while (i + n < used && res->cts[i + n].level == res->cts[i].level) n++;
+        const size_t j0 = std::min(nq, i * per_ct), m = std::min(nq - j0, n * per_ct);
+        st = decrypt_bits(c, k, &res->cts[i], (int)n, (int)m, seg_layout(f), bits + j0 * n_out, s);
+    }
+    if (st) {
+        if (!on_device) dev_free(bits, s);
+        return st;
     }
     if (!on_device) {
         CUDA_TRY(cudaMemcpyAsync(out_bits, bits, nq * n_out, cudaMemcpyDeviceToHost, s));
         dev_free(bits, s);
     }
-    dev_free(slots, s);
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(s));
     return COPSE_OK;
 }
@@ -1050,16 +1048,12 @@ static copse_status item_body(copse_session *S, size_t i, cudaStream_t s, int la
     copse_ctbuf feats;
     feats.ctx = c;
     feats.stream = s;
-    STATUS_TRY(encrypt_planes(c, S->keys, S->d_feats + it.feat_off, (int)it.nq, (int)f.n_features, (int)f.K,
+    STATUS_TRY(encrypt_planes(c, S->keys, S->d_feats + it.feat_off, (int)it.nq, 1, (int)f.n_features, (int)f.K,
                               (int)f.q, (int)f.pd(), (int)f.block, (int)f.n_seg, (int)f.precision, (u64)i, feats.cts, s,
                               S->d_seed));
     DCt res;
     STATUS_TRY(infer_impl(c, S->evk, it.m, &feats, &res, s, lane));
-    u64 *slots = nullptr;
-    STATUS_TRY(dev_alloc(c, (void **)&slots, (size_t)c->N * 8, s));
-    STATUS_TRY(decrypt_slots_dev(c, S->keys, res, slots, s));
-    STATUS_TRY(extract_bits(c, slots, (int)it.nq, seg_layout(f), S->d_bits + it.bit_off, s));
-    dev_free(slots, s);
+    STATUS_TRY(decrypt_bits(c, S->keys, &res, 1, (int)it.nq, seg_layout(f), S->d_bits + it.bit_off, s));
     ct_free(&res, s);
     return COPSE_OK;  // feats frees its ciphertexts on s when it goes out of scope
 }

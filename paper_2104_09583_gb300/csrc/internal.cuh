@@ -682,12 +682,13 @@ copse_status op_matmul_bsgs(copse_ctx *c, const copse_evk *evk, const DCt &v, co
 copse_status encode_patterns(copse_ctx *c, const std::vector<uint32_t> &patterns, int n, int len, int period,
                              int level, int ext_alpha, u64 *out, cudaStream_t s);
 copse_status keygen_dev(copse_ctx *c, u64 seed, const std::vector<u64> &galois, copse_keys **keys, copse_evk **evk);
-// p planes for n queries: feats [n][nf] (device), layout of the model given by
-// K, q, pd, block
-// (d_seed: when set, the seed is read from that device word instead of `seed`)
-copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d_feats, int nq, int nf, int K,
+// p planes of nct query ciphertexts for nq queries: feats [nq][nf] (device), layout of the model
+// given by K, q, pd, block; ciphertext i holds queries [i per, (i + 1) per), per = N / (block nseg),
+// its plane j is encryption index i p + j
+// (d_seed: when set, the seed is read from that device word, plus `seed`)
+copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d_feats, int nq, int nct, int nf, int K,
                             int q, int pd, int block, int nseg, int p, u64 seed, std::vector<DCt> &out,
-                            cudaStream_t s, const u64 *d_seed = nullptr, int index0 = 0);
+                            cudaStream_t s, const u64 *d_seed = nullptr);
 // decrypt to N slot values (device output, NTT(mod t) order remapped to slot order)
 copse_status decrypt_slots_dev(copse_ctx *c, const copse_keys *k, const DCt &ct, u64 *d_slots, cudaStream_t s);
 // where each query's result bits sit: query j owns blocks j nseg .. j nseg + nseg - 1; its
@@ -698,8 +699,9 @@ struct SegLayout {
     int off[COPSE_MAX_SEG + 1];
 };
 SegLayout seg_layout(const CompiledForest &f);
-copse_status extract_bits(copse_ctx *c, const u64 *d_slots, int nq, const SegLayout &lay, uint8_t *d_bits,
-                          cudaStream_t s);
+// decrypt n result ciphertexts (one level) of nq queries to their output bits
+copse_status decrypt_bits(copse_ctx *c, const copse_keys *k, const DCt *cts, int n, int nq, const SegLayout &lay,
+                          uint8_t *d_bits, cudaStream_t s);
 // sessions (copse.cu): asynchronous launch with feature/bit buffers in pinned host or
 // device memory; seed_slot is pinned host memory holding the run's seed until it completes
 copse_status session_launch(copse_session *S, const uint32_t *feats, uint64_t seed, uint8_t *bits, cudaStream_t s,

@@ -630,12 +630,14 @@ __global__ void k_lift(const u64 *in, u64 *out, int npoly, int level, int nres, 
 }
 
 // bit-planes of the replicated, block-periodic feature vectors, NTT(mod t) order
-// block beta of the ciphertext belongs to query beta / nseg (its segment beta mod nseg)
-__global__ void k_feature_planes(const uint32_t *feats, int nq, int nf, int K, int q, int pd, int block, int nseg,
-                                 int p, int logN, const uint32_t *slot_index, u64 *out) {
+// block beta of a ciphertext belongs to its query beta / nseg (segment beta mod nseg); ciphertext
+// blockIdx.y of the launch holds queries blockIdx.y per_ct ..
+__global__ void k_feature_planes(const uint32_t *feats, int nq, int per_ct, int nf, int K, int q, int pd, int block,
+                                 int nseg, int p, int logN, const uint32_t *slot_index, u64 *out) {
     size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= (1ull << logN)) return;
-    const int j = (int)(s / block) / nseg, x = (int)(s % block);
+    const int j = (int)blockIdx.y * per_ct + (int)(s / block) / nseg, x = (int)(s % block);
+    out += ((size_t)blockIdx.y * p) << logN;
     uint32_t val = 0;
     if (j < nq && x < pd) val = feats[(size_t)j * nf + (x % q) / K];
     const uint32_t pos = slot_index[s];
@@ -669,29 +671,44 @@ __global__ void k_enc_prep(const u64 *mt, int p, int index0, u64 seed_val, const
     }
 }
 
-// ct_i = (pk0 u + x0, pk1 u + x1), out [p][2][L][N]
-__global__ void k_enc_combine(const u64 *pk, const u64 *U, const u64 *X0, const u64 *X1, u64 *out, int p, int L,
+// ct_i = (pk0 u + x0, pk1 u + x1) straight into the ciphertexts out.ct[i] ([2][L][N]) of the
+// planes of blockIdx.y; W: the transformed samples u, x0, x1, each [p][L][N]; two elements a thread
+#define ENC_CTS 64
+constexpr size_t ENC_SCRATCH = (size_t)1 << 30;
+struct EncOut {
+    u64 *ct[ENC_CTS];
+};
+__global__ void k_enc_combine(const u64 *pk, const u64 *W, size_t wstride, const __grid_constant__ EncOut out, int L,
                               int logN, const PrimeDev *pr) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t per = (size_t)L << logN;
-    if (e >= (size_t)p * per) return;
-    const size_t i = e / per, k = e - i * per;
+    const size_t per = (size_t)L << logN, k = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (k >= per) return;
     const PrimeDev P = pr[k >> logN];
-    const u64 u = U[e];
-    out[(2 * i) * per + k] = add_mod(mul_mod(pk[k], u, P), X0[e], P.q);
-    out[(2 * i + 1) * per + k] = add_mod(mul_mod(pk[per + k], u, P), X1[e], P.q);
+    const u64 *w = W + blockIdx.y * per + k;
+    u64 *o = out.ct[blockIdx.y] + k;
+    const Pair2 u = ld_pair(w);
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        const Pair2 a = ld_pair(pk + c * per + k), x = ld_pair(w + (c + 1) * wstride);
+        st_pair(o + c * per, Pair2{add_mod(mul_mod(a.x0, u.x0, P), x.x0, P.q), add_mod(mul_mod(a.x1, u.x1, P), x.x1, P.q)});
+    }
 }
 
-__global__ void k_dec_dot(const u64 *ct, const u64 *s, u64 *x, int logN, const PrimeDev *pr) {
+// c0 + c1 s at the first prime, ciphertext blockIdx.y at in.ct (components one residue apart)
+#define DEC_CTS 64
+struct DecIn {
+    const u64 *ct[DEC_CTS];
+};
+__global__ void k_dec_dot(const __grid_constant__ DecIn in, const u64 *s, u64 *x, int logN, const PrimeDev *pr) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (1ull << logN)) return;
     const PrimeDev P = pr[0];
-    x[e] = add_mod(ct[e], mul_mod(ct[(1ull << logN) + e], s[e], P), P.q);
+    const u64 *ct = in.ct[blockIdx.y];
+    x[((size_t)blockIdx.y << logN) + e] = add_mod(ct[e], mul_mod(ct[(1ull << logN) + e], s[e], P), P.q);
 }
 
-__global__ void k_dec_to_t(const u64 *x, u64 *out, int logN, u64 t, const PrimeDev *pr) {
+__global__ void k_dec_to_t(const u64 *x, u64 *out, size_t n, u64 t, const PrimeDev *pr) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (1ull << logN)) return;
+    if (e >= n) return;
     const u64 q = pr[0].q, v = x[e];
     if (v > (q - 1) / 2) {
         const u64 m = (q - v) % t;  // centred value is -(q - v)
@@ -708,15 +725,18 @@ __global__ void k_gather_slots(const u64 *ntt_t, const uint32_t *slot_index, u64
 }
 
 // output bit x of query j: segment s with off[s] <= x < off[s] + len[s], slot x - off[s] of
-// block j nseg + s
-__global__ void k_extract_bits(const u64 *slots, int nq, const SegLayout lay, uint8_t *bits) {
+// block j nseg + s of its ciphertext (j counted within it, per_ct queries each); straight from the
+// transform mod t, slot s at position slot_index[s]
+__global__ void k_extract_bits(const u64 *ntt_t, const uint32_t *slot_index, int nq, int per_ct, int logN,
+                               const __grid_constant__ SegLayout lay, uint8_t *bits) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)nq * lay.total) return;
     const size_t j = e / lay.total;
     const int x = (int)(e - j * lay.total);
     int sg = 0;
     while (sg + 1 < lay.nseg && x >= lay.off[sg + 1]) sg++;
-    const u64 v = slots[(j * lay.nseg + sg) * lay.block + (x - lay.off[sg])];
+    const size_t ct = j / per_ct, jc = j - ct * per_ct;
+    const u64 v = ntt_t[(ct << logN) + slot_index[(jc * lay.nseg + sg) * lay.block + (x - lay.off[sg])]];
     bits[e] = v == 0 ? 0 : (v == 1 ? 1 : 2);
 }
 
@@ -1631,67 +1651,104 @@ copse_status keygen_dev(copse_ctx *c, u64 seed, const std::vector<u64> &galois, 
     return COPSE_OK;
 }
 
-copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d_feats, int nq, int nf, int K,
+copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d_feats, int nq, int nct, int nf, int K,
                             int q, int pd, int block, int nseg, int p, u64 seed, std::vector<DCt> &out,
-                            cudaStream_t s, const u64 *d_seed, int index0) {
-    const int N = c->N, L = c->L;
-    Scratch sc(s);
-    u64 *mt = nullptr, *U = nullptr, *X0 = nullptr, *X1 = nullptr, *cts = nullptr;
-    STATUS_TRY(sc.get(c, &mt, (size_t)p * N));
-    STATUS_TRY(sc.get(c, &U, (size_t)p * L * N));
-    STATUS_TRY(sc.get(c, &X0, (size_t)p * L * N));
-    STATUS_TRY(sc.get(c, &X1, (size_t)p * L * N));
-    k_feature_planes<<<nblk(N), TPB, 0, s>>>(d_feats, nq, nf, K, q, pd, block, nseg, p, c->logN, c->d_slot_index, mt);
-    LAUNCH_CHECK();
-    STATUS_TRY(ntt_inverse(c, batch(mt, N, p, 0, 1, 0, c->t_index()), s));
-    if (index0 < 0 || index0 + p > 0x100000) { set_error("encryption index out of range"); return COPSE_EINVAL; }
-    k_enc_prep<<<nblk((size_t)p * N), TPB, 0, s>>>(mt, p, index0, seed, d_seed, L, c->logN, c->t, c->d_prime, U, X0, X1);
-    LAUNCH_CHECK();
-    STATUS_TRY(ntt_forward(c, batch(U, (size_t)L * N, p, 0, L, L), s));
-    STATUS_TRY(ntt_forward(c, batch(X0, (size_t)L * N, p, 0, L, L), s));
-    STATUS_TRY(ntt_forward(c, batch(X1, (size_t)L * N, p, 0, L, L), s));
-    STATUS_TRY(dev_alloc(c, (void **)&cts, (size_t)p * 2 * L * N * 8, s));
-    k_enc_combine<<<nblk((size_t)p * L * N), TPB, 0, s>>>(k->pk, U, X0, X1, cts, p, L, c->logN, c->d_prime);
-    LAUNCH_CHECK();
-    // appended to `out`
-    for (int i = 0; i < p; i++) {
-        DCt ct;
-        ct.level = L;
-        ct.ncomp = 2;
-        STATUS_TRY(ct_alloc(c, &ct, L, 2, s));
-        CUDA_TRY(cudaMemcpyAsync(ct.data, cts + (size_t)i * 2 * L * N, (size_t)2 * L * N * 8, cudaMemcpyDeviceToDevice, s));
-        out.push_back(ct);
+                            cudaStream_t s, const u64 *d_seed) {
+    const int N = c->N, L = c->L, per_ct = N / (block * nseg);
+    if ((size_t)nct * p > 0x100000) { set_error("encryption index out of range"); return COPSE_EINVAL; }
+    // as many ciphertexts at a time as keep the samples of their planes below ENC_SCRATCH
+    const size_t ct_words = (size_t)p * L * N;
+    const int step = (int)std::max<size_t>(1, std::min<size_t>(nct, ENC_SCRATCH / (3 * ct_words * sizeof(u64))));
+    for (int q0 = 0; q0 < nct; q0 += step) {
+        const int nc = std::min(step, nct - q0), np = nc * p, j0 = q0 * per_ct;
+        Scratch sc(s);
+        const size_t words = (size_t)np * L * N;
+        u64 *mt = nullptr, *W = nullptr;
+        STATUS_TRY(sc.get(c, &mt, (size_t)np * N));
+        STATUS_TRY(sc.get(c, &W, 3 * words));  // the samples u, t e0 + m, t e1 of every plane
+        k_feature_planes<<<dim3(nblk(N), nc), TPB, 0, s>>>(d_feats + (size_t)j0 * nf, nq - j0, per_ct, nf, K, q, pd, block,
+                                                           nseg, p, c->logN, c->d_slot_index, mt);
+        LAUNCH_CHECK();
+        STATUS_TRY(ntt_inverse(c, batch(mt, N, np, 0, 1, 0, c->t_index()), s));
+        k_enc_prep<<<nblk((size_t)np * N), TPB, 0, s>>>(mt, np, q0 * p, seed, d_seed, L, c->logN, c->t, c->d_prime, W,
+                                                        W + words, W + 2 * words);
+        LAUNCH_CHECK();
+        STATUS_TRY(ntt_forward(c, batch(W, (size_t)L * N, 3 * np, 0, L, L), s));
+        // appended to `out`
+        for (int i0 = 0; i0 < np; i0 += ENC_CTS) {
+            const int n = std::min(ENC_CTS, np - i0);
+            EncOut o;
+            for (int i = 0; i < n; i++) {
+                DCt ct;
+                STATUS_TRY(ct_alloc(c, &ct, L, 2, s));
+                out.push_back(ct);
+                o.ct[i] = ct.data;
+            }
+            k_enc_combine<<<dim3(nblk((size_t)L * N / 2), n), TPB, 0, s>>>(k->pk, W + (size_t)i0 * L * N, words, o, L,
+                                                                          c->logN, c->d_prime);
+            LAUNCH_CHECK();
+        }
     }
-    dev_free(cts, s);
     return COPSE_OK;
+}
+
+// n ciphertexts (one level) to their polynomials mod t, transformed: xt [n][N]
+static copse_status decrypt_ntt(copse_ctx *c, const copse_keys *k, const DCt *cts, int n, u64 *xt, cudaStream_t s) {
+    const int N = c->N;
+    // down to one prime
+    std::vector<DCt> cur;
+    std::vector<const DCt *> at;
+    for (int i = 0; i < n; i++) at.push_back(&cts[i]);
+    copse_status st = COPSE_OK;
+    while (at[0]->level > 1 && st == COPSE_OK) {
+        std::vector<DCt> nx;
+        st = op_modswitch_cts(c, at, nx, s);
+        for (DCt &x : cur) ct_free(&x, s);
+        cur.swap(nx);
+        for (int i = 0; i < n; i++) at[i] = &cur[i];
+    }
+    auto body = [&]() -> copse_status {
+        Scratch sc(s);
+        u64 *x = nullptr;
+        STATUS_TRY(sc.get(c, &x, (size_t)n * N));
+        for (int i0 = 0; i0 < n; i0 += DEC_CTS) {
+            const int m = std::min(DEC_CTS, n - i0);
+            DecIn in;
+            for (int i = 0; i < m; i++) in.ct[i] = at[i0 + i]->data;
+            k_dec_dot<<<dim3(nblk(N), m), TPB, 0, s>>>(in, k->s_hat, x + (size_t)i0 * N, c->logN, c->d_prime);
+            LAUNCH_CHECK();
+        }
+        STATUS_TRY(ntt_inverse(c, batch(x, N, n, 0, 1, 1), s));
+        k_dec_to_t<<<nblk((size_t)n * N), TPB, 0, s>>>(x, xt, (size_t)n * N, c->t, c->d_prime);
+        LAUNCH_CHECK();
+        return ntt_forward(c, batch(xt, N, n, 0, 1, 0, c->t_index()), s);
+    };
+    if (st == COPSE_OK) st = body();
+    for (DCt &x : cur)
+        if (x.data) ct_free(&x, s);
+    return st;
 }
 
 copse_status decrypt_slots_dev(copse_ctx *c, const copse_keys *k, const DCt &ct, u64 *d_slots, cudaStream_t s) {
-    const int N = c->N;
-    DCt cur;
-    STATUS_TRY(ct_copy(c, ct, &cur, s));
-    copse_status st = op_to_level(c, &cur, 1, s);
-    if (st) { ct_free(&cur, s); return st; }
     Scratch sc(s);
-    u64 *x = nullptr, *xt = nullptr;
-    STATUS_TRY(sc.get(c, &x, N));
-    STATUS_TRY(sc.get(c, &xt, N));
-    k_dec_dot<<<nblk(N), TPB, 0, s>>>(cur.data, k->s_hat, x, c->logN, c->d_prime);
-    LAUNCH_CHECK();
-    ct_free(&cur, s);
-    STATUS_TRY(ntt_inverse(c, batch(x, N, 1, 0, 1, 1), s));
-    k_dec_to_t<<<nblk(N), TPB, 0, s>>>(x, xt, c->logN, c->t, c->d_prime);
-    LAUNCH_CHECK();
-    STATUS_TRY(ntt_forward(c, batch(xt, N, 1, 0, 1, 0, c->t_index()), s));
-    k_gather_slots<<<nblk(N), TPB, 0, s>>>(xt, c->d_slot_index, d_slots, c->logN);
+    u64 *xt = nullptr;
+    STATUS_TRY(sc.get(c, &xt, c->N));
+    STATUS_TRY(decrypt_ntt(c, k, &ct, 1, xt, s));
+    k_gather_slots<<<nblk(c->N), TPB, 0, s>>>(xt, c->d_slot_index, d_slots, c->logN);
     LAUNCH_CHECK();
     return COPSE_OK;
 }
 
-copse_status extract_bits(copse_ctx *c, const u64 *d_slots, int nq, const SegLayout &lay, uint8_t *d_bits,
-                          cudaStream_t s) {
+copse_status decrypt_bits(copse_ctx *c, const copse_keys *k, const DCt *cts, int n, int nq, const SegLayout &lay,
+                          uint8_t *d_bits, cudaStream_t s) {
+    if (n == 0) return COPSE_OK;
+    Scratch sc(s);
+    u64 *xt = nullptr;
+    STATUS_TRY(sc.get(c, &xt, (size_t)n * c->N));
+    STATUS_TRY(decrypt_ntt(c, k, cts, n, xt, s));
     if (nq * lay.total == 0) return COPSE_OK;
-    k_extract_bits<<<nblk((size_t)nq * lay.total), TPB, 0, s>>>(d_slots, nq, lay, d_bits);
+    k_extract_bits<<<nblk((size_t)nq * lay.total), TPB, 0, s>>>(xt, c->d_slot_index, nq, c->N / (lay.block * lay.nseg),
+                                                               c->logN, lay, d_bits);
     LAUNCH_CHECK();
     return COPSE_OK;
 }
