@@ -16,6 +16,7 @@
 // rotating first and key switching after.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -25,11 +26,12 @@ constexpr int TPB = 256;
 constexpr int KS_TPB = 128;           // threads of the key-switch kernels (two elements each)
 constexpr int MAX_ALPHA = 40;
 constexpr int MM_ACC = 32;            // accumulators per launch (their diagonals' addresses are kernel parameters)
-constexpr int MM_DEEP = 2;            // rotations a thread loads at a time
+constexpr int MM_TPB = 128;
+constexpr int MM_DEEP = 4;            // rotations a thread loads at a time
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
 constexpr int MM_PARTS = 8;           // rotation ranges with their own partial sums at most
-constexpr int MM_BLOCKS = 1400;       // blocks that a launch is split up to (about three waves)
+constexpr int MM_BLOCKS = 2800;       // blocks that a launch is split up to (several waves)
 constexpr int RS_CHUNK = 32; // giant-step terms per k_rotsum launch
 
 inline unsigned nblk(size_t n) { return (unsigned)((n + TPB - 1) / TPB); }
@@ -317,18 +319,18 @@ __global__ void k_moddown_conv(const u64 *u, size_t ustride, u64 *W, size_t wstr
 // The diagonal products are summed exactly from split 28-bit products (at most CHUNK_ROT terms)
 // and reduced once.  grid.y / the block's part splits the chunk's rotations into contiguous
 // ranges with their own partial sums at acc + part * part_stride (summed later).
-struct MmJob {
-    const u64 *ksk;  // [ndig][2][L+alpha][N] NTT domain
-    u64 g;           // Galois element
-    const u64 *R;    // when set: R_k already computed, [2][ell+alpha][N]
-};
 struct MmTable {
-    MmJob job[CHUNK_ROT];
     const u64 *pt[MM_ACC * CHUNK_ROT];  // [acc][rotation], [ell+alpha][N], null = zero diagonal
+    const u64 *R;                       // R_k of the chunk, [rotation][2][ell+alpha][N]
     u64 *acc;                           // [acc][2][ell+alpha][N]
+    uint32_t dense;                     // bit x: accumulator x's diagonals are adjacent, none is zero
 };
 
 // one accumulator: the key switch of each rotation inline, so that no R_k is written
+struct MmJob {
+    const u64 *ksk;  // [ndig][2][L+alpha][N] NTT domain
+    u64 g;           // Galois element
+};
 struct MmFusedTable {
     MmJob job[CHUNK_ROT];
     const u64 *pt[CHUNK_ROT];
@@ -373,60 +375,88 @@ __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 
     }
 }
 
-// The same sums for a tile of NA accumulators per thread over precomputed R_k: two residue
-// products per diagonal word.  Reduced products made this the integer pipe's at 2.0 TB/s; exact
-// sums (six multiply-adds and no reduction per word) reach 4.0 TB/s (69 + 378 accumulators of 64
-// rotations at N = 2^15: 8.5 -> 4.2 ms), the multiplier's pipe 65-70% busy.  Blocks run over the
+// The same sums for a tile of NA accumulators per thread over precomputed R_k (adjacent in
+// memory, [k][2][ell+alpha][N]): two residue products per diagonal word.  Blocks run over the
 // launch's accumulator tiles fastest, so that the tiles of one element range find its R_k in L2;
-// each thread has the loads of MM_DEEP rotations in flight (four at two blocks per SM: 1% slower).
+// each thread has the loads of MM_DEEP rotations in flight.
+//
+// The diagonals of an accumulator usually lie one after another (a model stores them in that
+// order, zero ones left out): then their addresses are one pointer that advances (DENSE), and
+// only accumulators with zero diagonals look them up.
+//
+// 69 + 378 accumulators of 64 rotations at N = 2^15: 8.5 ms with a reduction per product, 4.2 with
+// exact sums, 3.4 (5 TB/s) with the addresses above and blocks of 128 threads (4.2 with 256 and
+// two rotations at a time; three at a time 3.5 to 3.8).
+template <int NA, bool DENSE>
+__device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, int x0, int k0, int k1, size_t n_el,
+                                        size_t e, AccK (&a)[NA][2]) {
+    const u64 *R = tab.R + (size_t)k0 * 2 * n_el + e;
+    const u64 *p[NA];
+#pragma unroll
+    for (int x = 0; x < NA; x++) {
+        a[x][0] = a[x][1] = AccK{0, 0, 0};
+        if (DENSE) p[x] = tab.pt[(x0 + x) * nrot] + (size_t)k0 * n_el + e;
+    }
+    auto step = [&](int k, auto n) {
+        constexpr int D = decltype(n)::value;
+        u64 Rv[D][2], pv[D][NA];
+#pragma unroll
+        for (int i = 0; i < D; i++) {
+            Rv[i][0] = R[0];
+            Rv[i][1] = R[n_el];
+            R += 2 * n_el;
+#pragma unroll
+            for (int x = 0; x < NA; x++) {
+                if (DENSE) {
+                    pv[i][x] = __ldcs(p[x]);
+                    p[x] += n_el;
+                } else {
+                    const u64 *q = x0 + x < nacc ? tab.pt[(x0 + x) * nrot + k + i] : nullptr;
+                    pv[i][x] = q ? __ldcs(q + e) : 0;
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < D; i++) {
+            const uint2 r0 = split_k(Rv[i][0]), r1 = split_k(Rv[i][1]);
+            const uint32_t s0 = r0.x + r0.y, s1 = r1.x + r1.y;
+#pragma unroll
+            for (int x = 0; x < NA; x++) {
+                const uint2 w = split_k(pv[i][x]);
+                mac_k(a[x][0], w, w.x + w.y, r0, s0);
+                mac_k(a[x][1], w, w.x + w.y, r1, s1);
+            }
+        }
+    };
+    int k = k0;
+    for (; k + MM_DEEP <= k1; k += MM_DEEP) step(k, std::integral_constant<int, MM_DEEP>{});
+    for (; k < k1; k++) step(k, std::integral_constant<int, 1>{});
+}
+
 template <int NA>
-__global__ void __launch_bounds__(256, 3) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
+__global__ void __launch_bounds__(MM_TPB, 4) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
                                                    size_t part_stride, int ell, int alpha, int L, int logN,
                                                    const PrimeDev *pr) {
     const int nx = ell + alpha, tiles = (nacc + NA - 1) / NA;
     const size_t n_el = (size_t)nx << logN;
-    const int x0 = (int)(blockIdx.x % tiles) * NA, na = min(NA, nacc - x0);
+    const int x0 = (int)(blockIdx.x % tiles) * NA;
     const size_t e = (size_t)(blockIdx.x / tiles) * blockDim.x + threadIdx.x;
     if (e >= n_el) return;
     const int per = (nrot + (int)gridDim.y - 1) / (int)gridDim.y;
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
+    AccK a[NA][2];
+    // every accumulator of the tile dense (bits of tab.dense)
+    if (x0 + NA <= nacc && ((tab.dense >> x0) & ((1u << NA) - 1)) == (1u << NA) - 1)
+        mm_tile<NA, true>(tab, nrot, nacc, x0, k0, k1, n_el, e, a);
+    else
+        mm_tile<NA, false>(tab, nrot, nacc, x0, k0, k1, n_el, e, a);
     const int r = (int)(e >> logN);
     const PrimeDev P = pr[r < ell ? r : L + (r - ell)];
-    AccK a[NA][2];
-#pragma unroll
-    for (int x = 0; x < NA; x++) a[x][0] = a[x][1] = AccK{0, 0, 0};
-    for (int kb = k0; kb < k1; kb += MM_DEEP) {
-        u64 R[MM_DEEP][2], pv[MM_DEEP][NA];
-#pragma unroll
-        for (int i = 0; i < MM_DEEP; i++) {
-            const int k = kb + i;
-            R[i][0] = R[i][1] = 0;
-            if (k < k1) {
-                R[i][0] = tab.job[k].R[e];
-                R[i][1] = tab.job[k].R[n_el + e];
-            }
-#pragma unroll
-            for (int x = 0; x < NA; x++) {
-                const u64 *p = k < k1 && x < na ? tab.pt[(x0 + x) * nrot + k] : nullptr;
-                pv[i][x] = p ? __ldcs(p + e) : 0;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < MM_DEEP; i++) {
-            const uint2 r0 = split_k(R[i][0]), r1 = split_k(R[i][1]);
-#pragma unroll
-            for (int x = 0; x < NA; x++) {
-                const uint2 p = split_k(pv[i][x]);
-                mac_k(a[x][0], p, p.x + p.y, r0, r0.x + r0.y);
-                mac_k(a[x][1], p, p.x + p.y, r1, r1.x + r1.y);
-            }
-        }
-    }
     u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride + (size_t)x0 * 2 * n_el + e;
 #pragma unroll
     for (int x = 0; x < NA; x++)
-        if (x < na) {
+        if (x0 + x < nacc) {
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 u64 *o = acc + (size_t)(2 * x + c) * n_el;
@@ -1269,7 +1299,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
         // partial sums where the elements and accumulators alone make too few blocks
         const size_t blocks = nacc < MM_PRECOMPUTE_ACC ? ks_blocks((size_t)nx * N)
-                                                       : (size_t)nblk((size_t)nx * N) * ((std::min(nacc, MM_ACC) + 3) / 4);
+                                                       : ((size_t)nx * N + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 3) / 4);
         const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
                                                  (MM_BLOCKS + blocks - 1) / blocks});
         const size_t part_stride = (size_t)nacc * ext;
@@ -1306,18 +1336,24 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
             for (int a0 = 0; a0 < nacc; a0 += MM_ACC) {
                 const int na = std::min(MM_ACC, nacc - a0);
                 int nz_pt = 0;
-                auto point = [&](int a, int x) {
-                    const u64 *p = pt[a0 + a][ks_idx[k0 + x]];
-                    nz_pt += p != nullptr;
-                    return p;
-                };
                 MmTable tab;
                 MmFusedTable ftab;
                 tab.acc = ftab.acc = part + (size_t)a0 * ext;
+                tab.R = Rall ? Rall + k0 * ext : nullptr;
+                tab.dense = 0;
+                for (int a = 0; a < na; a++) {
+                    bool dense = true;
+                    for (int x = 0; x < nr; x++) {
+                        const u64 *p = pt[a0 + a][ks_idx[k0 + x]];
+                        tab.pt[a * nr + x] = p;
+                        nz_pt += p != nullptr;
+                        dense = dense && p && p == tab.pt[a * nr] + (size_t)x * nx * N;
+                    }
+                    if (dense) tab.dense |= 1u << a;
+                }
                 for (int x = 0; x < nr; x++) {
-                    const int r = ks_idx[k0 + x];
-                    tab.job[x] = ftab.job[x] = MmJob{evk->find(gal[r]), gal[r], Rall ? Rall + (k0 + x) * ext : nullptr};
-                    for (int a = 0; a < na; a++) tab.pt[a * nr + x] = point(a, x);
+                    const u64 g = gal[ks_idx[k0 + x]];
+                    ftab.job[x] = MmJob{evk->find(g), g};
                     ftab.pt[x] = tab.pt[x];
                 }
                 // algorithmic bytes: keys, diagonals, accumulators in and out, the rotated
@@ -1325,9 +1361,9 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                 const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * na * nx * parts +
                                                 (Rall ? (double)nr * 2 * nx
                                                       : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
-                const unsigned eb = nblk((size_t)nx * N);
+                const unsigned eb = (unsigned)(((size_t)nx * N + MM_TPB - 1) / MM_TPB);
 #define MM_MAC(K)                                                                                              \
-    k_mm_mac<K><<<dim3(eb * (unsigned)((na + K - 1) / K), parts), TPB, 0, s>>>(nr, na, first, tab, part_stride, \
+    k_mm_mac<K><<<dim3(eb * (unsigned)((na + K - 1) / K), parts), MM_TPB, 0, s>>>(nr, na, first, tab, part_stride, \
                                                                                ell, A, c->L, c->logN, c->d_prime)
                 if (!Rall)
                     TIMED("mm_fused", bytes, s,
