@@ -36,6 +36,22 @@ constexpr int RS_CHUNK = 32; // giant-step terms per k_rotsum launch
 
 inline unsigned nblk(size_t n) { return (unsigned)((n + TPB - 1) / TPB); }
 
+// two adjacent elements: every access 16 bytes
+struct Pair2 {
+    u64 x0, x1;
+};
+__device__ __forceinline__ Pair2 ld_pair(const u64 *p, bool flip = false) {
+    const ulonglong2 v = *(const ulonglong2 *)p;
+    return flip ? Pair2{v.y, v.x} : Pair2{v.x, v.y};
+}
+__device__ __forceinline__ void st_pair(u64 *p, Pair2 v) { *(ulonglong2 *)p = make_ulonglong2(v.x0, v.x1); }
+__device__ __forceinline__ Pair2 add_pair(Pair2 a, Pair2 b, u64 q) {
+    return Pair2{add_mod(a.x0, b.x0, q), add_mod(a.x1, b.x1, q)};
+}
+__device__ __forceinline__ Pair2 mul_pair(u64 c, Pair2 a, const PrimeDev &P) {
+    return Pair2{mul_mod(c, a.x0, P), mul_mod(c, a.x1, P)};
+}
+
 // Position n of the bit-reversed NTT holds the evaluation at psi^(2 brev(n) + 1);
 // tau_g(a) there equals a at psi^((2 brev(n) + 1) g).
 
@@ -67,33 +83,43 @@ struct TensorJobs {
     const u64 *a[MDD_CTS];
     const u64 *b[MDD_CTS];
 };
-__global__ void k_tensor_many(const TensorJobs J, u64 *out, int level, int logN, const PrimeDev *pr) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)level << logN;
+__global__ void k_tensor_many(const __grid_constant__ TensorJobs J, u64 *out, int level, int logN, const PrimeDev *pr) {
+    const size_t n = (size_t)level << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= n) return;
     const u64 *a = J.a[blockIdx.y], *b = J.b[blockIdx.y];
-    u64 *o = out + (size_t)blockIdx.y * 3 * n;
+    u64 *o = out + (size_t)blockIdx.y * 3 * n + e;
     const PrimeDev P = pr[e >> logN];
-    u64 a0 = a[e], a1 = a[n + e], b0 = b[e], b1 = b[n + e];
-    o[e] = mul_mod(a0, b0, P);
-    o[n + e] = add_mod(mul_mod(a0, b1, P), mul_mod(a1, b0, P), P.q);
-    o[2 * n + e] = mul_mod(a1, b1, P);
+    const Pair2 a0 = ld_pair(a + e), a1 = ld_pair(a + n + e), b0 = ld_pair(b + e), b1 = ld_pair(b + n + e);
+    st_pair(o, Pair2{mul_mod(a0.x0, b0.x0, P), mul_mod(a0.x1, b0.x1, P)});
+    // the two cross products summed exactly, reduced once
+    AccK c[2] = {AccK{0, 0, 0}, AccK{0, 0, 0}};
+    const u64 x[2][2] = {{a0.x0, a0.x1}, {a1.x0, a1.x1}}, y[2][2] = {{b1.x0, b1.x1}, {b0.x0, b0.x1}};
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            const uint2 u = split_k(x[h][i]), w = split_k(y[h][i]);
+            mac_k(c[i], u, u.x + u.y, w, w.x + w.y);
+        }
+    st_pair(o + n, Pair2{acc_reduce(c[0], P), acc_reduce(c[1], P)});
+    st_pair(o + 2 * n, Pair2{mul_mod(a1.x0, b1.x0, P), mul_mod(a1.x1, b1.x1, P)});
 }
 
 #define AFF_JOBS 64
 struct AffineJobsDev {
     const u64 *x[AFF_JOBS], *m[AFF_JOBS], *add[AFF_JOBS];
 };
-__global__ void k_affine_many(const AffineJobsDev J, u64 *out, int level, int logN, const PrimeDev *pr) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)level << logN;
+__global__ void k_affine_many(const __grid_constant__ AffineJobsDev J, u64 *out, int level, int logN,
+                              const PrimeDev *pr) {
+    const size_t n = (size_t)level << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= 2 * n) return;
     const int j = blockIdx.y;
-    size_t k = e < n ? e : e - n;
+    const size_t k = e < n ? e : e - n;
     const PrimeDev P = pr[k >> logN];
-    u64 v = mul_mod(J.x[j][e], J.m[j][k], P);
-    if (J.add[j] && e < n) v = add_mod(v, J.add[j][k], P.q);
-    out[(size_t)j * 2 * n + e] = v;
+    const Pair2 x = ld_pair(J.x[j] + e), m = ld_pair(J.m[j] + k);
+    Pair2 v{mul_mod(x.x0, m.x0, P), mul_mod(x.x1, m.x1, P)};
+    if (J.add[j] && e < n) v = add_pair(v, ld_pair(J.add[j] + k), P.q);
+    st_pair(out + (size_t)j * 2 * n + e, v);
 }
 
 __global__ void k_mul_elem(const u64 *a, const u64 *b, u64 *out, int nres, int logN, const PrimeDev *pr) {
@@ -160,20 +186,6 @@ __global__ void k_modup(const u64 *x, const u64 *x_ntt, size_t xs, u64 *y, int e
 // (flip) exchanged: an automorphism takes an aligned pair of positions of the bit-reversed
 // transform to an aligned pair (their exponents differ by N, and so do the images').  Key
 // component c of digit j at key + (2 j + c) * kstride.  Every access is 16 bytes.
-struct Pair2 {
-    u64 x0, x1;
-};
-__device__ __forceinline__ Pair2 ld_pair(const u64 *p, bool flip = false) {
-    const ulonglong2 v = *(const ulonglong2 *)p;
-    return flip ? Pair2{v.y, v.x} : Pair2{v.x, v.y};
-}
-__device__ __forceinline__ void st_pair(u64 *p, Pair2 v) { *(ulonglong2 *)p = make_ulonglong2(v.x0, v.x1); }
-__device__ __forceinline__ Pair2 add_pair(Pair2 a, Pair2 b, u64 q) {
-    return Pair2{add_mod(a.x0, b.x0, q), add_mod(a.x1, b.x1, q)};
-}
-__device__ __forceinline__ Pair2 mul_pair(u64 c, Pair2 a, const PrimeDev &P) {
-    return Pair2{mul_mod(c, a.x0, P), mul_mod(c, a.x1, P)};
-}
 __device__ __forceinline__ u64 mont_acc(const AccK &a, const PrimeDev &P) {
     const unsigned __int128 v = acc_value(a);
     return mont_reduce(Acc128{(u64)v, (u64)(v >> 64)}, P);
@@ -516,13 +528,13 @@ __global__ void __launch_bounds__(KS_TPB) k_rotsum(const __grid_constant__ RsTab
 // polynomials ([npoly][ell+alpha][N] each)
 __global__ void k_sum_parts(const u64 *part, size_t stride, int nparts, u64 *out, size_t words, int ell, int alpha,
                             int L, int logN, const PrimeDev *pr) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t i = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= words) return;
     const int r = (int)((i >> logN) % (size_t)(ell + alpha));
     const u64 q = pr[r < ell ? r : L + (r - ell)].q;
-    u64 s = part[i];
-    for (int y = 1; y < nparts; y++) s = add_mod(s, part[(size_t)y * stride + i], q);
-    out[i] = s;
+    Pair2 s = ld_pair(part + i);
+    for (int y = 1; y < nparts; y++) s = add_pair(s, ld_pair(part + (size_t)y * stride + i), q);
+    st_pair(out + i, s);
 }
 
 // The last step of matrix products for a batch of outputs (blockIdx.y = output a):
@@ -536,19 +548,21 @@ struct FinTable {
     const u64 *pt_add[FIN_MAX];    // [ell][N]
 };
 
-__global__ void k_finish(const FinTable tab, const u64 *v, int ell, int logN, const PrimeDev *pr) {
-    const size_t n = (size_t)ell << logN;
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_finish(const __grid_constant__ FinTable tab, const u64 *v, int ell, int logN, const PrimeDev *pr) {
+    const size_t n = (size_t)ell << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= 2 * n) return;
     const int a = blockIdx.y;
     const size_t k = e < n ? e : e - n;
     const PrimeDev P = pr[k >> logN];
-    u64 x = tab.res[a][e];
-    if (tab.pt_mul[a]) x = add_mod(x, mul_mod(tab.pt_mul[a][k], v[e], P), P.q);
-    if (tab.ct_add[a]) x = add_mod(x, tab.ct_add[a][e], P.q);
-    if (tab.ct_add2[a]) x = add_mod(x, tab.ct_add2[a][e], P.q);
-    if (e < n && tab.pt_add[a]) x = add_mod(x, tab.pt_add[a][k], P.q);
-    tab.res[a][e] = x;
+    Pair2 x = ld_pair(tab.res[a] + e);
+    if (tab.pt_mul[a]) {
+        const Pair2 m = ld_pair(tab.pt_mul[a] + k), w = ld_pair(v + e);
+        x = add_pair(x, Pair2{mul_mod(m.x0, w.x0, P), mul_mod(m.x1, w.x1, P)}, P.q);
+    }
+    if (tab.ct_add[a]) x = add_pair(x, ld_pair(tab.ct_add[a] + e), P.q);
+    if (tab.ct_add2[a]) x = add_pair(x, ld_pair(tab.ct_add2[a] + e), P.q);
+    if (e < n && tab.pt_add[a]) x = add_pair(x, ld_pair(tab.pt_add[a] + k), P.q);
+    st_pair(tab.res[a] + e, x);
 }
 
 // modulus switch, conversion step: last [ncomp][N] coefficients of q_{ell-1} ->
@@ -1085,7 +1099,7 @@ static copse_status mul_group(copse_ctx *c, const copse_evk *evk, const std::vec
         tj.b[k] = b[idx[k]]->data;
     }
     TIMED("tensor", 8.0 * N * 7.0 * ell * nj, s,
-          k_tensor_many<<<dim3(nblk((size_t)ell * N), nj), TPB, 0, s>>>(tj, d, ell, c->logN, c->d_prime));
+          k_tensor_many<<<dim3(nblk((size_t)ell * N / 2), nj), TPB, 0, s>>>(tj, d, ell, c->logN, c->d_prime));
     LAUNCH_CHECK();
     STATUS_TRY(ks_modup_batch(c, d + (size_t)2 * ell * N, per3, nj, ell, sc, &yhat, s));
     STATUS_TRY(sc.get(c, &U, (size_t)nj * 2 * nx * N));
@@ -1227,7 +1241,7 @@ copse_status op_affine_many(copse_ctx *c, const std::vector<AffineJob> &jobs, cu
         u64 *r = nullptr;
         STATUS_TRY(sc.get(c, &r, (size_t)nj * 2 * ell * N));
         TIMED("affine", 8.0 * N * 6.0 * ell * nj, s,
-              k_affine_many<<<dim3(nblk((size_t)2 * ell * N), nj), TPB, 0, s>>>(J, r, ell, c->logN, c->d_prime));
+              k_affine_many<<<dim3(nblk((size_t)ell * N), nj), TPB, 0, s>>>(J, r, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
         std::vector<DCt> o;
         STATUS_TRY(op_modswitch_many(c, r, nj, ell, o, s));
@@ -1382,7 +1396,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         }
         if (parts > 1) {
             TIMED("sum_parts", 8.0 * (double)(parts + 1) * part_stride, s,
-                  k_sum_parts<<<nblk(part_stride), TPB, 0, s>>>(part, part_stride, parts, acc, part_stride, ell, A,
+                  k_sum_parts<<<nblk(part_stride / 2), TPB, 0, s>>>(part, part_stride, parts, acc, part_stride, ell, A,
                                                                 c->L, c->logN, c->d_prime));
             LAUNCH_CHECK();
         }
@@ -1409,7 +1423,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         }
         if (!any) continue;
         TIMED("mm_finish", 8.0 * N * 5.0 * ell * na, s,
-              k_finish<<<dim3(nblk(per), na), TPB, 0, s>>>(tab, v.data, ell, c->logN, c->d_prime));
+              k_finish<<<dim3(nblk(per / 2), na), TPB, 0, s>>>(tab, v.data, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
     }
     if (raw_out) return COPSE_OK;
@@ -1492,7 +1506,7 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
             tab.ct_add2[i] = add_ct.size() > (size_t)a ? add_ct[a] : nullptr;
         }
         TIMED("add", 8.0 * N * 5.0 * ell * na, s,
-              k_finish<<<dim3(nblk(per), na), TPB, 0, s>>>(tab, nullptr, ell, c->logN, c->d_prime));
+              k_finish<<<dim3(nblk(per / 2), na), TPB, 0, s>>>(tab, nullptr, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
     }
     return op_modswitch_many(c, res, n_mat, ell, out, s);
