@@ -264,6 +264,32 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
+// Dependent launches: a kernel launched by launch_dep may start while the kernel before it on the
+// stream still runs, up to its dep_wait(), which returns once that kernel (and so every earlier
+// one) has completed.  Every thread of such a kernel calls dep_wait before it touches memory that
+// another kernel writes or reads; only tables fixed at context creation are read ahead of it.
+// dep_trigger lets the next kernel start as soon as every block of this one has.  In a stream this
+// hides a kernel's launch behind the one before (a negacyclic product at N = 2^12 37 -> 31 us);
+// while a graph is recorded the launches are ordinary ones (between graph memory nodes such edges
+// cost more than they hide: the toy session 279 -> 322 us).
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    cfg.numAttrs = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // errors: LAUNCH_CHECK after the launch
+}
+
 // ---------------------------------------------------------------- context
 // Base-conversion constants.  Primes are addressed by a global index g:
 // 0..L-1 ciphertext primes, L..L+alpha-1 special primes, L+alpha = t.

@@ -364,6 +364,8 @@ template <int LOGN, class IO>
 __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_cols(const __grid_constant__ NttBatch b, NttTables tb,
                                                                    const __grid_constant__ IO io, Mid mid) {
     using S = Shape<LOGN>;
+    dep_trigger();
+    dep_wait();
     __shared__ u64 sm[TILE];
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) {
@@ -382,6 +384,8 @@ template <int LOGN, class IO>
 __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_rows(const __grid_constant__ NttBatch b, NttTables tb,
                                                                    const __grid_constant__ IO io, Mid mid) {
     using S = Shape<LOGN>;
+    dep_trigger();
+    dep_wait();
     __shared__ u64 sm[PTILE];
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) return;
@@ -400,6 +404,8 @@ template <int LOGN, class IO>
 __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_rows(const __grid_constant__ NttBatch b, NttTables tb,
                                                                    const __grid_constant__ IO io, Mid mid) {
     using S = Shape<LOGN>;
+    dep_trigger();
+    dep_wait();
     __shared__ u64 sm[PTILE];
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) return;
@@ -417,6 +423,8 @@ template <int LOGN, class IO>
 __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_cols(const __grid_constant__ NttBatch b, NttTables tb,
                                                                    const __grid_constant__ IO io, Mid mid) {
     using S = Shape<LOGN>;
+    dep_trigger();
+    dep_wait();
     __shared__ u64 sm[TILE];
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) return;
@@ -467,12 +475,15 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     ClusterSmem<LOGN> &M = *reinterpret_cast<ClusterSmem<LOGN> *>(dyn_smem);
     cg::cluster_group cl = cg::this_cluster();
     const TileAt t = tile_at(b, tb.L, S::TILES);  // tile = the block's rank
+    dep_trigger();
     if (ntt_skipped(b, t.p, t.r)) {  // the same for every block of the cluster
+        dep_wait();
         io.skip(t.p, t.r, t.tile, S::TILES);
         return;
     }
     cl.barrier_arrive();  // every block runs: its row tile may be written
     copy_twiddles<LOGN>(M, tb, t);
+    dep_wait();
     const PrimeDev P = tb.pr[t.g];
     u64 v[16];
     fwd_cols<LOGN, 8, true>(io, t.p, t.r, t.g, t.tile, M.col, P.q, M.colt, v, [] {
@@ -504,9 +515,14 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     ClusterSmem<LOGN> &M = *reinterpret_cast<ClusterSmem<LOGN> *>(dyn_smem);
     cg::cluster_group cl = cg::this_cluster();
     const TileAt t = tile_at(b, tb.L, S::TILES);
-    if (ntt_skipped(b, t.p, t.r)) return;
+    dep_trigger();
+    if (ntt_skipped(b, t.p, t.r)) {
+        dep_wait();
+        return;
+    }
     cl.barrier_arrive();
     copy_twiddles<LOGN>(M, tb, t);
+    dep_wait();
     const PrimeDev P = tb.pr[t.g];
     const int th = threadIdx.x, i = th & (S::SB - 1), gr = th / S::SB, c = th & (S::C - 1), ic = th >> S::LC;
     u64 v[16];
@@ -545,11 +561,14 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_co
     __shared__ u64 sm[(1 << LOGN) + NT];
     __shared__ ulonglong2 T[1 << LOGN];
     const TileAt t = tile_at(b, tb.L, 1);
+    dep_trigger();
     if (ntt_skipped(b, t.p, t.r)) {
+        dep_wait();
         io.skip(t.p, t.r, 0, 1);
         return;
     }
     copy_pairs<LOGN>(T, tb.tw + ((size_t)t.g << LOGN));
+    dep_wait();
     const PrimeDev P = tb.pr[t.g];
     const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
     u64 v[16], u[4][4];
@@ -601,8 +620,13 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
     __shared__ u64 sm[(1 << LOGN) + NT];
     __shared__ ulonglong2 T[1 << LOGN];
     const TileAt t = tile_at(b, tb.L, 1);
-    if (ntt_skipped(b, t.p, t.r)) return;
+    dep_trigger();
+    if (ntt_skipped(b, t.p, t.r)) {
+        dep_wait();
+        return;
+    }
     copy_pairs<LOGN>(T, tb.tw + ((size_t)t.g << LOGN));
+    dep_wait();
     const PrimeDev P = tb.pr[t.g];
     const u64 q = P.q;
     const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;

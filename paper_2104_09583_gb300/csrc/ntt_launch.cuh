@@ -55,9 +55,9 @@ copse_status launch_cluster(copse_ctx *ctx, const NttBatch &b, const IO &io, cud
         STATUS_TRY(cluster_attr<LOGN>(k_ntt_fwd_cluster<LOGN, IO>, ctx->device, done));
     TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
         if constexpr (INV)
-            k_ntt_inv_cluster<LOGN, IO><<<grid, NTHR, smem, s>>>(b, tables<true>(ctx), io);
+            launch_dep(k_ntt_inv_cluster<LOGN, IO>, grid, NTHR, smem, s, b, tables<true>(ctx), io);
         else
-            k_ntt_fwd_cluster<LOGN, IO><<<grid, NTHR, smem, s>>>(b, tables<false>(ctx), io);
+            launch_dep(k_ntt_fwd_cluster<LOGN, IO>, grid, NTHR, smem, s, b, tables<false>(ctx), io);
     });
     LAUNCH_CHECK();
     return COPSE_OK;
@@ -70,11 +70,11 @@ copse_status launch_tiled(copse_ctx *ctx, const NttBatch &b, const IO &io, const
     const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;
     TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
         if constexpr (INV) {
-            k_ntt_inv_rows<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io, mid);
-            k_ntt_inv_cols<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<true>(ctx), io, mid);
+            launch_dep(k_ntt_inv_rows<LOGN, IO>, grid, NTHR, 0, s, b, tables<true>(ctx), io, mid);
+            launch_dep(k_ntt_inv_cols<LOGN, IO>, grid, NTHR, 0, s, b, tables<true>(ctx), io, mid);
         } else {
-            k_ntt_fwd_cols<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io, mid);
-            k_ntt_fwd_rows<LOGN, IO><<<grid, NTHR, 0, s>>>(b, tables<false>(ctx), io, mid);
+            launch_dep(k_ntt_fwd_cols<LOGN, IO>, grid, NTHR, 0, s, b, tables<false>(ctx), io, mid);
+            launch_dep(k_ntt_fwd_rows<LOGN, IO>, grid, NTHR, 0, s, b, tables<false>(ctx), io, mid);
         }
     });
     LAUNCH_CHECK();
@@ -87,9 +87,9 @@ copse_status launch_one(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStr
     const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;
     TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
         if constexpr (INV)
-            k_ntt_inv_one<LOGN, IO><<<grid, 1 << (LOGN - 4), 0, s>>>(b, tables<true>(ctx), io);
+            launch_dep(k_ntt_inv_one<LOGN, IO>, grid, 1 << (LOGN - 4), 0, s, b, tables<true>(ctx), io);
         else
-            k_ntt_fwd_one<LOGN, IO><<<grid, 1 << (LOGN - 4), 0, s>>>(b, tables<false>(ctx), io);
+            launch_dep(k_ntt_fwd_one<LOGN, IO>, grid, 1 << (LOGN - 4), 0, s, b, tables<false>(ctx), io);
     });
     LAUNCH_CHECK();
     return COPSE_OK;

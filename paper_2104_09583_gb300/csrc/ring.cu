@@ -84,6 +84,8 @@ struct TensorJobs {
     const u64 *b[MDD_CTS];
 };
 __global__ void k_tensor_many(const __grid_constant__ TensorJobs J, u64 *out, int level, int logN, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const size_t n = (size_t)level << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= n) return;
     const u64 *a = J.a[blockIdx.y], *b = J.b[blockIdx.y];
@@ -111,6 +113,8 @@ struct AffineJobsDev {
 };
 __global__ void k_affine_many(const __grid_constant__ AffineJobsDev J, u64 *out, int level, int logN,
                               const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const size_t n = (size_t)level << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= 2 * n) return;
     const int j = blockIdx.y;
@@ -270,6 +274,8 @@ struct InnerJobs {
 template <int ND>
 __global__ void __launch_bounds__(KS_TPB) k_ks_inner(const u64 *yhat, const __grid_constant__ InnerJobs jobs, int ell,
                                                   int alpha, int L, int logN, const PrimeDev *pr, const u64 *mdP) {
+    dep_trigger();
+    dep_wait();
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x), n_el = (size_t)nx << logN;
     if (e >= n_el) return;
@@ -352,6 +358,8 @@ template <int ND>
 __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 *c0, int nrot, int first,
                                                   const __grid_constant__ MmFusedTable tab, size_t part_stride, int ell,
                                                   int alpha, int L, int logN, const PrimeDev *pr, KsTables T) {
+    dep_trigger();
+    dep_wait();
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t n_el = (size_t)nx << logN;
     const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
@@ -449,6 +457,8 @@ template <int NA>
 __global__ void __launch_bounds__(MM_TPB, 4) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
                                                    size_t part_stride, int ell, int alpha, int L, int logN,
                                                    const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const int nx = ell + alpha, tiles = (nacc + NA - 1) / NA;
     const size_t n_el = (size_t)nx << logN;
     const int x0 = (int)(blockIdx.x % tiles) * NA;
@@ -495,6 +505,8 @@ struct RsTable {
 template <int ND>
 __global__ void __launch_bounds__(KS_TPB) k_rotsum(const __grid_constant__ RsTable tab, int nterm, int first, u64 *acc,
                                                 int ell, int alpha, int L, int logN, const PrimeDev *pr, KsTables T) {
+    dep_trigger();
+    dep_wait();
     const int nx = ell + alpha, nd = (ell + alpha - 1) / alpha, NB = L + alpha;
     const size_t n_el = (size_t)nx << logN;
     const size_t e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
@@ -528,6 +540,8 @@ __global__ void __launch_bounds__(KS_TPB) k_rotsum(const __grid_constant__ RsTab
 // polynomials ([npoly][ell+alpha][N] each)
 __global__ void k_sum_parts(const u64 *part, size_t stride, int nparts, u64 *out, size_t words, int ell, int alpha,
                             int L, int logN, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const size_t i = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= words) return;
     const int r = (int)((i >> logN) % (size_t)(ell + alpha));
@@ -549,6 +563,8 @@ struct FinTable {
 };
 
 __global__ void k_finish(const __grid_constant__ FinTable tab, const u64 *v, int ell, int logN, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const size_t n = (size_t)ell << logN, e = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e >= 2 * n) return;
     const int a = blockIdx.y;
@@ -678,6 +694,8 @@ __global__ void k_lift(const u64 *in, u64 *out, int npoly, int level, int nres, 
 // blockIdx.y of the launch holds queries blockIdx.y per_ct ..
 __global__ void k_feature_planes(const uint32_t *feats, int nq, int per_ct, int nf, int K, int q, int pd, int block,
                                  int nseg, int p, int logN, const uint32_t *slot_index, u64 *out) {
+    dep_trigger();
+    dep_wait();
     size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= (1ull << logN)) return;
     const int j = (int)blockIdx.y * per_ct + (int)(s / block) / nseg, x = (int)(s % block);
@@ -693,6 +711,8 @@ __global__ void k_feature_planes(const uint32_t *feats, int nq, int per_ct, int 
 // read from device memory when seed_ptr is set (replayed graphs)
 __global__ void k_enc_prep(const u64 *mt, int p, int index0, u64 seed_val, const u64 *seed_ptr, int L, int logN, u64 t,
                            const PrimeDev *pr, u64 *U, u64 *X0, u64 *X1) {
+    dep_trigger();
+    dep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ((size_t)p << logN)) return;
     // replayed graphs: the run's seed from device memory plus the item's offset
@@ -724,6 +744,8 @@ struct EncOut {
 };
 __global__ void k_enc_combine(const u64 *pk, const u64 *W, size_t wstride, const __grid_constant__ EncOut out, int L,
                               int logN, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     const size_t per = (size_t)L << logN, k = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (k >= per) return;
     const PrimeDev P = pr[k >> logN];
@@ -743,6 +765,8 @@ struct DecIn {
     const u64 *ct[DEC_CTS];
 };
 __global__ void k_dec_dot(const __grid_constant__ DecIn in, const u64 *s, u64 *x, int logN, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (1ull << logN)) return;
     const PrimeDev P = pr[0];
@@ -751,6 +775,8 @@ __global__ void k_dec_dot(const __grid_constant__ DecIn in, const u64 *s, u64 *x
 }
 
 __global__ void k_dec_to_t(const u64 *x, u64 *out, size_t n, u64 t, const PrimeDev *pr) {
+    dep_trigger();
+    dep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     const u64 q = pr[0].q, v = x[e];
@@ -763,6 +789,8 @@ __global__ void k_dec_to_t(const u64 *x, u64 *out, size_t n, u64 t, const PrimeD
 }
 
 __global__ void k_gather_slots(const u64 *ntt_t, const uint32_t *slot_index, u64 *slots, int logN) {
+    dep_trigger();
+    dep_wait();
     size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= (1ull << logN)) return;
     slots[s] = ntt_t[slot_index[s]];
@@ -773,6 +801,8 @@ __global__ void k_gather_slots(const u64 *ntt_t, const uint32_t *slot_index, u64
 // transform mod t, slot s at position slot_index[s]
 __global__ void k_extract_bits(const u64 *ntt_t, const uint32_t *slot_index, int nq, int per_ct, int logN,
                                const __grid_constant__ SegLayout lay, uint8_t *bits) {
+    dep_trigger();
+    dep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)nq * lay.total) return;
     const size_t j = e / lay.total;
@@ -795,18 +825,18 @@ __global__ void k_add_one(u64 *c0, int ell, int logN, const PrimeDev *pr) {
 // ---------------------------------------------------------------- helpers
 inline unsigned ks_blocks(size_t n_el) { return (unsigned)((n_el / 2 + KS_TPB - 1) / KS_TPB); }
 // a key-switch kernel by its number of digits
-#define KS_DISPATCH(nd, kernel, grid, args)                          \
+#define KS_DISPATCH(nd, kernel, grid, ...)                           \
     switch (nd) {                                                    \
-        case 1: kernel<1><<<grid, KS_TPB, 0, s>>> args; break;       \
-        case 2: kernel<2><<<grid, KS_TPB, 0, s>>> args; break;       \
-        case 3: kernel<3><<<grid, KS_TPB, 0, s>>> args; break;       \
-        case 4: kernel<4><<<grid, KS_TPB, 0, s>>> args; break;       \
-        default: kernel<0><<<grid, KS_TPB, 0, s>>> args; break;      \
+        case 1: launch_dep(kernel<1>, grid, KS_TPB, 0, s, __VA_ARGS__); break;  \
+        case 2: launch_dep(kernel<2>, grid, KS_TPB, 0, s, __VA_ARGS__); break;  \
+        case 3: launch_dep(kernel<3>, grid, KS_TPB, 0, s, __VA_ARGS__); break;  \
+        case 4: launch_dep(kernel<4>, grid, KS_TPB, 0, s, __VA_ARGS__); break;  \
+        default: launch_dep(kernel<0>, grid, KS_TPB, 0, s, __VA_ARGS__); break; \
     }
 void ks_inner_launch(copse_ctx *c, const u64 *yhat, const InnerJobs &jobs, int nj, int ell, cudaStream_t s) {
     const int A = c->alpha, nd = (ell + A - 1) / A;
     KS_DISPATCH(nd, k_ks_inner, dim3(ks_blocks((size_t)(ell + A) * c->N), nj),
-                (yhat, jobs, ell, A, c->L, c->logN, c->d_prime, c->ks.md_P));
+                yhat, jobs, ell, A, c->L, c->logN, c->d_prime, c->ks.md_P);
 }
 
 NttBatch batch(u64 *data, size_t stride, int npoly, int r0, int nr, int ell, int fixed = -1) {
@@ -1099,7 +1129,7 @@ static copse_status mul_group(copse_ctx *c, const copse_evk *evk, const std::vec
         tj.b[k] = b[idx[k]]->data;
     }
     TIMED("tensor", 8.0 * N * 7.0 * ell * nj, s,
-          k_tensor_many<<<dim3(nblk((size_t)ell * N / 2), nj), TPB, 0, s>>>(tj, d, ell, c->logN, c->d_prime));
+          launch_dep(k_tensor_many, dim3(nblk((size_t)ell * N / 2), nj), TPB, 0, s, tj, d, ell, c->logN, c->d_prime));
     LAUNCH_CHECK();
     STATUS_TRY(ks_modup_batch(c, d + (size_t)2 * ell * N, per3, nj, ell, sc, &yhat, s));
     STATUS_TRY(sc.get(c, &U, (size_t)nj * 2 * nx * N));
@@ -1241,7 +1271,7 @@ copse_status op_affine_many(copse_ctx *c, const std::vector<AffineJob> &jobs, cu
         u64 *r = nullptr;
         STATUS_TRY(sc.get(c, &r, (size_t)nj * 2 * ell * N));
         TIMED("affine", 8.0 * N * 6.0 * ell * nj, s,
-              k_affine_many<<<dim3(nblk((size_t)ell * N), nj), TPB, 0, s>>>(J, r, ell, c->logN, c->d_prime));
+              launch_dep(k_affine_many, dim3(nblk((size_t)ell * N), nj), TPB, 0, s, J, r, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
         std::vector<DCt> o;
         STATUS_TRY(op_modswitch_many(c, r, nj, ell, o, s));
@@ -1377,13 +1407,13 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                                                       : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
                 const unsigned eb = (unsigned)(((size_t)nx * N + MM_TPB - 1) / MM_TPB);
 #define MM_MAC(K)                                                                                              \
-    k_mm_mac<K><<<dim3(eb * (unsigned)((na + K - 1) / K), parts), MM_TPB, 0, s>>>(nr, na, first, tab, part_stride, \
+    launch_dep(k_mm_mac<K>, dim3(eb * (unsigned)((na + K - 1) / K), parts), MM_TPB, 0, s, nr, na, first, tab, part_stride, \
                                                                                ell, A, c->L, c->logN, c->d_prime)
                 if (!Rall)
                     TIMED("mm_fused", bytes, s,
                           KS_DISPATCH(nd, k_mm_fused, dim3(ks_blocks((size_t)nx * N), parts),
-                                      (yhat, v.data, nr, first, ftab, part_stride, ell, A, c->L, c->logN, c->d_prime,
-                                       c->ks)));
+                                      yhat, v.data, nr, first, ftab, part_stride, ell, A, c->L, c->logN, c->d_prime,
+                                      c->ks));
                 else if (na <= 2)
                     TIMED("mm_fused", bytes, s, MM_MAC(2));
                 else if (na == 3)
@@ -1396,7 +1426,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         }
         if (parts > 1) {
             TIMED("sum_parts", 8.0 * (double)(parts + 1) * part_stride, s,
-                  k_sum_parts<<<nblk(part_stride / 2), TPB, 0, s>>>(part, part_stride, parts, acc, part_stride, ell, A,
+                  launch_dep(k_sum_parts, nblk(part_stride / 2), TPB, 0, s, part, part_stride, parts, acc, part_stride, ell, A,
                                                                 c->L, c->logN, c->d_prime));
             LAUNCH_CHECK();
         }
@@ -1423,7 +1453,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         }
         if (!any) continue;
         TIMED("mm_finish", 8.0 * N * 5.0 * ell * na, s,
-              k_finish<<<dim3(nblk(per / 2), na), TPB, 0, s>>>(tab, v.data, ell, c->logN, c->d_prime));
+              launch_dep(k_finish, dim3(nblk(per / 2), na), TPB, 0, s, tab, v.data, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
     }
     if (raw_out) return COPSE_OK;
@@ -1485,7 +1515,7 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
                 const double bytes = 8.0 * N * ((double)nt * (2.0 * nd * nx + (double)nd * nx + ell) + 4.0 * nx);
                 TIMED("rotsum", bytes, s,
                       KS_DISPATCH(nd, k_rotsum, ks_blocks((size_t)nx * N),
-                                  (tab, nt, k0 == x0, acc + (size_t)a * ext, ell, A, c->L, c->logN, c->d_prime, c->ks)));
+                                  tab, nt, k0 == x0, acc + (size_t)a * ext, ell, A, c->L, c->logN, c->d_prime, c->ks));
                 LAUNCH_CHECK();
             }
         }
@@ -1506,7 +1536,7 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
             tab.ct_add2[i] = add_ct.size() > (size_t)a ? add_ct[a] : nullptr;
         }
         TIMED("add", 8.0 * N * 5.0 * ell * na, s,
-              k_finish<<<dim3(nblk(per / 2), na), TPB, 0, s>>>(tab, nullptr, ell, c->logN, c->d_prime));
+              launch_dep(k_finish, dim3(nblk(per / 2), na), TPB, 0, s, tab, nullptr, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
     }
     return op_modswitch_many(c, res, n_mat, ell, out, s);
@@ -1716,11 +1746,11 @@ copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d
         u64 *mt = nullptr, *W = nullptr;
         STATUS_TRY(sc.get(c, &mt, (size_t)np * N));
         STATUS_TRY(sc.get(c, &W, 3 * words));  // the samples u, t e0 + m, t e1 of every plane
-        k_feature_planes<<<dim3(nblk(N), nc), TPB, 0, s>>>(d_feats + (size_t)j0 * nf, nq - j0, per_ct, nf, K, q, pd, block,
+        launch_dep(k_feature_planes, dim3(nblk(N), nc), TPB, 0, s, d_feats + (size_t)j0 * nf, nq - j0, per_ct, nf, K, q, pd, block,
                                                            nseg, p, c->logN, c->d_slot_index, mt);
         LAUNCH_CHECK();
         STATUS_TRY(ntt_inverse(c, batch(mt, N, np, 0, 1, 0, c->t_index()), s));
-        k_enc_prep<<<nblk((size_t)np * N), TPB, 0, s>>>(mt, np, q0 * p, seed, d_seed, L, c->logN, c->t, c->d_prime, W,
+        launch_dep(k_enc_prep, nblk((size_t)np * N), TPB, 0, s, mt, np, q0 * p, seed, d_seed, L, c->logN, c->t, c->d_prime, W,
                                                         W + words, W + 2 * words);
         LAUNCH_CHECK();
         STATUS_TRY(ntt_forward(c, batch(W, (size_t)L * N, 3 * np, 0, L, L), s));
@@ -1734,7 +1764,7 @@ copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d
                 out.push_back(ct);
                 o.ct[i] = ct.data;
             }
-            k_enc_combine<<<dim3(nblk((size_t)L * N / 2), n), TPB, 0, s>>>(k->pk, W + (size_t)i0 * L * N, words, o, L,
+            launch_dep(k_enc_combine, dim3(nblk((size_t)L * N / 2), n), TPB, 0, s, k->pk, W + (size_t)i0 * L * N, words, o, L,
                                                                           c->logN, c->d_prime);
             LAUNCH_CHECK();
         }
@@ -1765,11 +1795,11 @@ static copse_status decrypt_ntt(copse_ctx *c, const copse_keys *k, const DCt *ct
             const int m = std::min(DEC_CTS, n - i0);
             DecIn in;
             for (int i = 0; i < m; i++) in.ct[i] = at[i0 + i]->data;
-            k_dec_dot<<<dim3(nblk(N), m), TPB, 0, s>>>(in, k->s_hat, x + (size_t)i0 * N, c->logN, c->d_prime);
+            launch_dep(k_dec_dot, dim3(nblk(N), m), TPB, 0, s, in, k->s_hat, x + (size_t)i0 * N, c->logN, c->d_prime);
             LAUNCH_CHECK();
         }
         STATUS_TRY(ntt_inverse(c, batch(x, N, n, 0, 1, 1), s));
-        k_dec_to_t<<<nblk((size_t)n * N), TPB, 0, s>>>(x, xt, (size_t)n * N, c->t, c->d_prime);
+        launch_dep(k_dec_to_t, nblk((size_t)n * N), TPB, 0, s, x, xt, (size_t)n * N, c->t, c->d_prime);
         LAUNCH_CHECK();
         return ntt_forward(c, batch(xt, N, n, 0, 1, 0, c->t_index()), s);
     };
@@ -1784,7 +1814,7 @@ copse_status decrypt_slots_dev(copse_ctx *c, const copse_keys *k, const DCt &ct,
     u64 *xt = nullptr;
     STATUS_TRY(sc.get(c, &xt, c->N));
     STATUS_TRY(decrypt_ntt(c, k, &ct, 1, xt, s));
-    k_gather_slots<<<nblk(c->N), TPB, 0, s>>>(xt, c->d_slot_index, d_slots, c->logN);
+    launch_dep(k_gather_slots, nblk(c->N), TPB, 0, s, xt, c->d_slot_index, d_slots, c->logN);
     LAUNCH_CHECK();
     return COPSE_OK;
 }
@@ -1797,7 +1827,7 @@ copse_status decrypt_bits(copse_ctx *c, const copse_keys *k, const DCt *cts, int
     STATUS_TRY(sc.get(c, &xt, (size_t)n * c->N));
     STATUS_TRY(decrypt_ntt(c, k, cts, n, xt, s));
     if (nq * lay.total == 0) return COPSE_OK;
-    k_extract_bits<<<nblk((size_t)nq * lay.total), TPB, 0, s>>>(xt, c->d_slot_index, nq, c->N / (lay.block * lay.nseg),
+    launch_dep(k_extract_bits, nblk((size_t)nq * lay.total), TPB, 0, s, xt, c->d_slot_index, nq, c->N / (lay.block * lay.nseg),
                                                                c->logN, lay, d_bits);
     LAUNCH_CHECK();
     return COPSE_OK;
