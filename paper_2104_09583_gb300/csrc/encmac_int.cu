@@ -26,9 +26,11 @@
 namespace {
 
 constexpr int IM_JC = 32;        // baby steps per chunk
-constexpr int IM_FOLD = 16;      // products between folds: (x0 + x1)(y0 + y1) < 2.25 2^58 for 56-bit sums
-constexpr int IM_THREADS = 256;  // threads per block at most
-constexpr size_t IM_SMEM = 48 * 1024;
+// products between folds: with masks below 2^57 the middle product's sums of halves are below
+// 2^30.2 and 2^29.6, sixteen of their products below 2^64
+constexpr int IM_FOLD = 16;
+constexpr int IM_THREADS = 128;  // threads per block at most
+constexpr size_t IM_SMEM = 40 * 1024;
 constexpr int IM_QT = 16;        // query ciphertexts per tile at most
 
 struct IntMacArgs {
@@ -55,7 +57,7 @@ __device__ __forceinline__ u128 shfl_down_u128(u128 v, int d) {
 
 // QP query ciphertexts per thread (1 or 2)
 template <int QP>
-__global__ void __launch_bounds__(IM_THREADS, QP == 1 ? 3 : 2) k_enc_mac_int(const IntMacArgs P) {
+__global__ void __launch_bounds__(IM_THREADS, QP == 1 ? 6 : 4) k_enc_mac_int(const IntMacArgs P) {
     extern __shared__ uint4 sm_int[];
     const int E = 1 << P.logE, JP = P.JP;
     const size_t n_el = (size_t)P.ell << P.logN;
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(IM_THREADS, QP == 1 ? 3 : 2) k_enc_mac_int(con
                     const u64 c0 = *src;
                     const uint32_t id = __ldg(id0 + x * P.nb);
                     if (id != ~0u) {
-                        const u64 c1 = mask_at(mask_state(P.seed, r, pos, P.logN), id, pd);
+                        const u64 c1 = mask_at_lazy(mask_state(P.seed, r, pos, P.logN), id, pd);  // below 4q < 2^57
                         w = make_uint4((uint32_t)c0 & 0x0FFFFFFFu, (uint32_t)(c0 >> 28), (uint32_t)c1 & 0x0FFFFFFFu,
                                        (uint32_t)(c1 >> 28));
                     }
@@ -201,16 +203,16 @@ __global__ void __launch_bounds__(IM_THREADS, QP == 1 ? 3 : 2) k_enc_mac_int(con
 
 // Time of one element in SM nanoseconds, fitted to both kernels on a GB300 (the 7 launches of an
 // encrypted model's matrices, N = 2^15, 64 to 1536 (accumulator, baby step) products, 1 to 64
-// query ciphertexts): here 1.0 a product and tile of query ciphertexts (its mask) and 0.35 a
+// query ciphertexts): here 1.0 a product and tile of query ciphertexts (its mask) and 0.32 a
 // product and query ciphertext; the tensor cores 2800 a tile of 16 accumulators and run of 256
 // baby steps, 1930 a pass of 8 query ciphertexts and 0.8 a product.  Measured, ms here / there:
-// 64 products 2.5 / 74.6 at 1, 9.9 / 74.6 at 8, 12.6 / 98 at 16, 22 / 137 at 24; 1024-1536
-// products 22 / 87 at 1, 61 / 88 at 8, 108 / 127 at 16, 173 / 155 at 24.
+// 64 products 1.9 / 74.6 at 1, 6.5 / 74.6 at 8, 11.6 / 98 at 16; 1024-1536 products 23 / 87 at 1,
+// 57 / 88 at 8, 100 / 127 at 16 (before the blocks were halved 173 / 155 at 24).
 bool enc_mac_use_int(const std::vector<EncModel::MacMat> &mats, int nq) {
     double t_int = 0, t_tc = 0;
     for (const EncModel::MacMat &M : mats) {
         const double prod = (double)M.nm * M.nb;
-        t_int += prod * ((nq + IM_QT - 1) / IM_QT + 0.35 * nq);
+        t_int += prod * ((nq + IM_QT - 1) / IM_QT + 0.32 * nq);
         t_tc += ((M.nm + 15) / 16) * ((M.nb + 255) / 256) * (2800.0 + 1930.0 * ((nq + 7) / 8)) + 0.8 * prod;
     }
     return t_int <= t_tc;
@@ -236,7 +238,9 @@ copse_status enc_mac_int(copse_ctx *c, const EncModel::MacMat &M, const u64 *R, 
     P.pr = c->d_prime;
     // tiles: at most 16 query ciphertexts and 64 (accumulator, thread's query ciphertexts) slots,
     // evenly divided; then as many elements (up to 16) and parts of the baby steps (up to 16) as
-    // fill the block
+    // fill the block.  Small blocks, so that the staging of some overlaps the products of others:
+    // with 256 threads 5 query ciphertexts of a 252-branch model took 22.2 ms, with 128 14.7; 16 of
+    // a 1008-branch model 111 and 100
     const int qp = nq > 1 ? 2 : 1;
     const int nqt = (nq + IM_QT - 1) / IM_QT;
     P.qt = (nq + nqt - 1) / nqt;
@@ -246,8 +250,8 @@ copse_status enc_mac_int(copse_ctx *c, const EncModel::MacMat &M, const u64 *R, 
     P.mt = (M.nm + nmt - 1) / nmt;
     const int slots = P.mt * qs;
     auto bytes = [&](int E, int JP) { return (size_t)E * (P.mt + qs * qp) * (IM_JC + (JP & 7)) * sizeof(uint4); };
-    int E = 4;
-    P.logE = 2;
+    int E = 2;
+    P.logE = 1;
     P.JP = 1;
     while (E < 16 && E * 2 * slots <= IM_THREADS && bytes(E * 2, 7) <= IM_SMEM) {
         E *= 2;

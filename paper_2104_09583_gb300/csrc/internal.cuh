@@ -136,10 +136,13 @@ __device__ __forceinline__ u64 reduce64_lazy(u64 x, const PrimeDev &P) {
     const uint32_t h = (uint32_t)(((x >> 32) * c + __umulhi((uint32_t)x, c)) >> 32);
     return x - (u64)h * P.q;
 }
-// (hi 2^64 + lo) mod q in [0, q) for any two words: hi (2^64 mod q) by its Shoup quotient and lo
-// each below 2q, one correction of their sum
+// (hi 2^64 + lo) mod q for any two words: hi (2^64 mod q) by its Shoup quotient and lo each below
+// 2q, their sum below 4q, or (reduce_words) corrected to [0, q)
+__device__ __forceinline__ u64 reduce_words_lazy(u64 hi, u64 lo, const PrimeDev &P) {
+    return mul_shoup_lazy(hi, P.r64, P.r64_sh, P.q) + reduce64_lazy(lo, P);
+}
 __device__ __forceinline__ u64 reduce_words(u64 hi, u64 lo, const PrimeDev &P) {
-    u64 s = mul_shoup_lazy(hi, P.r64, P.r64_sh, P.q) + reduce64_lazy(lo, P);
+    u64 s = reduce_words_lazy(hi, lo, P);
     if (s >= 2 * P.q) s -= 2 * P.q;
     return s >= P.q ? s - P.q : s;
 }
@@ -237,6 +240,10 @@ constexpr u64 MODEL_STREAM = 0x800000ull;
 __device__ __forceinline__ u64 mask_state(u64 seed, int r, uint32_t pos, int logN) {
     const u64 j = bit_reverse(pos, logN);
     return seed + RNG_STEP * ((MODEL_STREAM << 40) + 2 * (((u64)r << logN) + j) + 1ULL);
+}
+__device__ __forceinline__ u64 mask_at_lazy(u64 state, uint32_t id, const PrimeDev &P) {  // below 4q
+    const u64 z = state + ((u64)((uint32_t)RNG_STEP * id) << 41);
+    return reduce_words_lazy(rng_mix(z), rng_mix(z + RNG_STEP), P);
 }
 __device__ __forceinline__ u64 mask_at(u64 state, uint32_t id, const PrimeDev &P) {
     const u64 z = state + ((u64)((uint32_t)RNG_STEP * id) << 41);
