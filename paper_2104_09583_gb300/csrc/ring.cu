@@ -26,8 +26,8 @@ constexpr int TPB = 256;
 constexpr int KS_TPB = 128;           // threads of the key-switch kernels (two elements each)
 constexpr int MAX_ALPHA = 40;
 constexpr int MM_ACC = 32;            // accumulators per launch (their diagonals' addresses are kernel parameters)
-constexpr int MM_TPB = 128;
-constexpr int MM_DEEP = 4;            // rotations a thread loads at a time
+constexpr int MM_TPB = 64;            // two elements a thread
+constexpr int MM_RING = 4;            // rotations that a thread has in flight or in shared memory
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
 constexpr int MM_PARTS = 8;           // rotation ranges with their own partial sums at most
@@ -395,66 +395,69 @@ __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 
     }
 }
 
-// The same sums for a tile of NA accumulators per thread over precomputed R_k (adjacent in
-// memory, [k][2][ell+alpha][N]): two residue products per diagonal word.  Blocks run over the
-// launch's accumulator tiles fastest, so that the tiles of one element range find its R_k in L2;
-// each thread has the loads of MM_DEEP rotations in flight.
+// The same sums for a tile of NA accumulators and two adjacent elements per thread over
+// precomputed R_k (adjacent in memory, [k][2][ell+alpha][N]): two residue products per diagonal
+// word.  Blocks run over the launch's accumulator tiles fastest, so that the tiles of one element
+// range find its R_k in L2.  The bound is the diagonals' stream from memory; each thread keeps
+// MM_RING - 1 rotations of its own words arriving in its own shared memory (asynchronous copies,
+// so neither registers nor barriers) while it multiplies the one before.
 //
 // The diagonals of an accumulator usually lie one after another (a model stores them in that
 // order, zero ones left out): then their addresses are one pointer that advances (DENSE), and
-// only accumulators with zero diagonals look them up.
+// only accumulators with zero diagonals look them up (and copy zeros in their place).
 //
-// 69 + 378 accumulators of 64 rotations at N = 2^15: 8.5 ms with a reduction per product, 4.2 with
-// exact sums, 3.4 (5 TB/s) with the addresses above and blocks of 128 threads (4.2 with 256 and
-// two rotations at a time; three at a time 3.5 to 3.8).
+// 24 accumulators of 60 rotations, 10 residues, N = 2^15: 0.94 ms (4.0 TB/s of diagonals) with
+// plain loads of four rotations at a time and one element a thread, 0.65 (5.8) so; one element a
+// thread 0.71, three accumulators 0.67, eight rotations in flight the same.  Of the first step
+// half were instructions that split_k now avoids (117 -> 72 per rotation and warp).
 template <int NA, bool DENSE>
 __device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, int x0, int k0, int k1, size_t n_el,
-                                        size_t e, AccK (&a)[NA][2]) {
+                                        size_t e, Pair2 (*ring)[NA + 2][MM_TPB], DotAcc (&a)[NA]) {
+    const int t = threadIdx.x;
     const u64 *R = tab.R + (size_t)k0 * 2 * n_el + e;
     const u64 *p[NA];
 #pragma unroll
     for (int x = 0; x < NA; x++) {
-        a[x][0] = a[x][1] = AccK{0, 0, 0};
+#pragma unroll
+        for (int c = 0; c < 2; c++) a[x].a[c][0] = a[x].a[c][1] = AccK{0, 0, 0};
         if (DENSE) p[x] = tab.pt[(x0 + x) * nrot] + (size_t)k0 * n_el + e;
     }
-    auto step = [&](int k, auto n) {
-        constexpr int D = decltype(n)::value;
-        u64 Rv[D][2], pv[D][NA];
-#pragma unroll
-        for (int i = 0; i < D; i++) {
-            Rv[i][0] = R[0];
-            Rv[i][1] = R[n_el];
+    auto load = [&](int k) {
+        if (k < k1) {
+            Pair2(&d)[NA + 2][MM_TPB] = ring[(k - k0) % MM_RING];
+            cp_async16(&d[0][t], R);
+            cp_async16(&d[1][t], R + n_el);
             R += 2 * n_el;
 #pragma unroll
             for (int x = 0; x < NA; x++) {
                 if (DENSE) {
-                    pv[i][x] = __ldcs(p[x]);
+                    cp_async16(&d[2 + x][t], p[x]);
                     p[x] += n_el;
                 } else {
-                    const u64 *q = x0 + x < nacc ? tab.pt[(x0 + x) * nrot + k + i] : nullptr;
-                    pv[i][x] = q ? __ldcs(q + e) : 0;
+                    const u64 *q = x0 + x < nacc ? tab.pt[(x0 + x) * nrot + k] : nullptr;
+                    if (q)
+                        cp_async16(&d[2 + x][t], q + e);
+                    else
+                        d[2 + x][t] = Pair2{0, 0};
                 }
             }
         }
-#pragma unroll
-        for (int i = 0; i < D; i++) {
-            const uint2 r0 = split_k(Rv[i][0]), r1 = split_k(Rv[i][1]);
-            const uint32_t s0 = r0.x + r0.y, s1 = r1.x + r1.y;
-#pragma unroll
-            for (int x = 0; x < NA; x++) {
-                const uint2 w = split_k(pv[i][x]);
-                mac_k(a[x][0], w, w.x + w.y, r0, s0);
-                mac_k(a[x][1], w, w.x + w.y, r1, s1);
-            }
-        }
+        cp_async_commit();
     };
-    int k = k0;
-    for (; k + MM_DEEP <= k1; k += MM_DEEP) step(k, std::integral_constant<int, MM_DEEP>{});
-    for (; k < k1; k++) step(k, std::integral_constant<int, 1>{});
+#pragma unroll
+    for (int i = 0; i < MM_RING - 1; i++) load(k0 + i);
+    for (int k = k0; k < k1; k++) {
+        load(k + MM_RING - 1);
+        cp_async_wait<MM_RING - 1>();
+        const Pair2(&d)[NA + 2][MM_TPB] = ring[(k - k0) % MM_RING];
+        const Pair2 r0 = d[0][t], r1 = d[1][t];
+#pragma unroll
+        for (int x = 0; x < NA; x++) dot_term(a[x], d[2 + x][t], r0, r1);
+    }
 }
 
 template <int NA>
-__global__ void __launch_bounds__(MM_TPB, 4) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
+__global__ void __launch_bounds__(MM_TPB, 6) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
                                                    size_t part_stride, int ell, int alpha, int L, int logN,
                                                    const PrimeDev *pr) {
     dep_trigger();
@@ -462,17 +465,18 @@ __global__ void __launch_bounds__(MM_TPB, 4) k_mm_mac(int nrot, int nacc, int fi
     const int nx = ell + alpha, tiles = (nacc + NA - 1) / NA;
     const size_t n_el = (size_t)nx << logN;
     const int x0 = (int)(blockIdx.x % tiles) * NA;
-    const size_t e = (size_t)(blockIdx.x / tiles) * blockDim.x + threadIdx.x;
+    const size_t e = 2 * ((size_t)(blockIdx.x / tiles) * blockDim.x + threadIdx.x);
     if (e >= n_el) return;
     const int per = (nrot + (int)gridDim.y - 1) / (int)gridDim.y;
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
-    AccK a[NA][2];
+    __shared__ __align__(16) Pair2 ring[MM_RING][NA + 2][MM_TPB];
+    DotAcc a[NA];
     // every accumulator of the tile dense (bits of tab.dense)
     if (x0 + NA <= nacc && ((tab.dense >> x0) & ((1u << NA) - 1)) == (1u << NA) - 1)
-        mm_tile<NA, true>(tab, nrot, nacc, x0, k0, k1, n_el, e, a);
+        mm_tile<NA, true>(tab, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
     else
-        mm_tile<NA, false>(tab, nrot, nacc, x0, k0, k1, n_el, e, a);
+        mm_tile<NA, false>(tab, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
     const int r = (int)(e >> logN);
     const PrimeDev P = pr[r < ell ? r : L + (r - ell)];
     u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride + (size_t)x0 * 2 * n_el + e;
@@ -482,8 +486,9 @@ __global__ void __launch_bounds__(MM_TPB, 4) k_mm_mac(int nrot, int nacc, int fi
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 u64 *o = acc + (size_t)(2 * x + c) * n_el;
-                const u64 s = acc_reduce(a[x][c], P);
-                *o = first ? s : add_mod(*o, s, P.q);
+                Pair2 s{acc_reduce(a[x].a[c][0], P), acc_reduce(a[x].a[c][1], P)};
+                if (!first) s = add_pair(s, ld_pair(o), P.q);
+                st_pair(o, s);
             }
         }
 }
@@ -1343,7 +1348,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
         // partial sums where the elements and accumulators alone make too few blocks
         const size_t blocks = nacc < MM_PRECOMPUTE_ACC ? ks_blocks((size_t)nx * N)
-                                                       : ((size_t)nx * N + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 3) / 4);
+                                                       : ((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 3) / 4);
         const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
                                                  (MM_BLOCKS + blocks - 1) / blocks});
         const size_t part_stride = (size_t)nacc * ext;
@@ -1405,7 +1410,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                 const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * na * nx * parts +
                                                 (Rall ? (double)nr * 2 * nx
                                                       : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
-                const unsigned eb = (unsigned)(((size_t)nx * N + MM_TPB - 1) / MM_TPB);
+                const unsigned eb = (unsigned)(((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB);
 #define MM_MAC(K)                                                                                              \
     launch_dep(k_mm_mac<K>, dim3(eb * (unsigned)((na + K - 1) / K), parts), MM_TPB, 0, s, nr, na, first, tab, part_stride, \
                                                                                ell, A, c->L, c->logN, c->d_prime)
@@ -1416,7 +1421,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                                       c->ks));
                 else if (na <= 2)
                     TIMED("mm_fused", bytes, s, MM_MAC(2));
-                else if (na == 3)
+                else if (na == 3 || na == 5 || na == 6 || na == 9)  // as many tiles as of four, fuller
                     TIMED("mm_fused", bytes, s, MM_MAC(3));
                 else
                     TIMED("mm_fused", bytes, s, MM_MAC(4));

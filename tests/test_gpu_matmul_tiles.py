@@ -1,7 +1,8 @@
 """The diagonal products of a plaintext model (csrc/ring.cu) at the edges of their tiles, against
 the oracle coefficient for coefficient (tolerance zero: exact modular arithmetic): one
 accumulator (the key switch inline), two, three, four and more with a remainder, more than 32 (two
-launches), rotations in one chunk of 64 and in several, and partial sums over rotation ranges."""
+launches), rotations in one chunk of 64 and in several, fewer than a thread keeps in flight, and
+partial sums over rotation ranges."""
 import pytest
 
 from oracle import bgv as B
@@ -21,7 +22,8 @@ FOREST = (92, 8, 4, 4, 3, 3)  # seed, trees, depth, features, precision, classes
 LOG_N = 10
 
 
-@pytest.mark.parametrize("g", [(0, 0), (90, 70), (60, 40), (40, 64), (4, 9), (64, 16)])
+@pytest.mark.parametrize("g", [(0, 0), (90, 70), (60, 40), (40, 64), (4, 9), (64, 16), (2, 3), (3, 2), (66, 67),
+                               (27, 17), (22, 14)])
 def test_diagonal_products_match_the_oracle(g):
     seed, nt, dp, nf, p, nc = FOREST
     text = synth.random_forest(seed, nt, dp, nf, p, nc, complete=True)
