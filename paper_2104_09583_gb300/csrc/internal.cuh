@@ -262,10 +262,14 @@ __device__ __forceinline__ u64 seeded_mask(u64 seed, u64 stream, int r, uint32_t
     return reduce_words(rng_word(seed, stream, idx), rng_word(seed, stream, idx + 1), P);
 }
 
-// 16-byte asynchronous copies global -> shared (cp.async, grouped per thread)
+// 16- and 8-byte asynchronous copies global -> shared (cp.async, grouped per thread)
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -362,10 +366,14 @@ struct copse_ctx {
     u64 *d_psi_sh = nullptr;
     u64 *d_ipsi = nullptr;            // [NP][N] psi^-brev(k)
     u64 *d_ipsi_sh = nullptr;
-    u64 *d_tw_f = nullptr;            // N >= 2^8: (w, w') pairs of psi^brev(k), [NP][N][2],
-    u64 *d_tw_i = nullptr;            //   and of psi^-brev(k)
-    u64 *d_low_f = nullptr;           // N >= 2^12: the low row stages' pairs in the order of the threads that use
-    u64 *d_low_i = nullptr;           //   them, [NP][N / 2048][pairs][128][2] (ntt_core.cuh)
+    // transform twiddles psi^brev(k), and psi^-brev(k), [NP][N] (ntt_core.cuh): for 2^8 <= N < 2^12
+    // (w, w') pairs; for N >= 2^12 the words (w, 2v) and (wq, vq) of split ones, and the low row
+    // stages' twiddles in the order of the threads that use them, [NP][N / 2048][pairs][128], pairs
+    // or (N = 2^15) split
+    u64 *d_tw_f = nullptr, *d_tw_i = nullptr;
+    u64 *d_twq_f = nullptr, *d_twq_i = nullptr;
+    u64 *d_low_f = nullptr, *d_low_i = nullptr;
+    u64 *d_lowq_f = nullptr, *d_lowq_i = nullptr;
     uint32_t *d_slot_index = nullptr; // [N] NTT(mod t) position of slot s
     KsTables ks{};
     std::vector<void *> owned;        // device allocations freed with the context

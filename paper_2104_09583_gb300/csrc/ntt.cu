@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(512) k_ntt_fwd(NttBatch b, const PrimeDev *__r
     const int p = blockIdx.x / b.nr, r = b.r0 + blockIdx.x % b.nr;
     if (ntt_skipped(b, p, r)) return;
     const int g = ntt_prime(b, r, L);
-    const u64 q = primes[g].q, q2 = 2 * q;
+    const u64 q = primes[g].q;
     u64 *data = b.data + (size_t)p * b.stride + (size_t)r * N;
     const u64 *W = tw + (size_t)g * N, *Wp = tw_sh + (size_t)g * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) sm[i] = data[i];
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(512) k_ntt_fwd(NttBatch b, const PrimeDev *__r
         for (int x = threadIdx.x; x < half; x += blockDim.x) {
             const int i = x >> lt, j = x & (tt - 1);
             const int idx = (i << (lt + 1)) + j;
-            bf_fwd(sm[idx], sm[idx + tt], make_ulonglong2(W[m + i], Wp[m + i]), q, q2);
+            bf_fwd(sm[idx], sm[idx + tt], make_ulonglong2(W[m + i], Wp[m + i]), q);
         }
         __syncthreads();
     }
@@ -124,16 +124,28 @@ __global__ void k_md_finish_io(const MdFuse f, const u64 *W, int njobs, const Pr
 }
 
 
-// (w, w') pairs in natural order, and the low row stages' pairs in thread order (ntt_core.cuh):
-// forward stage s of thread t takes 16 >> (K - s) pairs of transform stage A + 4 + s from
-// coefficient 16 t of its tile on, inverse stage s takes 8 >> s pairs of distance 2^s
-// (K = LB - 4 low stages).
+// The tables of ntt_core.cuh: (w, w') pairs in natural order, or the split twiddles (2^31 w mod q
+// and the two quotients follow from the Shoup quotient w' = floor(w 2^64 / q): floor(w 2^31 / q) is
+// its upper 31 bits and floor((2^31 w mod q) 2^32 / q) the 32 below), and the low row stages'
+// twiddles (pairs of modulus 2q, or split) in thread order: forward stage s of thread t takes 16 >> (K - s) pairs of
+// transform stage A + 4 + s from coefficient 16 t of its tile on, inverse stage s takes 8 >> s
+// pairs of distance 2^s (K = LB - 4 low stages).
 constexpr long CLUSTER_BLOCKS = 400;
 __global__ void k_pairs(const u64 *W, const u64 *Wp, ulonglong2 *out, size_t n) {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e < n) out[e] = make_ulonglong2(W[e], Wp[e]);
 }
-__global__ void k_low_pairs(const u64 *W, const u64 *Wp, ulonglong2 *out, int np, int logN, int pairs, int inverse) {
+__device__ __forceinline__ void split_tw(u64 w, u64 wp, u64 q, ulonglong2 *out, uint2 *outq) {
+    *out = make_ulonglong2(w, 2 * mul_shoup(1ull << 31, w, wp, q));
+    *outq = make_uint2((uint32_t)(wp >> 33), (uint32_t)(wp >> 1));
+}
+__global__ void k_split_tw(const u64 *W, const u64 *Wp, ulonglong2 *out, uint2 *outq, size_t n, int logN,
+                           const PrimeDev *pr) {
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) split_tw(W[e], Wp[e], pr[e >> logN].q, out + e, outq + e);
+}
+__global__ void k_low_tw(const u64 *W, const u64 *Wp, ulonglong2 *out, uint2 *outq, int np, int logN, int pairs, int inverse,
+                         const PrimeDev *pr) {
     const int tiles = 1 << (logN - 11), K = logN - logN / 2 - 4;
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)np * tiles * pairs * NTHR) return;
@@ -145,7 +157,8 @@ __global__ void k_low_pairs(const u64 *W, const u64 *Wp, ulonglong2 *out, int np
     for (; k >= (inverse ? 8 >> s : 16 >> (K - s)); s++) k -= inverse ? 8 >> s : 16 >> (K - s);
     const int U = inverse ? logN - 1 - s : logN - K + s;  // transform stage: 2^U groups
     const size_t at = ((size_t)g << logN) + (1 << U) + (pos >> (logN - U)) + k;
-    out[e] = make_ulonglong2(W[at], Wp[at]);
+    if (outq) split_tw(W[at], Wp[at], pr[g].q, out + e, outq + e);
+    else out[e] = make_ulonglong2(W[at], Wp[at] >> 1);
 }
 
 }  // namespace
@@ -206,15 +219,30 @@ copse_status ntt_stage_tables(copse_ctx *ctx) {
         CUDA_TRY(cudaMalloc(&p, n * sizeof(ulonglong2)));
         ctx->owned.push_back(p);
         const u64 *W = inv ? ctx->d_ipsi : ctx->d_psi, *Wp = inv ? ctx->d_ipsi_sh : ctx->d_psi_sh;
-        k_pairs<<<(unsigned)((n + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)p, n);
-        CUDA_TRY(cudaGetLastError());
         (inv ? ctx->d_tw_i : ctx->d_tw_f) = (u64 *)p;
-        if (!nl) continue;
+        if (!nl) {
+            k_pairs<<<(unsigned)((n + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)p, n);
+            CUDA_TRY(cudaGetLastError());
+            continue;
+        }
+        void *pq = nullptr;
+        CUDA_TRY(cudaMalloc(&pq, n * sizeof(uint2)));
+        ctx->owned.push_back(pq);
+        (inv ? ctx->d_twq_i : ctx->d_twq_f) = (u64 *)pq;
+        k_split_tw<<<(unsigned)((n + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)p, (uint2 *)pq, n, ctx->logN, ctx->d_prime);
+        CUDA_TRY(cudaGetLastError());
         CUDA_TRY(cudaMalloc(&l, nl * sizeof(ulonglong2)));
         ctx->owned.push_back(l);
-        k_low_pairs<<<(unsigned)((nl + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)l, ctx->NP, ctx->logN, pairs, inv);
+        void *lq = nullptr;
+        if (lb == 8) {
+            CUDA_TRY(cudaMalloc(&lq, nl * sizeof(uint2)));
+            ctx->owned.push_back(lq);
+        }
+        k_low_tw<<<(unsigned)((nl + 255) / 256), 256>>>(W, Wp, (ulonglong2 *)l, (uint2 *)lq, ctx->NP, ctx->logN, pairs,
+                                                        inv, ctx->d_prime);
         CUDA_TRY(cudaGetLastError());
         (inv ? ctx->d_low_i : ctx->d_low_f) = (u64 *)l;
+        (inv ? ctx->d_lowq_i : ctx->d_lowq_f) = (u64 *)lq;
     }
     CUDA_TRY(cudaDeviceSynchronize());
     return COPSE_OK;

@@ -21,9 +21,10 @@
 //
 // Measured (us, forward / inverse; before = a radix-4 / radix-8 pass per two or three stages with
 // 512 / 256 threads and every twiddle staged through shared memory): N = 2^15, 1024 residue
-// polynomials 616 / 644 before, 331 / 359 now (0.76 / 0.70 T butterflies/s of the 0.95 that the
-// multiplier alone reaches), 64: 43 / 47 before, 29 / 31 now; N = 2^14, 1024 in clusters
-// 269 / 313 before, 163 / 178 tiled now.
+// polynomials 616 / 644 before, 318 / 355 with exact products, 288 / 325 with split ones (0.87 /
+// 0.77 T butterflies/s of the 1.24 that the multiplier alone reaches: the rest is additions,
+// exchanges, and 4 TB/s of memory traffic in the column half), 128: 44 / 50 and 39 / 47; N = 2^14,
+// 1024 in clusters 269 / 313 before, 153 / 173 tiled, 147 / 162 split.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -57,26 +58,65 @@ __device__ __forceinline__ bool ntt_skipped(const NttBatch &b, int p, int r) {
     return b.skip_alpha > 0 && r >= j * b.skip_alpha && r < min((j + 1) * b.skip_alpha, b.ell);
 }
 
-// Forward butterfly without a correction step: the Shoup product V is below 2q for any
-// 64-bit input, so x' = U + V and y' = U - V + 2q only grow by 2q per stage.  From inputs
-// below 2q, values stay below (2 log2 N + 2) q <= 32 q <= 2^60 for primes below 2^55 (the
+// Twiddle factors w of modulus m, in two forms.
+//
+// Exact: the pair (w, w' = floor(w 2^64 / m)); the Shoup product of any 64-bit value is below 2m.
+// Ten multiply instructions.
+//
+// Split (N >= 2^12): the values carry a factor of two, X = 2x, and the modulus is m = 2q.  With
+// x = x1 2^31 + x0, so that X's words are x1 and 2 x0 without any shift, and v = w 2^31 mod q,
+//   x w = x1 v + x0 w,   X w = x1 (2v) + (2 x0) w  (mod m),
+// and the quotient by q is x1 v / q + x0 w / q, below 2^32 for x < 2^62: from
+// vq = floor(v 2^32 / q) and wq = floor(w 2^31 / q) with two high words,
+//   h = floor(x1 vq / 2^32) + floor(2 x0 wq / 2^32),
+// short by less than x1 / 2^32 + 1 (the truncated constants) + 2 (the floors), so that
+// X w - h m is below 2 (3.5 q) < 4m.  Eight multiply instructions: 1.24 T butterflies/s of the
+// multiplier alone (152 SMs), 1.04 exact ones.
+struct Tw3 {
+    u64 w, v;         // w, 2 (w 2^31 mod q)
+    uint32_t wq, vq;  // floor(w 2^31 / q), floor((w 2^31 mod q) 2^32 / q)
+};
+__device__ __forceinline__ u64 tw_mul(u64 x, ulonglong2 w, u64 m) { return mul_shoup_lazy(x, w.x, w.y, m); }
+__device__ __forceinline__ u64 tw_mul(u64 x, const Tw3 &w, u64 m) {
+    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32);
+    const uint32_t h = __umulhi(x1, w.vq) + __umulhi(x0, w.wq);
+    return (u64)x1 * w.v + (u64)x0 * w.w - (u64)h * m;
+}
+// what a product stays below, in units of m
+__device__ __forceinline__ constexpr u64 tw_bound(const ulonglong2 &) { return 2; }
+__device__ __forceinline__ constexpr u64 tw_bound(const Tw3 &) { return 4; }
+
+// Forward butterfly without a correction step: the product V is below B m (B = 2 or 4), so
+// x' = U + V and y' = U - V + B m only grow by B m per stage.  From inputs below 2m, exact values
+// stay below (2 log2 N + 2) m <= 24m (N <= 2^11, m = q) and split ones (the last two to four
+// stages of which are exact) below 54m < 2^62 (m = 2q, x < 2^61) for primes below 2^55 (the
 // context's limit); the final store reduces them once.
-__device__ __forceinline__ void bf_fwd(u64 &x, u64 &y, ulonglong2 w, u64 q, u64 q2) {
+template <class TW>
+__device__ __forceinline__ void bf_fwd(u64 &x, u64 &y, const TW &w, u64 m) {
     const u64 U = x;
-    const u64 V = mul_shoup_lazy(y, w.x, w.y, q);
+    const u64 V = tw_mul(y, w, m);
     x = U + V;
-    y = U - V + q2;
+    y = U - V + tw_bound(w) * m;
 }
 
 // Inverse butterfly without a correction step, for a stage whose inputs are below c (a
-// multiple of q): U - V + c is positive and below 2c, so the product is the same residue,
-// x' = U + V < 2c and y' < 2q.  From inputs below c0 (q or 2q), stage u of a pass takes
-// c = 2^u c0; a pass of at most 8 stages from q, or 7 from 2q, stays below 2^63 for primes below
-// 2^55 (the context's limit) and is reduced once before the next pass or the scaling.
-__device__ __forceinline__ void bf_inv(u64 &x, u64 &y, ulonglong2 w, u64 q, u64 c) {
+// multiple of m, at least B m / 2): U - V + c is positive and below 2c, so the product is the
+// same residue, x' = U + V < 2c and y' < B m <= 2c.  From inputs below c0, stage u of a pass takes
+// c = 2^u c0.  The products' inputs stay below 2^63: passes of more than four stages lower the
+// values that four stages from 8m would take past that (inv_cap).
+template <class TW>
+__device__ __forceinline__ void bf_inv(u64 &x, u64 &y, const TW &w, u64 m, u64 c) {
     const u64 U = x, V = y;
     x = U + V;
-    y = mul_shoup_lazy(U - V + c, w.x, w.y, q);
+    y = tw_mul(U - V + c, w, m);
+}
+
+// a doubled value reduced below 2m = 4q (reduce64_lazy of modulus 2q)
+__device__ __forceinline__ u64 reduce2_lazy(u64 x, const PrimeDev &P) {
+    if (P.one_sh >> 33) return mul_shoup_lazy(x, 1, P.one_sh >> 1, 2 * P.q);
+    const uint32_t c = (uint32_t)(P.one_sh >> 1);
+    const uint32_t h = (uint32_t)(((x >> 32) * c + __umulhi((uint32_t)x, c)) >> 32);
+    return x - (u64)h * (2 * P.q);
 }
 
 // a transform's lazy value reduced to [0, q)
@@ -88,32 +128,45 @@ __device__ __forceinline__ u64 fwd_reduce(u64 v, const PrimeDev &P) {
 // K forward stages (distances 2^(K-1), .., 1 within groups of 2^K) on 16 registers;
 // tw(s, il): the pair of stage s, group il < 16 >> (K - s)
 template <int K, class TW>
-__device__ __forceinline__ void stages_fwd(u64 (&v)[16], u64 q, u64 q2, TW tw) {
+__device__ __forceinline__ void stages_fwd(u64 (&v)[16], u64 m, TW tw) {
 #pragma unroll
     for (int s = 0; s < K; s++) {
         const int ld = K - 1 - s, d = 1 << ld;
-        ulonglong2 w;
+        decltype(tw(0, 0)) w;
 #pragma unroll
         for (int x = 0; x < 8; x++) {
             const int il = x >> ld, j = x & (d - 1);
             if (j == 0) w = tw(s, il);
-            bf_fwd(v[2 * d * il + j], v[2 * d * il + d + j], w, q, q2);
+            bf_fwd(v[2 * d * il + j], v[2 * d * il + d + j], w, m);
         }
     }
 }
 // K inverse stages (distances 1, .., 2^(K-1)); inputs below c0; tw(s, il): il < 8 >> s
 template <int K, class TW>
-__device__ __forceinline__ void stages_inv(u64 (&v)[16], u64 q, u64 c0, TW tw) {
+__device__ __forceinline__ void stages_inv(u64 (&v)[16], u64 m, u64 c0, TW tw) {
 #pragma unroll
     for (int s = 0; s < K; s++) {
         const int d = 1 << s;
-        ulonglong2 w;
+        decltype(tw(0, 0)) w;
 #pragma unroll
         for (int x = 0; x < 8; x++) {
             const int il = x >> s, j = x & (d - 1);
             if (j == 0) w = tw(s, il);
-            bf_inv(v[2 * d * il + j], v[2 * d * il + d + j], w, q, c0 << s);
+            bf_inv(v[2 * d * il + j], v[2 * d * il + d + j], w, m, c0 << s);
         }
+    }
+}
+
+// After K inverse stages from inputs below C m with products below B m, value j of a group of 2^K
+// is below C 2^K m (j = 0: sums only) or B 2^(K - 1 - b) m (b: its highest bit, the last stage at
+// which it was the product).  Those that can pass 8m are reduced below 2m.
+template <int K, int C, int B>
+__device__ __forceinline__ void inv_cap(u64 (&v)[16], const PrimeDev &P) {
+#pragma unroll
+    for (int x = 0; x < 16; x++) {
+        const int j = x & ((1 << K) - 1);
+        const int bound = j == 0 ? C << K : (B << (K - 1)) >> (j >= 8 ? 3 : j >= 4 ? 2 : j >= 2 ? 1 : 0);
+        if (bound > 8) v[x] = reduce2_lazy(v[x], P);
     }
 }
 
@@ -127,76 +180,104 @@ __device__ __forceinline__ ulonglong2 pair_at(const ulonglong2 *p) {
 // read 16 consecutive coefficients each hit different banks, as do 16 that read a run.
 constexpr int PTILE = TILE + TILE / 16;
 __device__ __forceinline__ int pad(int f) { return f + (f >> 4); }
+// pad(f + d) - pad(f) where f mod 16 + d mod 16 < 16
+__device__ __forceinline__ constexpr int padc(int d) { return d + (d >> 4); }
 
-// twiddles of the passes (T: the prime's pairs in natural order, low: this tile's low row pairs
-// of this thread, [pair][thread]); the column stages use the first 2^A pairs only
+// a table of split twiddles: (w, 2v) and (wq, vq)
+struct Tab3 {
+    const ulonglong2 *w;
+    const uint2 *q;
+    __device__ __forceinline__ Tab3 operator+(size_t k) const { return Tab3{w + k, q + k}; }
+};
+template <bool SH>
+__device__ __forceinline__ Tw3 tw3_at(const Tab3 &t, int k) {
+    ulonglong2 a;
+    uint2 b;
+    if constexpr (SH) {
+        a = t.w[k];
+        b = t.q[k];
+    } else {
+        a = __ldg(t.w + k);
+        b = __ldg(t.q + k);
+    }
+    return Tw3{a.x, a.y, b.x, b.y};
+}
+
+// twiddles of the passes (T: the prime's split twiddles in natural order, low: this tile's low
+// row twiddles of this thread, [pair][thread]); the column stages use the first 2^A twiddles only.
+// The low ones are one per butterfly, so that their bytes count: split ones gain for the four low
+// stages of N = 2^15 (1024 residue polynomials forward / inverse 295 / 334 us with exact pairs,
+// 288 / 325 split) and lose for the three of N = 2^14 (147 / 162 exact, 145 / 165 split).
 //
 // forward column stages 0..3: the whole transform's first 15 twiddles
 template <bool SH>
 struct TwColTop {
-    const ulonglong2 *T;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return pair_at<SH>(T + (1 << s) + il); }
+    Tab3 T;
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const { return tw3_at<SH>(T, (1 << s) + il); }
 };
 // forward column stages 4..A-1 of rows 16 b ..
 template <int A, bool SH>
 struct TwColLow {
-    const ulonglong2 *T;
+    Tab3 T;
     int b;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return pair_at<SH>(T + (1 << (4 + s)) + ((16 * b) >> (A - 4 - s)) + il);
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const {
+        return tw3_at<SH>(T, (1 << (4 + s)) + ((16 * b) >> (A - 4 - s)) + il);
     }
 };
 // forward row stages 0..3 of one row
 template <int A>
 struct TwRowTop {
-    const ulonglong2 *T;
+    Tab3 T;
     int row;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return pair_at<false>(T + (1 << (A + s)) + (row << s) + il);
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const {
+        return tw3_at<false>(T, (1 << (A + s)) + (row << s) + il);
     }
 };
 // the same, and the last four inverse row stages, from a copy of the 15 pairs of each of a tile's
 // R rows, those of 2^u groups per row at R (2^u - 1) (gr: the row within the tile)
 template <int R, bool INV>
 struct TwRowTopSh {
-    const ulonglong2 *W;
+    Tab3 T;
     int gr;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const {
         const int u = INV ? 3 - s : s;
-        return W[R * ((1 << u) - 1) + (gr << u) + il];
+        return tw3_at<true>(T, R * ((1 << u) - 1) + (gr << u) + il);
     }
 };
-// low row stages in thread order: the pairs of stage s follow those of the stages before
+// low row stages in thread order: the twiddles of stage s follow those of the stages before
 template <int K, bool INV, bool SH>
 struct TwRowLow {
-    const ulonglong2 *low;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        const int off = INV ? 16 - (16 >> s) : (16 >> (K - s)) - (16 >> K);
-        return pair_at<SH>(low + (off + il) * NTHR);
+    static constexpr bool SPLIT = K == 4;  // LB = 8
+    static constexpr int B = SPLIT ? 4 : 2;
+    Tab3 low;
+    __device__ __forceinline__ auto operator()(int s, int il) const {
+        const int k = ((INV ? 16 - (16 >> s) : (16 >> (K - s)) - (16 >> K)) + il) * NTHR;
+        if constexpr (SPLIT) return tw3_at<SH>(low, k);
+        else return pair_at<SH>(low.w + k);
     }
 };
 // inverse column stages of distance 2^s rows, rows 16 b ..
 template <int A, bool SH>
 struct TwInvColLow {
-    const ulonglong2 *T;
+    Tab3 T;
     int b;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return pair_at<SH>(T + (1 << (A - 1 - s)) + ((16 * b) >> (s + 1)) + il);
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const {
+        return tw3_at<SH>(T, (1 << (A - 1 - s)) + ((16 * b) >> (s + 1)) + il);
     }
 };
 // the last four inverse column stages
 template <bool SH>
 struct TwInvColTop {
-    const ulonglong2 *T;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const { return pair_at<SH>(T + (1 << (3 - s)) + il); }
+    Tab3 T;
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const { return tw3_at<SH>(T, (1 << (3 - s)) + il); }
 };
 // the last four inverse row stages of one row
 template <int A>
 struct TwInvRowTop {
-    const ulonglong2 *T;
+    Tab3 T;
     int row;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int il) const {
-        return pair_at<false>(T + (1 << (A + 3 - s)) + (row << (3 - s)) + il);
+    __device__ __forceinline__ Tw3 operator()(int s, int il) const {
+        return tw3_at<false>(T, (1 << (A + 3 - s)) + (row << (3 - s)) + il);
     }
 };
 
@@ -205,7 +286,7 @@ struct TwInvRowTop {
 // the thread ends with rows 16 b .. 16 b + 15 of its column.  SH: the first 2^A pairs at T are
 // the block's copy, complete after `arrived`.
 template <int LOGN, int KL, bool SH, class IO, class ARR>
-__device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T, u64 q,
+__device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int tile, Tab3 T, u64 q,
                                          u64 *sm, u64 (&v)[16], ARR arrived) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
@@ -215,16 +296,16 @@ __device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int 
         u64 x[KL];
         load_n(io, p, r, g, n0 + KL * h * dn, dn, x);
 #pragma unroll
-        for (int m = 0; m < KL; m++) v[KL * h + m] = x[m];
+        for (int m = 0; m < KL; m++) v[KL * h + m] = 2 * x[m];
     }
     arrived();
-    stages_fwd<4>(v, q, 2 * q, TwColTop<SH>{T});
+    stages_fwd<4>(v, 2 * q, TwColTop<SH>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[((i + m * S::SA) << S::LC) + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((16 * i + m) << S::LC) + c];
-    stages_fwd<S::A - 4>(v, q, 2 * q, TwColLow<S::A, SH>{T, i});
+    stages_fwd<S::A - 4>(v, 2 * q, TwColLow<S::A, SH>{T, i});
 }
 
 // Forward row half: v holds coefficients i + m SB of the thread's row (i = t mod SB); all LB row
@@ -235,24 +316,25 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
                                          const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, i = t & (S::SB - 1), gr = t / S::SB;
-    const u64 q = P.q;
+    const u64 m2 = 2 * P.q;
     const int f0 = (t & ~31) * 16 + (t & 31);
+    u64 *seq = sm + pad((gr << S::LB) + i), *own = sm + pad(16 * t), *run = sm + pad(f0);
     const size_t k0 = ((size_t)tile << 11) + f0;
     u64 u[4][4];
     if (EARLY) {
 #pragma unroll
         for (int h = 0; h < 4; h++) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
     }
-    stages_fwd<4>(v, q, 2 * q, top);
+    stages_fwd<4>(v, m2, top);
 #pragma unroll
-    for (int m = 0; m < 16; m++) sm[pad((gr << S::LB) + i + m * S::SB)] = v[m];
+    for (int m = 0; m < 16; m++) seq[padc(m * S::SB)] = v[m];
     __syncthreads();
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * t + m)];
-    stages_fwd<S::LB - 4>(v, q, 2 * q, low);
+    for (int m = 0; m < 16; m++) v[m] = own[m];
+    stages_fwd<S::LB - 4>(v, m2, low);
     // to runs of 32 coefficients per warp access, within the warp's 512
 #pragma unroll
-    for (int m = 0; m < 16; m++) sm[pad(16 * t + m)] = v[m];
+    for (int m = 0; m < 16; m++) own[m] = v[m];
     __syncwarp();
 #pragma unroll
     for (int h = 0; h < 4; h++) {
@@ -260,7 +342,7 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
         if (!EARLY) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
 #pragma unroll
         for (int m = 0; m < 4; m++) {
-            x[m] = sm[pad(f0 + 32 * (4 * h + m))];
+            x[m] = run[padc(32 * (4 * h + m))] >> 1;
             if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
         }
         store_n(io, p, r, g, k0 + 128 * h, 32, x, u[h]);
@@ -268,31 +350,33 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
 }
 
 // Inverse row half: the tile through io.load, all LB row stages; the thread ends with
-// coefficients i + m SB of its row, reduced below 2q.  `arrived`: the twiddles' copies complete.
+// coefficients i + m SB of its row, doubled, below 4q.  `arrived`: the twiddles' copies complete.
 template <int LOGN, class IO, class TOP, class LOW, class ARR>
 __device__ __forceinline__ void inv_rows(const IO &io, int p, int r, int g, int tile, TOP top, LOW low,
                                          const PrimeDev &P, u64 *sm, u64 (&v)[16], ARR arrived) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, i = t & (S::SB - 1), gr = t / S::SB;
-    const u64 q = P.q;
+    const u64 m2 = 2 * P.q;
     const int f0 = (t & ~31) * 16 + (t & 31);
+    u64 *seq = sm + pad((gr << S::LB) + i), *own = sm + pad(16 * t), *run = sm + pad(f0);
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = io.load(p, r, g, ((size_t)tile << 11) + f0 + 32 * m);
+    for (int m = 0; m < 16; m++) v[m] = 2 * io.load(p, r, g, ((size_t)tile << 11) + f0 + 32 * m);
 #pragma unroll
-    for (int m = 0; m < 16; m++) sm[pad(f0 + 32 * m)] = v[m];
+    for (int m = 0; m < 16; m++) run[padc(32 * m)] = v[m];
     arrived();
     __syncwarp();
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * t + m)];
-    stages_inv<S::LB - 4>(v, q, q, low);
+    for (int m = 0; m < 16; m++) v[m] = own[m];
+    stages_inv<S::LB - 4>(v, m2, LOW::B / 2 * m2, low);
+    inv_cap<S::LB - 4, LOW::B / 2, LOW::B>(v, P);
 #pragma unroll
-    for (int m = 0; m < 16; m++) sm[pad(16 * t + m)] = v[m];
+    for (int m = 0; m < 16; m++) own[m] = v[m];
     __syncthreads();
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = sm[pad((gr << S::LB) + i + m * S::SB)];
-    stages_inv<4>(v, q, q << (S::LB - 4), top);
+    for (int m = 0; m < 16; m++) v[m] = seq[padc(m * S::SB)];
+    stages_inv<4>(v, m2, 8 * m2, top);
 #pragma unroll
-    for (int m = 0; m < 16; m++) v[m] = reduce64_lazy(v[m], P);
+    for (int m = 0; m < 16; m++) v[m] = reduce2_lazy(v[m], P);
 }
 
 // an inverse transform's result: scaled, and stored as a conversion's digit where asked (centred,
@@ -306,23 +390,25 @@ __device__ __forceinline__ u64 inv_result(u64 v, Shoup sc, bool digits, u64 q) {
     return x;
 }
 
-// Inverse column half: v holds rows 16 b .. 16 b + 15 of the thread's column (below 2q); all A
+// Inverse column half: v holds rows 16 b .. 16 b + 15 of the thread's column (doubled, below 4q); all A
 // column stages, scaled and stored through io.
 template <int LOGN, bool SH, class IO>
-__device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int tile, const ulonglong2 *T, Shoup sc,
-                                         bool digits, u64 q, u64 *sm, u64 (&v)[16]) {
+__device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int tile, Tab3 T, Shoup sc,
+                                         bool digits, const PrimeDev &P, u64 *sm, u64 (&v)[16]) {
     using S = Shape<LOGN>;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
-    stages_inv<S::A - 4>(v, q, 2 * q, TwInvColLow<S::A, SH>{T, i});
+    const u64 m2 = 2 * P.q;
+    stages_inv<S::A - 4>(v, m2, 2 * m2, TwInvColLow<S::A, SH>{T, i});
+    inv_cap<S::A - 4, 2, 4>(v, P);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[((16 * i + m) << S::LC) + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((i + m * S::SA) << S::LC) + c];
-    stages_inv<4>(v, q, (2 * q) << (S::A - 4), TwInvColTop<SH>{T});
+    stages_inv<4>(v, m2, 8 * m2, TwInvColTop<SH>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++)
-        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m], sc, digits, q));
+        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m] >> 1, sc, digits, P.q));
 }
 
 // ---------------------------------------------------------------- tiled: two launches
@@ -346,17 +432,20 @@ __device__ __forceinline__ TileAt tile_at(const NttBatch &b, int L, int tiles) {
     t.g = ntt_prime(b, t.r, L);
     return t;
 }
-// the low row pairs of a tile within their table
-template <int LOGN>
-__device__ __forceinline__ size_t low_at(const TileAt &t) {
-    return ((size_t)t.g * Shape<LOGN>::TILES + t.tile) * Shape<LOGN>::PAIRS * NTHR;
-}
 // constant tables of a launch
 struct NttTables {
     const PrimeDev *pr;
-    const ulonglong2 *tw;   // [NP][N] pairs in natural order
-    const ulonglong2 *low;  // [NP][N / 2048][PAIRS][128] low row pairs
+    const ulonglong2 *tw;   // [NP][N] in natural order: exact pairs of q, or (N >= 2^12) (w, 2v) of split twiddles
+    const uint2 *twq;       // and their (wq, vq)
+    const ulonglong2 *low;  // [NP][N / 2048][PAIRS][128] low row twiddles: exact pairs of 2q, or (N = 2^15)
+    const uint2 *lowq;      // split
     int L;
+    // the low row twiddles of a tile
+    template <int LOGN>
+    __device__ __forceinline__ Tab3 low_of(const TileAt &t) const {
+        return Tab3{low, lowq} + ((size_t)t.g * Shape<LOGN>::TILES + t.tile) * Shape<LOGN>::PAIRS * NTHR;
+    }
+    __device__ __forceinline__ Tab3 tab(int g, int logN) const { return Tab3{tw, twq} + ((size_t)g << logN); }
 };
 constexpr int FWD_BLOCKS = 6, INV_BLOCKS = 6;  // blocks per SM that the register count allows for (5: 2% slower, 4: 4%)
 
@@ -373,7 +462,7 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_cols(const __grid_
         return;
     }
     u64 v[16];
-    fwd_cols<LOGN, 4, false>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), tb.pr[t.g].q, sm, v, [] {});
+    fwd_cols<LOGN, 4, false>(io, t.p, t.r, t.g, t.tile, tb.tab(t.g, LOGN), tb.pr[t.g].q, sm, v, [] {});
     const int c = threadIdx.x & (S::C - 1), i = threadIdx.x >> S::LC;
     u64 *o = mid.base + t.p * mid.ps + ((size_t)(t.r - mid.r0) << LOGN) + ((size_t)t.tile << S::LC) + c;
 #pragma unroll
@@ -396,8 +485,8 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_rows(const __grid_
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = in[m * S::SB];
     fwd_rows<LOGN, false>(io, t.p, t.r, t.g, t.tile,
-                          TwRowTop<S::A>{tb.tw + ((size_t)t.g << LOGN), (t.tile << S::LR) + gr},
-                          TwRowLow<S::LB - 4, false, false>{tb.low + low_at<LOGN>(t) + th}, tb.pr[t.g], sm, v);
+                          TwRowTop<S::A>{tb.tab(t.g, LOGN), (t.tile << S::LR) + gr},
+                          TwRowLow<S::LB - 4, false, false>{tb.low_of<LOGN>(t) + th}, tb.pr[t.g], sm, v);
 }
 
 template <int LOGN, class IO>
@@ -412,8 +501,8 @@ __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_rows(const __grid_
     const int th = threadIdx.x, i = th & (S::SB - 1), gr = th / S::SB;
     u64 v[16];
     inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile,
-                   TwInvRowTop<S::A>{tb.tw + ((size_t)t.g << LOGN), (t.tile << S::LR) + gr},
-                   TwRowLow<S::LB - 4, true, false>{tb.low + low_at<LOGN>(t) + th}, tb.pr[t.g], sm, v, [] {});
+                   TwInvRowTop<S::A>{tb.tab(t.g, LOGN), (t.tile << S::LR) + gr},
+                   TwRowLow<S::LB - 4, true, false>{tb.low_of<LOGN>(t) + th}, tb.pr[t.g], sm, v, [] {});
     u64 *o = mid.base + t.p * mid.ps + ((size_t)(t.r - mid.r0) << LOGN) + ((size_t)t.tile << 11) + (gr << S::LB) + i;
 #pragma unroll
     for (int m = 0; m < 16; m++) o[m * S::SB] = v[m];
@@ -435,7 +524,7 @@ __global__ void __launch_bounds__(NTHR, INV_BLOCKS) k_ntt_inv_cols(const __grid_
     for (int m = 0; m < 16; m++) v[m] = in[(size_t)(16 * i + m) << S::LB];
     const PrimeDev P = tb.pr[t.g];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN, false>(io, t.p, t.r, t.g, t.tile, tb.tw + ((size_t)t.g << LOGN), sc, b.digits, P.q, sm, v);
+    inv_cols<LOGN, false>(io, t.p, t.r, t.g, t.tile, tb.tab(t.g, LOGN), sc, b.digits, P, sm, v);
 }
 
 // ---------------------------------------------------------------- clusters: one launch
@@ -448,23 +537,34 @@ template <int LOGN>
 struct ClusterSmem {
     u64 colt[TILE], rowt[PTILE];
     ulonglong2 low[Shape<LOGN>::PAIRS * NTHR];  // [pair][thread]
+    uint2 lowq[LOGN == 15 ? Shape<LOGN>::PAIRS * NTHR : 1];
     ulonglong2 top[15 * Shape<LOGN>::R];        // TwRowTopSh
-    ulonglong2 col[1 << Shape<LOGN>::A];        // the prime's first 2^A pairs
+    ulonglong2 col[1 << Shape<LOGN>::A];        // the prime's first 2^A twiddles
+    uint2 topq[15 * Shape<LOGN>::R], colq[1 << Shape<LOGN>::A];
 };
 // each thread copies the low pairs that it uses itself
 template <int LOGN>
 __device__ __forceinline__ void copy_twiddles(ClusterSmem<LOGN> &S, const NttTables &tb, const TileAt &t) {
     using H = Shape<LOGN>;
     const int th = threadIdx.x;
-    const ulonglong2 *T = tb.tw + ((size_t)t.g << LOGN), *low = tb.low + low_at<LOGN>(t);
-    for (int e = th; e < (1 << H::A); e += NTHR) cp_async16(&S.col[e], T + e);
+    const Tab3 T = tb.tab(t.g, LOGN);
+    const Tab3 low = tb.low_of<LOGN>(t);
+    for (int e = th; e < (1 << H::A); e += NTHR) {
+        cp_async16(&S.col[e], T.w + e);
+        cp_async8(&S.colq[e], T.q + e);
+    }
     for (int e = th; e < 15 * H::R; e += NTHR) {
         // entry R (2^u - 1) + k: pair 2^(A + u) + (row0 << u) + k
         const int u = 31 - __clz(e / H::R + 1), k = e - H::R * ((1 << u) - 1);
-        cp_async16(&S.top[e], T + (1 << (H::A + u)) + ((t.tile << H::LR) << u) + k);
+        const int at = (1 << (H::A + u)) + ((t.tile << H::LR) << u) + k;
+        cp_async16(&S.top[e], T.w + at);
+        cp_async8(&S.topq[e], T.q + at);
     }
 #pragma unroll
-    for (int k = 0; k < H::PAIRS; k++) cp_async16(&S.low[k * NTHR + th], low + k * NTHR + th);
+    for (int k = 0; k < H::PAIRS; k++) {
+        cp_async16(&S.low[k * NTHR + th], low.w + k * NTHR + th);
+        if (LOGN == 15) cp_async8(&S.lowq[k * NTHR + th], low.q + k * NTHR + th);
+    }
     cp_async_commit();
 }
 
@@ -487,7 +587,7 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     dep_wait();
     const PrimeDev P = tb.pr[t.g];
     u64 v[16];
-    fwd_cols<LOGN, 16, true>(io, t.p, t.r, t.g, t.tile, M.col, P.q, M.colt, v, [] {
+    fwd_cols<LOGN, 16, true>(io, t.p, t.r, t.g, t.tile, Tab3{M.col, M.colq}, P.q, M.colt, v, [] {
         cp_async_wait<0>();
         __syncthreads();
     });
@@ -504,8 +604,8 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     cl.sync();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = M.rowt[pad((gr << S::LB) + i + m * S::SB)];
-    fwd_rows<LOGN, true>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, false>{M.top, gr},
-                         TwRowLow<S::LB - 4, false, true>{M.low + th}, P, M.rowt, v);
+    fwd_rows<LOGN, true>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, false>{Tab3{M.top, M.topq}, gr},
+                         TwRowLow<S::LB - 4, false, true>{Tab3{M.low, M.lowq} + th}, P, M.rowt, v);
 }
 
 template <int LOGN, class IO>
@@ -528,8 +628,8 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     const int th = threadIdx.x, i = th & (S::SB - 1), gr = th / S::SB, c = th & (S::C - 1), ic = th >> S::LC;
     u64 v[16];
     // the low pairs are the thread's own copies; the others' are complete after the exchange's barrier
-    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, true>{M.top, gr},
-                   TwRowLow<S::LB - 4, true, true>{M.low + th}, P, M.rowt, v, [] { cp_async_wait<0>(); });
+    inv_rows<LOGN>(io, t.p, t.r, t.g, t.tile, TwRowTopSh<S::R, true>{Tab3{M.top, M.topq}, gr},
+                   TwRowLow<S::LB - 4, true, true>{Tab3{M.low, M.lowq} + th}, P, M.rowt, v, [] { cp_async_wait<0>(); });
     cl.barrier_wait();
     const int row = (t.tile << S::LR) + gr;
 #pragma unroll
@@ -541,7 +641,7 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = M.colt[((16 * ic + m) << S::LC) + c];
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
-    inv_cols<LOGN, true>(io, t.p, t.r, t.g, t.tile, M.col, sc, b.digits, P.q, M.colt, v);
+    inv_cols<LOGN, true>(io, t.p, t.r, t.g, t.tile, Tab3{M.col, M.colq}, sc, b.digits, P, M.colt, v);
 }
 
 // ---------------------------------------------------------------- 2^8 <= N <= 2^11: one block
@@ -578,20 +678,20 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_co
     __syncthreads();
 #pragma unroll
     for (int h = 0; h < 4; h++) operand_n(io, t.p, t.r, (size_t)(th + 4 * h * NT), NT, u[h]);
-    stages_fwd<4>(v, P.q, 2 * P.q, TwColTop<true>{T});
+    stages_fwd<4>(v, P.q, [&](int s, int il) { return T[(1 << s) + il]; });
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
-    stages_fwd<4>(v, P.q, 2 * P.q, [&](int s, int il) { return T[(1 << (4 + s)) + (blk << s) + il]; });
+    stages_fwd<4>(v, P.q, [&](int s, int il) { return T[(1 << (4 + s)) + (blk << s) + il]; });
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = v[m];
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
-        stages_fwd<LS>(v, P.q, 2 * P.q, [&](int s, int il) { return T[(1 << (8 + s)) + ((16 * th) >> (LS - s)) + il]; });
+        stages_fwd<LS>(v, P.q, [&](int s, int il) { return T[(1 << (8 + s)) + ((16 * th) >> (LS - s)) + il]; });
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
@@ -648,7 +748,7 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(th + m * NT)];
-    stages_inv<4>(v, q, 2 * q, TwInvColTop<true>{T});
+    stages_inv<4>(v, q, 2 * q, [&](int s, int il) { return T[(1 << (3 - s)) + il]; });
     const Shoup sc = b.scale ? b.scale[t.r - b.r0] : Shoup{P.ninv, P.ninv_sh};
 #pragma unroll
     for (int m = 0; m < 16; m++) io.store(t.p, t.r, t.g, (size_t)(th + m * NT), inv_result(v[m], sc, b.digits, q));

@@ -28,7 +28,8 @@ inline double butterflies(const copse_ctx *ctx, const NttBatch &b) {
 template <bool INV>
 NttTables tables(const copse_ctx *c) {
     return NttTables{c->d_prime, (const ulonglong2 *)(INV ? c->d_tw_i : c->d_tw_f),
-                     (const ulonglong2 *)(INV ? c->d_low_i : c->d_low_f), c->L};
+                     (const uint2 *)(INV ? c->d_twq_i : c->d_twq_f), (const ulonglong2 *)(INV ? c->d_low_i : c->d_low_f),
+                     (const uint2 *)(INV ? c->d_lowq_i : c->d_lowq_f), c->L};
 }
 
 // A cluster kernel's shared memory, and the opt-in to 16-block clusters (N = 2^15, above the

@@ -79,3 +79,47 @@ def test_negacyclic_product_matches_the_oracle(log_n, most):
         assert_same(dc.cpu().numpy().view(np.uint64), want, "negacyclic product")
     finally:
         K.copse_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("log_n,bits", [(8, 36), (11, 36), (12, 36), (13, 36), (14, 40), (15, 40), (8, 55), (11, 55),
+                                        (12, 55), (13, 55), (14, 55), (15, 55)])
+def test_transforms_at_the_ends_of_their_lazy_ranges(log_n, bits):
+    """Forward and inverse of residues all q - 1, all zero but one, alternating 0 and q - 1, and
+    random ones, at the smallest and the largest primes, in clusters and tiled."""
+    L, N = 2, 1 << log_n
+    P = B.Params(logN=log_n, L=L, bits=bits, dnum=2)
+    ctx = K.copse_ctx_create(log_n, bits, L, 2)
+    try:
+        rng = np.random.default_rng(log_n + bits)
+        x = np.zeros((4, L, N), np.uint64)
+        for r, q in enumerate(P.q):
+            x[0, r] = q - 1
+            x[1, r, N - 1] = q - 1
+            x[2, r, ::2] = q - 1
+            x[3, r] = rng.integers(0, q, size=N, dtype=np.uint64)
+        for most in (ALWAYS, 0):
+            K.copse_ctx_set_ntt_cluster_max(ctx, most)
+            d = torch.from_numpy(x.view(np.int64)).cuda()
+            K.copse_ntt(ctx, d.data_ptr(), 4, L)
+            f = d.clone()
+            K.copse_ntt(ctx, d.data_ptr(), 4, L, inverse=True)
+            # the inverse of the largest values, forward again
+            e = torch.from_numpy(x.view(np.int64)).cuda()
+            K.copse_ntt(ctx, e.data_ptr(), 4, L, inverse=True)
+            K.copse_ntt(ctx, e.data_ptr(), 4, L)
+            torch.cuda.synchronize()
+            got = f.cpu().numpy().view(np.uint64)
+            assert_same(d.cpu().numpy().view(np.uint64), x, "forward and back")
+            assert_same(e.cpu().numpy().view(np.uint64), x, "inverse and forward")
+            for r, q in enumerate(P.q):
+                assert (got[:, r] < q).all()
+                # products of the transforms are the transforms of the products
+                out = np.zeros(N, np.uint64)
+                B.lib().or_negacyclic_mul(x[0, r].copy(), x[3, r].copy(), log_n, q, out)
+                prod = np.array([int(a) * int(b) % q for a, b in zip(got[0, r], got[3, r])], np.uint64)
+                t = torch.from_numpy(np.stack([prod] * L).view(np.int64)).cuda()
+                K.copse_ntt(ctx, t.data_ptr(), 1, L, inverse=True)
+                torch.cuda.synchronize()
+                assert_same(t.cpu().numpy().view(np.uint64)[r], out, f"product, prime {r}")
+    finally:
+        K.copse_ctx_destroy(ctx)
