@@ -27,6 +27,7 @@ constexpr int KS_TPB = 128;           // threads of the key-switch kernels (two 
 constexpr int MAX_ALPHA = 40;
 constexpr int MM_ACC = 32;            // accumulators per launch (their diagonals' addresses are kernel parameters)
 constexpr int MM_TPB = 64;            // two elements a thread
+constexpr int MM_PER_SM = 9;          // blocks per SM that the registers are cut for
 constexpr int MM_RING = 4;            // rotations that a thread has in flight or in shared memory
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
@@ -404,12 +405,15 @@ __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 
 //
 // The diagonals of an accumulator usually lie one after another (a model stores them in that
 // order, zero ones left out): then their addresses are one pointer that advances (DENSE), and
-// only accumulators with zero diagonals look them up (and copy zeros in their place).
+// only accumulators with zero diagonals look them up (and leave those out).
 //
-// 24 accumulators of 60 rotations, 10 residues, N = 2^15: 0.94 ms (4.0 TB/s of diagonals) with
-// plain loads of four rotations at a time and one element a thread, 0.65 (5.8) so; one element a
-// thread 0.71, three accumulators 0.67, eight rotations in flight the same.  Of the first step
-// half were instructions that split_k now avoids (117 -> 72 per rotation and warp).
+// Bytes of diagonals per second over a 64-branch forest's 69 + 378 accumulators of 64 rotations at
+// N = 2^15, one of the two matrices half zero (14 GB): 4.1 TB/s with plain loads of four rotations
+// at a time and one element a thread; 4.8 by asynchronous copies with tiles of four accumulators
+// (158 registers, six blocks an SM: too few warps for the latencies of shared memory and of the
+// multiplier); three accumulators 5.3 at eight blocks, 6.2 at nine (96 registers) of the 6.8 that
+// a copy reaches; two 5.9 at ten.  Rings of three and four rotations measure the same.  Half of
+// the first step was instructions that split_k now avoids (117 -> 72 per rotation and warp).
 template <int NA, bool DENSE>
 __device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, int x0, int k0, int k1, size_t n_el,
                                         size_t e, Pair2 (*ring)[NA + 2][MM_TPB], DotAcc (&a)[NA]) {
@@ -422,9 +426,9 @@ __device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, 
         for (int c = 0; c < 2; c++) a[x].a[c][0] = a[x].a[c][1] = AccK{0, 0, 0};
         if (DENSE) p[x] = tab.pt[(x0 + x) * nrot] + (size_t)k0 * n_el + e;
     }
-    auto load = [&](int k) {
+    auto load = [&](int k, int slot) {
         if (k < k1) {
-            Pair2(&d)[NA + 2][MM_TPB] = ring[(k - k0) % MM_RING];
+            Pair2(&d)[NA + 2][MM_TPB] = ring[slot];
             cp_async16(&d[0][t], R);
             cp_async16(&d[1][t], R + n_el);
             R += 2 * n_el;
@@ -435,29 +439,53 @@ __device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, 
                     p[x] += n_el;
                 } else {
                     const u64 *q = x0 + x < nacc ? tab.pt[(x0 + x) * nrot + k] : nullptr;
-                    if (q)
-                        cp_async16(&d[2 + x][t], q + e);
-                    else
-                        d[2 + x][t] = Pair2{0, 0};
+                    if (q) cp_async16(&d[2 + x][t], q + e);
                 }
             }
         }
         cp_async_commit();
     };
+    auto products = [&](int k, int slot) {
+        const Pair2(&d)[NA + 2][MM_TPB] = ring[slot];
+        const Pair2 r[2] = {d[0][t], d[1][t]};
+        uint2 y[2][2];
+        uint32_t ys[2][2];
 #pragma unroll
-    for (int i = 0; i < MM_RING - 1; i++) load(k0 + i);
-    for (int k = k0; k < k1; k++) {
-        load(k + MM_RING - 1);
-        cp_async_wait<MM_RING - 1>();
-        const Pair2(&d)[NA + 2][MM_TPB] = ring[(k - k0) % MM_RING];
-        const Pair2 r0 = d[0][t], r1 = d[1][t];
+        for (int c = 0; c < 2; c++) {
+            y[c][0] = split_k(r[c].x0);
+            y[c][1] = split_k(r[c].x1);
+            ys[c][0] = y[c][0].x + y[c][0].y;
+            ys[c][1] = y[c][1].x + y[c][1].y;
+        }
 #pragma unroll
-        for (int x = 0; x < NA; x++) dot_term(a[x], d[2 + x][t], r0, r1);
+        for (int x = 0; x < NA; x++) {
+            if (!DENSE && !(x0 + x < nacc && tab.pt[(x0 + x) * nrot + k])) continue;  // the same for every thread
+            const Pair2 w = d[2 + x][t];
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const uint2 u = split_k(e ? w.x1 : w.x0);
+                const uint32_t us = u.x + u.y;
+                mac_k(a[x].a[0][e], u, us, y[0][e], ys[0][e]);
+                mac_k(a[x].a[1][e], u, us, y[1][e], ys[1][e]);
+            }
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < MM_RING - 1; i++) load(k0 + i, i);
+    for (int k = k0; k < k1; k += MM_RING) {
+#pragma unroll
+        for (int i = 0; i < MM_RING; i++) {
+            if (k + i < k1) {
+                load(k + i + MM_RING - 1, (i + MM_RING - 1) % MM_RING);
+                cp_async_wait<MM_RING - 1>();
+                products(k + i, i);
+            }
+        }
     }
 }
 
 template <int NA>
-__global__ void __launch_bounds__(MM_TPB, 6) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
+__global__ void __launch_bounds__(MM_TPB, MM_PER_SM) k_mm_mac(int nrot, int nacc, int first, const __grid_constant__ MmTable tab,
                                                    size_t part_stride, int ell, int alpha, int L, int logN,
                                                    const PrimeDev *pr) {
     dep_trigger();
@@ -1348,7 +1376,7 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
         // partial sums where the elements and accumulators alone make too few blocks
         const size_t blocks = nacc < MM_PRECOMPUTE_ACC ? ks_blocks((size_t)nx * N)
-                                                       : ((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 3) / 4);
+                                                       : ((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 2) / 3);
         const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
                                                  (MM_BLOCKS + blocks - 1) / blocks});
         const size_t part_stride = (size_t)nacc * ext;
@@ -1421,10 +1449,8 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                                       c->ks));
                 else if (na <= 2)
                     TIMED("mm_fused", bytes, s, MM_MAC(2));
-                else if (na == 3 || na == 5 || na == 6 || na == 9)  // as many tiles as of four, fuller
-                    TIMED("mm_fused", bytes, s, MM_MAC(3));
                 else
-                    TIMED("mm_fused", bytes, s, MM_MAC(4));
+                    TIMED("mm_fused", bytes, s, MM_MAC(3));
 #undef MM_MAC
                 LAUNCH_CHECK();
             }
