@@ -320,10 +320,11 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
     const int f0 = (t & ~31) * 16 + (t & 31);
     u64 *seq = sm + pad((gr << S::LB) + i), *own = sm + pad(16 * t), *run = sm + pad(f0);
     const size_t k0 = ((size_t)tile << 11) + f0;
-    u64 u[4][4];
+    constexpr int H = EARLY ? 4 : 8;  // coefficients stored together
+    u64 u[16 / H][H];
     if (EARLY) {
 #pragma unroll
-        for (int h = 0; h < 4; h++) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
+        for (int h = 0; h < 16 / H; h++) operand_n(io, p, r, k0 + 32 * H * h, 32, u[h]);
     }
     stages_fwd<4>(v, m2, top);
 #pragma unroll
@@ -337,15 +338,15 @@ __device__ __forceinline__ void fwd_rows(const IO &io, int p, int r, int g, int 
     for (int m = 0; m < 16; m++) own[m] = v[m];
     __syncwarp();
 #pragma unroll
-    for (int h = 0; h < 4; h++) {
-        u64 x[4];
-        if (!EARLY) operand_n(io, p, r, k0 + 128 * h, 32, u[h]);
+    for (int h = 0; h < 16 / H; h++) {
+        u64 x[H];
+        if (!EARLY) operand_n(io, p, r, k0 + 32 * H * h, 32, u[h]);
 #pragma unroll
-        for (int m = 0; m < 4; m++) {
-            x[m] = run[padc(32 * (4 * h + m))] >> 1;
+        for (int m = 0; m < H; m++) {
+            x[m] = run[padc(32 * (H * h + m))] >> 1;
             if (!IO::RAW) x[m] = fwd_reduce(x[m], P);
         }
-        store_n(io, p, r, g, k0 + 128 * h, 32, x, u[h]);
+        store_n(io, p, r, g, k0 + 32 * H * h, 32, x, u[h]);
     }
 }
 
