@@ -207,8 +207,8 @@ copse_status ntt_stage_tables(copse_ctx *ctx) {
     // Clusters up to about the blocks that fit the GPU at once (three of a cluster kernel's blocks
     // per SM), two launches above; the tuner or the caller may set other crossovers.  Measured at
     // N = 2^14 (us a forward transform in a graph, clusters / tiled): 16 residue polynomials
-    // 9.5 / 8.1, 32: 9.8 / 10.1, 48: 12.5 / 12.9, 64: 22.2 / 15.5, 128: 32.9 / 23.7; whole
-    // inferences are flat between 32 and 64.
+    // 8.7 / 8.0, 32: 9.2 / 9.6, 48: 11.6 / 11.6, 64: 20.2 / 14.3, 128: 29.8 / 21.8; whole
+    // inferences are flat between 300 and 400 blocks.
     if (ctx->logN >= 12 && ctx->logN < 15) ctx->ntt_cluster_max = ctx->ntt_fused_max = CLUSTER_BLOCKS >> (ctx->logN - 11);
     // one block per transform below 2^12: no low row stages
     const int lb = ctx->logN - ctx->logN / 2, pairs = lb == 8 ? 15 : (lb == 7 ? 14 : 12);
