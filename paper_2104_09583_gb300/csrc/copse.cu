@@ -548,12 +548,12 @@ extern "C" copse_status copse_encrypt_features(copse_ctx *c, const copse_keys *k
     return COPSE_OK;
 }
 
-// The products of one vector with a group of matrices: the plain diagonal method,
-// or its baby-step / giant-step form.
-static copse_status group_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const DeviceModel::Group &G,
-                                 const std::vector<const u64 *> &add, std::vector<DCt> &out, cudaStream_t s) {
-    if (G.plan.plain()) return op_matmul(c, evk, v, G.plan.baby, G.pt, add, out, s);
-    return op_matmul_bsgs(c, evk, v, G.plan.baby, G.pt, G.acc_mat, G.acc_giant, (int)G.plan.n_mat, add, out, s);
+// The products of every query ciphertext's vector with a group of matrices: the plain diagonal
+// method, or its baby-step / giant-step form.
+static copse_status group_matmul(copse_ctx *c, const copse_evk *evk, const std::vector<DCt> &v, const DeviceModel::Group &G,
+                                 const std::vector<const u64 *> &add, std::vector<std::vector<DCt>> &out, cudaStream_t s) {
+    const MatmulGiant giant{&G.acc_mat, &G.acc_giant, (int)G.plan.n_mat};
+    return op_matmul_many(c, evk, v, G.plan.baby, G.pt, add, out, s, G.plan.plain() ? nullptr : &giant);
 }
 
 // SecComp (Section 4.1.2) of nct query ciphertexts, p feature planes each (x[q p + i]):
@@ -742,7 +742,7 @@ static copse_status infer_multi(copse_ctx *c, const copse_evk *evk, copse_model 
     if (m->f.fused) {
         // fused level products: (S_k R) * Decisions XOR Mask_k, no Branches vector
         STATUS_TRY(mark(2));
-        for (int q = 0; q < nct; q++) STATUS_TRY(group_matmul(c, evk, Dc[q], D->Lv, D->mask, lvs[q], s));
+        STATUS_TRY(group_matmul(c, evk, Dc, D->Lv, D->mask, lvs, s));
         for (DCt &x : Dc) ct_free(&x, s);
         STATUS_TRY(mark(3));
         return aggregate(c, evk, m, lvs, nct, results, s, mark);
@@ -752,7 +752,7 @@ static copse_status infer_multi(copse_ctx *c, const copse_evk *evk, copse_model 
     if (enc) {
         STATUS_TRY(enc_matmul(c, evk, *m->enc, Dc, 0, br, s));
     } else {
-        for (int q = 0; q < nct; q++) STATUS_TRY(group_matmul(c, evk, Dc[q], D->R, {nullptr}, br[q], s));
+        STATUS_TRY(group_matmul(c, evk, Dc, D->R, {nullptr}, br, s));
     }
     for (DCt &x : Dc) ct_free(&x, s);
     STATUS_TRY(mark(2));
@@ -762,7 +762,7 @@ static copse_status infer_multi(copse_ctx *c, const copse_evk *evk, copse_model 
     if (enc) {
         STATUS_TRY(enc_matmul(c, evk, *m->enc, B, 1, lvs, s));
     } else {
-        for (int q = 0; q < nct; q++) STATUS_TRY(group_matmul(c, evk, B[q], D->Lv, D->mask, lvs[q], s));
+        STATUS_TRY(group_matmul(c, evk, B, D->Lv, D->mask, lvs, s));
     }
     for (DCt &x : B) ct_free(&x, s);
     STATUS_TRY(mark(3));
@@ -794,11 +794,11 @@ static copse_status aggregate(copse_ctx *c, const copse_evk *evk, copse_model *m
     // label shuffle with padding (Section 7.2): one more plaintext matrix product
     if (!m->f.shuffle_src.empty()) {
         STATUS_TRY(upload_shuffle(c, m, s));
+        std::vector<std::vector<DCt>> o;
+        STATUS_TRY(op_matmul_many(c, evk, results, m->shuf->rots, m->shuf->pt, {nullptr}, o, s));
         for (int q = 0; q < nct; q++) {
-            std::vector<DCt> o;
-            STATUS_TRY(op_matmul(c, evk, results[q], m->shuf->rots, m->shuf->pt, {nullptr}, o, s));
             ct_free(&results[q], s);
-            results[q] = o[0];
+            results[q] = o[q][0];
         }
     }
     STATUS_TRY(mark(4));

@@ -607,22 +607,26 @@ struct AffineJob {
 };
 copse_status op_affine_many(copse_ctx *c, const std::vector<AffineJob> &jobs, cudaStream_t s);
 copse_status op_rotate(copse_ctx *c, const copse_evk *evk, const DCt &a, uint32_t k, DCt *out, cudaStream_t s);
-// Diagonal products sharing the rotations of v: for each accumulator a,
-//   out[a] = modswitch(ModDown(sum_{k: rots[k] != 0} pt[a][k] * R_k) + pt[a][k0] * v + add[a])
+// Diagonal products of several ciphertexts v[q]: those of one level that run together read each
+// diagonal from memory once.  For each v = v[q] and accumulator a, out[q][a] is
+//   modswitch(ModDown(sum_{k: rots[k] != 0} pt[a][k] * R_k) + pt[a][k0] * v + add[a])
 // with R_k the rotation by rots[k] before its ModDown (one ModUp of v serves all k)
 // and k0 the zero rotation if present.  pt[a][k] may be null (zero diagonal);
 // pt pointers are NTT-domain [v.level + alpha][N] (extended basis), add[a] [v.level][N].
-// raw_out set: the sums ModDown(...) + pt[a][k0] * v go to raw_out [nacc][2][v.level][N]
-// (no add, no modswitch) and `out` stays empty.
-copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const std::vector<uint32_t> &rots,
-                       const std::vector<std::vector<const u64 *>> &pt, const std::vector<const u64 *> &add,
-                       std::vector<DCt> &out, cudaStream_t s, u64 *raw_out = nullptr);
-// Baby-step / giant-step products: the baby-step sums of every accumulator
-// (matrix acc_mat[x], giant step acc_giant[x]) share the rotations of v by the
-// baby amounts (op_matmul, raw); then for each matrix a
+// With `giant`, baby-step / giant-step products: the baby-step sums of every accumulator
+// (matrix acc_mat[x], giant step acc_giant[x]), raw (no add, no modswitch), share the rotations of v
+// by the baby amounts; then for each matrix a
 //   out[a] = modswitch(ModDown(sum_{k != 0} R_k(inner[a, k])) + inner[a, 0] + add[a]),
 // R_k the rotation by k before its ModDown; accumulators of one matrix are
 // contiguous with giant steps ascending.
+struct MatmulGiant {
+    const std::vector<int> *acc_mat;
+    const std::vector<uint32_t> *acc_giant;
+    int n_mat;
+};
+copse_status op_matmul_many(copse_ctx *c, const copse_evk *evk, const std::vector<DCt> &v, const std::vector<uint32_t> &rots,
+                            const std::vector<std::vector<const u64 *>> &pt, const std::vector<const u64 *> &add,
+                            std::vector<std::vector<DCt>> &out, cudaStream_t s, const MatmulGiant *giant = nullptr);
 // ---------------------------------------------------------------- encrypted models
 // The model's ciphertexts in canonical order (threshold planes, reshuffle diagonals,
 // level-k diagonals for k = 1..d, masks), each a secret-key encryption at its level
@@ -718,10 +722,6 @@ copse_status op_rotations(copse_ctx *c, const copse_evk *evk, const DCt &v, cons
 copse_status relin_batch(copse_ctx *c, const copse_evk *evk, const u64 *d3, int n, int ell, u64 *out, cudaStream_t s);
 // c0 += 1 in place
 copse_status op_add_one(copse_ctx *c, DCt &x, cudaStream_t s);
-copse_status op_matmul_bsgs(copse_ctx *c, const copse_evk *evk, const DCt &v, const std::vector<uint32_t> &baby,
-                            const std::vector<std::vector<const u64 *>> &pt, const std::vector<int> &acc_mat,
-                            const std::vector<uint32_t> &acc_giant, int n_mat, const std::vector<const u64 *> &add,
-                            std::vector<DCt> &out, cudaStream_t s);
 
 // encode host slot patterns: n patterns of `len` values mod t, repeated every
 // `period` slots (period divides N; len <= period), into NTT-domain plaintexts

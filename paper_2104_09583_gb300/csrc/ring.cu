@@ -31,6 +31,8 @@ constexpr int MM_PER_SM = 9;          // blocks per SM that the registers are cu
 constexpr int MM_RING = 4;            // rotations that a thread has in flight or in shared memory
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
+constexpr int MM_LANES = 8;           // ciphertexts multiplied together by the same diagonals at most
+constexpr size_t MM_LANE_BYTES = 2ull << 30;  // their rotations and sums at most
 constexpr int MM_PARTS = 8;           // rotation ranges with their own partial sums at most
 constexpr int MM_BLOCKS = 2800;       // blocks that a launch is split up to (several waves)
 constexpr int RS_CHUNK = 32; // giant-step terms per k_rotsum launch
@@ -340,8 +342,9 @@ __global__ void k_moddown_conv(const u64 *u, size_t ustride, u64 *W, size_t wstr
 // ranges with their own partial sums at acc + part * part_stride (summed later).
 struct MmTable {
     const u64 *pt[MM_ACC * CHUNK_ROT];  // [acc][rotation], [ell+alpha][N], null = zero diagonal
-    const u64 *R;                       // R_k of the chunk, [rotation][2][ell+alpha][N]
-    u64 *acc;                           // [acc][2][ell+alpha][N]
+    const u64 *R;                       // R_k of the chunk, [rotation][2][ell+alpha][N], lanes R_lane apart
+    u64 *acc;                           // [acc][2][ell+alpha][N], lanes acc_lane apart
+    size_t R_lane, acc_lane;
     uint32_t dense;                     // bit x: accumulator x's diagonals are adjacent, none is zero
 };
 
@@ -399,7 +402,9 @@ __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 
 // The same sums for a tile of NA accumulators and two adjacent elements per thread over
 // precomputed R_k (adjacent in memory, [k][2][ell+alpha][N]): two residue products per diagonal
 // word.  Blocks run over the launch's accumulator tiles fastest, so that the tiles of one element
-// range find its R_k in L2.  The bound is the diagonals' stream from memory; each thread keeps
+// range find its R_k in L2; blockIdx.z is the lane (the ciphertexts that are multiplied by the same
+// diagonals; lanes fastest, so that one reads a diagonal from memory and the others find it in L2,
+// measure the same for four and cost one lane 10 %).  The bound is the diagonals' stream from memory; each thread keeps
 // MM_RING - 1 rotations of its own words arriving in its own shared memory (asynchronous copies,
 // so neither registers nor barriers) while it multiplies the one before.
 //
@@ -415,10 +420,10 @@ __global__ void __launch_bounds__(KS_TPB) k_mm_fused(const u64 *yhat, const u64 
 // a copy reaches; two 5.9 at ten.  Rings of three and four rotations measure the same.  Half of
 // the first step was instructions that split_k now avoids (117 -> 72 per rotation and warp).
 template <int NA, bool DENSE>
-__device__ __forceinline__ void mm_tile(const MmTable &tab, int nrot, int nacc, int x0, int k0, int k1, size_t n_el,
+__device__ __forceinline__ void mm_tile(const MmTable &tab, const u64 *R0, int nrot, int nacc, int x0, int k0, int k1, size_t n_el,
                                         size_t e, Pair2 (*ring)[NA + 2][MM_TPB], DotAcc (&a)[NA]) {
     const int t = threadIdx.x;
-    const u64 *R = tab.R + (size_t)k0 * 2 * n_el + e;
+    const u64 *R = R0 + (size_t)k0 * 2 * n_el + e;
     const u64 *p[NA];
 #pragma unroll
     for (int x = 0; x < NA; x++) {
@@ -499,15 +504,16 @@ __global__ void __launch_bounds__(MM_TPB, MM_PER_SM) k_mm_mac(int nrot, int nacc
     const int k0 = (int)blockIdx.y * per, k1 = min(nrot, k0 + per);
     if (k0 >= k1) return;
     __shared__ __align__(16) Pair2 ring[MM_RING][NA + 2][MM_TPB];
+    const u64 *R = tab.R + blockIdx.z * tab.R_lane;
     DotAcc a[NA];
     // every accumulator of the tile dense (bits of tab.dense)
     if (x0 + NA <= nacc && ((tab.dense >> x0) & ((1u << NA) - 1)) == (1u << NA) - 1)
-        mm_tile<NA, true>(tab, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
+        mm_tile<NA, true>(tab, R, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
     else
-        mm_tile<NA, false>(tab, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
+        mm_tile<NA, false>(tab, R, nrot, nacc, x0, k0, k1, n_el, e, ring, a);
     const int r = (int)(e >> logN);
     const PrimeDev P = pr[r < ell ? r : L + (r - ell)];
-    u64 *acc = tab.acc + (size_t)blockIdx.y * part_stride + (size_t)x0 * 2 * n_el + e;
+    u64 *acc = tab.acc + blockIdx.z * tab.acc_lane + (size_t)blockIdx.y * part_stride + (size_t)x0 * 2 * n_el + e;
 #pragma unroll
     for (int x = 0; x < NA; x++)
         if (x0 + x < nacc) {
@@ -1351,10 +1357,10 @@ static copse_status moddown_batch(copse_ctx *c, u64 *acc, int n, int ell, u64 *r
     return COPSE_OK;
 }
 
-copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const std::vector<uint32_t> &rots,
+static copse_status matmul_lanes(copse_ctx *c, const copse_evk *evk, const DCt *v, int nv, const std::vector<uint32_t> &rots,
                        const std::vector<std::vector<const u64 *>> &pt, const std::vector<const u64 *> &add,
                        std::vector<DCt> &out, cudaStream_t s, u64 *raw_out) {
-    const int ell = v.level, N = c->N, A = c->alpha, nx = ell + A, nacc = (int)pt.size(), nrot = (int)rots.size();
+    const int ell = v[0].level, N = c->N, A = c->alpha, nx = ell + A, nacc = (int)pt.size(), nrot = (int)rots.size();
     const size_t ext = (size_t)2 * nx * N, per = (size_t)2 * ell * N;
     Scratch sc(s);
     std::vector<u64> gal(nrot);
@@ -1367,40 +1373,53 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
         for (int a = 0; a < nacc; a++) used |= pt[a][r] != nullptr;
         if (used) ks_idx.push_back(r);
     }
-    // extended-basis accumulators [nacc][2][ell+alpha][N] and the Q-basis results [nacc][2][ell][N]
+    // extended-basis accumulators [nv][nacc][2][ell+alpha][N] and the Q-basis results [nv][nacc][2][ell][N]
     u64 *acc = nullptr, *res = raw_out;
-    if (!res) STATUS_TRY(sc.get(c, &res, (size_t)nacc * per));
+    if (!res) STATUS_TRY(sc.get(c, &res, (size_t)nv * nacc * per));
     if (ks_idx.empty()) {
-        CUDA_TRY(cudaMemsetAsync(res, 0, (size_t)nacc * per * sizeof(u64), s));
+        CUDA_TRY(cudaMemsetAsync(res, 0, (size_t)nv * nacc * per * sizeof(u64), s));
     } else {
         // rotations of a chunk are split into `parts` ranges (of at least eight) with their own
         // partial sums where the elements and accumulators alone make too few blocks
         const size_t blocks = nacc < MM_PRECOMPUTE_ACC ? ks_blocks((size_t)nx * N)
-                                                       : ((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 2) / 3);
+                                                       : ((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB * ((std::min(nacc, MM_ACC) + 2) / 3) * nv;
         const int parts = (int)std::min<size_t>({(size_t)MM_PARTS, (std::min<size_t>(ks_idx.size(), CHUNK_ROT) + 7) / 8,
                                                  (MM_BLOCKS + blocks - 1) / blocks});
-        const size_t part_stride = (size_t)nacc * ext;
+        const size_t part_stride = (size_t)nv * nacc * ext;
         u64 *part = nullptr;
-        STATUS_TRY(sc.get(c, &acc, (size_t)nacc * ext));
+        STATUS_TRY(sc.get(c, &acc, part_stride));
         if (parts > 1)
             STATUS_TRY(sc.get(c, &part, (size_t)parts * part_stride));
         else
             part = acc;
-        u64 *yhat = nullptr;
-        STATUS_TRY(ks_modup(c, v.data + (size_t)ell * N, ell, sc, &yhat, s));
+        u64 *yhat = nullptr;  // [nv][nd][ell+alpha][N]
         const int nd = (ell + A - 1) / A;
+        const size_t ydig = (size_t)nd * nx * N;
+        if (nv == 1) {
+            STATUS_TRY(ks_modup(c, v[0].data + (size_t)ell * N, ell, sc, &yhat, s));
+        } else {
+            u64 *c1 = nullptr;
+            STATUS_TRY(sc.get(c, &c1, (size_t)nv * ell * N));
+            for (int l = 0; l < nv; l++)
+                CUDA_TRY(cudaMemcpyAsync(c1 + (size_t)l * ell * N, v[l].data + (size_t)ell * N, (size_t)ell * N * sizeof(u64),
+                                         cudaMemcpyDeviceToDevice, s));
+            STATUS_TRY(ks_modup_batch(c, c1, (size_t)ell * N, nv, ell, sc, &yhat, s));
+        }
         // several accumulators: compute every rotation's key-switched
         // R_k = KSraw(tau_k c1) + (P tau_k c0, 0) once in one wide launch (instead of once
         // per accumulator chunk, inside the accumulation loop), then stream the products
         u64 *Rall = nullptr;
         if (nacc >= MM_PRECOMPUTE_ACC) {
-            STATUS_TRY(sc.get(c, &Rall, ks_idx.size() * ext));
-            for (size_t k0 = 0; k0 < ks_idx.size(); k0 += CHUNK_ROT) {
-                const int nj = (int)std::min<size_t>(CHUNK_ROT, ks_idx.size() - k0);
+            // the lanes of a rotation one after another: the later ones find its key in L2
+            STATUS_TRY(sc.get(c, &Rall, nv * ks_idx.size() * ext));
+            const size_t jobs_all = nv * ks_idx.size();
+            for (size_t j0 = 0; j0 < jobs_all; j0 += CHUNK_ROT) {
+                const int nj = (int)std::min<size_t>(CHUNK_ROT, jobs_all - j0);
                 InnerJobs jobs;
                 for (int i = 0; i < nj; i++) {
-                    const int r = ks_idx[k0 + i];
-                    jobs.j[i] = InnerJob{evk->find(gal[r]), Rall + (k0 + i) * ext, gal[r], nullptr, nullptr, v.data};
+                    const size_t k = (j0 + i) / nv, l = (j0 + i) % nv;
+                    const u64 g = gal[ks_idx[k]];
+                    jobs.j[i] = InnerJob{evk->find(g), Rall + (l * ks_idx.size() + k) * ext, g, yhat + l * ydig, nullptr, v[l].data};
                 }
                 TIMED_OPS("ks_inner", 8.0 * N * nj * (2.0 * nd * nx + 2.0 * nx + ell), 2.0 * N * (double)nj * nd * nx, s,
                           ks_inner_launch(c, yhat, jobs, nj, ell, s));
@@ -1418,6 +1437,8 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                 tab.acc = ftab.acc = part + (size_t)a0 * ext;
                 tab.R = Rall ? Rall + k0 * ext : nullptr;
                 tab.dense = 0;
+                tab.R_lane = ks_idx.size() * ext;
+                tab.acc_lane = (size_t)nacc * ext;
                 for (int a = 0; a < na; a++) {
                     bool dense = true;
                     for (int x = 0; x < nr; x++) {
@@ -1435,18 +1456,21 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
                 }
                 // algorithmic bytes: keys, diagonals, accumulators in and out, the rotated
                 // digits and c0 once (with R_k precomputed: R_k in place of the keys, digits and c0)
-                const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * na * nx * parts +
-                                                (Rall ? (double)nr * 2 * nx
+                const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * nv * na * nx * parts +
+                                                (Rall ? (double)nv * nr * 2 * nx
                                                       : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
                 const unsigned eb = (unsigned)(((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB);
 #define MM_MAC(K)                                                                                              \
-    launch_dep(k_mm_mac<K>, dim3(eb * (unsigned)((na + K - 1) / K), parts), MM_TPB, 0, s, nr, na, first, tab, part_stride, \
+    launch_dep(k_mm_mac<K>, dim3(eb * (unsigned)((na + K - 1) / K), parts, nv), MM_TPB, 0, s, nr, na, first, tab, part_stride, \
                                                                                ell, A, c->L, c->logN, c->d_prime)
                 if (!Rall)
-                    TIMED("mm_fused", bytes, s,
-                          KS_DISPATCH(nd, k_mm_fused, dim3(ks_blocks((size_t)nx * N), parts),
-                                      yhat, v.data, nr, first, ftab, part_stride, ell, A, c->L, c->logN, c->d_prime,
-                                      c->ks));
+                    for (int l = 0; l < nv; l++) {
+                        ftab.acc = part + ((size_t)l * nacc + a0) * ext;
+                        TIMED("mm_fused", bytes, s,
+                              KS_DISPATCH(nd, k_mm_fused, dim3(ks_blocks((size_t)nx * N), parts),
+                                          yhat + l * ydig, v[l].data, nr, first, ftab, part_stride, ell, A, c->L, c->logN,
+                                          c->d_prime, c->ks));
+                    }
                 else if (na <= 2)
                     TIMED("mm_fused", bytes, s, MM_MAC(2));
                 else
@@ -1462,33 +1486,64 @@ copse_status op_matmul(copse_ctx *c, const copse_evk *evk, const DCt &v, const s
             LAUNCH_CHECK();
         }
         // one ModDown per accumulator (both components)
-        STATUS_TRY(moddown_batch(c, acc, nacc, ell, res, s));
+        STATUS_TRY(moddown_batch(c, acc, nv * nacc, ell, res, s));
     }
-    out.assign(raw_out ? 0 : nacc, DCt());
+    out.assign(raw_out ? 0 : nv * nacc, DCt());
     // the zero-rotation terms and the addends of every accumulator in one launch, then the
     // modulus switch of all of them together
     int r0 = -1;
     for (int r = 0; r < nrot; r++)
         if (gal[r] == 1) r0 = r;
-    for (int a0 = 0; a0 < nacc; a0 += FIN_MAX) {
-        const int na = std::min(FIN_MAX, nacc - a0);
+    for (int i0 = 0; i0 < nv * ((nacc + FIN_MAX - 1) / FIN_MAX); i0++) {
+        const int l = i0 % nv, a0 = i0 / nv * FIN_MAX, na = std::min(FIN_MAX, nacc - a0);
         FinTable tab;
         memset(&tab, 0, sizeof(tab));
         bool any = false;
         for (int i = 0; i < na; i++) {
             const int a = a0 + i;
-            tab.res[i] = res + (size_t)a * per;
+            tab.res[i] = res + ((size_t)l * nacc + a) * per;
             tab.pt_mul[i] = r0 >= 0 ? pt[a][r0] : nullptr;
             tab.pt_add[i] = (!raw_out && add.size() > (size_t)a) ? add[a] : nullptr;
             any |= tab.pt_mul[i] || tab.pt_add[i];
         }
         if (!any) continue;
         TIMED("mm_finish", 8.0 * N * 5.0 * ell * na, s,
-              launch_dep(k_finish, dim3(nblk(per / 2), na), TPB, 0, s, tab, v.data, ell, c->logN, c->d_prime));
+              launch_dep(k_finish, dim3(nblk(per / 2), na), TPB, 0, s, tab, v[l].data, ell, c->logN, c->d_prime));
         LAUNCH_CHECK();
     }
     if (raw_out) return COPSE_OK;
-    return op_modswitch_many(c, res, nacc, ell, out, s);
+    return op_modswitch_many(c, res, nv * nacc, ell, out, s);
+}
+
+copse_status op_matmul_many(copse_ctx *c, const copse_evk *evk, const std::vector<DCt> &v, const std::vector<uint32_t> &rots,
+                            const std::vector<std::vector<const u64 *>> &pt, const std::vector<const u64 *> &add,
+                            std::vector<std::vector<DCt>> &out, cudaStream_t s, const MatmulGiant *giant) {
+    const int nv = (int)v.size(), nacc = (int)pt.size();
+    out.resize(nv);
+    for (int q0 = 0, n; q0 < nv; q0 += n) {
+        const int ell = v[q0].level;
+        const size_t per = (size_t)2 * ell * c->N, ext = (size_t)2 * (ell + c->alpha) * c->N;
+        // lanes of one level together while their rotations and sums fit MM_LANE_BYTES, evenly divided
+        const size_t lane_bytes = (rots.size() + nacc) * ext * sizeof(u64);
+        const int most = (int)std::max<size_t>(1, std::min<size_t>(MM_LANES, MM_LANE_BYTES / lane_bytes));
+        int same = 1;
+        while (q0 + same < nv && v[q0 + same].level == ell) same++;
+        const int groups = (same + most - 1) / most;
+        n = (same + groups - 1) / groups;
+        Scratch sc(s);
+        u64 *inner = nullptr;
+        if (giant) STATUS_TRY(sc.get(c, &inner, (size_t)n * nacc * per));
+        std::vector<DCt> o;
+        STATUS_TRY(matmul_lanes(c, evk, v.data() + q0, n, rots, pt, giant ? std::vector<const u64 *>{} : add, o, s, inner));
+        for (int l = 0; l < n; l++) {
+            if (giant)
+                STATUS_TRY(giant_phase(c, evk, inner + (size_t)l * nacc * per, ell, *giant->acc_mat, *giant->acc_giant,
+                                       giant->n_mat, add, {}, out[q0 + l], s));
+            else
+                out[q0 + l].assign(o.begin() + (size_t)l * nacc, o.begin() + (size_t)(l + 1) * nacc);
+        }
+    }
+    return COPSE_OK;
 }
 
 copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, int ell, const std::vector<int> &acc_mat,
@@ -1571,20 +1626,6 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
         LAUNCH_CHECK();
     }
     return op_modswitch_many(c, res, n_mat, ell, out, s);
-}
-
-copse_status op_matmul_bsgs(copse_ctx *c, const copse_evk *evk, const DCt &v, const std::vector<uint32_t> &baby,
-                            const std::vector<std::vector<const u64 *>> &pt, const std::vector<int> &acc_mat,
-                            const std::vector<uint32_t> &acc_giant, int n_mat, const std::vector<const u64 *> &add,
-                            std::vector<DCt> &out, cudaStream_t s) {
-    const int ell = v.level, nacc = (int)pt.size();
-    Scratch sc(s);
-    // baby steps: inner[x] = sum_j d'_{x,j} * rot(v, j), one ModDown each
-    u64 *inner = nullptr;
-    STATUS_TRY(sc.get(c, &inner, (size_t)nacc * 2 * ell * c->N));
-    std::vector<DCt> none;
-    STATUS_TRY(op_matmul(c, evk, v, baby, pt, {}, none, s, inner));
-    return giant_phase(c, evk, inner, ell, acc_mat, acc_giant, n_mat, add, {}, out, s);
 }
 
 copse_status op_rotations(copse_ctx *c, const copse_evk *evk, const DCt &v, const std::vector<uint32_t> &amounts,
