@@ -21,10 +21,10 @@
 //
 // Measured (us, forward / inverse; before = a radix-4 / radix-8 pass per two or three stages with
 // 512 / 256 threads and every twiddle staged through shared memory): N = 2^15, 1024 residue
-// polynomials 616 / 644 before, 318 / 355 with exact products, 288 / 325 with split ones (0.87 /
+// polynomials 616 / 644 before, 318 / 355 with exact products, 277 / 325 with split ones (0.91 /
 // 0.77 T butterflies/s of the 1.24 that the multiplier alone reaches: the rest is additions,
 // exchanges, and 4 TB/s of memory traffic in the column half), 128: 44 / 50 and 39 / 47; N = 2^14,
-// 1024 in clusters 269 / 313 before, 153 / 173 tiled, 147 / 162 split.
+// 1024 in clusters 269 / 313 before, 153 / 173 tiled, 138 / 161 split.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -286,9 +286,10 @@ struct TwInvRowTop {
 // the thread ends with rows 16 b .. 16 b + 15 of its column.  SH: the first 2^A pairs at T are
 // the block's copy, complete after `arrived`.
 template <int LOGN, int KL, bool SH, class IO, class ARR>
-__device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int tile, Tab3 T, u64 q,
-                                         u64 *sm, u64 (&v)[16], ARR arrived) {
+__device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int tile, Tab3 T,
+                                         const PrimeDev &P, u64 *sm, u64 (&v)[16], ARR arrived) {
     using S = Shape<LOGN>;
+    const u64 m2 = 2 * P.q;
     const int t = threadIdx.x, c = t & (S::C - 1), i = t >> S::LC;
     const size_t n0 = ((size_t)i << S::LB) + (tile << S::LC) + c, dn = (size_t)S::SA << S::LB;
 #pragma unroll
@@ -296,16 +297,31 @@ __device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int 
         u64 x[KL];
         load_n(io, p, r, g, n0 + KL * h * dn, dn, x);
 #pragma unroll
-        for (int m = 0; m < KL; m++) v[KL * h + m] = 2 * x[m];
+        for (int m = 0; m < KL; m++) v[KL * h + m] = x[m];
     }
+    if constexpr (std::is_same<IO, PlainIO>::value) {
+        // a caller's coefficients need not be residues: any 64-bit value, lowered where the bounds
+        // of split twiddles (x + 54q < 2^62) need it.  One test for the thread's sixteen, which
+        // also puts all loads before the first butterfly: 277 us for 1024 residue polynomials of
+        // 2^15 (288 without a test, 313 with one per four)
+        uint32_t any = 0;
+#pragma unroll
+        for (int m = 0; m < 16; m++) any |= (uint32_t)(v[m] >> 32);
+        if (any >> 29) {
+#pragma unroll
+            for (int m = 0; m < 16; m++) v[m] = reduce64_lazy(v[m], P);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] *= 2;
     arrived();
-    stages_fwd<4>(v, 2 * q, TwColTop<SH>{T});
+    stages_fwd<4>(v, m2, TwColTop<SH>{T});
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[((i + m * S::SA) << S::LC) + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((16 * i + m) << S::LC) + c];
-    stages_fwd<S::A - 4>(v, 2 * q, TwColLow<S::A, SH>{T, i});
+    stages_fwd<S::A - 4>(v, m2, TwColLow<S::A, SH>{T, i});
 }
 
 // Forward row half: v holds coefficients i + m SB of the thread's row (i = t mod SB); all LB row
@@ -463,7 +479,7 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_cols(const __grid_
         return;
     }
     u64 v[16];
-    fwd_cols<LOGN, 4, false>(io, t.p, t.r, t.g, t.tile, tb.tab(t.g, LOGN), tb.pr[t.g].q, sm, v, [] {});
+    fwd_cols<LOGN, 4, false>(io, t.p, t.r, t.g, t.tile, tb.tab(t.g, LOGN), tb.pr[t.g], sm, v, [] {});
     const int c = threadIdx.x & (S::C - 1), i = threadIdx.x >> S::LC;
     u64 *o = mid.base + t.p * mid.ps + ((size_t)(t.r - mid.r0) << LOGN) + ((size_t)t.tile << S::LC) + c;
 #pragma unroll
@@ -588,7 +604,7 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     dep_wait();
     const PrimeDev P = tb.pr[t.g];
     u64 v[16];
-    fwd_cols<LOGN, 16, true>(io, t.p, t.r, t.g, t.tile, Tab3{M.col, M.colq}, P.q, M.colt, v, [] {
+    fwd_cols<LOGN, 16, true>(io, t.p, t.r, t.g, t.tile, Tab3{M.col, M.colq}, P, M.colt, v, [] {
         cp_async_wait<0>();
         __syncthreads();
     });

@@ -123,3 +123,27 @@ def test_transforms_at_the_ends_of_their_lazy_ranges(log_n, bits):
                 assert_same(t.cpu().numpy().view(np.uint64)[r], out, f"product, prime {r}")
     finally:
         K.copse_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("log_n", [8, 11, 12, 14, 15])
+def test_forward_of_words_that_are_not_residues(log_n):
+    """The forward transform of x + k q is that of x, up to words of 2^64 - 2^60."""
+    L, N = 2, 1 << log_n
+    P = B.Params(logN=log_n, L=L, bits=55, dnum=2)
+    ctx = K.copse_ctx_create(log_n, 55, L, 2)
+    try:
+        rng = np.random.default_rng(log_n)
+        x = np.stack([rng.integers(0, q, size=N, dtype=np.uint64) for q in P.q])
+        for most in (ALWAYS, 0):
+            K.copse_ctx_set_ntt_cluster_max(ctx, most)
+            for top in (1 << 57, 1 << 61, 1 << 62, 1 << 63, (1 << 64) - (1 << 60)):
+                y = x.copy()
+                for r, q in enumerate(P.q):
+                    y[r, ::3] += np.uint64(top // q - 1) * np.uint64(q)
+                a, b = (torch.from_numpy(z.view(np.int64)).cuda() for z in (x, y))
+                for d in (a, b):
+                    K.copse_ntt(ctx, d.data_ptr(), 1, L)
+                torch.cuda.synchronize()
+                assert_same(b.cpu().numpy().view(np.uint64), a.cpu().numpy().view(np.uint64), f"words below {top}")
+    finally:
+        K.copse_ctx_destroy(ctx)
