@@ -188,7 +188,7 @@ def ncu_traffic(family, workload, alg_bytes_per_launch, key="dram_bytes_per_unit
 
 # ---------------------------------------------------------------- CUDA arm
 # kernel families -> the measured integer rate their algorithmic operations are priced at
-PEAK_KIND = {"enc_mac": "tensor", "ks_inner": "mac", **{f: "butterfly" for f in (
+PEAK_KIND = {"enc_mac": "tensor", "enc_mac_int": "mac", "ks_inner": "mac", **{f: "butterfly" for f in (
     "ntt_fwd", "ntt_inv", "ntt_inv_copy", "ntt_fwd_ms", "ntt_fwd_md", "ntt_fwd_mu", "ntt_fwd_mdd")}}
 PEAK_UNIT = {"mac": ("G modular products/s", "exact 64-bit residue products in lazily reduced sums"),
              "butterfly": ("G butterflies/s", "lazy Shoup NTT butterflies"),
