@@ -5,9 +5,9 @@
 // A tile is 2048 coefficients (columns x all rows, or rows x all columns) and a block of 128
 // threads holds one in registers, 16 coefficients a thread: four stages in registers, one
 // exchange through shared memory, the remaining two to four stages in registers.  What bounds a
-// large batch is the integer multiplier (a butterfly is a 64-bit Shoup product), so the layout
+// large batch is the integer multiplier (a butterfly is a 64-bit modular product), so the layout
 // spends as little else as it can: an 8-stage pass has one exchange instead of one per two or
-// three stages, and no index arithmetic between the stages.  Twiddles are read as (w, w') pairs
+// three stages, and no index arithmetic between the stages.  Twiddles are read with their quotients
 // straight from global memory: those of a tile's top stages are shared by the threads of a
 // sequence, those of the low stages, one per butterfly, are stored in thread order
 // ([tile][pair][thread]), so that every load of a warp is contiguous.
