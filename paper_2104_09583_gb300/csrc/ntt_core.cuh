@@ -407,6 +407,16 @@ __device__ __forceinline__ u64 inv_result(u64 v, Shoup sc, bool digits, u64 q) {
     return x;
 }
 
+// sc w mod q as a Shoup pair: with 2^64 = one_sh q + r64, floor(sw 2^64 / q) is sw one_sh +
+// floor(sw r64 / q), the last term by its own quotient and possibly one short, so that a product
+// of a value below 2^62 stays below 2q
+__device__ __forceinline__ Shoup scaled_twiddle(Shoup sc, const Tw3 &w, const PrimeDev &P) {
+    u64 s = tw_mul(2 * sc.w, w, 2 * P.q) >> 1;  // below 4q
+    if (s >= 2 * P.q) s -= 2 * P.q;
+    if (s >= P.q) s -= P.q;
+    return Shoup{s, s * P.one_sh + __umul64hi(s, P.r64_sh)};
+}
+
 // Inverse column half: v holds rows 16 b .. 16 b + 15 of the thread's column (doubled, below 4q); all A
 // column stages, scaled and stored through io.
 template <int LOGN, bool SH, class IO>
@@ -422,10 +432,26 @@ __device__ __forceinline__ void inv_cols(const IO &io, int p, int r, int g, int 
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[((i + m * S::SA) << S::LC) + c];
-    stages_inv<4>(v, m2, 8 * m2, TwInvColTop<SH>{T});
+    const TwInvColTop<SH> top{T};
+    Shoup sw = sc;
+    if constexpr (SH) {
+        // the last stage's products are by one twiddle: it takes the scaling with it (queries of 75
+        // and 90 launches 1035 -> 1027 us and 1675 -> 1666; tiled, where the eight products saved
+        // meet the register limit, 325 us either way)
+        stages_inv<3>(v, m2, 8 * m2, top);
+        sw = scaled_twiddle(sc, top(3, 0), P);
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const u64 U = v[m], V = v[m + 8];
+            v[m] = U + V;
+            v[m + 8] = U - V + 64 * m2;
+        }
+    } else {
+        stages_inv<4>(v, m2, 8 * m2, top);
+    }
 #pragma unroll
     for (int m = 0; m < 16; m++)
-        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m] >> 1, sc, digits, P.q));
+        io.store(p, r, g, ((size_t)(i + m * S::SA) << S::LB) + (tile << S::LC) + c, inv_result(v[m] >> 1, m < 8 ? sc : sw, digits, P.q));
 }
 
 // ---------------------------------------------------------------- tiled: two launches
