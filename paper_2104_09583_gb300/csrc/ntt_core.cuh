@@ -691,7 +691,8 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
 // A block of N / 16 threads holds one residue polynomial, 16 coefficients a thread: the first
 // four stages, the next four and the remaining LOGN - 8 in registers, with an exchange through
 // shared memory between them (a stage per exchange before: 5.6 us at N = 2^10 and 9.6 us at
-// N = 2^11 for any batch that fits the GPU).
+// N = 2^11 for any batch that fits the GPU).  The inverse takes words below 2q, as the rings below
+// do: its passes of LOGN - 4 <= 7 stages start from c0 = 2q and stay below 2^8 q < 2^63.
 template <int LOGN>
 __device__ __forceinline__ void copy_pairs(ulonglong2 *dst, const ulonglong2 *src) {
 #pragma unroll
@@ -778,14 +779,14 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
-        stages_inv<LS>(v, q, q, [&](int s, int il) { return T[(1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il]; });
+        stages_inv<LS>(v, q, 2 * q, [&](int s, int il) { return T[(1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il]; });
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
         __syncthreads();
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
-    stages_inv<4>(v, q, q << LS, [&](int s, int il) { return T[(1 << (7 - s)) + (blk << (3 - s)) + il]; });
+    stages_inv<4>(v, q, (2 * q) << LS, [&](int s, int il) { return T[(1 << (7 - s)) + (blk << (3 - s)) + il]; });
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = reduce64_lazy(v[m], P);
     __syncthreads();
