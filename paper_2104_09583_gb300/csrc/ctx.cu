@@ -73,6 +73,7 @@ copse_status dev_alloc(copse_ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
     if (e != cudaSuccess) {
         set_error(std::string("device allocation of ") + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e));
         cudaGetLastError();
+        *p = nullptr;
         return COPSE_ENOMEM;
     }
     return COPSE_OK;

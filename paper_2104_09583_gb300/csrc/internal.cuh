@@ -431,6 +431,25 @@ struct Scratch {
     }
 };
 
+// body(first, count) for n items in evenly divided groups of at most `most`.  A group whose memory
+// the device does not have is tried again at half the size, and the groups after it too, down to
+// one item: a call on several ciphertexts runs wherever one after the other would.  The body gives
+// back what it made of a group that fails.
+template <class Body>
+copse_status in_groups(int n, int most, Body body) {
+    for (int i = 0, m; i < n; i += m) {
+        const int groups = (n - i + most - 1) / most;
+        m = (n - i + groups - 1) / groups;
+        copse_status st = body(i, m);
+        while (st == COPSE_ENOMEM && m > 1) {
+            most = m = (m + 1) / 2;
+            st = body(i, m);
+        }
+        STATUS_TRY(st);
+    }
+    return COPSE_OK;
+}
+
 // ---------------------------------------------------------------- ciphertexts
 // A ciphertext at level ell with ncomp components, each [ell][N] residues
 // (residue r modulo q_r), stored in the bit-reversed NTT (evaluation) domain.

@@ -32,7 +32,9 @@ constexpr int MM_RING = 4;            // rotations that a thread has in flight o
 constexpr int MM_PRECOMPUTE_ACC = 2;  // accumulators from which the rotations are key-switched first
 constexpr int CHUNK_ROT = 64;
 constexpr int MM_LANES = 8;           // ciphertexts multiplied together by the same diagonals at most
-constexpr size_t MM_LANE_BYTES = 2ull << 30;  // their rotations and sums at most
+// their rotations and one set of sums at most (a lane's digits, results and inner sums come on top:
+// where the device does not hold them, fewer run together)
+constexpr size_t MM_LANE_BYTES = 2ull << 30;
 constexpr int MM_PARTS = 8;           // rotation ranges with their own partial sums at most
 constexpr int MM_BLOCKS = 2800;       // blocks that a launch is split up to (several waves)
 constexpr int RS_CHUNK = 32; // giant-step terms per k_rotsum launch
@@ -1520,28 +1522,36 @@ copse_status op_matmul_many(copse_ctx *c, const copse_evk *evk, const std::vecto
                             std::vector<std::vector<DCt>> &out, cudaStream_t s, const MatmulGiant *giant) {
     const int nv = (int)v.size(), nacc = (int)pt.size();
     out.resize(nv);
-    for (int q0 = 0, n; q0 < nv; q0 += n) {
+    for (int q0 = 0, same; q0 < nv; q0 += same) {
         const int ell = v[q0].level;
         const size_t per = (size_t)2 * ell * c->N, ext = (size_t)2 * (ell + c->alpha) * c->N;
-        // lanes of one level together while their rotations and sums fit MM_LANE_BYTES, evenly divided
+        same = 1;
+        while (q0 + same < nv && v[q0 + same].level == ell) same++;
+        // lanes of one level together while their rotations and sums fit MM_LANE_BYTES
         const size_t lane_bytes = (rots.size() + nacc) * ext * sizeof(u64);
         const int most = (int)std::max<size_t>(1, std::min<size_t>(MM_LANES, MM_LANE_BYTES / lane_bytes));
-        int same = 1;
-        while (q0 + same < nv && v[q0 + same].level == ell) same++;
-        const int groups = (same + most - 1) / most;
-        n = (same + groups - 1) / groups;
-        Scratch sc(s);
-        u64 *inner = nullptr;
-        if (giant) STATUS_TRY(sc.get(c, &inner, (size_t)n * nacc * per));
-        std::vector<DCt> o;
-        STATUS_TRY(matmul_lanes(c, evk, v.data() + q0, n, rots, pt, giant ? std::vector<const u64 *>{} : add, o, s, inner));
-        for (int l = 0; l < n; l++) {
-            if (giant)
-                STATUS_TRY(giant_phase(c, evk, inner + (size_t)l * nacc * per, ell, *giant->acc_mat, *giant->acc_giant,
-                                       giant->n_mat, add, {}, out[q0 + l], s));
-            else
-                out[q0 + l].assign(o.begin() + (size_t)l * nacc, o.begin() + (size_t)(l + 1) * nacc);
-        }
+        auto lanes = [&](int q, int n) -> copse_status {
+            Scratch sc(s);
+            u64 *inner = nullptr;
+            if (giant) STATUS_TRY(sc.get(c, &inner, (size_t)n * nacc * per));
+            std::vector<DCt> o;
+            copse_status st = matmul_lanes(c, evk, v.data() + q, n, rots, pt, giant ? std::vector<const u64 *>{} : add, o, s, inner);
+            for (int l = 0; l < n && st == COPSE_OK; l++) {
+                if (giant)
+                    st = giant_phase(c, evk, inner + (size_t)l * nacc * per, ell, *giant->acc_mat, *giant->acc_giant,
+                                     giant->n_mat, add, {}, out[q + l], s);
+                else
+                    out[q + l].assign(o.begin() + (size_t)l * nacc, o.begin() + (size_t)(l + 1) * nacc);
+            }
+            if (st == COPSE_OK) return st;
+            for (DCt &x : o) ct_free(&x, s);
+            for (int l = 0; l < n; l++) {
+                for (DCt &x : out[q + l]) ct_free(&x, s);
+                out[q + l].clear();
+            }
+            return st;
+        };
+        STATUS_TRY(in_groups(same, most, [&](int i, int n) { return lanes(q0 + i, n); }));
     }
     return COPSE_OK;
 }

@@ -1,0 +1,79 @@
+"""Calls on several ciphertexts when device memory is short: what runs together needs scratch for all
+of them, and where the device has less, the call runs on smaller groups with the same results.  Each
+test holds all memory but a slack that suffices for one ciphertext after the other (measured: a half
+more than that takes) and not for all at once."""
+import numpy as np
+import pytest
+
+from paper_2104_09583_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+K = pytest.importorskip("paper_2104_09583_gb300.copse")
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+MB = 1 << 20
+
+
+class Held:
+    """All free device memory but `slack` MB, held while the block runs."""
+
+    def __init__(self, slack):
+        self.slack = slack
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        self.blocks = []
+        left, size = torch.cuda.mem_get_info()[0] - self.slack * MB, 1 << 38
+        while size >= 2 * MB:
+            if size <= left:
+                try:
+                    self.blocks.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+                    left -= size
+                    continue
+                except torch.OutOfMemoryError:
+                    pass
+            size //= 2
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        self.blocks.clear()
+        torch.cuda.empty_cache()
+
+
+def test_matrix_products_of_several_query_ciphertexts():
+    """Four query ciphertexts at N = 2^15: one after the other they take 0.6 GB beside the queries
+    and the model, together 2 GB."""
+    log_n, L, p, nf, n_ct = 15, 10, 8, 16, 4
+    ctx = K.copse_ctx_create(log_n, 55, L, 2)
+    made = []
+    try:
+        model = K.copse_compile_forest(synth.random_forest(5, 16, 6, nf, p, 3), p, nf, log_n)
+        made.append((K.copse_model_destroy, model))
+        K.copse_model_set_bsgs(model, 64, 64)
+        keys, evk = K.copse_keygen(ctx, 7, [model])
+        made += [(K.copse_keys_destroy, keys), (K.copse_evk_destroy, evk)]
+        i = K.copse_model_info_get(model)
+        qs = synth.random_queries(3, n_ct * ((1 << log_n) // (i["block"] * i["n_segments"])), nf, p)
+        # one ciphertext first: the model's plaintexts are resident from here on
+        none = K.copse_encrypt_features(ctx, keys, model, np.zeros((0, nf), np.uint32), 1)
+        made.append((K.copse_ctbuf_destroy, none))
+        made.append((K.copse_ctbuf_destroy, K.copse_infer(ctx, evk, model, none)))
+        feats = K.copse_encrypt_features(ctx, keys, model, qs, 2)
+        made.append((K.copse_ctbuf_destroy, feats))
+        assert K.copse_ctbuf_count(feats) == n_ct * p
+        with Held(900):
+            res = K.copse_infer(ctx, evk, model, feats)
+            made.append((K.copse_ctbuf_destroy, res))
+        assert np.array_equal(K.copse_decrypt_labels(ctx, keys, model, res, len(qs)), K.copse_classify_plain(model, qs))
+        again = K.copse_infer(ctx, evk, model, feats)
+        made.append((K.copse_ctbuf_destroy, again))
+        for c in range(n_ct):
+            assert np.array_equal(K.copse_ctbuf_export(ctx, res, c, 1 << log_n), K.copse_ctbuf_export(ctx, again, c, 1 << log_n))
+    finally:
+        for destroy, h in reversed(made):
+            destroy(h)
+        K.copse_ctx_destroy(ctx)
