@@ -98,15 +98,17 @@ copse_status launch_one(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStr
 
 // A batch of b with this IO: clusters up to max_cluster residue polynomials (N = 2^15 only where
 // 16-block clusters are opted in), else two launches through `data` (in place) or, when it is
-// null, through scratch.
+// null, through scratch; where the device does not hold that scratch, clusters, which need none.
 template <int LOGN, bool INV, class IO>
 copse_status launch_ring(copse_ctx *ctx, const NttBatch &b, const IO &io, u64 *data, long max_cluster, cudaStream_t s) {
-    if (ctx->ntt_clusters && (long)b.npoly * b.nr <= max_cluster && (LOGN < 15 || ctx->ntt_cluster16))
-        return launch_cluster<LOGN, INV, IO>(ctx, b, io, s);
+    const bool clusters = ctx->ntt_clusters && (LOGN < 15 || ctx->ntt_cluster16);
+    if (clusters && (long)b.npoly * b.nr <= max_cluster) return launch_cluster<LOGN, INV, IO>(ctx, b, io, s);
     if (data) return launch_tiled<LOGN, INV, IO>(ctx, b, io, Mid{data, b.stride, 0}, s);
     u64 *scratch = nullptr;
-    STATUS_TRY(dev_alloc(ctx, (void **)&scratch, ((size_t)b.npoly * b.nr << LOGN) * sizeof(u64), s));
-    const copse_status st = launch_tiled<LOGN, INV, IO>(ctx, b, io, Mid{scratch, (size_t)b.nr << LOGN, b.r0}, s);
+    copse_status st = dev_alloc(ctx, (void **)&scratch, ((size_t)b.npoly * b.nr << LOGN) * sizeof(u64), s);
+    if (st == COPSE_ENOMEM && clusters) return launch_cluster<LOGN, INV, IO>(ctx, b, io, s);
+    STATUS_TRY(st);
+    st = launch_tiled<LOGN, INV, IO>(ctx, b, io, Mid{scratch, (size_t)b.nr << LOGN, b.r0}, s);
     dev_free(scratch, s);
     return st;
 }

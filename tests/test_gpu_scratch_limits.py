@@ -44,16 +44,16 @@ class Held:
         torch.cuda.empty_cache()
 
 
-def test_matrix_products_of_several_query_ciphertexts():
-    """Four query ciphertexts at N = 2^15: one after the other they take 0.6 GB beside the queries
-    and the model, together 2 GB."""
-    log_n, L, p, nf, n_ct = 15, 10, 8, 16, 4
-    ctx = K.copse_ctx_create(log_n, 55, L, 2)
+def infer_in(slack, log_n, dnum, forest, nf, g):
+    """Inference of four full query ciphertexts with `slack` MB free beside the queries and the
+    model: its labels and ciphertexts are those of a call with all memory."""
+    L, p, n_ct = 10, 8, 4
+    ctx = K.copse_ctx_create(log_n, 55, L, dnum)
     made = []
     try:
-        model = K.copse_compile_forest(synth.random_forest(5, 16, 6, nf, p, 3), p, nf, log_n)
+        model = K.copse_compile_forest(forest, p, nf, log_n)
         made.append((K.copse_model_destroy, model))
-        K.copse_model_set_bsgs(model, 64, 64)
+        K.copse_model_set_bsgs(model, *g)
         keys, evk = K.copse_keygen(ctx, 7, [model])
         made += [(K.copse_keys_destroy, keys), (K.copse_evk_destroy, evk)]
         i = K.copse_model_info_get(model)
@@ -65,7 +65,7 @@ def test_matrix_products_of_several_query_ciphertexts():
         feats = K.copse_encrypt_features(ctx, keys, model, qs, 2)
         made.append((K.copse_ctbuf_destroy, feats))
         assert K.copse_ctbuf_count(feats) == n_ct * p
-        with Held(900):
+        with Held(slack):
             res = K.copse_infer(ctx, evk, model, feats)
             made.append((K.copse_ctbuf_destroy, res))
         assert np.array_equal(K.copse_decrypt_labels(ctx, keys, model, res, len(qs)), K.copse_classify_plain(model, qs))
@@ -77,3 +77,14 @@ def test_matrix_products_of_several_query_ciphertexts():
         for destroy, h in reversed(made):
             destroy(h)
         K.copse_ctx_destroy(ctx)
+
+
+def test_matrix_products_of_several_query_ciphertexts():
+    """N = 2^15: one after the other the four take 0.6 GB, together 2 GB."""
+    infer_in(900, 15, 2, synth.random_forest(5, 16, 6, 16, 8, 3), 16, (64, 64))
+
+
+def test_transforms_without_room_for_the_partial_transform():
+    """N = 2^14: with scratch for the tiled transforms' partial results 0.69 GB, in clusters, which
+    need none, 0.54 GB."""
+    infer_in(600, 14, 3, synth.random_forest(5, 4, 5, 8, 8, 3, complete=False), 8, (32, 32))
