@@ -1821,8 +1821,8 @@ copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d
     // as many ciphertexts at a time as keep the samples of their planes below ENC_SCRATCH
     const size_t ct_words = (size_t)p * L * N;
     const int step = (int)std::max<size_t>(1, std::min<size_t>(nct, ENC_SCRATCH / (3 * ct_words * sizeof(u64))));
-    for (int q0 = 0; q0 < nct; q0 += step) {
-        const int nc = std::min(step, nct - q0), np = nc * p, j0 = q0 * per_ct;
+    auto planes = [&](int q0, int nc) -> copse_status {
+        const int np = nc * p, j0 = q0 * per_ct;
         Scratch sc(s);
         const size_t words = (size_t)np * L * N;
         u64 *mt = nullptr, *W = nullptr;
@@ -1850,8 +1850,14 @@ copse_status encrypt_planes(copse_ctx *c, const copse_keys *k, const uint32_t *d
                                                                           c->logN, c->d_prime);
             LAUNCH_CHECK();
         }
-    }
-    return COPSE_OK;
+        return COPSE_OK;
+    };
+    return in_groups(nct, step, [&](int q0, int nc) {
+        const size_t made = out.size();
+        const copse_status st = planes(q0, nc);
+        for (; st != COPSE_OK && out.size() > made; out.pop_back()) ct_free(&out.back(), s);
+        return st;
+    });
 }
 
 // n ciphertexts (one level) to their polynomials mod t, transformed: xt [n][N]

@@ -88,3 +88,36 @@ def test_transforms_without_room_for_the_partial_transform():
     """N = 2^14: with scratch for the tiled transforms' partial results 0.69 GB, in clusters, which
     need none, 0.54 GB."""
     infer_in(600, 14, 3, synth.random_forest(5, 4, 5, 8, 8, 3, complete=False), 8, (32, 32))
+
+
+def codec(log_n, n_ct, body):
+    """body(ctx, keys, model, queries) with a small model and n_ct full query ciphertexts."""
+    L, p, nf = 10, 8, 4
+    ctx = K.copse_ctx_create(log_n, 55, L, 3)
+    made = []
+    try:
+        model = K.copse_compile_forest(synth.random_forest(5, 2, 4, nf, p, 3, complete=False), p, nf, log_n)
+        made.append((K.copse_model_destroy, model))
+        keys, evk = K.copse_keygen(ctx, 7, [model])
+        made += [(K.copse_keys_destroy, keys), (K.copse_evk_destroy, evk)]
+        i = K.copse_model_info_get(model)
+        body(ctx, keys, model, synth.random_queries(3, n_ct * ((1 << log_n) // i["block"]), nf, p), made)
+    finally:
+        for destroy, h in reversed(made):
+            destroy(h)
+        K.copse_ctx_destroy(ctx)
+
+
+def test_encryption_of_several_query_ciphertexts():
+    """Eight query ciphertexts of eight planes at N = 2^15 (0.32 GB): all samples at once 0.76 GB."""
+    def body(ctx, keys, model, qs, made):
+        with Held(550):
+            few = K.copse_encrypt_features(ctx, keys, model, qs, 2)
+            made.append((K.copse_ctbuf_destroy, few))
+        all_ = K.copse_encrypt_features(ctx, keys, model, qs, 2)
+        made.append((K.copse_ctbuf_destroy, all_))
+        assert K.copse_ctbuf_count(few) == K.copse_ctbuf_count(all_) == 64
+        for i in range(64):
+            assert np.array_equal(K.copse_ctbuf_export(ctx, few, i, 1 << 15), K.copse_ctbuf_export(ctx, all_, i, 1 << 15)), i
+
+    codec(15, 8, body)
