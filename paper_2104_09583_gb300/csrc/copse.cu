@@ -874,8 +874,10 @@ extern "C" copse_status copse_decrypt_labels(copse_ctx *c, const copse_keys *k, 
     for (size_t i = 0, n; i < used && st == COPSE_OK; i += n) {
         n = 1;
         while (i + n < used && res->cts[i + n].level == res->cts[i].level) n++;
-        const size_t j0 = std::min(nq, i * per_ct), m = std::min(nq - j0, n * per_ct);
-        st = decrypt_bits(c, k, &res->cts[i], (int)n, (int)m, seg_layout(f), bits + j0 * n_out, s);
+        st = in_groups((int)n, (int)n, [&](int g, int ng) {
+            const size_t j0 = std::min(nq, (i + g) * per_ct), m = std::min(nq - j0, ng * per_ct);
+            return decrypt_bits(c, k, &res->cts[i + g], ng, (int)m, seg_layout(f), bits + j0 * n_out, s);
+        });
     }
     if (st) {
         if (!on_device) dev_free(bits, s);

@@ -121,3 +121,27 @@ def test_encryption_of_several_query_ciphertexts():
             assert np.array_equal(K.copse_ctbuf_export(ctx, few, i, 1 << 15), K.copse_ctbuf_export(ctx, all_, i, 1 << 15)), i
 
     codec(15, 8, body)
+
+
+def test_decryption_of_several_ciphertexts():
+    """Forty ciphertexts of ten primes at N = 2^15: switched down together 0.6 GB, one after the other
+    less than what is always left.  They come from another context, whose idle memory is gone."""
+    cts = []
+
+    def encrypt(ctx, keys, model, qs, made):
+        planes = K.copse_encrypt_features(ctx, keys, model, qs, 2)
+        made.append((K.copse_ctbuf_destroy, planes))
+        cts.extend(K.copse_ctbuf_export(ctx, planes, i, 1 << 15) for i in range(K.copse_ctbuf_count(planes)))
+
+    def decrypt(ctx, keys, model, qs, made):
+        buf = K.copse_ctbuf_import(ctx, np.stack(cts))
+        made.append((K.copse_ctbuf_destroy, buf))
+        nq = 8 * len(qs)  # eight planes a query ciphertext, each read as a result
+        with Held(300):
+            few = K.copse_decrypt_labels(ctx, keys, model, buf, nq)
+        assert few.any() and (few <= 1).all()
+        assert np.array_equal(few, K.copse_decrypt_labels(ctx, keys, model, buf, nq))
+
+    codec(15, 5, encrypt)
+    assert len(cts) == 40
+    codec(15, 5, decrypt)
