@@ -191,21 +191,29 @@ def ncu_traffic(family, workload, alg_bytes_per_launch, key="dram_bytes_per_unit
 PEAK_KIND = {"enc_mac": "tensor", "enc_mac_int": "mac", "ks_inner": "mac", **{f: "butterfly" for f in (
     "ntt_fwd", "ntt_inv", "ntt_inv_copy", "ntt_fwd_ms", "ntt_fwd_md", "ntt_fwd_mu", "ntt_fwd_mdd")}}
 PEAK_UNIT = {"mac": ("G modular products/s", "exact 64-bit residue products in lazily reduced sums"),
-             "butterfly": ("G butterflies/s", "lazy Shoup NTT butterflies"),
+             "butterfly": ("G butterflies/s", "forward NTT butterflies by split twiddles"),
+             "butterfly_exact": ("G butterflies/s", "forward NTT butterflies by exact Shoup twiddles"),
              "tensor": ("G flop/s", "dense f16 tensor-core multiply-adds (2 flops each)")}
+
+
+def peak_kind(family, log_n):
+    """The measured rate a family is priced at on a ring of degree 2^log_n: transforms below
+    2^12 take exact twiddles, larger ones split ones."""
+    kind = PEAK_KIND.get(family)
+    return "butterfly_exact" if kind == "butterfly" and log_n < 12 else kind
 
 
 def int_peaks(K, local):
     """Measured rates of the arithmetic the kernels are priced at: the modular arithmetic on
     this GPU (register-only microbenchmarks, best of 5 CUDA-event timed runs: exact products
-    in lazily reduced sums, lazy Shoup butterflies, Barrett products), and the dense f16
-    tensor-core rate, the sustained bf16 figure of MEASURED_PEAKS.json (f16 and bf16 have the
+    in lazily reduced sums, the transforms' butterflies by split and by exact twiddles, Barrett
+    products), and the dense f16 tensor-core rate, the sustained bf16 figure of MEASURED_PEAKS.json (f16 and bf16 have the
     same nominal dense rate, so the ratio is 1; sustained because the kernel runs inside a
     seconds-long step)."""
     ctx = K.copse_ctx_create(10, 55, 4, 2, device=local)
     try:
         out = {}
-        for kind in ("mac", "butterfly", "barrett"):
+        for kind in ("mac", "butterfly", "barrett", "butterfly_exact"):
             ops, ms = K.copse_measure_int_peak(ctx, kind, 5)
             out[kind] = {"ops_per_s": ops, "best_ms": ms}
     finally:
@@ -216,7 +224,7 @@ def int_peaks(K, local):
     return out
 
 
-def family_roofline(fam, ops, peaks_hbm, how, ipk, workload, steps):
+def family_roofline(fam, ops, peaks_hbm, how, ipk, workload, steps, log_n):
     """Roofline of the dominant kernel family (largest summed CUDA-event time) of an
     instrumented step: HBM bytes (algorithmic) and, where the family counts its modular
     products, the integer roof from the measured rate of that arithmetic."""
@@ -227,7 +235,7 @@ def family_roofline(fam, ops, peaks_hbm, how, ipk, workload, steps):
     hbm = {"achieved": achieved, "peak": peaks_hbm, "unit": "GB/s", "frac": achieved / peaks_hbm,
            "peak_source": f"{how} hbm_gbs (copy)"}
     tr = ncu_traffic(top, workload, v["bytes"] / v["launches"])
-    kind = PEAK_KIND.get(top)
+    kind = peak_kind(top, log_n)
     if ops.get(top) and kind and ipk:
         ach = ops[top] / sec
         peak = ipk[kind]["ops_per_s"]
@@ -250,7 +258,7 @@ def family_roofline(fam, ops, peaks_hbm, how, ipk, workload, steps):
     return roof
 
 
-def family_table(fam, steps, ops=None, ipk=None, hbm=None):
+def family_table(fam, steps, log_n, ops=None, ipk=None, hbm=None):
     """Per kernel family: launches, time and share per step, HBM GB/s of its algorithmic bytes and,
     where it counts modular operations, their rate and its fraction of the measured peak."""
     tot = max(1e-9, sum(x["ms"] for x in fam.values()))
@@ -262,7 +270,7 @@ def family_table(fam, steps, ops=None, ipk=None, hbm=None):
                "gbs": v["bytes"] / (v["ms"] * 1e-3) / 1e9 if v["ms"] else 0.0}
         if hbm:
             row["hbm_frac"] = row["gbs"] / hbm
-        kind = PEAK_KIND.get(k)
+        kind = peak_kind(k, log_n)
         if ops and ops.get(k) and kind and ipk and v["ms"]:
             rate = ops[k] / (v["ms"] * 1e-3)
             row["int_rate_g"] = rate / 1e9
@@ -385,7 +393,7 @@ def run_headline(args, ws, rank, local, ipk):
         fam = {k: v for k, v in K.copse_stats_all().items() if v["launches"]}
         ops = {k: K.copse_stats_get_ops(k) for k in fam}
     peaks, how = measured_peaks()
-    roof = family_roofline(fam, ops, peaks["hbm_gbs"], how, ipk, W.name, 1) if fam else None
+    roof = family_roofline(fam, ops, peaks["hbm_gbs"], how, ipk, W.name, 1, W.log_n) if fam else None
     launches_step = int(sum(v["launches"] for v in fam.values()))
 
     # end to end through the C ABI: pinned host features in, leaf bits back to pinned host memory
@@ -422,7 +430,7 @@ def run_headline(args, ws, rank, local, ipk):
     K.copse_model_destroy(model)
     K.copse_ctx_destroy(ctx)
     value = ws * nq * args.steps / (total_ms / 1e3)
-    ktab = family_table(fam, 1, ops, ipk, peaks["hbm_gbs"])
+    ktab = family_table(fam, 1, W.log_n, ops, ipk, peaks["hbm_gbs"])
     return {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": total_ms / args.steps, "p50_ms": float(np.percentile(per, 50)),
@@ -578,8 +586,8 @@ def run_forest100(args, ws, rank, local, ipk):
     key_gb = n_rot * dnum * 2 * (W.primes + alpha) * N * 8 / 1e9
     return {"workload": W.name, "ring_degree": N, "ciphertext_primes": W.primes, "dnum": dnum, "tuning": tuning,
             "branches": info["b"], "leaves": L, "depth": info["depth"], "one_query": one, "batched": batched,
-            "plain_ops": plain, "kernels": family_table(fam, steps, ops, ipk, peaks["hbm_gbs"]),
-            "roofline": family_roofline(fam, ops, peaks["hbm_gbs"], how, ipk, W.name, steps) if fam else None,
+            "plain_ops": plain, "kernels": family_table(fam, steps, W.log_n, ops, ipk, peaks["hbm_gbs"]),
+            "roofline": family_roofline(fam, ops, peaks["hbm_gbs"], how, ipk, W.name, steps, W.log_n) if fam else None,
             "rotation_keys": n_rot,
             "key_working_set_gb": round(key_gb, 2), "l2": "working set > L2 (rotation keys %.1f GB)" % key_gb}
 

@@ -488,7 +488,8 @@ copse_status copse_tune_dnum(const copse_params *base, int device, copse_model *
  * its family (transforms: "ntt_fwd", "ntt_inv", "ntt_inv_copy" and the fused
  * forms "ntt_fwd_ms", "ntt_fwd_md", "ntt_fwd_mu", "ntt_fwd_mdd"; key switching
  * and products: "modup", "ks_inner", "mm_fused", "mm_finish", "rotsum",
- * "sum_parts", "enc_mac", "moddown_conv", "ks_finish", "ms_conv", "ms_finish";
+ * "sum_parts", "enc_mac", "enc_mac_int", "rot_layout", "moddown_conv", "ks_finish", "ms_conv",
+ * "ms_finish";
  * elementwise: "tensor", "affine", "add") and its algorithmic bytes (each
  * operand read once, each result written once).  The paper's own measurement is per-stage wall time
  * (Section 8.4); this gives the per-kernel view. */
@@ -500,7 +501,8 @@ copse_status copse_stats_reset(void);
 copse_status copse_stats_get(const char *name, uint64_t *launches, double *ms, double *bytes);
 /* Wait for the device; algorithmic modular products of family `name` (NULL or
  * "" = all families): the 64-bit residue products the launches' method needs
- * (a ciphertext tensor counts 4 per element), the unit of the integer roof. */
+ * (a ciphertext tensor counts 4 per element; "enc_mac_int", which takes three
+ * residue products per ciphertext product, 3), the unit of the integer roof. */
 copse_status copse_stats_get_ops(const char *name, double *ops);
 /* Newline-separated family names seen so far into buf[cap]. */
 copse_status copse_stats_names(char *buf, size_t cap);
@@ -538,10 +540,13 @@ copse_status copse_worklist_run(copse_ctx *ctx, const copse_ctbuf *in, const cop
  * microbenchmarks on the context's device, CUDA-event timed, best of `reps`
  * runs after one warm-up run:
  *   kind 0: exact products x*y of residues below 2^55 added to a lazily reduced
- *           sum (split 28-bit multiply-adds), the unit of the dot-product kernels;
- *   kind 1: lazy forward NTT butterflies with a constant twiddle (Shoup/Harvey);
- *   kind 2: Barrett products of two residues, fully reduced.
- * *ops_per_s: products (kind 0, 2) or butterflies (kind 1) per second over the
+ *           sum (split 28-bit, three multiply-adds), the unit of the dot-product kernels;
+ *   kind 1: forward NTT butterflies with a constant split twiddle, the unit of the
+ *           transforms of N >= 2^12;
+ *   kind 2: Barrett products of two residues, fully reduced;
+ *   kind 3: forward NTT butterflies with a constant exact twiddle (Shoup/Harvey),
+ *           the unit of the smaller transforms.
+ * *ops_per_s: products (kind 0, 2) or butterflies (kind 1, 3) per second over the
  * whole device; *best_ms (may be NULL) the best run.  Allocates a small sink
  * buffer; synchronous.  EINVAL on a bad kind or reps < 1. */
 copse_status copse_measure_int_peak(copse_ctx *ctx, int kind, int reps, double *ops_per_s, float *best_ms);

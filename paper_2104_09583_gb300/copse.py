@@ -513,12 +513,12 @@ def copse_worklist_run(ctx, inbuf, items, timeout_ms=1000, stream=None):
     return h
 
 
-INT_PEAK_KINDS = {"mac": 0, "butterfly": 1, "barrett": 2}
+INT_PEAK_KINDS = {"mac": 0, "butterfly": 1, "barrett": 2, "butterfly_exact": 3}
 
 
 def copse_measure_int_peak(ctx, kind, reps=5):
     """Measured device rate of one kind of modular arithmetic ("mac", "butterfly",
-    "barrett"): (operations per second, best run in ms)."""
+    "barrett", "butterfly_exact"): (operations per second, best run in ms)."""
     ops, ms = C.c_double(), C.c_float()
     _check(_lib.copse_measure_int_peak(ctx, INT_PEAK_KINDS[kind], reps, C.byref(ops), C.byref(ms)))
     return ops.value, ms.value

@@ -343,7 +343,7 @@ copse_status enc_matmul(copse_ctx *c, const copse_evk *evk, const EncModel &E, c
                     for (int j = 0; j < nb; j++) present += G.acc[x0 + y].diag[j] >= 0;
                 const double bytes = 8.0 * (double)n_el * ((double)present + 2.0 * nb * ng + 3.0 * nm * ng);
                 if (on_int)
-                    TIMED_OPS("enc_mac_int", bytes, 4.0 * (double)n_el * (double)present * ng, s,
+                    TIMED_OPS("enc_mac_int", bytes, 3.0 * (double)n_el * (double)present * ng, s,
                               st = enc_mac_int(c, M, Rb, ng, acc3, (size_t)nm * per3, E.seed, s));
                 else
                     TIMED_OPS("enc_mac", bytes, enc_mac_tc_flops(M, ng, c->logN), s,

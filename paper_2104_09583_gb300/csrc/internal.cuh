@@ -147,37 +147,10 @@ __device__ __forceinline__ u64 reduce_words(u64 hi, u64 lo, const PrimeDev &P) {
     return s >= P.q ? s - P.q : s;
 }
 __device__ __forceinline__ u64 reduce128(const Acc128 &a, const PrimeDev &P) { return reduce_words(a.hi, a.lo, P); }
-// Exact sums of products of operands below 2^56 (residues of primes below 2^55 and
-// sums of two of them) from 32 x 32 -> 64-bit multiply-adds: x = x1 2^28 + x0 with
-// x0, x1 < 2^28, so x y = x1 y1 2^56 + (x1 y0 + x0 y1) 2^28 + x0 y0 and every partial
-// product is below 2^56.  Three 64-bit partial sums hold 64 such products exactly
-// (lo, hi < 2^62, mid < 2^63); one reduction at the end gives the residue.
-struct Sp28 {
-    uint32_t lo, hi;
-};
-__device__ __forceinline__ Sp28 split28(u64 x) { return Sp28{(uint32_t)x & 0x0FFFFFFFu, (uint32_t)(x >> 28)}; }
-struct Acc3w {
-    u64 lo, mid, hi;
-};
-__device__ __forceinline__ void mac_sp(Acc3w &a, Sp28 x, Sp28 y) {
-    a.lo += (u64)x.lo * y.lo;
-    a.mid += (u64)x.lo * y.hi;
-    a.mid += (u64)x.hi * y.lo;
-    a.hi += (u64)x.hi * y.hi;
-}
-// lo + mid 2^28 + hi 2^56 (< 2^119) as a 128-bit value
-__device__ __forceinline__ Acc128 acc3w_value(const Acc3w &a) {
-    Acc128 v{a.lo, 0};
-    const u64 m = a.mid << 28;
-    v.lo += m;
-    v.hi += (a.mid >> 36) + (v.lo < m);
-    const u64 h = a.hi << 56;
-    v.lo += h;
-    v.hi += (a.hi >> 8) + (v.lo < h);
-    return v;
-}
-// The same sums with three multiply-adds a product (Karatsuba): x0 y0, x1 y1 and
-// (x0 + x1)(y0 + y1), the middle term by subtraction when the sums are taken as a 128-bit value.
+// Exact sums of products of operands below 2^56 (residues of primes below 2^55 and sums of two of
+// them) from 32 x 32 -> 64-bit multiply-adds, three a product (Karatsuba): x = x1 2^28 + x0, the sums
+// of x0 y0, x1 y1 and (x0 + x1)(y0 + y1), the middle term by subtraction when the sums are taken as a
+// 128-bit value; one reduction at the end gives the residue.
 // Operands below 2^55 (x0 + x1 < 1.5 2^28): 64 products at most; sums of two such operands: 16.
 struct AccK {
     u64 lo, hi, s;
