@@ -1456,11 +1456,11 @@ static copse_status matmul_lanes(copse_ctx *c, const copse_evk *evk, const DCt *
                     ftab.job[x] = MmJob{evk->find(g), g};
                     ftab.pt[x] = tab.pt[x];
                 }
-                // algorithmic bytes: keys, diagonals, accumulators in and out, the rotated
-                // digits and c0 once (with R_k precomputed: R_k in place of the keys, digits and c0)
-                const double bytes = 8.0 * N * (nz_pt * (double)nx + 4.0 * nv * na * nx * parts +
-                                                (Rall ? (double)nv * nr * 2 * nx
-                                                      : (double)nr * 2 * nd * nx + (double)nd * nx + ell));
+                // algorithmic bytes of a launch: diagonals, the sums out (and in after the first chunk) and
+                // R_k of every lane, or, one accumulator and one lane a launch, keys, rotated digits and c0
+                const double sums = (first ? 2.0 : 4.0) * na * nx * parts;
+                const double bytes = 8.0 * N * (nz_pt * (double)nx + (Rall ? nv * (sums + (double)nr * 2 * nx)
+                                                                           : sums + (double)nr * 2 * nd * nx + (double)nd * nx + ell));
                 const unsigned eb = (unsigned)(((size_t)nx * N / 2 + MM_TPB - 1) / MM_TPB);
 #define MM_MAC(K)                                                                                              \
     launch_dep(k_mm_mac<K>, dim3(eb * (unsigned)((na + K - 1) / K), parts, nv), MM_TPB, 0, s, nr, na, first, tab, part_stride, \
@@ -1608,7 +1608,7 @@ copse_status giant_phase(copse_ctx *c, const copse_evk *evk, const u64 *inner, i
                     tab.t[i] = RsTerm{yhat + (size_t)(x - x0) * nd * nx * N, inner + (size_t)x * per,
                                       evk->find(gal[x]), gal[x]};
                 }
-                const double bytes = 8.0 * N * ((double)nt * (2.0 * nd * nx + (double)nd * nx + ell) + 4.0 * nx);
+                const double bytes = 8.0 * N * ((double)nt * (2.0 * nd * nx + (double)nd * nx + ell) + (k0 == x0 ? 2.0 : 4.0) * nx);
                 TIMED("rotsum", bytes, s,
                       KS_DISPATCH(nd, k_rotsum, ks_blocks((size_t)nx * N),
                                   tab, nt, k0 == x0, acc + (size_t)a * ext, ell, A, c->L, c->logN, c->d_prime, c->ks));
