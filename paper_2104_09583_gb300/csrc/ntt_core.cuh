@@ -46,6 +46,10 @@ struct Shape {
     static constexpr int TILES = 1 << (LOGN - 11);
     static constexpr int SA = 1 << (A - 4), SB = 1 << (LB - 4);  // threads per column, per row
     static constexpr int PAIRS = LB == 8 ? 15 : (LB == 7 ? 14 : 12);  // low row twiddles of a thread
+    // What the forward stages add to a value, in units of the modulus m = 2q < 2^56 (bf_fwd): all
+    // column and the first four row stages are split, the low row stages exact or (LB = 8) split.
+    static constexpr int GROWTH = 4 * (A + 4) + (LB == 8 ? 4 : 2) * (LB - 4);
+    static_assert(GROWTH < 64, "a doubled word below 2^62 leaves 2^63");
 };
 
 __device__ __forceinline__ int ntt_prime(const NttBatch &b, int r, int L) {
@@ -87,10 +91,12 @@ __device__ __forceinline__ constexpr u64 tw_bound(const ulonglong2 &) { return 2
 __device__ __forceinline__ constexpr u64 tw_bound(const Tw3 &) { return 4; }
 
 // Forward butterfly without a correction step: the product V is below B m (B = 2 or 4), so
-// x' = U + V and y' = U - V + B m only grow by B m per stage.  From inputs below 2m, exact values
-// stay below (2 log2 N + 2) m <= 24m (N <= 2^11, m = q) and split ones (the last two to four
-// stages of which are exact) below 54m < 2^62 (m = 2q, x < 2^61) for primes below 2^55 (the
-// context's limit); the final store reduces them once.
+// x' = U + V and y' = U - V + B m only grow by B m per stage.  One-block transforms (N <= 2^11,
+// m = q, every stage exact): from inputs below 2q, values stay below (2 log2 N + 2) q <= 24q.  From
+// 2^12 on (m = 2q < 2^56 for primes below 2^55, the context's limit; Shape::GROWTH): from doubled
+// inputs below 2m, values stay below 46m, 48m, 52m and 62m at N = 2^12 .. 2^15 (halved, below 2^61);
+// from doubled words below 2^62, below 2^62 + 60m < 2^63, which is what a split product takes.  The
+// final store reduces them once.
 template <class TW>
 __device__ __forceinline__ void bf_fwd(u64 &x, u64 &y, const TW &w, u64 m) {
     const u64 U = x;
@@ -301,7 +307,7 @@ __device__ __forceinline__ void fwd_cols(const IO &io, int p, int r, int g, int 
     }
     if constexpr (std::is_same<IO, PlainIO>::value) {
         // a caller's coefficients need not be residues: any 64-bit value, lowered where the bounds
-        // of split twiddles (x + 54q < 2^62) need it.  One test for the thread's sixteen, which
+        // of split twiddles (x + 60q < 2^62) need it.  One test for the thread's sixteen, which
         // also puts all loads before the first butterfly: 277 us for 1024 residue polynomials of
         // 2^15 (288 without a test, 313 with one per four)
         uint32_t any = 0;

@@ -63,7 +63,7 @@ __device__ __forceinline__ void mdd_store(const MddFuse &f, const PrimeDev *pr, 
 }
 
 // Load / store of the transforms: coefficient n of residue r (global prime g) of batch
-// polynomial p in; value v at position k out, in [0, q), or (RAW) unreduced below 2^60.
+// polynomial p in; value v at position k out, in [0, q), or (RAW) unreduced below 62q < 2^61.
 struct PlainIO {
     static constexpr bool RAW = false;
     u64 *data;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void operand_n(const IO &io, int p, int r, size_t k0,
 // is summed exactly (digits and factors are stored split at 28 bits: three multiply-adds a
 // product, at most 64 products) and reduced once, S 2^-64 mod q (Montgomery).
 // S < m 2^(2 bits) + q < q 2^64 for m < 2^(63 - bits) terms of residues below 2^bits; the result
-// stays below 2q, which the transform takes (its values stay below (2 log2 N + 2) q).
+// stays below 2q, which the transform takes (the bounds are at bf_fwd, ntt_core.cuh).
 // The digits of the next factor are loaded while this one's are multiplied.
 // Taking the centring out of the sums (a comparison and a count per product before) and the
 // factors and digits apart beforehand, with finishes of one combined reduction: ModDown with six
@@ -286,8 +286,8 @@ __device__ __forceinline__ void load_n(const MsIO &io, int p, int r, int, size_t
     }
 }
 
-// x a + v b mod q for constants a, b (Shoup pairs), x < q and any v < 2^60, in [0, q): the two
-// quotients are subtracted together, so the sum lies below 3q
+// x a + v b mod q for constants a, b (Shoup pairs), x < q and v < 2^61, in [0, q): the two quotients
+// are subtracted together; x's part is below q + q x / 2^64, v's below q + q v / 2^64, the sum below 3q
 __device__ __forceinline__ u64 mul2_shoup(u64 x, Shoup a, u64 v, Shoup b, u64 q) {
     const u64 h = __umul64hi(x, a.wp) + __umul64hi(v, b.wp);
     u64 r = x * a.w + v * b.w - h * q;
