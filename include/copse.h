@@ -397,7 +397,10 @@ copse_status copse_ct_mul_plain(copse_ctx *ctx, const copse_ctbuf *a, size_t ia,
 /* Forward (inverse = 0) or inverse negacyclic NTT, in place, of n_polys
  * polynomials laid out [n_polys][n_res][N] in device memory, residue r taken
  * modulo ciphertext prime r (n_res <= n_primes).  Coefficient order in,
- * bit-reversed evaluation order out (and back).  Async. */
+ * bit-reversed evaluation order out (and back); results lie in [0, q_r).
+ * Input words: forward, any word below 2^64 - 2^60 stands for its residue (from
+ * N = 2^12 on any word); inverse, residues in [0, q_r) (below N = 2^12 any word
+ * below 2 q_r).  Others give wrong residues.  Async. */
 copse_status copse_ntt(copse_ctx *ctx, uint64_t *data, size_t n_polys, uint32_t n_res, int inverse, void *stream);
 
 /* Negacyclic product c = a * b in Z_q[X]/(X^N + 1), coefficient form in and

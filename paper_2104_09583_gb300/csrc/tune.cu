@@ -246,7 +246,8 @@ extern "C" copse_status copse_tune_fused(copse_ctx *c, copse_model *m, const uin
     const long before = c->ntt_fused_max;
     *best = (uint32_t)std::min<long>(before, 0xffffffffL);
     if (c->logN < 12 || c->logN > 14) {
-        // no fused transform at this ring degree: nothing to choose
+        // one form only: below 2^12 a block per transform; at 2^15 two launches (where 16-block clusters
+        // are opted in, copse_ctx_set_ntt_fused_max sets their crossover)
         for (size_t i = 0; i < n; i++) ms[i] = -1.f;
         return COPSE_OK;
     }
