@@ -19,7 +19,8 @@
 // so nothing is dead code.  How many chains a kind takes is measured, the
 // fastest of 2 to 16 (T/s): split butterflies 1.23 with two, 1.22 with four,
 // 1.12 to 1.19 with more, where registers are allocated less well; exact ones
-// 1.04 with two to eight; sums 2.15 with two, 2.52 with four, 2.71 with twelve.
+// 1.04 with two to eight; sums 2.15 with two, 2.52 with four, 2.71 with twelve
+// (another card: 1.28, 1.08 and 2.85).
 #include <algorithm>
 
 #include "ntt_core.cuh"
