@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(NTHR, FWD_BLOCKS) k_ntt_fwd_cols(const __grid_
     __shared__ u64 sm[TILE];
     const TileAt t = tile_at(b, tb.L, S::TILES);
     if (ntt_skipped(b, t.p, t.r)) {
-        io.skip(t.p, t.r, t.tile, S::TILES);
+        io.skip(t.p, t.r, t.tile, S::TILES, threadIdx.x, NTHR);
         return;
     }
     u64 v[16];
@@ -628,7 +628,7 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
     dep_trigger();
     if (ntt_skipped(b, t.p, t.r)) {  // the same for every block of the cluster
         dep_wait();
-        io.skip(t.p, t.r, t.tile, S::TILES);
+        io.skip(t.p, t.r, t.tile, S::TILES, threadIdx.x, NTHR);
         return;
     }
     cl.barrier_arrive();  // every block runs: its row tile may be written
@@ -699,53 +699,83 @@ __global__ void __cluster_dims__(Shape<LOGN>::TILES, 1, 1) __launch_bounds__(NTH
 // shared memory between them (a stage per exchange before: 5.6 us at N = 2^10 and 9.6 us at
 // N = 2^11 for any batch that fits the GPU).  The inverse takes words below 2q, as the rings below
 // do: its passes of LOGN - 4 <= 7 stages start from c0 = 2q and stay below 2^8 q < 2^63.
+// At N = 2^8 a transform is half a warp: two of them share a block, which is then one warp, each half
+// synchronised by itself.  With a block of 16 threads each, the inverse of 1024 / 2048 residue
+// polynomials took 9.9 / 13.5 us (128 threads a block and a stage per barrier: 8.3 / 12.4), now
+// 6.1 / 10.2; four and eight to a block measure the same.
+template <int LOGN>
+struct One {
+    static constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;  // SP: threads per sixteenth
+    static constexpr int PER = LOGN == 8 ? 2 : 1;                            // transforms per block
+    // the transform's place in its block, the thread's in its transform
+    static __device__ __forceinline__ int place() { return PER == 1 ? 0 : threadIdx.x / NT; }
+    static __device__ __forceinline__ int thread() { return PER == 1 ? threadIdx.x : threadIdx.x % NT; }
+    static __device__ __forceinline__ void sync() {
+        if constexpr (PER == 2) __syncwarp(0xffffu << (threadIdx.x & 16));
+        else __syncthreads();
+    }
+    // the transform of this thread; false past the last one
+    static __device__ __forceinline__ bool at(const NttBatch &b, int L, TileAt &t) {
+        const int pr = (int)blockIdx.x * PER + place();
+        t.tile = 0;
+        t.p = pr / b.nr;
+        t.r = b.r0 + pr % b.nr;
+        t.g = ntt_prime(b, t.r, L);
+        return PER == 1 || pr < b.npoly * b.nr;
+    }
+};
 template <int LOGN>
 __device__ __forceinline__ void copy_pairs(ulonglong2 *dst, const ulonglong2 *src) {
+    const int th = One<LOGN>::thread();
 #pragma unroll
-    for (int k = 0; k < 16; k++) cp_async16(dst + threadIdx.x + (k << (LOGN - 4)), src + threadIdx.x + (k << (LOGN - 4)));
+    for (int k = 0; k < 16; k++) cp_async16(dst + th + (k << (LOGN - 4)), src + th + (k << (LOGN - 4)));
     cp_async_commit();
 }
 template <int LOGN, class IO>
-__global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_constant__ NttBatch b, NttTables tb,
-                                                                 const __grid_constant__ IO io) {
-    constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;  // SP: threads per sixteenth
-    __shared__ u64 sm[(1 << LOGN) + NT];
-    __shared__ ulonglong2 T[1 << LOGN];
-    const TileAt t = tile_at(b, tb.L, 1);
+__global__ void __launch_bounds__(One<LOGN>::NT *One<LOGN>::PER)
+    k_ntt_fwd_one(const __grid_constant__ NttBatch b, NttTables tb, const __grid_constant__ IO io) {
+    using O = One<LOGN>;
+    constexpr int NT = O::NT, LS = O::LS, SP = O::SP;
+    __shared__ u64 sms[O::PER][(1 << LOGN) + NT];
+    __shared__ ulonglong2 Ts[O::PER][1 << LOGN];
+    u64 *sm = sms[O::place()];
+    ulonglong2 *T = Ts[O::place()];
+    TileAt t;
+    const bool some = O::at(b, tb.L, t);
     dep_trigger();
-    if (ntt_skipped(b, t.p, t.r)) {
+    if (!some || ntt_skipped(b, t.p, t.r)) {
         dep_wait();
-        io.skip(t.p, t.r, 0, 1);
+        if (some) io.skip(t.p, t.r, 0, 1, O::thread(), NT);
         return;
     }
     copy_pairs<LOGN>(T, tb.tw + ((size_t)t.g << LOGN));
     dep_wait();
     const PrimeDev P = tb.pr[t.g];
-    const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
+    const int th = O::thread(), i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
     u64 v[16], u[4][4];
     load_n(io, t.p, t.r, t.g, (size_t)th, NT, v);
     cp_async_wait<0>();
-    __syncthreads();
+    O::sync();
 #pragma unroll
     for (int h = 0; h < 4; h++) operand_n(io, t.p, t.r, (size_t)(th + 4 * h * NT), NT, u[h]);
     stages_fwd<4>(v, P.q, [&](int s, int il) { return T[(1 << s) + il]; });
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
-    __syncthreads();
+    O::sync();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
     stages_fwd<4>(v, P.q, [&](int s, int il) { return T[(1 << (4 + s)) + (blk << s) + il]; });
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = v[m];
-        __syncthreads();
+        O::sync();
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
         stages_fwd<LS>(v, P.q, [&](int s, int il) { return T[(1 << (8 + s)) + ((16 * th) >> (LS - s)) + il]; });
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
-    __syncthreads();
+    O::sync();
 #pragma unroll
     for (int h = 0; h < 4; h++) {
         u64 x[4];
@@ -759,14 +789,18 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_fwd_one(const __grid_co
 }
 
 template <int LOGN, class IO>
-__global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_constant__ NttBatch b, NttTables tb,
-                                                                 const __grid_constant__ IO io) {
-    constexpr int NT = 1 << (LOGN - 4), LS = LOGN - 8, SP = 1 << LS;
-    __shared__ u64 sm[(1 << LOGN) + NT];
-    __shared__ ulonglong2 T[1 << LOGN];
-    const TileAt t = tile_at(b, tb.L, 1);
+__global__ void __launch_bounds__(One<LOGN>::NT *One<LOGN>::PER)
+    k_ntt_inv_one(const __grid_constant__ NttBatch b, NttTables tb, const __grid_constant__ IO io) {
+    using O = One<LOGN>;
+    constexpr int NT = O::NT, LS = O::LS, SP = O::SP;
+    __shared__ u64 sms[O::PER][(1 << LOGN) + NT];
+    __shared__ ulonglong2 Ts[O::PER][1 << LOGN];
+    u64 *sm = sms[O::place()];
+    ulonglong2 *T = Ts[O::place()];
+    TileAt t;
+    const bool some = O::at(b, tb.L, t);
     dep_trigger();
-    if (ntt_skipped(b, t.p, t.r)) {
+    if (!some || ntt_skipped(b, t.p, t.r)) {
         dep_wait();
         return;
     }
@@ -774,28 +808,28 @@ __global__ void __launch_bounds__(1 << (LOGN - 4)) k_ntt_inv_one(const __grid_co
     dep_wait();
     const PrimeDev P = tb.pr[t.g];
     const u64 q = P.q;
-    const int th = threadIdx.x, i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
+    const int th = O::thread(), i = th & (SP - 1), blk = th >> LS, f0 = (blk << (LOGN - 4)) + i;
     u64 v[16];
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = io.load(t.p, t.r, t.g, (size_t)(th + m * NT));
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(th + m * NT)] = v[m];
     cp_async_wait<0>();
-    __syncthreads();
+    O::sync();
     if (LS > 0) {
 #pragma unroll
         for (int m = 0; m < 16; m++) v[m] = sm[pad(16 * th + m)];
         stages_inv<LS>(v, q, 2 * q, [&](int s, int il) { return T[(1 << (LOGN - 1 - s)) + ((16 * th) >> (s + 1)) + il]; });
 #pragma unroll
         for (int m = 0; m < 16; m++) sm[pad(16 * th + m)] = v[m];
-        __syncthreads();
+        O::sync();
     }
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(f0 + m * SP)];
     stages_inv<4>(v, q, (2 * q) << LS, [&](int s, int il) { return T[(1 << (7 - s)) + (blk << (3 - s)) + il]; });
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[pad(f0 + m * SP)] = reduce64_lazy(v[m], P);
-    __syncthreads();
+    O::sync();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[pad(th + m * NT)];
     stages_inv<4>(v, q, 2 * q, [&](int s, int il) { return T[(1 << (3 - s)) + il]; });

@@ -75,7 +75,7 @@ struct PlainIO {
     __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
         data[(size_t)p * stride + ((size_t)r << logN) + k] = v;
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // out-of-place transform: residue r of polynomial p from src into dst
@@ -92,7 +92,7 @@ struct CopyIO {
     __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
         dst[(size_t)p * dstride + ((size_t)r << logN) + k] = v;
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // one residue of polynomials at separate addresses in, contiguous residues out
@@ -105,7 +105,7 @@ struct GatherIO {
     __device__ __forceinline__ void store(int p, int, int, size_t k, u64 v) const {
         dst[((size_t)p << logN) + k] = v;
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // ModUp (polynomial p = item nd + digit j, residue r of the extended basis): load the
@@ -124,12 +124,13 @@ struct MuIO {
     __device__ __forceinline__ void store(int p, int r, int, size_t k, u64 v) const {
         y[(((size_t)p * (ell + alpha) + r) << logN) + k] = v;
     }
-    __device__ __forceinline__ void skip(int p, int r, int rank, int cl) const {
+    // part `rank` of `cl`, by thread t of nt
+    __device__ __forceinline__ void skip(int p, int r, int rank, int cl, int t, int nt) const {
         const int item = p / nd;
         const size_t n = (size_t)1 << logN, part = n / cl, k0 = (size_t)rank * part;
         const u64 *src = x_ntt + (size_t)item * xs + ((size_t)r << logN) + k0;
         u64 *dst = y + (((size_t)p * (ell + alpha) + r) << logN) + k0;
-        for (size_t k = threadIdx.x; k < part / 2; k += blockDim.x) ((ulonglong2 *)dst)[k] = ((const ulonglong2 *)src)[k];
+        for (size_t k = t; k < part / 2; k += nt) ((ulonglong2 *)dst)[k] = ((const ulonglong2 *)src)[k];
     }
 };
 
@@ -143,7 +144,7 @@ struct MsIO {
     __device__ __forceinline__ const u64 *operand(int p, int r) const {
         return (f.xp[0] ? f.xp[p] : f.x + (size_t)p * f.ell * ((size_t)1 << logN)) + ((size_t)r << logN);
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // ModDown: load the conversion of the alpha special residues, store the finish
@@ -156,7 +157,7 @@ struct MdIO {
     __device__ __forceinline__ const u64 *operand(int p, int r) const {
         return f.U + (size_t)p * f.ustride + ((size_t)r << logN);
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // relinearise-and-drop ModDown: load the conversion from the q_{ell-1} P basis, store the finish
@@ -169,7 +170,7 @@ struct MddIO {
     __device__ __forceinline__ const u64 *operand(int p, int r) const {
         return f.U + (size_t)p * f.ustride + ((size_t)r << logN);
     }
-    __device__ __forceinline__ void skip(int, int, int, int) const {}
+    __device__ __forceinline__ void skip(int, int, int, int, int, int) const {}
 };
 
 // ---------------------------------------------------------------- a thread's coefficients of a tile

@@ -84,13 +84,14 @@ copse_status launch_tiled(copse_ctx *ctx, const NttBatch &b, const IO &io, const
 
 template <int LOGN, bool INV, class IO>
 copse_status launch_one(copse_ctx *ctx, const NttBatch &b, const IO &io, cudaStream_t s) {
-    const unsigned grid = (unsigned)b.npoly * (unsigned)b.nr;
+    using O = One<LOGN>;
+    const unsigned grid = ((unsigned)b.npoly * (unsigned)b.nr + O::PER - 1) / O::PER;
     const double bytes = (double)b.npoly * b.nr * ctx->N * 16.0;
     TIMED_OPS(io_family<IO>(INV), bytes, butterflies(ctx, b), s, {
         if constexpr (INV)
-            launch_dep(k_ntt_inv_one<LOGN, IO>, grid, 1 << (LOGN - 4), 0, s, b, tables<true>(ctx), io);
+            launch_dep(k_ntt_inv_one<LOGN, IO>, grid, O::NT * O::PER, 0, s, b, tables<true>(ctx), io);
         else
-            launch_dep(k_ntt_fwd_one<LOGN, IO>, grid, 1 << (LOGN - 4), 0, s, b, tables<false>(ctx), io);
+            launch_dep(k_ntt_fwd_one<LOGN, IO>, grid, O::NT * O::PER, 0, s, b, tables<false>(ctx), io);
     });
     LAUNCH_CHECK();
     return COPSE_OK;
