@@ -37,7 +37,8 @@ __global__ void __launch_bounds__(512) k_ntt_fwd(NttBatch b, const PrimeDev *__r
     const int p = blockIdx.x / b.nr, r = b.r0 + blockIdx.x % b.nr;
     if (ntt_skipped(b, p, r)) return;
     const int g = ntt_prime(b, r, L);
-    const u64 q = primes[g].q;
+    const PrimeDev P = primes[g];
+    const u64 q = P.q;
     u64 *data = b.data + (size_t)p * b.stride + (size_t)r * N;
     const u64 *W = tw + (size_t)g * N, *Wp = tw_sh + (size_t)g * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) sm[i] = data[i];
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(512) k_ntt_fwd(NttBatch b, const PrimeDev *__r
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         u64 v = sm[i];
-        data[i] = fwd_reduce(v, primes[g]);
+        data[i] = fwd_reduce(v, P);
     }
 }
 
